@@ -278,7 +278,7 @@ extern "C" pm_status pm_predict(pm_ctx *c, const int64_t *F, int64_t R, int32_t 
   if (precision != PM_PREC_FP64 && precision != PM_PREC_NATIVE_FP64)
     return pm_set_error(PM_ERR_INVALID_ARG, "unknown precision");
   if (precision == PM_PREC_FP64 && (k > 40 || M > 64)) return pm_set_error(PM_ERR_INVALID_ARG, "k <= 40 and M <= 64");
-  CU(pmd::launch_predict(F, R, k, W, M, precision, T, (cudaStream_t)stream));
+  CU(pmd::launch_predict(F, R, k, W, M, precision, T, c->d_status, (cudaStream_t)stream));
   return PM_OK;
 }
 
@@ -294,7 +294,7 @@ extern "C" pm_status pm_predict_argmin(pm_ctx *c, const int64_t *F, int64_t R, i
   void *scr = nullptr;
   pm_status s = ctx_scratch(c, pmd::argmin_scratch_bytes(M, pmd::argmin_parts()), &scr);
   if (s) return s;
-  CU(pmd::launch_predict_argmin(F, R, k, W, M, precision, scr, arg, mn, (cudaStream_t)stream));
+  CU(pmd::launch_predict_argmin(F, R, k, W, M, precision, scr, arg, mn, c->d_status, (cudaStream_t)stream));
   return PM_OK;
 }
 

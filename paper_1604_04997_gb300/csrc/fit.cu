@@ -556,7 +556,7 @@ cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int 
   k_chol_solve<<<M, 32, 0, st>>>(G, rhs, k, M, cmax, x, info, ratio);
   for (int it = 0; it < steps; it++) {
     k_unscale<<<(k * M + 255) / 256, 256, 0, st>>>(x, k, M, cmax, amax, W_out);
-    if ((e = launch_predict(F, R, k, W_out, M, PM_PREC_FP64, P, st)) != cudaSuccess) return e;
+    if ((e = launch_predict(F, R, k, W_out, M, PM_PREC_FP64, P, status, st)) != cudaSuccess) return e;
     cudaMemsetAsync(rr, 0, (size_t)M * 8, st);
     cudaMemsetAsync(bb, 0, (size_t)M * 8, st);
     cudaMemsetAsync(g, 0, (size_t)M * FIT_MAXK * 8, st);
@@ -566,7 +566,7 @@ cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int 
   }
   k_unscale<<<(k * M + 255) / 256, 256, 0, st>>>(x, k, M, cmax, amax, W_out);
   // final residual for the report
-  if ((e = launch_predict(F, R, k, W_out, M, PM_PREC_FP64, P, st)) != cudaSuccess) return e;
+  if ((e = launch_predict(F, R, k, W_out, M, PM_PREC_FP64, P, status, st)) != cudaSuccess) return e;
   cudaMemsetAsync(rr, 0, (size_t)M * 8, st);
   cudaMemsetAsync(bb, 0, (size_t)M * 8, st);
   k_residual<<<sms * 4, 256, 0, st>>>(P, T, rf, R, M, objective, Q, rr, bb);

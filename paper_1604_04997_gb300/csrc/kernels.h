@@ -72,12 +72,20 @@ struct ArgPart { double t; int64_t r; };   // a partial per-model minimum: time 
 // n_part == 0 gives -1 and +inf
 cudaError_t launch_argmin_reduce(const ArgPart *part, int n_part, int M, int64_t *arg, double *mn, cudaStream_t st);
 cudaError_t launch_predict(const int64_t *F, int64_t R, int k, const double *W, int M, int precision, double *T,
-                           cudaStream_t st);
+                           int *status, cudaStream_t st);
 // argmin: per-model partial results go to scratch (n_part [M] (double, int64) pairs), then reduced.
 size_t argmin_scratch_bytes(int M, int n_part);
 int argmin_parts();
 cudaError_t launch_predict_argmin(const int64_t *F, int64_t R, int k, const double *W, int M, int precision,
-                                  void *scratch, int64_t *arg, double *mn, cudaStream_t st);
+                                  void *scratch, int64_t *arg, double *mn, int *status, cudaStream_t st);
+
+// predict_exact.cu: the same exact sums from digit products on the tensor cores, for
+// k <= 32 (exact_tc_ok); status (may be null) receives ST_TIMEOUT
+bool exact_tc_ok(int k, int M);
+cudaError_t launch_predict_exact(const int64_t *F, int64_t R, int k, const double *W, int M, double *T, int *status,
+                                 int sms, cudaStream_t st);
+cudaError_t launch_argmin_exact(const int64_t *F, int64_t R, int k, const double *W, int M, ArgPart *part, int n_part,
+                                int *status, cudaStream_t st);
 
 // top-k rows per (group, model): work units of at most TOPK_CHUNK positions of one
 // group; a group of one unit is written directly (part < 0), the partial lists of the

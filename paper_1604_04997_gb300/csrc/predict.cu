@@ -153,7 +153,7 @@ static int num_sms() {
 }
 
 cudaError_t launch_predict(const int64_t *F, int64_t R, int k, const double *W, int M, int precision, double *T,
-                           cudaStream_t st) {
+                           int *status, cudaStream_t st) {
   if (R == 0) return cudaSuccess;
   if (precision == PM_PREC_NATIVE_FP64) {
     int64_t n = R * M;
@@ -161,6 +161,7 @@ cudaError_t launch_predict(const int64_t *F, int64_t R, int k, const double *W, 
     return cudaGetLastError();
   }
   if (k > PR_MAXK || M > PR_MAXM) return cudaErrorInvalidValue;
+  if (exact_tc_ok(k, M)) return launch_predict_exact(F, R, k, W, M, T, status, num_sms(), st);
   size_t sm = sizeof(PredictSmem);
   cudaFuncSetAttribute(k_predict_ff, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   int64_t ntiles = (R + PR_ROWS - 1) / PR_ROWS;
@@ -263,7 +264,12 @@ int argmin_parts() { return num_sms() * 4; }
 size_t argmin_scratch_bytes(int M, int n_part) { return (size_t)M * n_part * sizeof(ArgPart); }
 
 static cudaError_t launch_argmin_parts(const int64_t *F, int64_t R, int k, const double *W, int M, void *scratch,
-                                       int np, int64_t *arg, double *mn, cudaStream_t st) {
+                                       int np, int64_t *arg, double *mn, int *status, cudaStream_t st) {
+  if (exact_tc_ok(k, M)) {
+    np = std::min(np, num_sms());   // one CTA per SM
+    cudaError_t e = launch_argmin_exact(F, R, k, W, M, (ArgPart *)scratch, np, status, st);
+    return e != cudaSuccess ? e : launch_argmin_reduce((const ArgPart *)scratch, np, M, arg, mn, st);
+  }
   size_t sm = sizeof(PredictSmem);
   cudaFuncSetAttribute(k_predict_argmin_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   k_predict_argmin_part<<<np, PR_WARPS * 32, sm, st>>>(F, R, k, W, M, (ArgPart *)scratch);
@@ -271,9 +277,9 @@ static cudaError_t launch_argmin_parts(const int64_t *F, int64_t R, int k, const
 }
 
 cudaError_t launch_predict_argmin(const int64_t *F, int64_t R, int k, const double *W, int M, int precision,
-                                  void *scratch, int64_t *arg, double *mn, cudaStream_t st) {
+                                  void *scratch, int64_t *arg, double *mn, int *status, cudaStream_t st) {
   if (k > PR_MAXK || M > PR_MAXM || precision != PM_PREC_FP64) return cudaErrorInvalidValue;
-  return launch_argmin_parts(F, R, k, W, M, scratch, argmin_parts(), arg, mn, st);
+  return launch_argmin_parts(F, R, k, W, M, scratch, argmin_parts(), arg, mn, status, st);
 }
 
 // ---------------------------------------------------------------- top-k rows per (group, model)
@@ -636,7 +642,7 @@ extern "C" pm_status pm_predict_argmin_static(const int64_t *d_F, int64_t R, int
   const int cap = (int)(STATIC_ARGMIN_BYTES / ((size_t)M * sizeof(ArgPart)));
   const int np = std::min(4 * sms, cap);
   if (np < 1) return pm_set_error_c(PM_ERR_INVALID_ARG, "pm_predict_argmin_static: M too large for the scratch array");
-  if (launch_argmin_parts(d_F, R, k, d_W, M, scratch, np, d_arg, d_min, (cudaStream_t)stream) != cudaSuccess)
+  if (launch_argmin_parts(d_F, R, k, d_W, M, scratch, np, d_arg, d_min, nullptr, (cudaStream_t)stream) != cudaSuccess)
     return pm_set_error_c(PM_ERR_CUDA, "pm_predict_argmin_static: kernel launch failed");
   return PM_OK;
 }
