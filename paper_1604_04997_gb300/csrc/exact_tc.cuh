@@ -13,13 +13,14 @@
 // forms it: the same sums, the same times bit for bit.
 //
 // Four diagonals d = 4 g .. 4 g + 3 make one group (one 32-bit limb of S) and lie side by
-// side in tensor memory, 4 x nb columns (nb: models rounded up to 16).  With the weight
-// digits stored one after another, and zero blocks before and after them, the digits
+// side in tensor memory, 4 x nb columns (nb: the models of one pass, 16 or 32).  With the
+// weight digits stored one after another, and zero blocks before and after them, the digits
 // 4 g - q .. 4 g - q + 3 that digit q of the counts meets are one window of the B operand:
 // one MMA (M = 128 rows, N = 4 nb, K = 16) per (group, digit q, 16 features), at most 44
-// per 128-row tile, all of a group with the same shape and accumulator.  Two groups
-// alternate between two column ranges, so the MMAs of the next groups run while a
-// group's sums are read back; a tile's operands are double-buffered likewise.
+// per 128-row tile and pass, all of a group with the same shape and accumulator.  Four
+// column ranges are used in turn, so the MMAs of a pass run while the sums of the one before
+// are read back; a tile's operands are double-buffered likewise.  More than 32 models take
+// two passes: 8 sums per thread, so that four limbs of each stay in registers.
 //
 // Digits that no count of the tile reaches are skipped (counts below 2^46 need 6 of 8).
 #pragma once
@@ -34,34 +35,46 @@
 namespace pmd {
 
 constexpr int XP_ROWS = 128;      // MMA M: rows per tile
-constexpr int XP_THREADS = 512;   // 16 warps: warp w reads TMEM lanes 32 (w % 4) .., models 16 (w / 4) ..
+constexpr int XP_WARPS = 16;      // working warps: warp w reads TMEM lanes 32 (w % 4) .., models 8 (w / 4) .. of a pass
+constexpr int XP_THREADS = 32 * XP_WARPS + 32;   // and one warp of which a thread issues the MMAs
+constexpr int XP_RING = 4;        // column ranges in TMEM
 constexpr int XP_DIG = 8;
 constexpr int XP_MAXK = 32;
 constexpr int XP_MAXM = 64;
 constexpr int XP_BLOCKS = 14;     // weight-digit blocks: three zero, eight digits, three zero
-constexpr float XP_MAGIC = 12582912.0f;        // 1.5 2^23: (P + XP_MAGIC) has P + 0x4B400000 as its bits
+// Every accumulator starts at XP_BIAS's float 1.5 2^23 = 4096 x 3072, the third of a group
+// at 2^15 more (one more MMA per group): |P| <= 3,936,256 keeps the sum inside [2^23, 2^24),
+// so the bits read back are P + XP_BIAS (+ 2^15), an integer.
 constexpr uint32_t XP_BIAS = 0x4B400000u;
-// the bias of the four limbs: XP_BIAS (1 + 256 + ... + 256^15) modulo 2^128
-constexpr uint64_t XP_BIAS_W = (uint64_t)XP_BIAS * 0x01010101u;
-constexpr uint32_t XP_B0 = (uint32_t)XP_BIAS_W;
-constexpr uint64_t XP_S1 = (XP_BIAS_W >> 32) + XP_BIAS_W;
-constexpr uint32_t XP_B1 = (uint32_t)XP_S1;
-constexpr uint64_t XP_S2 = (XP_S1 >> 32) + XP_BIAS_W;
-constexpr uint32_t XP_B2 = (uint32_t)XP_S2;
-constexpr uint32_t XP_B3 = (uint32_t)((XP_S2 >> 32) + XP_BIAS_W);
+constexpr uint32_t XP_BIAS_A = 0x3C006C00u, XP_BIAS_B = 0x6A00u, XP_BIAS_B2 = 0x78006A00u;   // f16: 4096, 1; 3072, 0; 3072, 32768
+// Gathering a limb (xp_limb) leaves the high word at its value plus XP_HI.
+constexpr uint32_t XP_HI = 0x8B41u;
 
-// sizes that depend on the problem: K-steps of 16 features and padded models
+// sizes that depend on the problem: KS K-steps of 16 features, NB models per pass (padded),
+// PASSES passes; offsets in bytes from the operands' start
+template <int KS_, int NB_, int PASSES_>
 struct XpGeom {
-  int ks, nb;
-  __host__ __device__ uint32_t a_dig() const { return (uint32_t)(XP_ROWS * 32 * ks); }   // one digit of a row tile
-  __host__ __device__ uint32_t a_buf() const { return XP_DIG * a_dig(); }
-  __host__ __device__ uint32_t b_blk() const { return (uint32_t)(nb * 32 * ks); }        // one digit of the weights
-  __host__ __device__ uint32_t sbo() const { return (uint32_t)(256 * ks); }              // between 8-row groups
-  __host__ __device__ size_t smem() const { return 2 * a_buf() + XP_BLOCKS * b_blk() + 128; }
-  __host__ __device__ uint32_t tmem_cols() const { return nb <= 16 ? 128u : nb <= 32 ? 256u : 512u; }
+  static constexpr int KS = KS_, NB = NB_, PASSES = PASSES_;
+  static constexpr uint32_t SBO = 256 * KS;                      // between 8-row groups
+  static constexpr uint32_t A_DIG = XP_ROWS * 32 * KS;           // one digit of a row tile
+  static constexpr uint32_t A_BUF = XP_DIG * A_DIG;
+  static constexpr uint32_t B_BLK = NB * 32 * KS;                // one digit of a pass's weights
+  static constexpr uint32_t B_PASS = XP_BLOCKS * B_BLK;
+  static constexpr uint32_t OFF_B = 2 * A_BUF;
+  // operands of the bias MMA, K = 16: 128 rows and 4 NB models, element 0 of each row set
+  static constexpr uint32_t OFF_BIAS_A = OFF_B + PASSES * B_PASS;
+  static constexpr uint32_t OFF_BIAS_B = OFF_BIAS_A + XP_ROWS * 32;
+  static constexpr size_t SMEM = OFF_BIAS_B + NB * 128 + 128;
+  static constexpr uint32_t RANGE = 4 * NB;                      // TMEM columns of one group
+  static constexpr uint32_t TMEM_COLS = XP_RING * RANGE;         // 256 or 512
 };
 
-__host__ __device__ inline XpGeom xp_geom(int k, int M) { return XpGeom{k <= 16 ? 1 : 2, (M + 15) & ~15}; }
+// the geometry of a problem: f(XpGeom) with k <= 16 or 32 and M <= 16, 32 or 64
+template <class Fn>
+inline cudaError_t xp_dispatch(int k, int M, Fn &&f) {
+  if (k <= 16) return M <= 16 ? f(XpGeom<1, 16, 1>{}) : M <= 32 ? f(XpGeom<1, 32, 1>{}) : f(XpGeom<1, 32, 2>{});
+  return M <= 16 ? f(XpGeom<2, 16, 1>{}) : M <= 32 ? f(XpGeom<2, 32, 1>{}) : f(XpGeom<2, 32, 2>{});
+}
 
 __device__ __forceinline__ uint32_t xp_saddr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -79,15 +92,12 @@ __device__ __forceinline__ void xp_mma(uint32_t tmem, uint64_t a, uint64_t b, ui
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
-// 16 TMEM lanes x 16 columns: thread t holds lanes t/4 and t/4 + 8, columns 8 j + 2 (t%4)
-// and + 1 (j = 0, 1) as v[4 j + {0, 1}] (lane t/4) and v[4 j + {2, 3}] (lane t/4 + 8)
-__device__ __forceinline__ void xp_ld16x16(uint32_t taddr, float (&v)[8]) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+// 16 TMEM lanes x 8 columns: thread t holds lanes t/4 and t/4 + 8, columns 2 (t%4) and + 1
+// as words {0, 1} (lane t/4) and {2, 3} (lane t/4 + 8)
+__device__ __forceinline__ void xp_ld16x8(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 8; i++) v[i] = __uint_as_float(r[i]);
 }
 
 // ---------------------------------------------------------------- digits
@@ -164,44 +174,55 @@ __device__ __forceinline__ int xp_feature(int kg, int c, int e, int ks) { return
 // ---------------------------------------------------------------- operands
 
 // Weights (fp64 [M][k], staged through `scratch`, M k doubles in shared memory) to the
-// digit blocks sB and the exponents sE.  Every thread of the CTA calls it.
-__device__ __forceinline__ void xp_load_weights(const XpGeom &g, const double *__restrict__ W, int M, int k,
+// digit blocks sB and the exponents sE, and the operands of the bias MMA.  Every thread of
+// the CTA calls it.
+template <class G>
+__device__ __forceinline__ void xp_load_weights(const double *__restrict__ W, int M, int k,
                                                 double *scratch, uint8_t *sB, int *sE) {
-  for (int i = threadIdx.x; i < M * k; i += XP_THREADS) scratch[i] = W[i];
-  for (uint32_t i = threadIdx.x; i < XP_BLOCKS * g.b_blk() / 16; i += XP_THREADS)
+  for (int i = threadIdx.x; i < M * k; i += blockDim.x) scratch[i] = W[i];
+  for (uint32_t i = threadIdx.x; i < G::PASSES * G::B_PASS / 16; i += blockDim.x)
     ((uint4 *)sB)[i] = make_uint4(0, 0, 0, 0);
+  uint8_t *bias = sB + G::PASSES * G::B_PASS;   // rows of 2 x 16 bytes, 8-row groups of 2 x 128
+  for (int i = threadIdx.x; i < 2 * (XP_ROWS + 4 * G::NB); i += blockDim.x) {
+    const int kg = (i >> 3) & 1, r = (i >> 4) * 8 + (i & 7);
+    const int n = r - XP_ROWS;   // column of the group: diagonal n / nb
+    ((uint4 *)bias)[i] = make_uint4(kg ? 0u : n < 0 ? XP_BIAS_A : n / G::NB == 2 ? XP_BIAS_B2 : XP_BIAS_B, 0, 0, 0);
+  }
   __syncthreads();
   if ((int)threadIdx.x < XP_MAXM) sE[threadIdx.x] = (int)threadIdx.x < M ? weight_exponent(scratch + threadIdx.x * k, k) : 0;
   __syncthreads();
-  const int kslots = 16 * g.ks;
-  for (int i = threadIdx.x; i < M * kslots / 2; i += XP_THREADS) {
+  const int kslots = 16 * G::KS;
+  for (int i = threadIdx.x; i < M * kslots / 2; i += blockDim.x) {
     const int m = i / (kslots / 2), p = i - m * (kslots / 2);   // slots 2 p and 2 p + 1
     const int kg = p >> 2, c = p & 3;
-    const int f = xp_feature(kg, c, 0, g.ks);
+    const int f = xp_feature(kg, c, 0, G::KS);
     const int64_t w0 = f < k ? xp_fixed_weight(scratch[m * k + f], sE[m]) : 0;
     const int64_t w1 = f + 1 < k ? xp_fixed_weight(scratch[m * k + f + 1], sE[m]) : 0;
     uint32_t d[XP_DIG];
     xp_digits(w0, w1, d);
-    uint8_t *dst = sB + (m >> 3) * g.sbo() + kg * 128 + (m & 7) * 16 + c * 4;
+    uint8_t *dst = sB + (m >> 5) * G::B_PASS + ((m & 31) >> 3) * G::SBO + kg * 128 + (m & 7) * 16 + c * 4;
 #pragma unroll
-    for (int q = 0; q < XP_DIG; q++) *(uint32_t *)(dst + (3 + q) * g.b_blk()) = d[q];
+    for (int q = 0; q < XP_DIG; q++) *(uint32_t *)(dst + (3 + q) * G::B_BLK) = d[q];
   }
 }
 
-// This thread's share of a row tile: row `xp_row` of the tile, K-group `xp_kg`, eight
+// A working thread's share of a row tile: row `xp_row` of the tile, K-group `xp_kg`, eight
 // counts.  With one K-step only the first eight warps have a share.
-__device__ __forceinline__ int xp_row(int ks) {
+template <class G>
+__device__ __forceinline__ int xp_row() {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  return ks == 2 ? warp * 8 + (lane & 7) : warp * 16 + (lane >> 4) * 8 + (lane & 7);
+  return G::KS == 2 ? warp * 8 + (lane & 7) : warp * 16 + (lane >> 4) * 8 + (lane & 7);
 }
-__device__ __forceinline__ int xp_kg(int ks) { return ((threadIdx.x & 31) >> 3) & (2 * ks - 1); }
+template <class G>
+__device__ __forceinline__ int xp_kg() { return ((threadIdx.x & 31) >> 3) & (2 * G::KS - 1); }
 
 // vec: k even and F 16-byte aligned
-__device__ __forceinline__ void xp_load_row(const int64_t *__restrict__ f, int k, int ks, bool vec, int64_t (&v)[8]) {
-  const int kg = xp_kg(ks);
+template <class G>
+__device__ __forceinline__ void xp_load_row(const int64_t *__restrict__ f, int k, bool vec, int64_t (&v)[8]) {
+  const int kg = xp_kg<G>();
 #pragma unroll
   for (int c = 0; c < 4; c++) {
-    const int j = xp_feature(kg, c, 0, ks);
+    const int j = xp_feature(kg, c, 0, G::KS);
     v[2 * c] = v[2 * c + 1] = 0;
     if (vec) {
       if (j < k) {
@@ -216,80 +237,125 @@ __device__ __forceinline__ void xp_load_row(const int64_t *__restrict__ f, int k
   }
 }
 
-// digits of this thread's eight counts into operand buffer sA; *s_nd collects the number
-// of digits the tile needs
-__device__ __forceinline__ void xp_store_digits(const XpGeom &g, const int64_t (&v)[8], uint8_t *sA, int *s_nd) {
-  if (g.ks == 1 && threadIdx.x >= XP_THREADS / 2) return;   // warp-uniform
+// digits of this thread's eight counts into operand buffer sA; s_nd[warp] receives the
+// number of digits the warp's counts need
+template <class G>
+__device__ __forceinline__ void xp_store_digits(const int64_t (&v)[8], uint8_t *sA, int *s_nd) {
+  if (G::KS == 1 && threadIdx.x >= 16 * XP_WARPS) return;   // warp-uniform; those warps' entries stay 1
   uint64_t mag = 0;
 #pragma unroll
   for (int c = 0; c < 8; c++) mag |= (uint64_t)(v[c] ^ (v[c] >> 63));
   const int nd = __reduce_max_sync(0xffffffffu, xp_ndigits(mag));
-  if ((threadIdx.x & 31) == 0) atomicMax(s_nd, nd);
-  const int row = xp_row(g.ks);
-  uint8_t *dst = sA + (row >> 3) * g.sbo() + xp_kg(g.ks) * 128 + (row & 7) * 16;
+  if ((threadIdx.x & 31) == 0) s_nd[threadIdx.x >> 5] = nd;
+  const int row = xp_row<G>();
+  uint8_t *dst = sA + (row >> 3) * G::SBO + xp_kg<G>() * 128 + (row & 7) * 16;
   uint32_t d[4][XP_DIG];
 #pragma unroll
   for (int c = 0; c < 4; c++) xp_digits(v[2 * c], v[2 * c + 1], d[c]);
 #pragma unroll
-  for (int q = 0; q < XP_DIG; q++) *(uint4 *)(dst + q * g.a_dig()) = make_uint4(d[0][q], d[1][q], d[2][q], d[3][q]);
+  for (int q = 0; q < XP_DIG; q++) *(uint4 *)(dst + q * G::A_DIG) = make_uint4(d[0][q], d[1][q], d[2][q], d[3][q]);
+}
+
+// the digits a tile needs: the largest of its warps' entries (any thread)
+__device__ __forceinline__ int xp_tile_digits(const int *s_nd) {
+  int n = 1;
+#pragma unroll
+  for (int w = 0; w < XP_WARPS; w += 4) {
+    const int4 x = *(const int4 *)(s_nd + w);
+    n = max(max(max(n, x.x), max(x.y, x.z)), x.w);
+  }
+  return n;
 }
 
 // groups of diagonals that have any digit product, for nd digits (a prefix of the four)
 __device__ __forceinline__ int xp_groups(int nd) { return nd >= 6 ? 4 : nd >= 2 ? 3 : 2; }
 
-// issue group gr's MMAs (one thread) into TMEM columns tmem .. and commit them to mbar
-__device__ __forceinline__ void xp_issue(const XpGeom &g, uint32_t sA, uint32_t sB, uint32_t tmem, int gr, int nd,
-                                         uint32_t mbar) {
+// Issue group gr's MMAs into TMEM columns tmem .. (one thread; s0: the operands' shared
+// address, sA: the tile's digits, sB: the pass's weight digits).  Their completion and this thread's own arrival complete
+// one phase of mbar (two arrivals): whoever waits for it sees the sums and everything this
+// thread has seen.
+template <class G>
+__device__ __forceinline__ void xp_issue(uint32_t s0, uint32_t sA, uint32_t sB, uint32_t tmem, int gr,
+                                         int nd, uint32_t mbar) {
   // kind::f16: D fp32, A and B f16, both K-major; the fourth diagonal of group 3 is empty
-  const uint32_t n = (uint32_t)((gr == 3 ? 3 : 4) * g.nb);
+  const uint32_t n = (uint32_t)((gr == 3 ? 3 : 4) * G::NB);
   const uint32_t idesc = (1u << 4) | (n >> 3) << 17 | (uint32_t)(XP_ROWS >> 4) << 24;
   const int q0 = max(0, 4 * gr - 7), q1 = min(nd - 1, 4 * gr + 3);
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-  uint32_t acc = 0;
+  xp_mma(tmem, xp_desc(s0 + G::OFF_BIAS_A, 256), xp_desc(s0 + G::OFF_BIAS_B, 256), idesc, 0);
   for (int q = q0; q <= q1; q++) {
-    const uint32_t a = sA + q * g.a_dig(), b = sB + (uint32_t)(3 + 4 * gr - q) * g.b_blk();
-    for (int kc = 0; kc < g.ks; kc++) {
-      xp_mma(tmem, xp_desc(a + kc * 256, g.sbo()), xp_desc(b + kc * 256, g.sbo()), idesc, acc);
-      acc = 1;
-    }
+    const uint32_t a = sA + q * G::A_DIG, b = sB + (uint32_t)(3 + 4 * gr - q) * G::B_BLK;
+    for (int kc = 0; kc < G::KS; kc++) xp_mma(tmem, xp_desc(a + kc * 256, G::SBO), xp_desc(b + kc * 256, G::SBO), idesc, 1);
   }
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar));
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(mbar) : "memory");
 }
 
-// One limb of this thread's 16 sums from group gr's diagonals (live: the group was issued;
-// else its sums are zero): limb = low word of carry + sum_j 256^j (P_j + bias), cy = high word.
-__device__ __forceinline__ void xp_limb(const XpGeom &g, uint32_t tmem, int gr, bool live, uint32_t (&limb)[16],
-                                        uint32_t (&cy)[16]) {
-#pragma unroll
-  for (int s = 0; s < 2; s++) {
-    float p[4][8];
-    if (live) {
-#pragma unroll
-      for (int j = 0; j < 4; j++)
-        if (gr < 3 || j < 3) xp_ld16x16(tmem + ((uint32_t)(16 * s) << 16) + (uint32_t)(j * g.nb), p[j]);
-      asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::);
-    }
-#pragma unroll
-    for (int o = 0; o < 8; o++) {
-      uint32_t b[4];
-#pragma unroll
-      for (int j = 0; j < 4; j++)
-        b[j] = live && (gr < 3 || j < 3) ? __float_as_uint(__fadd_rn(p[j][o], XP_MAGIC)) : XP_BIAS;
-      uint64_t t = (uint64_t)(b[0] + cy[8 * s + o]);   // below 2^31 + 2^24
-      asm("mad.wide.u32 %0, %1, 256, %0;" : "+l"(t) : "r"(b[1]));
-      asm("mad.wide.u32 %0, %1, 65536, %0;" : "+l"(t) : "r"(b[2]));
-      asm("mad.wide.u32 %0, %1, 16777216, %0;" : "+l"(t) : "r"(b[3]));
-      limb[8 * s + o] = (uint32_t)t;
-      cy[8 * s + o] = (uint32_t)(t >> 32);
+// One poll of mbar's phase that lets the hardware suspend the warp for a few microseconds,
+// so that waiting warps leave the issue slots to the others.
+__device__ __forceinline__ bool xp_try(uint32_t mbar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 4000;\nselp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(done)
+      : "r"(mbar), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+
+// Wait for one phase of mbar: false if it took longer than MBAR_WAIT_NS, or if another
+// thread has given up (*s_abort).
+__device__ __forceinline__ bool xp_wait_one(uint32_t mbar, uint32_t parity, volatile int *s_abort) {
+  bool ok = xp_try(mbar, parity);
+  if (!ok) {
+    const unsigned long long t0 = globaltimer_ns();
+    while (!ok && !*s_abort) {
+      ok = xp_try(mbar, parity);
+      if (!ok && globaltimer_ns() - t0 > MBAR_WAIT_NS) *s_abort = 1;
     }
   }
+  asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
+  return ok;
 }
 
-// Remove the bias from four limbs: the exact sum S, two's complement.
-__device__ __forceinline__ void xp_unbias(uint32_t &a, uint32_t &b, uint32_t &c, uint32_t &d) {
-  asm("sub.cc.u32 %0, %0, %4;\n\tsubc.cc.u32 %1, %1, %5;\n\tsubc.cc.u32 %2, %2, %6;\n\tsubc.u32 %3, %3, %7;\n\t"
-      : "+r"(a), "+r"(b), "+r"(c), "+r"(d)
-      : "n"(XP_B0), "n"(XP_B1), "n"(XP_B2), "n"(XP_B3));
+// the same for a whole warp, with the same result in all lanes
+__device__ __forceinline__ bool xp_wait(uint32_t mbar, uint32_t parity, volatile int *s_abort) {
+  return __all_sync(0xffffffffu, xp_wait_one(mbar, parity, s_abort));
+}
+
+__device__ __forceinline__ void xp_arrive(uint32_t mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(mbar) : "memory");
+}
+
+// One limb of this thread's 8 sums from group GR's diagonals:
+//   limb + 2^32 (cy' - XP_HI) = (cy - XP_HI) + P_0 + 256 P_1 + 256^2 P_2 + 256^3 P_3
+// (cy: the high word of the group before, none for group 0).  Sum 2 i + e: row 8 i of the
+// thread's four, model e of its two.
+// The pairs u = P_0 + 256 P_1 + carry and v = P_2 + 256 P_3 fit in 32 signed bits; as
+// unsigned words u + 2^31 and v + 0x8B408000 (the biases of b_2 + 256 b_3) they add up to
+// the limb's 64 bits plus 2^31 + 2^16 0x8B408000 = 2^32 XP_HI, which leaves the low word as
+// it is.  m256 is 256 as a kernel argument: a literal would become a shift and add on the
+// integer ALU, this kernel's busiest pipe.  (A 32 x 32 + 64-bit multiply-add is four
+// instructions on this GPU.)
+template <class G, int GR>
+__device__ __forceinline__ void xp_limb(uint32_t m256, uint32_t tmem, uint32_t (&limb)[8],
+                                        uint32_t (&cy)[8]) {
+  constexpr uint32_t K = 0x80000000u - XP_BIAS * 257u - (GR == 0 ? 0u : XP_HI);
+  uint32_t p[4][2][4];
+#pragma unroll
+  for (int s = 0; s < 2; s++)
+#pragma unroll
+    for (int j = 0; j < (GR == 3 ? 3 : 4); j++) xp_ld16x8(tmem + ((uint32_t)(16 * s) << 16) + (uint32_t)(j * G::NB), p[j][s]);
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::);
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    const int s = i >> 2, e = i & 3;
+    const uint32_t u = p[1][s][e] * m256 + (p[0][s][e] + (GR == 0 ? K : cy[i] + K));
+    const uint32_t v = GR == 3 ? p[2][s][e] : p[3][s][e] * m256 + p[2][s][e];
+    const uint64_t t = (uint64_t)u + ((uint64_t)v << 16);
+    limb[i] = (uint32_t)t;
+    cy[i] = (uint32_t)(t >> 32);
+  }
 }
 
 __device__ __noinline__ double xp_value_rare(uint32_t a, uint32_t b, uint32_t c, uint32_t d, int E) {
@@ -299,27 +365,38 @@ __device__ __noinline__ double xp_value_rare(uint32_t a, uint32_t b, uint32_t c,
   return key_value(acc_key(A), E);
 }
 
-// The time of an exact sum: key_value(acc_key(S), E) of eval_common.cuh (57 leading bits,
-// rounded once to FP64's 53) in one pass over the limbs.
-__device__ __forceinline__ double xp_value(uint32_t a, uint32_t b, uint32_t c, uint32_t d, int E) {
-  const uint32_t sg = (uint32_t)((int32_t)d >> 31);
-  uint32_t x0 = a ^ sg, x1 = b ^ sg, x2 = c ^ sg, x3 = d ^ sg;
-  asm("sub.cc.u32 %0, %0, %4;\n\tsubc.cc.u32 %1, %1, %4;\n\tsubc.cc.u32 %2, %2, %4;\n\tsubc.u32 %3, %3, %4;\n\t"
-      : "+r"(x0), "+r"(x1), "+r"(x2), "+r"(x3)
-      : "r"(sg));
-  // the three limbs from the leading one down
-  const bool p3 = x3 != 0, p2 = x2 != 0, p1 = x1 != 0;
-  const uint32_t h = p3 ? x3 : p2 ? x2 : p1 ? x1 : x0;
-  const uint32_t m = p3 ? x2 : p2 ? x1 : p1 ? x0 : 0;
-  const uint32_t l = p3 ? x1 : p2 ? x0 : 0;
-  const int lz = __clz((int)h);
-  const uint32_t nh = __funnelshift_l(m, h, lz), nl = __funnelshift_l(l, m, lz);   // bit 31 of nh: the leading one
-  const int x = (p3 ? 127 : p2 ? 95 : p1 ? 63 : 31) - lz - E + 1022;               // biased exponent - 1
-  if (h == 0 || x < 0 || x > 2043) return xp_value_rare(a, b, c, d, E);
-  uint64_t y = (((uint64_t)nh << 32) | nl) >> 7;   // 57 bits
-  y += 7 + ((y >> 4) & 1);                         // to nearest, ties to even, at bit 4
-  const uint64_t bits = (y >> 4) + ((uint64_t)(uint32_t)x << 52);
-  return __longlong_as_double((long long)(bits | ((uint64_t)sg << 63)));
+// The time of an exact sum S (limbs x0 .. x3, two's complement; NEG: S may be negative):
+// key_value(acc_key(S), E) of eval_common.cuh (57 leading bits, rounded once to FP64's 53)
+// in one pass over the limbs.  x: 1150 - E, the biased exponent of a leading one in bit 31
+// of x3, in [XP_XMIN, XP_XMAX], which keeps every time in FP64's normal range.  bad is set,
+// and the result is not to be used, for S = 0.
+constexpr int XP_XMIN = 130, XP_XMAX = 2044;
+template <bool NEG>
+__device__ __forceinline__ double xp_value(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, int x, bool &bad) {
+  uint32_t sg = 0;
+  if (NEG) {
+    sg = (uint32_t)((int32_t)x3 >> 31);
+    x0 ^= sg, x1 ^= sg, x2 ^= sg, x3 ^= sg;
+    asm("sub.cc.u32 %0, %0, %4;\n\tsubc.cc.u32 %1, %1, %4;\n\tsubc.cc.u32 %2, %2, %4;\n\tsubc.u32 %3, %3, %4;\n\t"
+        : "+r"(x0), "+r"(x1), "+r"(x2), "+r"(x3)
+        : "r"(sg));
+  }
+  // shift whole limbs out at the top until the leading one is in x3
+  if ((x3 | x2) == 0) { x3 = x1; x2 = x0; x1 = x0 = 0; x -= 64; }
+  if (x3 == 0) { x3 = x2; x2 = x1; x1 = x0; x -= 32; }
+  bad = bad || x3 == 0;
+  uint32_t lz;
+  asm("bfind.shiftamt.u32 %0, %1;" : "=r"(lz) : "r"(x3));
+  uint32_t nh, nl;   // the 64 bits from the leading one down
+  nh = __funnelshift_l(x2, x3, lz);
+  nl = __funnelshift_l(x1, x2, lz);
+  // drop the leading one and all below bit 7, round to nearest even at bit 11; a carry out
+  // of the fraction moves into the exponent
+  const uint32_t bit = (nl >> 11) & 1u;
+  uint64_t y = ((uint64_t)(nh & 0x7FFFFFFFu) << 32 | (nl & ~127u)) + (0x3FFu + bit);
+  const uint32_t lo = (uint32_t)(y >> 11);
+  const uint32_t hi = (uint32_t)(y >> 43) + ((uint32_t)(x - (int)lz) << 20);
+  return __hiloint2double((int)(NEG ? hi | (sg & 0x80000000u) : hi), (int)lo);
 }
 
 }  // namespace pmd

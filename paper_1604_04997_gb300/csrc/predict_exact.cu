@@ -9,6 +9,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "exact_tc.cuh"
 #include "kernels.h"
@@ -23,34 +24,40 @@ __device__ __forceinline__ int64_t xp_order(double t) {
 
 // ARG false: write T (fp64 [R][M]).  ARG true: per-model minimum over the CTA's rows
 // (smaller time, then smaller row) -> part[blockIdx.x][M].
-template <bool ARG>
+template <class G, bool ARG>
 __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *__restrict__ F, int64_t R, int k,
                                                                  const double *__restrict__ W, int M,
                                                                  double *__restrict__ T, ArgPart *__restrict__ part,
-                                                                 int *status) {
+                                                                 int *status, uint32_t m256) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((128u - (xp_saddr(smem_raw) & 127u)) & 127u);
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t full[XP_RING], empty[XP_RING], digits[2];   // sums ready / read, a tile's digits ready
+  __shared__ __align__(16) int s_nd[4][XP_WARPS];   // by tile modulo 4: a slow warp may still read an older tile's
   __shared__ uint32_t tmem_base;
-  __shared__ int s_E[XP_MAXM], s_nd[2];
-  const XpGeom g = xp_geom(k, M);
-  uint8_t *sA = smem, *sB = smem + 2 * g.a_buf();
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  __shared__ int s_E[XP_MAXM];
+  __shared__ volatile int s_abort;
+  uint8_t *sA = smem, *sB = smem + G::OFF_B;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform for the compiler: TMEM addresses stay in uniform registers
   const int quarter = warp & 3, slice = warp >> 2;
   const int64_t ntiles = (R + XP_ROWS - 1) / XP_ROWS;
   const bool vec = (k & 1) == 0 && ((uintptr_t)F & 15) == 0;
   const bool vst = (M & 1) == 0 && ((uintptr_t)T & 15) == 0;
-  const int row = xp_row(g.ks);   // this thread's row of a tile when it loads counts
+  const int row = xp_row<G>();   // this thread's row of a tile when it loads counts
 
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(xp_saddr(&mbar[0])));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(xp_saddr(&mbar[1])));
+    for (int b = 0; b < XP_RING; b++) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;\n" ::"r"(xp_saddr(&full[b])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(xp_saddr(&empty[b])), "n"(XP_WARPS));
+    }
+    for (int b = 0; b < 2; b++) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(xp_saddr(&digits[b])), "n"(XP_WARPS));
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
-    s_nd[0] = s_nd[1] = 0;
+    s_abort = 0;
   }
+  if (tid < 4 * XP_WARPS) s_nd[0][tid] = 1;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(xp_saddr(&tmem_base)),
-                 "r"(g.tmem_cols()));
+                 "r"(G::TMEM_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
   }
   int64_t v[8];
@@ -58,117 +65,160 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
     const int64_t r = tile * XP_ROWS + row;
 #pragma unroll
     for (int c = 0; c < 8; c++) v[c] = 0;
-    if (tile < ntiles && row < XP_ROWS && r < R) xp_load_row(F + r * k, k, g.ks, vec, v);
+    if (tile < ntiles && row < XP_ROWS && r < R) xp_load_row<G>(F + r * k, k, vec, v);
   };
   load(blockIdx.x);
-  xp_load_weights(g, W, M, k, (double *)sA, sB, s_E);
-  __syncthreads();   // the staged weights in sA have been read
-  xp_store_digits(g, v, sA, &s_nd[0]);
-  load((int64_t)blockIdx.x + gridDim.x);
-  xp_store_digits(g, v, sA + g.a_buf(), &s_nd[1]);
+  xp_load_weights<G>(W, M, k, (double *)sA, sB, s_E);
   asm volatile("fence.proxy.async.shared::cta;\n" ::);
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
-  __syncthreads();
+  __syncthreads();   // the staged weights in sA have been read
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-  const uint32_t tmem = tmem_base, sA32 = xp_saddr(sA), sB32 = xp_saddr(sB), half = 4u * (uint32_t)g.nb;
-  const uint32_t tread = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(slice * 16);
-  if (tid == 0 && blockIdx.x < ntiles) {
-    for (int gr = 0; gr < 2; gr++) xp_issue(g, sA32, sB32, tmem + gr * half, gr, s_nd[0], xp_saddr(&mbar[gr]));
-  }
-  const bool active = slice * 16 < g.nb;   // this warp has models
-  double bt[4];
-  int64_t br[4];
-  if (ARG) {
-#pragma unroll
-    for (int c = 0; c < 4; c++) { bt[c] = __longlong_as_double(0x7ff0000000000000ll); br[c] = INT64_MAX; }
-  }
-  uint32_t seq = 0;            // groups consumed so far: buffer seq & 1, phase parity (seq >> 1) & 1
-  int cur = 0;
-  bool aborted = false;
-  for (int64_t tile = blockIdx.x; tile < ntiles && !aborted; tile += gridDim.x, cur ^= 1) {
-    const int nd = s_nd[cur], ng = xp_groups(nd);
-    const bool more = tile + gridDim.x < ntiles;
-    const int nd_next = s_nd[cur ^ 1];
-    uint32_t limb[3][16], cy[16];
-#pragma unroll
-    for (int o = 0; o < 16; o++) cy[o] = 0;
-#pragma unroll
-    for (int gr = 0; gr < 4; gr++) {
-      const bool live = gr < ng;
-      const uint32_t buf = seq & 1;
-      if (live) {
-        if (!cta_wait_bounded(xp_saddr(&mbar[buf]), (seq >> 1) & 1)) { aborted = true; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-      }
-      if (active) {
-        uint32_t top[16];
-        xp_limb(g, tread + buf * half, gr, live, gr < 3 ? limb[gr < 3 ? gr : 0] : top, cy);
-        if (gr == 3) {
-#pragma unroll
-          for (int o = 0; o < 16; o++) cy[o] = top[o];   // the fourth limb
+  const uint32_t tmem = tmem_base, s0 = xp_saddr(smem);
+  uint32_t seq = 0;            // groups so far: columns seq % XP_RING, their (seq / XP_RING)-th use
+  uint32_t it = 0;             // tiles so far
+  bool ok = true;
+  const bool active = warp < XP_WARPS && slice * 8 < G::NB;   // this warp has models
+  double bt[2][2];
+  int64_t br[2][2];
+  if (warp == XP_WARPS) {
+    // one thread issues, ahead of the working warps as far as digits and columns allow
+    if (lane == 0) {
+      for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, it++) {
+        if (!(ok = xp_wait_one(xp_saddr(&digits[it & 1]), (it >> 1) & 1, &s_abort))) break;
+        const int nd = xp_tile_digits(s_nd[it & 3]), ng = xp_groups(nd);
+        for (int n = 0; n < G::PASSES * ng && ok; n++, seq++) {
+          const uint32_t b = seq % XP_RING;
+          const int ps = n >= ng;
+          if (seq >= XP_RING && !(ok = xp_wait_one(xp_saddr(&empty[b]), (seq / XP_RING - 1) & 1, &s_abort))) break;
+          xp_issue<G>(s0, s0 + (it & 1) * G::A_BUF, s0 + G::OFF_B + ps * G::B_PASS, tmem + b * G::RANGE, n - ps * ng, nd,
+                   xp_saddr(&full[b]));
         }
       }
-      if (live) {
-        asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
-        __syncthreads();   // this group's columns are read: the group after the next may use them
-        if (tid == 0) {
-          const int ahead = gr + 2;
-          if (ahead < ng)
-            xp_issue(g, sA32 + cur * g.a_buf(), sB32, tmem + buf * half, ahead, nd, xp_saddr(&mbar[buf]));
-          else if (more)
-            xp_issue(g, sA32 + (cur ^ 1) * g.a_buf(), sB32, tmem + buf * half, ahead - ng, nd_next,
-                     xp_saddr(&mbar[buf]));
-        }
-        seq++;
+      if (!ok) {
+        if (status) atomicOr(status, ST_TIMEOUT);
+        // let the MMAs in flight finish before TMEM is freed (bounded)
+        const unsigned long long t0 = globaltimer_ns();
+        for (uint32_t n = seq >= XP_RING ? seq - XP_RING : 0; n < seq; n++)
+          while (!xp_try(xp_saddr(&full[n % XP_RING]), (n / XP_RING) & 1) && globaltimer_ns() - t0 < MBAR_WAIT_NS) {}
       }
     }
-    if (aborted) break;
-    // every MMA of this tile is complete: its operand buffer takes the tile after the next
-    if (tid == 0) s_nd[cur] = 0;
-    load(tile + 2 * (int64_t)gridDim.x);
-    if (active) {
-      const int64_t r0 = tile * XP_ROWS + quarter * 32 + (lane >> 2);
-      const int c0 = slice * 16 + 2 * (lane & 3);
+    __syncwarp();
+  } else {
+    const int c0 = slice * 8 + 2 * (lane & 3);   // this thread's models of a pass: c0, c0 + 1
+    if (ARG) {
 #pragma unroll
-      for (int s = 0; s < 2; s++) {
+      for (int c = 0; c < 4; c++) { bt[c >> 1][c & 1] = __longlong_as_double(0x7ff0000000000000ll); br[c >> 1][c & 1] = INT64_MAX; }
+    }
+    const uint32_t tread = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(slice * 8);
+    // this warp's digits of the n-th tile are stored
+    auto stored = [&](uint32_t n) {
+      xp_store_digits<G>(v, sA + (n & 1) * G::A_BUF, s_nd[n & 3]);
+      asm volatile("fence.proxy.async.shared::cta;\n" ::);
+      __syncwarp();
+      if (lane == 0) xp_arrive(xp_saddr(&digits[n & 1]));
+    };
+    auto wait = [&]() { return xp_wait(xp_saddr(&full[seq % XP_RING]), (seq / XP_RING) & 1, &s_abort); };
+    auto done = [&]() {   // this warp has read its share of a group
+      asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
+      __syncwarp();
+      if (lane == 0) xp_arrive(xp_saddr(&empty[seq % XP_RING]));
+      seq++;
+    };
+    // the sums of one (tile, pass): four limbs, then the times
+    auto pass = [&](int ps, int64_t tile, double (&bt)[2], int64_t (&br)[2]) -> bool {
+      uint32_t limb[4][8];
+      uint32_t cy[8];
+      if (!wait()) return false;
+      const int ng = xp_groups(xp_tile_digits(s_nd[it & 3]));
+      if (active) xp_limb<G, 0>(m256, tread + (seq % XP_RING) * G::RANGE, limb[0], cy);
+      done();
+      if (!wait()) return false;
+      if (active) xp_limb<G, 1>(m256, tread + (seq % XP_RING) * G::RANGE, limb[1], cy);
+      done();
+      if (ng > 2) {
+        if (!wait()) return false;
+        if (active) xp_limb<G, 2>(m256, tread + (seq % XP_RING) * G::RANGE, limb[2], cy);
+        done();
+      } else {
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-          const int64_t r = r0 + 16 * s + 8 * h;
+        for (int o = 0; o < 8; o++) {
+          limb[2][o] = cy[o] - XP_HI;
+          cy[o] = (uint32_t)((int32_t)limb[2][o] >> 31) + XP_HI;
+        }
+      }
+      if (ng > 3) {
+        if (!wait()) return false;
+        if (active) xp_limb<G, 3>(m256, tread + (seq % XP_RING) * G::RANGE, limb[3], cy);
+        done();
+      } else {
 #pragma unroll
-          for (int j = 0; j < 2; j++) {
-            const int m = c0 + 8 * j, o = 8 * s + 4 * j + 2 * h;
-            double t[2];
+        for (int o = 0; o < 8; o++) limb[3][o] = cy[o] - XP_HI;
+      }
+      if (!active) return true;
+      const int64_t r0 = tile * XP_ROWS + quarter * 32 + (lane >> 2);   // this thread's rows: r0 + 8 i, i < 4
+      const int left = (int)min((int64_t)XP_ROWS, R - r0);               // row r0 + 8 i exists for 8 i < left
+      const int m = 32 * ps + c0;
+      double *out = ARG ? nullptr : T + r0 * M + m;
+      const int x0[2] = {1150 - s_E[m], 1150 - s_E[m + 1]};
+      const bool wide = min(x0[0], x0[1]) < XP_XMIN || max(x0[0], x0[1]) > XP_XMAX;   // times may leave the normal range
+      auto emit = [&](auto neg) {
 #pragma unroll
-            for (int e = 0; e < 2; e++) {
-              xp_unbias(limb[0][o + e], limb[1][o + e], limb[2][o + e], cy[o + e]);
-              t[e] = xp_value(limb[0][o + e], limb[1][o + e], limb[2][o + e], cy[o + e], s_E[m + e]);
-            }
+        for (int i = 0; i < 4; i++) {
+          double t[2];
+          bool bad = wide;
+#pragma unroll
+          for (int e = 0; e < 2; e++)
+            t[e] = xp_value<decltype(neg)::value>(limb[0][2 * i + e], limb[1][2 * i + e], limb[2][2 * i + e], limb[3][2 * i + e], x0[e], bad);
+          if (bad) {
+#pragma unroll
+            for (int e = 0; e < 2; e++)
+              t[e] = xp_value_rare(limb[0][2 * i + e], limb[1][2 * i + e], limb[2][2 * i + e], limb[3][2 * i + e], 1150 - x0[e]);
+          }
+          if (8 * i < left) {
             if (ARG) {
 #pragma unroll
               for (int e = 0; e < 2; e++)   // rows come in increasing order: only a smaller time improves
-                if (r < R && xp_order(t[e]) < xp_order(bt[2 * j + e])) { bt[2 * j + e] = t[e]; br[2 * j + e] = r; }
-            } else if (r < R) {
-              double *out = T + r * M + m;
-              if (vst) {
-                if (m < M) __stcs((double2 *)out, make_double2(t[0], t[1]));
-              } else {
-                if (m < M) __stcs(out, t[0]);
-                if (m + 1 < M) __stcs(out + 1, t[1]);
-              }
+                if (xp_order(t[e]) < xp_order(bt[e])) { bt[e] = t[e]; br[e] = r0 + 8 * i; }
+            } else if (vst) {
+              if (m < M) __stcs((double2 *)out, make_double2(t[0], t[1]));
+            } else {
+              if (m < M) __stcs(out, t[0]);
+              if (m + 1 < M) __stcs(out + 1, t[1]);
             }
           }
+          if (!ARG) out += 8 * M;
         }
+      };
+      uint32_t sg = 0;
+#pragma unroll
+      for (int o = 0; o < 8; o++) sg |= limb[3][o];
+      if (__any_sync(0xffffffffu, (int32_t)sg < 0)) emit(std::true_type{});
+      else emit(std::false_type{});
+      return true;
+    };
+    stored(0);
+    load((int64_t)blockIdx.x + gridDim.x);
+    stored(1);
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, it++) {
+      // the counts of the tile after the next on their way into L2
+      const int64_t next = tile + 2 * (int64_t)gridDim.x;
+      const int64_t off = (next * XP_ROWS + warp * (XP_ROWS / XP_WARPS)) * k * 8 + lane * 128;   // bytes: this warp's rows
+      if (lane * 128 < (XP_ROWS / XP_WARPS) * k * 8 && off < R * k * 8)
+        asm volatile("prefetch.global.L2 [%0];\n" ::"l"((const char *)F + off));
+      if (ARG) {   // the running minima of both passes stay in registers
+        if (!pass(0, tile, bt[0], br[0])) break;
+        if (G::PASSES > 1 && !pass(1, tile, bt[1], br[1])) break;
+      } else {
+        int ps = 0;
+#pragma unroll 1
+        for (; ps < G::PASSES; ps++)
+          if (!pass(ps, tile, bt[0], br[0])) break;
+        if (ps < G::PASSES) break;
       }
+      // every MMA of this tile is complete: its operand buffer takes the tile after the next
+      load(next);
+      stored(it + 2);
     }
-    __syncthreads();   // s_nd[cur] is cleared
-    xp_store_digits(g, v, sA + cur * g.a_buf(), &s_nd[cur]);
-    asm volatile("fence.proxy.async.shared::cta;\n" ::);
-    __syncthreads();
-  }
-  if (aborted) {
-    if (tid == 0 && status) atomicOr(status, ST_TIMEOUT);
-    // let the MMAs in flight finish before TMEM is freed (bounded)
-    cta_wait_bounded(xp_saddr(&mbar[(seq + 1) & 1]), ((seq + 1) >> 1) & 1);
   }
   if (ARG) {
     // the CTA's minimum per model over the 4 quarters x 8 row lanes, in the operand space
@@ -177,8 +227,8 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
     if (active) {
 #pragma unroll
       for (int c = 0; c < 4; c++)
-        red[(quarter * 8 + (lane >> 2)) * XP_MAXM + slice * 16 + 2 * (lane & 3) + 8 * (c >> 1) + (c & 1)] =
-            ArgPart{bt[c], br[c]};
+        red[(quarter * 8 + (lane >> 2)) * XP_MAXM + 32 * (c >> 1) + slice * 8 + 2 * (lane & 3) + (c & 1)] =
+            ArgPart{bt[c >> 1][c & 1], br[c >> 1][c & 1]};
     }
     __syncthreads();
     if (tid < M) {
@@ -194,29 +244,34 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
   __syncthreads();
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(g.tmem_cols()));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(G::TMEM_COLS));
 }
 
 bool exact_tc_ok(int k, int M) { return k >= 1 && k <= XP_MAXK && M >= 1 && M <= XP_MAXM; }
 
 cudaError_t launch_predict_exact(const int64_t *F, int64_t R, int k, const double *W, int M, double *T, int *status,
                                  int sms, cudaStream_t st) {
-  const size_t sm = xp_geom(k, M).smem();
-  cudaError_t e = cudaFuncSetAttribute(k_predict_exact<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  const int grid = (int)std::min<int64_t>(sms, (R + XP_ROWS - 1) / XP_ROWS);
-  k_predict_exact<false><<<grid, XP_THREADS, sm, st>>>(F, R, k, W, M, T, nullptr, status);
-  return cudaGetLastError();
+  return xp_dispatch(k, M, [&](auto g) {
+    using G = decltype(g);
+    cudaError_t e = cudaFuncSetAttribute(k_predict_exact<G, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+    if (e != cudaSuccess) return e;
+    const int grid = (int)std::min<int64_t>(sms, (R + XP_ROWS - 1) / XP_ROWS);
+    k_predict_exact<G, false><<<grid, XP_THREADS, G::SMEM, st>>>(F, R, k, W, M, T, nullptr, status, 256u);
+    return cudaGetLastError();
+  });
 }
 
 // per-CTA minima to part[n_part][M]; every entry is written (n_part CTAs, some without rows)
 cudaError_t launch_argmin_exact(const int64_t *F, int64_t R, int k, const double *W, int M, ArgPart *part, int n_part,
                                 int *status, cudaStream_t st) {
-  const size_t sm = std::max<size_t>(xp_geom(k, M).smem(), 32 * XP_MAXM * sizeof(ArgPart) + 128);
-  cudaError_t e = cudaFuncSetAttribute(k_predict_exact<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  k_predict_exact<true><<<n_part, XP_THREADS, sm, st>>>(F, R, k, W, M, nullptr, part, status);
-  return cudaGetLastError();
+  return xp_dispatch(k, M, [&](auto g) {
+    using G = decltype(g);
+    static_assert(G::SMEM >= 32 * XP_MAXM * sizeof(ArgPart) + 128, "the final reduction uses the operand space");
+    cudaError_t e = cudaFuncSetAttribute(k_predict_exact<G, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+    if (e != cudaSuccess) return e;
+    k_predict_exact<G, true><<<n_part, XP_THREADS, G::SMEM, st>>>(F, R, k, W, M, nullptr, part, status, 256u);
+    return cudaGetLastError();
+  });
 }
 
 }  // namespace pmd
