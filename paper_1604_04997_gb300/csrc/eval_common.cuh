@@ -248,6 +248,27 @@ __device__ __forceinline__ double key_value(int64_t k, int E) {
   return neg ? -v : v;
 }
 
+// W = round(w 2^E) to nearest even, as llrint(ldexp(w, E)), with integer operations (this
+// GPU's FP64 pipe is narrow); infinities and NaN take the FP64 path.
+__device__ __forceinline__ int64_t fixed_weight(double w, int E) {
+  const uint64_t b = (uint64_t)__double_as_longlong(w);
+  const int e = (int)((b >> 52) & 0x7FF);
+  if (e == 0x7FF) return llrint(ldexp(w, E));
+  const uint64_t mant = (b & 0xFFFFFFFFFFFFFull) | (e ? 1ull << 52 : 0ull);
+  const int s = (e ? e : 1) - 1075 + E;
+  uint64_t q;
+  if (s >= 0) {
+    q = mant << min(s, 63);
+  } else if (s > -55) {
+    const uint64_t half = 1ull << (-s - 1), rem = mant & (2 * half - 1);
+    q = mant >> -s;
+    if (rem > half || (rem == half && (q & 1))) q++;
+  } else {
+    q = 0;
+  }
+  return (b >> 63) ? -(int64_t)q : (int64_t)q;
+}
+
 // Exponent E of the fixed-point weights W_i = round(w_i 2^E): the largest with
 // sum_i |w_i| 2^E <= 2^62 (the sum is rounded up by 2^-40 relative to cover its own
 // rounding), so that sum_i |W_i| <= 2^62 + k/2.  Every kernel that ranks or converts

@@ -146,27 +146,6 @@ __device__ __forceinline__ int xp_ndigits(uint64_t mag) {   // mag: OR of v ^ (v
   return min(XP_DIG, (bits + 9) >> 3);
 }
 
-// W = round(w 2^E) to nearest even, as llrint(ldexp(w, E)), with integer operations (this
-// GPU's FP64 pipe is narrow); infinities and NaN take the FP64 path.
-__device__ __forceinline__ int64_t xp_fixed_weight(double w, int E) {
-  const uint64_t b = (uint64_t)__double_as_longlong(w);
-  const int e = (int)((b >> 52) & 0x7FF);
-  if (e == 0x7FF) return llrint(ldexp(w, E));
-  const uint64_t mant = (b & 0xFFFFFFFFFFFFFull) | (e ? 1ull << 52 : 0ull);
-  const int s = (e ? e : 1) - 1075 + E;
-  uint64_t q;
-  if (s >= 0) {
-    q = mant << min(s, 63);
-  } else if (s > -55) {
-    const uint64_t half = 1ull << (-s - 1), rem = mant & (2 * half - 1);
-    q = mant >> -s;
-    if (rem > half || (rem == half && (q & 1))) q++;
-  } else {
-    q = 0;
-  }
-  return (b >> 63) ? -(int64_t)q : (int64_t)q;
-}
-
 // feature of K slot 8 kg + 2 c + e (c: 16-byte chunk of the slot's K-group): lanes of
 // neighbouring K-groups read neighbouring 16-byte chunks of a row
 __device__ __forceinline__ int xp_feature(int kg, int c, int e, int ks) { return 2 * (2 * ks * c + kg) + e; }
@@ -196,8 +175,8 @@ __device__ __forceinline__ void xp_load_weights(const double *__restrict__ W, in
     const int m = i / (kslots / 2), p = i - m * (kslots / 2);   // slots 2 p and 2 p + 1
     const int kg = p >> 2, c = p & 3;
     const int f = xp_feature(kg, c, 0, G::KS);
-    const int64_t w0 = f < k ? xp_fixed_weight(scratch[m * k + f], sE[m]) : 0;
-    const int64_t w1 = f + 1 < k ? xp_fixed_weight(scratch[m * k + f + 1], sE[m]) : 0;
+    const int64_t w0 = f < k ? fixed_weight(scratch[m * k + f], sE[m]) : 0;
+    const int64_t w1 = f + 1 < k ? fixed_weight(scratch[m * k + f + 1], sE[m]) : 0;
     uint32_t d[XP_DIG];
     xp_digits(w0, w1, d);
     uint8_t *dst = sB + (m >> 5) * G::B_PASS + ((m & 31) >> 3) * G::SBO + kg * 128 + (m & 7) * 16 + c * 4;

@@ -32,39 +32,47 @@ cudaError_t launch_eval_counts(const uint32_t *arena, const int64_t *d_tab_off, 
 //       then [w0 w1 w2 entry] per term with a 96-bit weight (n64 terms whose basis value
 //       may leave [0, 2^32), then n32 terms), then [w0 w1 w2 w3][entry 0 0 0] per term
 //       with a 128-bit weight; the denominator block is [shift, 0, 0, 0, d^-1 mod 2^128];
-//   the walk order: variants sorted by program shape (every leaf of a program is padded
-//     to one count of 64-bit- and of 32-bit-class terms): per position its program's
-//     root record offset and its variant index in the group (16 bits each), and runs
-//     [shape = n64 | n32 << 8 (0xFFFF: 128-bit weights), first position, count, 0].
+//   the program table, in walk order (by shape: every leaf of a program is padded to one
+//     count of 64-bit- and of 32-bit-class terms): [root record offset | program id << 16],
+//     program ids in the order of their first variants;
+//   per program id its span [first entry | count << 16] in the list of variant indices (16
+//     bits each), which holds at most the first 16 variants of each program;
+//   runs of one shape [shape = n64 | n32 << 8 (0xFFFF: 128-bit weights), first position,
+//     count, first program]; H_STAGED: the words up to here, which the kernel stages;
+//   the whole walk, variant by variant (positions): per position the program's root record
+//     offset and the variant's index in the group (16 bits each).
 struct RankLayout {
   static constexpr int POINTS = 32;   // points per work unit: one per lane
   enum { H_B = 0, H_NLEV = 1, H_NCOND = 2, H_WORDS = 3, H_LEVEL_END = 4, H_OFF_BASIS = 12, H_OFF_COND = 13,
-         H_OFF_VARMAP = 14, H_OFF_VIDMAP = 15, H_OFF_RUNS = 16, H_NRUNS = 17, HDR_WORDS = 20 };
+         H_OFF_VARMAP = 14, H_OFF_VIDMAP = 15, H_OFF_RUNS = 16, H_NRUNS = 17, H_NPROGS = 18, H_OFF_PROGS = 19, H_OFF_SPAN = 20,
+         H_OFF_PVID = 21, H_STAGED = 22, HDR_WORDS = 24 };
+  static constexpr int SPAN_MAX = 16; // variants listed per program: the longest ranking
 };
 struct RankArgs {
   const uint32_t *img;         // every group's image (weights filled per call)
   const int4 *groups;          // [n_groups][2]: (image word offset, image words, first variant
-                               //   (template-relative), variants), (template, group index in template, 0, 0)
+                               //   (template-relative), variants), (template, group index in template, staged words, 0)
   const int4 *tmpl;            // [T][3]: (parameters, groups, 0, 0), box lo, box hi
   const int4 *chunks;          // [n_chunks] (template, first point, point count <= 32, first partial slot or -1)
   const int2 *units;           // [n_units] (chunk, group or -1 for a template without variants), schedule order
   int n_units;
-  int *unit_counter;           // reset to 0 before each launch
-  int *chunk_count;            // [n_chunks] groups finished, reset to 0 before each launch
+  int *unit_counter;           // units handed out beyond the first of each CTA; 0 before each launch
+  int *chunk_count;            // [n_chunks] groups finished; 0 before each launch
   int64_t *part_k;             // [slots][16][32] partial lists of chunks with several groups
   const int64_t *points;       // [total][4]
-  const double *w;             // [32]
+  const int *exponent;         // E of the fixed-point weights round(w 2^E)
   int topk;
   int32_t *top_idx;            // [total][topk]
   double *top_t;               // [total][topk]
   int *status;
-  int img_words, basis_cap;    // shared-memory layout: the largest image and basis of the plan
+  int img_words, basis_cap;    // shared-memory layout: the largest staged image and basis of the plan
 };
 cudaError_t launch_rank(const RankArgs &args, int nw, int grid, cudaStream_t st);
 int rank_max_blocks_per_sm(int nw, int img_words, int basis_cap);
-// fill the 128-bit term weights of the ranking programs from w (fp64 [32])
+// fill the 128-bit term weights of the ranking programs from w (fp64 [32]), zero the
+// launch's n_counters counters and write the weights' exponent E
 cudaError_t launch_k2_weights(uint32_t *prog, const uint4 *targets, const uint4 *contrib, int n_targets,
-                              const double *w, cudaStream_t st);
+                              const double *w, int *counters, int n_counters, int *exponent, cudaStream_t st);
 
 // predict.cu
 struct ArgPart { double t; int64_t r; };   // a partial per-model minimum: time and row

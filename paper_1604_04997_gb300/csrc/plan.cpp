@@ -87,7 +87,7 @@ namespace {
 constexpr int BASIS_MAX = 128;        // basis values per group (one byte per term index)
 constexpr int GCOND_MAX = 64;         // distinct conditions per group (two 32-bit masks per point)
 constexpr int LEVEL_MAX = 8;          // product depth of the basis
-constexpr int GROUP_MAX_WORDS = 12288; // a group's image, staged in shared memory (48 KB)
+constexpr int GROUP_MAX_WORDS = 12288; // a group's image as staged in shared memory (48 KB)
 constexpr int PROG_MAX_WORDS = 6144;  // one table's program (24 KB)
 constexpr i128 VALUE_LIM = (i128)1 << 62;
 
@@ -379,7 +379,7 @@ void pad4(std::vector<uint32_t> &o) {
 }
 
 // The group's image: header, basis definitions (ordered by level), condition
-// definitions, programs and the variant -> program map (layout in kernels.h).
+// definitions, programs, the program table and the walk (layout in kernels.h).
 // Weight words are left zero; `targets`/`contrib` say how to fill them per call
 // (word offsets relative to the image start).
 size_t emit_group(const Group &g0, std::vector<uint32_t> &img, std::vector<uint4> &targets,
@@ -539,36 +539,48 @@ size_t emit_group(const Group &g0, std::vector<uint32_t> &img, std::vector<uint4
       throw BuildError{PM_ERR_UNSUPPORTED, "a table's ranking program exceeds " + std::to_string(PROG_MAX_WORDS * 4) +
                                                " bytes"};
   }
-  // walk order: variants by shape (stable), as runs [shape, first position, count]; per
-  // position the program's root record and the variant's index in the group (16 bits each)
+  // walk order: variants by (shape, program), stable, so that a program's variants are
+  // neighbours in ascending order.  Program ids count up with the programs' first variants.
   const size_t nvar = g0.var_prog.size();
   std::vector<uint32_t> walk(nvar);
   std::iota(walk.begin(), walk.end(), 0u);
-  std::stable_sort(walk.begin(), walk.end(),
-                   [&](uint32_t a, uint32_t b) { return shape[g0.var_prog[a]] < shape[g0.var_prog[b]]; });
-  auto put16 = [&](auto value_of) {
-    for (size_t q = 0; q < nvar; q += 2) {
-      uint32_t x = value_of(walk[q]);
-      if (q + 1 < nvar) x |= value_of(walk[q + 1]) << 16;
-      img.push_back(x);
-    }
-    pad4(img);
-  };
-  img[RankLayout::H_OFF_VARMAP] = (uint32_t)img.size();
-  put16([&](uint32_t v) { return prog_off[g0.var_prog[v]]; });
-  img[RankLayout::H_OFF_VIDMAP] = (uint32_t)img.size();
-  put16([&](uint32_t v) { return v; });
-  img[RankLayout::H_OFF_RUNS] = (uint32_t)img.size();
-  uint32_t nruns = 0;
+  std::stable_sort(walk.begin(), walk.end(), [&](uint32_t a, uint32_t b) {
+    const int x = g0.var_prog[a], y = g0.var_prog[b];
+    return shape[x] != shape[y] ? shape[x] < shape[y] : x < y;
+  });
+  std::vector<uint32_t> span(progs.size(), 0), table, vids, runs;
   for (size_t q = 0; q < nvar;) {
+    const int pi = g0.var_prog[walk[q]];
     size_t e = q;
-    const uint32_t sh = shape[g0.var_prog[walk[q]]];
-    while (e < nvar && shape[g0.var_prog[walk[e]]] == sh) e++;
-    img.insert(img.end(), {sh, (uint32_t)q, (uint32_t)(e - q), 0u});
-    nruns++;
+    while (e < nvar && g0.var_prog[walk[e]] == pi) e++;
+    if (runs.empty() || runs[runs.size() - 4] != shape[pi])
+      runs.insert(runs.end(), {shape[pi], (uint32_t)q, 0u, (uint32_t)table.size()});
+    runs[runs.size() - 2] += (uint32_t)(e - q);
+    const uint32_t n = (uint32_t)std::min<size_t>(e - q, RankLayout::SPAN_MAX);
+    span[pi] = (uint32_t)vids.size() | (n << 16);
+    vids.insert(vids.end(), walk.begin() + q, walk.begin() + q + n);
+    table.push_back(prog_off[pi] | ((uint32_t)pi << 16));
     q = e;
   }
-  img[RankLayout::H_NRUNS] = nruns;
+  auto put = [&](int slot, const std::vector<uint32_t> &w) {
+    img[slot] = (uint32_t)img.size();
+    img.insert(img.end(), w.begin(), w.end());
+    pad4(img);
+  };
+  auto put16 = [&](int slot, size_t n, auto value_of) {
+    img[slot] = (uint32_t)img.size();
+    for (size_t q = 0; q < n; q += 2) img.push_back(value_of(q) | (q + 1 < n ? value_of(q + 1) << 16 : 0u));
+    pad4(img);
+  };
+  img[RankLayout::H_NPROGS] = (uint32_t)table.size();
+  put(RankLayout::H_OFF_PROGS, table);
+  put(RankLayout::H_OFF_SPAN, span);
+  img[RankLayout::H_NRUNS] = (uint32_t)runs.size() / 4;
+  put(RankLayout::H_OFF_RUNS, runs);
+  put16(RankLayout::H_OFF_PVID, vids.size(), [&](size_t q) { return vids[q]; });
+  img[RankLayout::H_STAGED] = (uint32_t)img.size();
+  put16(RankLayout::H_OFF_VARMAP, nvar, [&](size_t q) { return prog_off[g0.var_prog[walk[q]]]; });
+  put16(RankLayout::H_OFF_VIDMAP, nvar, [&](size_t q) { return walk[q]; });
   img[RankLayout::H_WORDS] = (uint32_t)img.size();
   return img.size();
 }
@@ -659,6 +671,7 @@ static pm_status build_host_plan(pm_ctx *c, const int32_t *tables, const int32_t
   std::vector<int4> &tmpl = hp.tmpl;
   tmpl.assign(3 * T, make_int4(0, 0, 0, 0));
   std::vector<std::vector<double>> gwork;    // per group: average work of one evaluation per variant
+  std::vector<double> gcost;                 // per group: work of one point (every program once)
   std::vector<int> gbasis;                   // per group: basis entries + conditions
   std::vector<int> first_group(T + 1, 0);
   int &max_words = hp.max_words, &max_basis = hp.max_basis;
@@ -706,20 +719,30 @@ static pm_status build_host_plan(pm_ctx *c, const int32_t *tables, const int32_t
         const uint32_t base = (uint32_t)img.size();
         for (auto &x : tg) targets.push_back(make_uint4(x.x + base, x.y, x.z, x.w));
         img.insert(img.end(), gi.begin(), gi.end());
-        max_words = std::max(max_words, (int)gi.size());
+        max_words = std::max(max_words, (int)gi[RankLayout::H_STAGED]);
         max_basis = std::max(max_basis, (int)cur.ents.size());
         const int nvar = (int)cur.var_prog.size();
         const int gidx = (int)groups.size() / 2;
         groups.push_back(make_int4((int)base, (int)gi.size(), cur.var_begin, nvar));
-        groups.push_back(make_int4(t, gidx - first_group[t], 0, 0));
+        groups.push_back(make_int4(t, gidx - first_group[t], (int)gi[RankLayout::H_STAGED], 0));
+        // each program is evaluated once per point; the evaluations its variants stand for
+        // are what the schedule reports
         std::vector<double> vw(nvar);
         for (int v = 0; v < nvar; v++) vw[v] = pw[cur.var_prog[v]];
         gwork.push_back(vw);
+        gcost.push_back(std::accumulate(pw.begin(), pw.end(), 0.0));
         gbasis.push_back((int)cur.ents.size() + (int)cur.conds.size());
       };
-      // image words of the group without its variant map, refreshed when a program is added
-      int fixed_words = 0;
-      auto map_words = [](size_t nvar) { return (int)(((nvar + 1) / 2 + 3) & ~(size_t)3); };
+      // staged image words of the group without its list of variants (at most SPAN_MAX per
+      // program), refreshed when a program is added
+      int fixed_words = 0, listed = 0;
+      std::vector<int> count;   // variants per program
+      auto list_words = [](int n) { return ((n + 1) / 2 + 3) & ~3; };
+      auto add_variant = [&](int prog) {
+        if ((int)count.size() <= prog) count.resize(prog + 1, 0);
+        if (count[prog]++ < RankLayout::SPAN_MAX) listed++;
+        cur.var_prog.push_back(prog);
+      };
       start(0);
       for (int v = v0; v < v1; v++) {
         const int id = tables[v];
@@ -734,7 +757,8 @@ static pm_status build_host_plan(pm_ctx *c, const int32_t *tables, const int32_t
         if ((int)cur.var_prog.size() >= slice_max && !cur.var_prog.empty()) {
           finish();
           start(v - v0);
-          fixed_words = 0;
+          fixed_words = listed = 0;
+          count.clear();
         }
         Group saved = cur;
         bool ok = true;
@@ -751,12 +775,12 @@ static pm_status build_host_plan(pm_ctx *c, const int32_t *tables, const int32_t
           std::vector<uint4> tg, cb;
           std::vector<double> pw;
           emit_group(cur, gi, tg, cb, pw);
-          fixed_new = (int)gi.size() - map_words(cur.var_prog.size());
+          fixed_new = (int)gi[RankLayout::H_STAGED] - list_words(listed);
         }
-        if (ok && fixed_new + map_words(cur.var_prog.size() + 1) > GROUP_MAX_WORDS) ok = false;
+        if (ok && fixed_new + list_words(listed + 1) > GROUP_MAX_WORDS) ok = false;
         if (ok) {
           fixed_words = fixed_new;
-          cur.var_prog.push_back(cur.prog_of_table[cid]);
+          add_variant(cur.prog_of_table[cid]);
           continue;
         }
         // this variant opens a new group
@@ -764,6 +788,8 @@ static pm_status build_host_plan(pm_ctx *c, const int32_t *tables, const int32_t
         cur = saved;
         finish();
         start(v - v0);
+        listed = 0;
+        count.clear();
         add_table(cur, cid, c->tables[cid]);
         check_limits(cur);
         {
@@ -771,11 +797,11 @@ static pm_status build_host_plan(pm_ctx *c, const int32_t *tables, const int32_t
           std::vector<uint4> tg, cb;
           std::vector<double> pw;
           emit_group(cur, gi, tg, cb, pw);
-          fixed_words = (int)gi.size() - map_words(0);
-          if (fixed_words + map_words(1) > GROUP_MAX_WORDS)
+          fixed_words = (int)gi[RankLayout::H_STAGED];
+          if (fixed_words + list_words(1) > GROUP_MAX_WORDS)
             return pm_set_error(PM_ERR_UNSUPPORTED, "a table too large for the ranking kernel");
         }
-        cur.var_prog.push_back(cur.prog_of_table[cid]);
+        add_variant(cur.prog_of_table[cid]);
       }
       finish();
       first_group[t + 1] = (int)groups.size() / 2;
@@ -807,7 +833,7 @@ static pm_status build_host_plan(pm_ctx *c, const int32_t *tables, const int32_t
         double gw = 0;
         for (double x : gwork[g]) gw += x;
         // about ten operations per basis value and condition, once per point of the unit
-        units.push_back({ch, g, (gw + 10.0 * gbasis[g]) * n});
+        units.push_back({ch, g, (gcost[g] + 10.0 * gbasis[g]) * n});
         total_work += gw * n;
         evals += (int64_t)gwork[g].size() * n;
       }
@@ -857,8 +883,8 @@ static pm_status build_plan(pm_ctx *c, const int32_t *tables, const int32_t *var
   p->d_chunks = (const int4 *)d;
   if ((s = alloc(hu.data(), hu.size() * sizeof(int2), &d))) return fail(s);
   p->d_units = (const int2 *)d;
-  if ((s = alloc(nullptr, sizeof(int) * (chunks.size() + 1), &d))) return fail(s);
-  p->d_counter = (int *)d;  // [0] unit counter, [1..] per-chunk group counters
+  if ((s = alloc(nullptr, sizeof(int) * (chunks.size() + 2), &d))) return fail(s);
+  p->d_counter = (int *)d;  // [0] unit counter, [1..] per-chunk group counters, then the weights' exponent
   if ((s = alloc(nullptr, (size_t)std::max(hp.slots, 1) * 16 * RankLayout::POINTS * 8, &d))) return fail(s);
   p->d_part_k = (int64_t *)d;
   p->n_chunks = (int)chunks.size();
@@ -945,8 +971,8 @@ pm_status ctx_plan_k2(pm_ctx *c, const int32_t *tables, const int32_t *var_off, 
 
 static pm_status launch_plan(pm_ctx *c, Plan *p, const int64_t *pts, const double *w, int topk, int32_t *idx,
                              double *t, cudaStream_t st, int nw, int grid) {
-  CU(cudaMemsetAsync(p->d_counter, 0, sizeof(int) * (p->n_chunks + 1), st));
-  CU(pmd::launch_k2_weights(p->d_img, p->d_targets, p->d_contrib, p->n_targets, w, st));
+  CU(pmd::launch_k2_weights(p->d_img, p->d_targets, p->d_contrib, p->n_targets, w, p->d_counter, p->n_chunks + 1,
+                            p->d_counter + p->n_chunks + 1, st));
   pmd::RankArgs a;
   a.img = p->d_img;
   a.groups = p->d_groups;
@@ -958,7 +984,7 @@ static pm_status launch_plan(pm_ctx *c, Plan *p, const int64_t *pts, const doubl
   a.chunk_count = p->d_counter + 1;
   a.part_k = p->d_part_k;
   a.points = pts;
-  a.w = w;
+  a.exponent = p->d_counter + p->n_chunks + 1;
   a.topk = topk;
   a.top_idx = idx;
   a.top_t = t;

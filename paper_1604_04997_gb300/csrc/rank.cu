@@ -9,13 +9,17 @@
 //      in shared memory;
 //   2. evaluate the group's basis (parameters, atoms floor((a.n + b)/c), monomials, in
 //      dependency levels) and its piece conditions once per point;
-//   3. each warp walks every NW-th variant: the piece from the condition bits, then the
+//   3. each warp walks every NW-th program (distinct table; variants that share a table
+//      share its prediction): the piece from the condition bits, then the
 //      exact fixed-point prediction S = sum_term Weff_term * basis_term (128 bits), the
 //      runtime min(loads, stores) post-ops and the exact division by the table's
 //      denominator; a candidate that beats the lane's threshold is buffered and the
 //      buffers are inserted into register-resident sorted lists of 16 when one fills;
 //   4. the warps share their 16th entries through shared memory (any warp's 16th
-//      entry bounds the unit's final 16th), then merge their lists.
+//      entry bounds the unit's final 16th), then merge their lists;
+//   5. the 16 best programs by (prediction, first variant) become the 16 best variants.
+//      (A variant among the 16 best has its program among the 16 best: otherwise 16
+//      programs come before it, each with a variant that comes before this one.)
 // A chunk whose template is split into several groups is finished by the last of its
 // units (partial lists in scratch, a fence and an atomic counter; no waiting).
 #include <cuda_runtime.h>
@@ -82,21 +86,30 @@ __device__ __forceinline__ void mac128_u32(uint32_t (&A)[4], const uint4 &W, uin
 // Fill the 128-bit term weights of the ranking programs: Weff = sum over contributions
 // of W_col * coef, with W_col = round(w_col 2^E) the fixed-point weights (sum |W| <=
 // 2^62, so with counts D * p_col < 2^62 a program's sum stays within +-2^124).
+// One target per thread.  The counters of the ranking launch that follows are zeroed here.
 __global__ void __launch_bounds__(128) k_k2_weights(uint32_t *__restrict__ prog, const uint4 *__restrict__ targets,
                                                     const uint4 *__restrict__ contrib, int n_targets,
-                                                    const double *__restrict__ w) {
+                                                    const double *__restrict__ w, int *__restrict__ counters,
+                                                    int n_counters, int *__restrict__ exponent) {
   __shared__ uint4 sW[32];   // each weight sign-extended to 128 bits
+  __shared__ double s_w[32];
   __shared__ int s_E;
-  if (threadIdx.x == 0) s_E = weight_exponent(w, 32);   // the same E as the ranking kernel's
+  const int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  if (threadIdx.x < 32) s_w[threadIdx.x] = w[threadIdx.x];
+  for (int i = first; i < n_counters; i += step) counters[i] = 0;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    const int64_t W = llrint(ldexp(w[lane], s_E));      // |W| <= 2^62
-    const uint32_t sx = W < 0 ? 0xFFFFFFFFu : 0u;
-    sW[lane] = make_uint4((uint32_t)W, (uint32_t)((uint64_t)W >> 32), sx, sx);
+  if (threadIdx.x == 0) {
+    s_E = weight_exponent(s_w, 32);
+    if (blockIdx.x == 0) *exponent = s_E;   // for the ranking kernel
   }
   __syncthreads();
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_targets; i += gridDim.x * blockDim.x) {
+  if (threadIdx.x < 32) {
+    const int64_t W = fixed_weight(s_w[threadIdx.x], s_E);   // |W| <= 2^62
+    const uint32_t sx = W < 0 ? 0xFFFFFFFFu : 0u;
+    sW[threadIdx.x] = make_uint4((uint32_t)W, (uint32_t)((uint64_t)W >> 32), sx, sx);
+  }
+  __syncthreads();
+  for (int i = first; i < n_targets; i += step) {
     const uint4 tg = targets[i];
     uint32_t A[4] = {0, 0, 0, 0};
     for (uint32_t c = 0; c < tg.z; c++) {
@@ -114,16 +127,16 @@ __global__ void __launch_bounds__(128) k_k2_weights(uint32_t *__restrict__ prog,
 }
 
 cudaError_t launch_k2_weights(uint32_t *prog, const uint4 *targets, const uint4 *contrib, int n_targets,
-                              const double *w, cudaStream_t st) {
+                              const double *w, int *counters, int n_counters, int *exponent, cudaStream_t st) {
   const int grid = std::max(1, std::min(1024, (n_targets + 127) / 128));
-  k_k2_weights<<<grid, 128, 0, st>>>(prog, targets, contrib, n_targets, w);
+  k_k2_weights<<<grid, 128, 0, st>>>(prog, targets, contrib, n_targets, w, counters, n_counters, exponent);
   return cudaGetLastError();
 }
 
 // A ranking entry packs the top 48 bits of the monotone key (sign, exponent and 40
-// mantissa bits: 2^-40 relative resolution) above a 16-bit variant index, so one
-// signed 64-bit comparison orders by (key, variant) and exact ties (variants with
-// equal predictions) fall to the smaller index.
+// mantissa bits: 2^-40 relative resolution) above a 16-bit index (of a program, in
+// the order of first variants, then of a variant), so one signed 64-bit comparison orders by
+// (key, index) and exact ties (equal predictions) fall to the smaller index.
 __device__ __forceinline__ int64_t pack_entry(int64_t key, int vid) {
   return (int64_t)(((uint64_t)(key >> 16) << 16) | (uint32_t)vid);
 }
@@ -192,7 +205,7 @@ struct TopK {
   }
 };
 
-// Candidate threshold: an entry e = (key48, variant) that the point's final 16th entry
+// Candidate threshold: an entry e = (key48, program) that the point's final 16th entry
 // cannot exceed.  For a positive key K, key48(S) < K <=> S < key_floor(K) = lo and
 // key48(S) == K <=> lo <= S < key_floor(K + 2^16) = hi, so the common test is one
 // 128-bit compare S < hi; only then is the entry formed (a tie at K takes K itself).
@@ -234,10 +247,15 @@ __device__ __forceinline__ int64_t pick4(int64_t h0, int64_t h1, int64_t h2, int
   return x;
 }
 
+// Shared memory: the staged image | the basis, then (after the walk) the warps' lists |
+// condition bits | 16th entries | candidate buffers, then the ranked variants [16][32]
+__host__ __device__ inline size_t rank_basis_bytes(int nw, int basis_cap) {
+  const size_t basis = (size_t)basis_cap * 32 * 8, lists = (size_t)(nw / 2) * RK_TOPK * 32 * 8;
+  return basis > lists ? basis : lists;
+}
 size_t rank_smem_bytes(int nw, int img_words, int basis_cap) {
-  const size_t a = (size_t)((img_words + 3) & ~3) * 4 + (size_t)basis_cap * 32 * 8;
-  const size_t lists = (size_t)(nw / 2) * RK_TOPK * 32 * 8;
-  return std::max(a, lists) + 64 * 4 + (size_t)nw * 32 * 8 + (size_t)nw * RK_BUF * 32 * 8;
+  return (size_t)((img_words + 3) & ~3) * 4 + rank_basis_bytes(nw, basis_cap) + 64 * 4 + (size_t)nw * 32 * 8 +
+         (size_t)nw * RK_BUF * 32 * 8;
 }
 
 template <int NW>
@@ -248,21 +266,18 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
   uint32_t *img = (uint32_t *)smem;                        // the group's image
   uint32_t *blo = img + img_cap;                           // basis, low words [basis_cap][32]
   uint32_t *bhi = blo + a.basis_cap * 32;                  // basis, high words
-  int64_t *lists = (int64_t *)smem;                        // after the walk: [NW][16][32]
-  const size_t region = max((size_t)img_cap * 4 + (size_t)a.basis_cap * 256, (size_t)(NW / 2) * RK_TOPK * 256);
-  uint32_t *mask = (uint32_t *)(smem + region);            // condition bits per point [2][32]
+  int64_t *lists = (int64_t *)blo;                         // after the walk: [NW / 2][16][32]
+  uint32_t *mask = (uint32_t *)((uint8_t *)blo + rank_basis_bytes(NW, a.basis_cap));   // condition bits per point [2][32]
   volatile int64_t *thrx = (int64_t *)(mask + 64);         // each warp's 16th entries [NW][32]
   int64_t *bufs = (int64_t *)(mask + 64) + NW * 32;        // [NW][RK_BUF][32]
   int64_t *mybuf = bufs + warp * RK_BUF * 32 + lane;
-  __shared__ int s_E, s_unit, s_last;
+  static_assert(NW * RK_BUF >= RK_TOPK, "the ranked variants take the buffers' place");
+  int64_t *ranked = bufs;
+  __shared__ int s_unit, s_last;
 
-  if (threadIdx.x == 0) s_E = weight_exponent(a.w, 32);   // the programs' weights are round(w 2^E)
-  while (true) {
-    __syncthreads();
-    if (threadIdx.x == 0) s_unit = atomicAdd(a.unit_counter, 1);
-    __syncthreads();
-    const int u = s_unit;
-    if (u >= a.n_units) break;
+  for (int u = blockIdx.x; u < a.n_units;) {
+    __syncthreads();   // the unit before is done with shared memory
+    if (threadIdx.x == 0) s_unit = (int)gridDim.x + atomicAdd(a.unit_counter, 1);   // the unit after this one
     const int2 U = a.units[u];
     const int4 C = a.chunks[U.x];          // template, first point, point count, first partial slot
     const int t = C.x;
@@ -274,7 +289,7 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
     tk.init();
     if (U.y >= 0) {
       const int4 G0 = a.groups[2 * U.y], G1 = a.groups[2 * U.y + 1];
-      for (int i = threadIdx.x; i < G0.y / 4; i += NW * 32) cp_async16(img + 4 * i, a.img + G0.x + 4 * i);
+      for (int i = threadIdx.x; i < G1.z / 4; i += NW * 32) cp_async16(img + 4 * i, a.img + G0.x + 4 * i);
       cp_async_commit();
       // this lane's point: two 16-byte loads, then the box check
       bool valid = live;
@@ -350,8 +365,8 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
       }
       __syncthreads();
       const uint32_t cm0 = mask[lane], cm1 = mask[32 + lane];
-      const uint16_t *vmap = (const uint16_t *)(img + img[RankLayout::H_OFF_VARMAP]);
-      const int nv = G0.w, vbase = G0.z;
+      const uint32_t *progs = img + img[RankLayout::H_OFF_PROGS];   // root record offset | program id << 16
+      const int np = (int)img[RankLayout::H_NPROGS], vbase = G0.z;
       const uint32_t bmax = img[RankLayout::H_B] - 1;   // every basis index is clamped to the basis
       Threshold th;
       th.set(RK_EMPTY);
@@ -373,7 +388,6 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
         nbuf = 0;
         if (tk.k[RK_TOPK - 1] < th.e) th.set(tk.k[RK_TOPK - 1]);
       };
-      const uint16_t *vidm = (const uint16_t *)(img + img[RankLayout::H_OFF_VIDMAP]);
       const uint4 *runs = (const uint4 *)(img + img[RankLayout::H_OFF_RUNS]);
       const int nruns = (int)img[RankLayout::H_NRUNS];
       // walk a program's nodes to its leaf at this lane's point: the table's conditions
@@ -422,7 +436,7 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
       };
       // any leaf: term counts read from the leaf record
       auto evaluate = [&](int pos) -> Acc128 {
-        const uint4 N = leaf_of(vmap[pos]);
+        const uint4 N = leaf_of(progs[pos] & 0xFFFF);
         const uint4 *rec = (const uint4 *)(img + N.y);
         const uint4 c0 = *rec++;
         uint32_t A[4] = {c0.x, c0.y, c0.z, c0.w};
@@ -457,7 +471,7 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
         bool stop = ++since >= RK_EXCHANGE;
         if (__any_sync(0xffffffffu, m)) {
           if (m) {
-            const int64_t e = th.entry(S, vbase + vidm[pos]);
+            const int64_t e = th.entry(S, (int)(progs[pos] >> 16));
             if (e < th.e) {
               mybuf[nbuf * 32] = e;
               nbuf++;
@@ -467,13 +481,13 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
         }
         return stop;
       };
-      // the first 16 positions of the warp fill its list, sorted once
-      const int fill_end = min(nv, RK_TOPK * NW);
+      // the first 16 programs of the warp fill its list, sorted once
+      const int fill_end = min(np, RK_TOPK * NW);
 #pragma unroll 1
-      for (int f = 0, pos = warp; f < RK_TOPK; f++, pos += NW) {
+      for (int pos = warp; pos < (fill_end + NW - 1) / NW * NW; pos += NW) {
         int64_t e = RK_EMPTY;
         if (pos < fill_end) {   // lanes without a valid point evaluate the box's corner
-          const int64_t x = pack_entry(acc_key(evaluate(pos)), vbase + vidm[pos]);
+          const int64_t x = pack_entry(acc_key(evaluate(pos)), (int)(progs[pos] >> 16));
           e = valid ? x : RK_EMPTY;
         }
 #pragma unroll
@@ -483,14 +497,14 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
       tk.sort();
       th.set(tk.k[RK_TOPK - 1]);
       exchange();
-      // the variants of a run of one shape (term counts fixed at compile time) from pos
+      // the programs of a run of one shape (term counts fixed at compile time) from pos
       // on, until the warp must stop; returns the next position.  The flush and the
       // exchange sit once in the run loop below, outside the per-shape code, which keeps
       // the kernel's hot code small.
       auto run_fixed = [&](auto c64, auto c32, int pos, int end) -> int {
         constexpr int N64 = decltype(c64)::value, N32 = decltype(c32)::value;
         while (pos < end) {
-          const uint4 N1 = leaf_of(vmap[pos]);
+          const uint4 N1 = leaf_of(progs[pos] & 0xFFFF);
           const uint4 *r1 = (const uint4 *)(img + N1.y);
           const uint4 c = r1[0];
           uint32_t A1[4] = {c.x, c.y, c.z, c.w};
@@ -514,7 +528,7 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
       };
       for (int r = 0; r < nruns; r++) {
         const uint4 R = runs[r];
-        const int start = max((int)R.y, fill_end), end = (int)(R.y + R.z);
+        const int start = max((int)R.w, fill_end), end = r + 1 < nruns ? (int)runs[r + 1].w : np;
         if (start >= end) continue;
         int pos = start + ((warp - start % NW) + NW) % NW;   // this warp's first position
         while (pos < end) {
@@ -534,7 +548,7 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
         }
       }
       flush();
-      // merge the warps' lists in a tree (the image and basis are no longer read)
+      // merge the warps' lists in a tree (the basis is no longer read)
       __syncthreads();
 #pragma unroll
       for (int half = NW / 2; half > 0; half >>= 1) {
@@ -546,38 +560,90 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
         if (warp < half) tk.merge(lists + warp * RK_TOPK * 32 + lane, 32);
         __syncthreads();
       }
+      // the best programs become the best variants: programs in order of their predictions,
+      // those with equal keys merged by variant index; the warps share the points
+      if (warp == 0) {
+#pragma unroll
+        for (int q = 0; q < RK_TOPK; q++) lists[q * 32 + lane] = tk.k[q];
+      }
+      __syncthreads();
+      if (lane % NW == warp) {
+        const uint32_t *span = img + img[RankLayout::H_OFF_SPAN];
+        const uint16_t *pvid = (const uint16_t *)(img + img[RankLayout::H_OFF_PVID]);
+        int o = 0, i = 0;
+        while (o < RK_TOPK && i < RK_TOPK) {
+          const int64_t e = lists[i * 32 + lane];
+          if (e == RK_EMPTY) break;
+          const int64_t key = entry_key(e);
+          int j = i + 1;
+          while (j < RK_TOPK && entry_key(lists[j * 32 + lane]) == key) j++;
+          if (j == i + 1) {
+            const uint32_t sp = span[entry_vid(e)], off = sp & 0xFFFF;
+            const int n = min((int)(sp >> 16), RK_TOPK - o);
+            for (int c = 0; c < n; c++) ranked[(o + c) * 32 + lane] = key | (uint32_t)(vbase + pvid[off + c]);
+            o += n;
+          } else {
+            // a tie of programs i .. j - 1: their next variants (4 bits each: at most 16 in all)
+            uint64_t next = 0;
+            while (o < RK_TOPK) {
+              int best = 0x10000, from = 0;
+              for (int r = i; r < j; r++) {
+                const uint32_t sp = span[entry_vid(lists[r * 32 + lane])];
+                const uint32_t c = (uint32_t)(next >> (4 * (r - i))) & 15;
+                if (c < (sp >> 16)) {
+                  const int v = pvid[(sp & 0xFFFF) + c];
+                  if (v < best) { best = v; from = r - i; }
+                }
+              }
+              if (best == 0x10000) break;
+              ranked[o * 32 + lane] = key | (uint32_t)(vbase + best);
+              next += 1ull << (4 * from);
+              o++;
+            }
+          }
+          i = j;
+        }
+        for (; o < RK_TOPK; o++) ranked[o * 32 + lane] = RK_EMPTY;
+      }
+      __syncthreads();
       if (S_groups > 1) {
-        // publish this group's lists; the last group of the chunk merges all of them
+        // publish this group's list; the last group of the chunk merges all of them
         if (warp == 0) {
           const int64_t slot0 = ((int64_t)C.w + G1.y) * RK_TOPK * 32 + lane;
 #pragma unroll
-          for (int q = 0; q < RK_TOPK; q++) a.part_k[slot0 + q * 32] = tk.k[q];
+          for (int q = 0; q < RK_TOPK; q++) a.part_k[slot0 + q * 32] = ranked[q * 32 + lane];
           __threadfence();
         }
         __syncthreads();
         if (threadIdx.x == 0) s_last = atomicAdd(a.chunk_count + U.x, 1) == S_groups - 1;
         __syncthreads();
-        if (!s_last) continue;
+        if (!s_last) {
+          u = s_unit;
+          continue;
+        }
         if (warp == 0) {
           __threadfence();
           tk.init();
           for (int g = 0; g < S_groups; g++) tk.merge(a.part_k + ((int64_t)C.w + g) * RK_TOPK * 32 + lane, 32);
-        }
-      }
-    }
-    if (warp == 0 && live) {
-      int32_t *oi = a.top_idx + p * a.topk;
-      double *ot = a.top_t + p * a.topk;
-      const int E = s_E;
 #pragma unroll
-      for (int q = 0; q < RK_TOPK; q++) {
-        if (q < a.topk) {
-          const bool real = tk.k[q] != RK_EMPTY;
-          oi[q] = real ? entry_vid(tk.k[q]) : -1;
-          ot[q] = real ? key_value(entry_key(tk.k[q]), E) : __longlong_as_double(0x7ff0000000000000ll);
+          for (int q = 0; q < RK_TOPK; q++) ranked[q * 32 + lane] = tk.k[q];
         }
+        __syncthreads();
       }
+    } else {
+      for (int i = threadIdx.x; i < RK_TOPK * 32; i += NW * 32) ranked[i] = RK_EMPTY;   // a template without variants
+      __syncthreads();
     }
+    // the unit's rows, written by all threads
+    const int E = *a.exponent;   // the programs' weights are round(w 2^E)
+    for (int i = threadIdx.x; i < C.z * a.topk; i += NW * 32) {
+      const int r = i / a.topk, q = i - r * a.topk;
+      const int64_t e = ranked[q * 32 + r], o = (int64_t)C.y * a.topk + i;
+      const bool real = e != RK_EMPTY;
+      a.top_idx[o] = real ? entry_vid(e) : -1;
+      a.top_t[o] = real ? key_value(entry_key(e), E) : __longlong_as_double(0x7ff0000000000000ll);
+    }
+    u = s_unit;
   }
 }
 
