@@ -282,4 +282,16 @@ __device__ __forceinline__ int weight_exponent(const double *w, int k) {
   return 62 - e;
 }
 
+// The same for 32 weights, one per lane of a warp: the sum by shuffles, in another order.
+// Both sums are within 2^-47 of the exact one, so they give the same exponent unless the
+// sum lies that close to a power of two; then the serial loop decides.
+__device__ __forceinline__ int weight_exponent_warp(const double *w32) {
+  double s = fabs(w32[threadIdx.x & 31]);
+#pragma unroll
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  const double lo = s * (1.0 + 0x1p-40 - 0x1p-45), hi = s * (1.0 + 0x1p-40 + 0x1p-45);
+  const uint64_t a = (uint64_t)__double_as_longlong(lo) >> 52, b = (uint64_t)__double_as_longlong(hi) >> 52;
+  return a == b && a > 0 && a < 0x7FF ? 62 - ((int)a - 1022) : weight_exponent(w32, 32);
+}
+
 }  // namespace pmd

@@ -23,6 +23,7 @@ cudaError_t launch_eval_counts(const uint32_t *arena, const int64_t *d_tab_off, 
 //   conditions (at most 64): [n_terms, const_lo, const_hi, (entry, coef_lo, coef_hi) *
 //     n_terms], bit q of a point's two mask words when const + sum coef * value >= 0:
 //     the tables' piece conditions and the signs of undecided post-op differences A - B;
+//     then the word offset of each condition in the image;
 //   programs (one per distinct table), as records of four words:
 //     condition node [1 | n << 8 | piece records << 16, condition ids 0-4 (6 bits each),
 //       ids 5-9, LUT offset]: the LUT byte of the n condition bits names a piece record;
@@ -45,7 +46,7 @@ struct RankLayout {
   static constexpr int POINTS = 32;   // points per work unit: one per lane
   enum { H_B = 0, H_NLEV = 1, H_NCOND = 2, H_WORDS = 3, H_LEVEL_END = 4, H_OFF_BASIS = 12, H_OFF_COND = 13,
          H_OFF_VARMAP = 14, H_OFF_VIDMAP = 15, H_OFF_RUNS = 16, H_NRUNS = 17, H_NPROGS = 18, H_OFF_PROGS = 19, H_OFF_SPAN = 20,
-         H_OFF_PVID = 21, H_STAGED = 22, HDR_WORDS = 24 };
+         H_OFF_PVID = 21, H_STAGED = 22, H_OFF_CINDEX = 23, HDR_WORDS = 24 };
   static constexpr int SPAN_MAX = 16; // variants listed per program: the longest ranking
 };
 struct RankArgs {

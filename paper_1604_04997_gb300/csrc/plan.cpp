@@ -419,7 +419,9 @@ size_t emit_group(const Group &g0, std::vector<uint32_t> &img, std::vector<uint4
     img.insert(img.end(), w, w + 8);
   }
   img[RankLayout::H_OFF_COND] = (uint32_t)img.size();
+  std::vector<uint32_t> cond_at;
   for (auto &cnd : g0.conds) {
+    cond_at.push_back((uint32_t)img.size());
     const int nt = (int)(cnd.size() - 1) / 2;
     img.push_back((uint32_t)nt);
     img.push_back((uint32_t)cnd[0]);
@@ -430,6 +432,8 @@ size_t emit_group(const Group &g0, std::vector<uint32_t> &img, std::vector<uint4
       img.push_back((uint32_t)((uint64_t)cnd[2 + 2 * t] >> 32));
     }
   }
+  img[RankLayout::H_OFF_CINDEX] = (uint32_t)img.size();
+  img.insert(img.end(), cond_at.begin(), cond_at.end());
   pad4(img);
   // flags of a target: 1 = a 96-bit weight (three words; the fourth holds the term's
   // basis entry)
@@ -658,7 +662,7 @@ struct HostPlan {
   std::vector<int4> tmpl;                    // per template: three int4 (see RankArgs)
   std::vector<int4> chunks;
   std::vector<int2> units;
-  int slots = 0, max_words = 0, max_basis = 0;
+  int slots = 0, max_words = 0, max_basis = 0, max_progs = 0;
   int64_t evals = 0;
   double total_work = 0;
 };
@@ -721,6 +725,7 @@ static pm_status build_host_plan(pm_ctx *c, const int32_t *tables, const int32_t
         img.insert(img.end(), gi.begin(), gi.end());
         max_words = std::max(max_words, (int)gi[RankLayout::H_STAGED]);
         max_basis = std::max(max_basis, (int)cur.ents.size());
+        hp.max_progs = std::max(hp.max_progs, (int)cur.progs.size());
         const int nvar = (int)cur.var_prog.size();
         const int gidx = (int)groups.size() / 2;
         groups.push_back(make_int4((int)base, (int)gi.size(), cur.var_begin, nvar));
@@ -896,6 +901,7 @@ static pm_status build_plan(pm_ctx *c, const int32_t *tables, const int32_t *var
   p->work_per_eval = hp.evals ? hp.total_work / (double)hp.evals : 0;
   p->img_words = hp.max_words;
   p->basis_cap = std::max(1, hp.max_basis);
+  p->max_progs = hp.max_progs;
   p->slice_max = slice_max;
   *out = p;
   return PM_OK;
@@ -944,7 +950,11 @@ static void default_shape(pm_ctx *c, Plan *p, int nw) {
 }
 
 static constexpr int DEFAULT_SLICE = 1 << 30;   // one group per template unless a limit splits it
-static constexpr int DEFAULT_NW = 8;
+// Warps per CTA by the programs of the largest group: with few programs a unit is mostly
+// its fixed steps (staging, basis, ranking), so four warps and twice the CTAs per SM are
+// faster (137 programs over 8 groups, 1,024 units: 52 us against 70); with more than 16 per
+// warp of eight the walk over the programs dominates and all eight share one basis.
+static int default_nw(const Plan *p) { return p->max_progs <= 128 ? 4 : 8; }
 
 pm_status ctx_plan_k2(pm_ctx *c, const int32_t *tables, const int32_t *var_off, int T, const int64_t *pt_off,
                       Plan **out) {
@@ -962,7 +972,7 @@ pm_status ctx_plan_k2(pm_ctx *c, const int32_t *tables, const int32_t *var_off, 
   Plan *p = nullptr;
   pm_status s = build_plan(c, tables, var_off, T, pt_off, DEFAULT_SLICE, &p);
   if (s) return s;
-  default_shape(c, p, DEFAULT_NW);
+  default_shape(c, p, default_nw(p));
   p->key = key;
   c->plans[key] = p;
   *out = p;

@@ -26,7 +26,8 @@ struct Plan {
   int *d_counter = nullptr;
   int64_t *d_part_k = nullptr;
   int n_units = 0, n_templates = 0, n_chunks = 0, n_groups = 0;
-  int img_words = 0, basis_cap = 1;  // the largest group image and basis (shared-memory layout)
+  int img_words = 0, basis_cap = 1;  // the largest staged image and basis (shared-memory layout)
+  int max_progs = 0;                 // programs of the largest group
   int slice_max = 0;                 // at most this many variants per group
   int64_t total_points = 0, total_evals = 0;
   double work_per_eval = 0;          // algorithmic integer operations per evaluation

@@ -36,6 +36,7 @@ constexpr int RK_TOPK = 16;
 constexpr int RK_BUF = 4;                   // buffered insertion candidates per lane
 constexpr int RK_EXCHANGE = 16;             // variants of a warp between threshold exchanges
 constexpr int64_t RK_EMPTY = INT64_MAX;     // an empty list entry
+constexpr int RK_COUNT = 32;                // up to this many programs are ranked by counting
 
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc) {
   unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
@@ -93,18 +94,14 @@ __global__ void __launch_bounds__(128) k_k2_weights(uint32_t *__restrict__ prog,
                                                     int n_counters, int *__restrict__ exponent) {
   __shared__ uint4 sW[32];   // each weight sign-extended to 128 bits
   __shared__ double s_w[32];
-  __shared__ int s_E;
   const int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
   if (threadIdx.x < 32) s_w[threadIdx.x] = w[threadIdx.x];
   for (int i = first; i < n_counters; i += step) counters[i] = 0;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    s_E = weight_exponent(s_w, 32);
-    if (blockIdx.x == 0) *exponent = s_E;   // for the ranking kernel
-  }
-  __syncthreads();
   if (threadIdx.x < 32) {
-    const int64_t W = fixed_weight(s_w[threadIdx.x], s_E);   // |W| <= 2^62
+    const int E = weight_exponent_warp(s_w);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *exponent = E;   // for the ranking kernel
+    const int64_t W = fixed_weight(s_w[threadIdx.x], E);      // |W| <= 2^62
     const uint32_t sx = W < 0 ? 0xFFFFFFFFu : 0u;
     sW[threadIdx.x] = make_uint4((uint32_t)W, (uint32_t)((uint64_t)W >> 32), sx, sx);
   }
@@ -248,14 +245,15 @@ __device__ __forceinline__ int64_t pick4(int64_t h0, int64_t h1, int64_t h2, int
 }
 
 // Shared memory: the staged image | the basis, then (after the walk) the warps' lists |
-// condition bits | 16th entries | candidate buffers, then the ranked variants [16][32]
+// condition bits | 16th entries | candidate buffers [NW][RK_BUF][32] or all candidates
+// [RK_COUNT][32], then the ranked variants [16][32]
 __host__ __device__ inline size_t rank_basis_bytes(int nw, int basis_cap) {
   const size_t basis = (size_t)basis_cap * 32 * 8, lists = (size_t)(nw / 2) * RK_TOPK * 32 * 8;
   return basis > lists ? basis : lists;
 }
 size_t rank_smem_bytes(int nw, int img_words, int basis_cap) {
   return (size_t)((img_words + 3) & ~3) * 4 + rank_basis_bytes(nw, basis_cap) + 64 * 4 + (size_t)nw * 32 * 8 +
-         (size_t)nw * RK_BUF * 32 * 8;
+         (size_t)std::max(nw * RK_BUF, RK_COUNT) * 32 * 8;
 }
 
 template <int NW>
@@ -348,19 +346,17 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
       // conditions: const + sum coef * value >= 0, one bit each (64-bit coefficients; the
       // sums are exact in 64 bits, wrapping included, since each true sum is below 2^63)
       {
-        const uint32_t *cd = img + img[RankLayout::H_OFF_COND];
-        for (int q = 0; q < ncond; q++) {
+        const uint32_t *at = img + img[RankLayout::H_OFF_CINDEX];
+        for (int q = warp; q < ncond; q += NW) {
+          const uint32_t *cd = img + at[q];
           const int nt = (int)cd[0];
-          if ((q % NW) == warp) {
-            uint64_t s = (uint64_t)ld64(cd + 1);
-            for (int k = 0; k < nt; k++) {
-              const uint32_t e = cd[3 + 3 * k];
-              const uint64_t x = (uint64_t)blo[e * 32 + lane] | ((uint64_t)bhi[e * 32 + lane] << 32);
-              s += x * (uint64_t)ld64(cd + 4 + 3 * k);
-            }
-            if ((int64_t)s >= 0) atomicOr(&mask[(q >> 5) * 32 + lane], 1u << (q & 31));
+          uint64_t s = (uint64_t)ld64(cd + 1);
+          for (int k = 0; k < nt; k++) {
+            const uint32_t e = cd[3 + 3 * k];
+            const uint64_t x = (uint64_t)blo[e * 32 + lane] | ((uint64_t)bhi[e * 32 + lane] << 32);
+            s += x * (uint64_t)ld64(cd + 4 + 3 * k);
           }
-          cd += 3 + 3 * nt;
+          if ((int64_t)s >= 0) atomicOr(&mask[(q >> 5) * 32 + lane], 1u << (q & 31));
         }
       }
       __syncthreads();
@@ -452,121 +448,149 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
         }
         return finish(A, N.z);
       };
-      auto exchange = [&]() {   // share 16th entries with the other warps
-        thrx[warp * 32 + lane] = tk.k[RK_TOPK - 1];
-        int64_t m = th.e;
+      if (np <= RK_COUNT) {
+        // Few programs (the common case once variants share tables): every candidate in
+        // shared memory, and each takes the place given by the number of smaller ones.  No
+        // lists, buffers or merges; np compares per candidate, np / NW candidates per warp.
+        for (int pos = warp; pos < np; pos += NW)
+          bufs[pos * 32 + lane] = pack_entry(acc_key(evaluate(pos)), (int)(progs[pos] >> 16));
+        __syncthreads();
+        constexpr int OWN = RK_COUNT / NW;
+        int64_t own[OWN];
+        int place[OWN];
 #pragma unroll
-        for (int w = 0; w < NW; w++) {
-          const int64_t x = thrx[w * 32 + lane];
-          m = x < m ? x : m;
+        for (int i = 0; i < OWN; i++) {
+          const int pos = warp + NW * i;
+          own[i] = pos < np ? bufs[pos * 32 + lane] : RK_EMPTY;
+          place[i] = 0;
         }
-        if (m < th.e) th.set(m);
-      };
-      int since = 0;
-      // one candidate after the fill: one 128-bit compare; the few that may pass are
-      // buffered.  Returns true when the warp should stop to flush its buffers (a lane's
-      // buffer is full) or to exchange thresholds (every RK_EXCHANGE variants).
-      auto offer = [&](const Acc128 &S, int pos) -> bool {
-        const bool m = valid && th.maybe(S);
-        bool stop = ++since >= RK_EXCHANGE;
-        if (__any_sync(0xffffffffu, m)) {
-          if (m) {
-            const int64_t e = th.entry(S, (int)(progs[pos] >> 16));
-            if (e < th.e) {
-              mybuf[nbuf * 32] = e;
-              nbuf++;
+        for (int j = 0; j < np; j++) {
+          const int64_t x = bufs[j * 32 + lane];
+#pragma unroll
+          for (int i = 0; i < OWN; i++) place[i] += x < own[i];
+        }
+#pragma unroll
+        for (int i = 0; i < OWN; i++)
+          if (warp + NW * i < np && place[i] < RK_TOPK) lists[place[i] * 32 + lane] = valid ? own[i] : RK_EMPTY;
+        for (int q = np + warp; q < RK_TOPK; q += NW) lists[q * 32 + lane] = RK_EMPTY;
+        __syncthreads();
+      } else {
+        auto exchange = [&]() {   // share 16th entries with the other warps
+          thrx[warp * 32 + lane] = tk.k[RK_TOPK - 1];
+          int64_t m = th.e;
+#pragma unroll
+          for (int w = 0; w < NW; w++) {
+            const int64_t x = thrx[w * 32 + lane];
+            m = x < m ? x : m;
+          }
+          if (m < th.e) th.set(m);
+        };
+        int since = 0;
+        // one candidate after the fill: one 128-bit compare; the few that may pass are
+        // buffered.  Returns true when the warp should stop to flush its buffers (a lane's
+        // buffer is full) or to exchange thresholds (every RK_EXCHANGE variants).
+        auto offer = [&](const Acc128 &S, int pos) -> bool {
+          const bool m = valid && th.maybe(S);
+          bool stop = ++since >= RK_EXCHANGE;
+          if (__any_sync(0xffffffffu, m)) {
+            if (m) {
+              const int64_t e = th.entry(S, (int)(progs[pos] >> 16));
+              if (e < th.e) {
+                mybuf[nbuf * 32] = e;
+                nbuf++;
+              }
+            }
+            stop = stop || __any_sync(0xffffffffu, nbuf == RK_BUF);
+          }
+          return stop;
+        };
+        // the first 16 programs of the warp fill its list, sorted once
+        const int fill_end = min(np, RK_TOPK * NW);
+#pragma unroll 1
+        for (int pos = warp; pos < (fill_end + NW - 1) / NW * NW; pos += NW) {
+          int64_t e = RK_EMPTY;
+          if (pos < fill_end) {   // lanes without a valid point evaluate the box's corner
+            const int64_t x = pack_entry(acc_key(evaluate(pos)), (int)(progs[pos] >> 16));
+            e = valid ? x : RK_EMPTY;
+          }
+#pragma unroll
+          for (int q = 0; q + 1 < RK_TOPK; q++) tk.k[q] = tk.k[q + 1];
+          tk.k[RK_TOPK - 1] = e;
+        }
+        tk.sort();
+        th.set(tk.k[RK_TOPK - 1]);
+        exchange();
+        // the programs of a run of one shape (term counts fixed at compile time) from pos
+        // on, until the warp must stop; returns the next position.  The flush and the
+        // exchange sit once in the run loop below, outside the per-shape code, which keeps
+        // the kernel's hot code small.
+        auto run_fixed = [&](auto c64, auto c32, int pos, int end) -> int {
+          constexpr int N64 = decltype(c64)::value, N32 = decltype(c32)::value;
+          while (pos < end) {
+            const uint4 N1 = leaf_of(progs[pos] & 0xFFFF);
+            const uint4 *r1 = (const uint4 *)(img + N1.y);
+            const uint4 c = r1[0];
+            uint32_t A1[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+            for (int i = 1; i <= N64; i++) term64(A1, r1[i]);
+#pragma unroll
+            for (int i = N64 + 1; i <= N64 + N32; i++) term32(A1, r1[i]);
+            const bool stop = offer(finish(A1, N1.z), pos);
+            pos += NW;
+            if (stop) break;
+          }
+          return pos;
+        };
+        auto run_generic = [&](int pos, int end) -> int {
+          while (pos < end) {
+            const bool stop = offer(evaluate(pos), pos);
+            pos += NW;
+            if (stop) break;
+          }
+          return pos;
+        };
+        for (int r = 0; r < nruns; r++) {
+          const uint4 R = runs[r];
+          const int start = max((int)R.w, fill_end), end = r + 1 < nruns ? (int)runs[r + 1].w : np;
+          if (start >= end) continue;
+          int pos = start + ((warp - start % NW) + NW) % NW;   // this warp's first position
+          while (pos < end) {
+            switch (R.x) {
+#define PM_RUN(a, b) case (a) | ((b) << 8): pos = run_fixed(IC<a>{}, IC<b>{}, pos, end); break;
+              PM_RUN(0, 1) PM_RUN(0, 2) PM_RUN(0, 3) PM_RUN(1, 1) PM_RUN(1, 2) PM_RUN(1, 3) PM_RUN(1, 6)
+              PM_RUN(1, 10) PM_RUN(2, 1) PM_RUN(2, 2) PM_RUN(3, 2) PM_RUN(3, 3) PM_RUN(4, 2) PM_RUN(5, 1)
+#undef PM_RUN
+              default:
+                pos = run_generic(pos, end);
+            }
+            if (__any_sync(0xffffffffu, nbuf == RK_BUF)) flush();
+            if (since >= RK_EXCHANGE) {
+              since = 0;
+              exchange();
             }
           }
-          stop = stop || __any_sync(0xffffffffu, nbuf == RK_BUF);
         }
-        return stop;
-      };
-      // the first 16 programs of the warp fill its list, sorted once
-      const int fill_end = min(np, RK_TOPK * NW);
-#pragma unroll 1
-      for (int pos = warp; pos < (fill_end + NW - 1) / NW * NW; pos += NW) {
-        int64_t e = RK_EMPTY;
-        if (pos < fill_end) {   // lanes without a valid point evaluate the box's corner
-          const int64_t x = pack_entry(acc_key(evaluate(pos)), (int)(progs[pos] >> 16));
-          e = valid ? x : RK_EMPTY;
-        }
-#pragma unroll
-        for (int q = 0; q + 1 < RK_TOPK; q++) tk.k[q] = tk.k[q + 1];
-        tk.k[RK_TOPK - 1] = e;
-      }
-      tk.sort();
-      th.set(tk.k[RK_TOPK - 1]);
-      exchange();
-      // the programs of a run of one shape (term counts fixed at compile time) from pos
-      // on, until the warp must stop; returns the next position.  The flush and the
-      // exchange sit once in the run loop below, outside the per-shape code, which keeps
-      // the kernel's hot code small.
-      auto run_fixed = [&](auto c64, auto c32, int pos, int end) -> int {
-        constexpr int N64 = decltype(c64)::value, N32 = decltype(c32)::value;
-        while (pos < end) {
-          const uint4 N1 = leaf_of(progs[pos] & 0xFFFF);
-          const uint4 *r1 = (const uint4 *)(img + N1.y);
-          const uint4 c = r1[0];
-          uint32_t A1[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-          for (int i = 1; i <= N64; i++) term64(A1, r1[i]);
-#pragma unroll
-          for (int i = N64 + 1; i <= N64 + N32; i++) term32(A1, r1[i]);
-          const bool stop = offer(finish(A1, N1.z), pos);
-          pos += NW;
-          if (stop) break;
-        }
-        return pos;
-      };
-      auto run_generic = [&](int pos, int end) -> int {
-        while (pos < end) {
-          const bool stop = offer(evaluate(pos), pos);
-          pos += NW;
-          if (stop) break;
-        }
-        return pos;
-      };
-      for (int r = 0; r < nruns; r++) {
-        const uint4 R = runs[r];
-        const int start = max((int)R.w, fill_end), end = r + 1 < nruns ? (int)runs[r + 1].w : np;
-        if (start >= end) continue;
-        int pos = start + ((warp - start % NW) + NW) % NW;   // this warp's first position
-        while (pos < end) {
-          switch (R.x) {
-#define PM_RUN(a, b) case (a) | ((b) << 8): pos = run_fixed(IC<a>{}, IC<b>{}, pos, end); break;
-            PM_RUN(0, 1) PM_RUN(0, 2) PM_RUN(0, 3) PM_RUN(1, 1) PM_RUN(1, 2) PM_RUN(1, 3) PM_RUN(1, 6)
-            PM_RUN(1, 10) PM_RUN(2, 1) PM_RUN(2, 2) PM_RUN(3, 2) PM_RUN(3, 3) PM_RUN(4, 2) PM_RUN(5, 1)
-#undef PM_RUN
-            default:
-              pos = run_generic(pos, end);
-          }
-          if (__any_sync(0xffffffffu, nbuf == RK_BUF)) flush();
-          if (since >= RK_EXCHANGE) {
-            since = 0;
-            exchange();
-          }
-        }
-      }
-      flush();
-      // merge the warps' lists in a tree (the basis is no longer read)
-      __syncthreads();
-#pragma unroll
-      for (int half = NW / 2; half > 0; half >>= 1) {
-        if (warp >= half && warp < 2 * half) {
-#pragma unroll
-          for (int q = 0; q < RK_TOPK; q++) lists[((warp - half) * RK_TOPK + q) * 32 + lane] = tk.k[q];
-        }
+        flush();
+        // merge the warps' lists in a tree (the basis is no longer read)
         __syncthreads();
-        if (warp < half) tk.merge(lists + warp * RK_TOPK * 32 + lane, 32);
+#pragma unroll
+        for (int half = NW / 2; half > 0; half >>= 1) {
+          if (warp >= half && warp < 2 * half) {
+#pragma unroll
+            for (int q = 0; q < RK_TOPK; q++) lists[((warp - half) * RK_TOPK + q) * 32 + lane] = tk.k[q];
+          }
+          __syncthreads();
+          if (warp < half) tk.merge(lists + warp * RK_TOPK * 32 + lane, 32);
+          __syncthreads();
+        }
+        if (warp == 0) {
+#pragma unroll
+          for (int q = 0; q < RK_TOPK; q++) lists[q * 32 + lane] = tk.k[q];
+        }
         __syncthreads();
       }
       // the best programs become the best variants: programs in order of their predictions,
       // those with equal keys merged by variant index; the warps share the points
-      if (warp == 0) {
-#pragma unroll
-        for (int q = 0; q < RK_TOPK; q++) lists[q * 32 + lane] = tk.k[q];
-      }
-      __syncthreads();
       if (lane % NW == warp) {
         const uint32_t *span = img + img[RankLayout::H_OFF_SPAN];
         const uint16_t *pvid = (const uint16_t *)(img + img[RankLayout::H_OFF_PVID]);
