@@ -398,17 +398,10 @@ extern "C" pm_status pm_fit_weights(pm_ctx *c, const int64_t *F, int64_t R, int3
   if (objective != PM_FIT_RELATIVE && objective != PM_FIT_ABSOLUTE) return pm_set_error(PM_ERR_INVALID_ARG, "objective");
   if (precision != PM_PREC_FP64 && precision != PM_PREC_BF16X3) return pm_set_error(PM_ERR_INVALID_ARG, "precision");
   void *scr = nullptr;
-  pm_status s = ctx_scratch(c, pmd::fit_scratch_bytes(R, k, M), &scr);
+  pm_status s = ctx_scratch(c, pmd::fit_scratch_bytes(R, M), &scr);
   if (s) return s;
-  if (!c->fit_host) {
-    CU(cudaMallocHost(&c->fit_host, 64 * (16 + 8 * 4)));
-  }
-  pmd::FitHost h;
-  h.info = (int *)c->fit_host;
-  h.ratio = (double *)((char *)c->fit_host + 64 * 16);
-  h.upd = h.ratio + 64;
-  h.rr = h.upd + 64;
-  h.bb = h.rr + 64;
+  if (!c->fit_host) CU(cudaMallocHost(&c->fit_host, 64 * pmd::FIT_REPORT_BYTES));
+  const pmd::FitHost h = pmd::fit_report(c->fit_host, M);
   cudaStream_t st = (cudaStream_t)stream;
   // PM_PREC_BF16X3: the Gram from three bf16 terms first; refinement with exact residuals
   // makes it accurate when cond(G) 2^-24 is well below one.  If some model's last
@@ -416,8 +409,7 @@ extern "C" pm_status pm_fit_weights(pm_ctx *c, const int64_t *F, int64_t R, int3
   // have), the fit is repeated with the exact digit Gram.
   int gram = precision == PM_PREC_BF16X3 ? 1 : 0;
   for (;;) {
-    CU(pmd::launch_fit(F, R, k, T, M, objective, gram, refine_steps, scr, W_out, &h, c->d_status, st));
-    CU(cudaStreamSynchronize(st));
+    CU(pmd::launch_fit(F, R, k, T, M, objective, gram, refine_steps, scr, W_out, c->fit_host, c->d_status, st));
     s = pm_sync_status(c, stream);
     if (s) return s;
     if (gram != 1 || refine_steps == 0) break;

@@ -337,7 +337,7 @@ __device__ __forceinline__ void xp_limb(uint32_t m256, uint32_t tmem, uint32_t (
   }
 }
 
-__device__ __noinline__ double xp_value_rare(uint32_t a, uint32_t b, uint32_t c, uint32_t d, int E) {
+static __device__ __noinline__ double xp_value_rare(uint32_t a, uint32_t b, uint32_t c, uint32_t d, int E) {
   Acc128 A;
   A.lo = (uint64_t)a | ((uint64_t)b << 32);
   A.hi = (uint64_t)c | ((uint64_t)d << 32);

@@ -7,13 +7,13 @@
 // in float-float arithmetic on the FP32 pipes (entries split exactly into hi + lo
 // pairs, error-free products by FMA, compensated sums; about 2^-44 relative) per row
 // chunk, chunks summed in FP64 (precision PM_PREC_FP64), or on the tensor cores from
-// three bf16 terms of A with FP32 accumulation (PM_PREC_BF16X3), or exactly from bf16
-// digits of a 47-bit fixed-point image of A when refinement on the three-term Gram
+// three bf16 terms with FP32 accumulation (PM_PREC_BF16X3, gram_pairs.cu), or exactly from
+// bf16 digits of a 47-bit fixed-point image of A when refinement on the three-term Gram
 // does not converge (gram_tc.cu);
 // the k x k systems are factored by FP64 Cholesky.  Iterative refinement then
 // recovers the accuracy: r = b - A x is formed from the exact fixed-point product
-// F w (the prediction kernel's arithmetic), t - F w in FP64 and float-float products
-// with 1/t (about 2^-45), the correction solves G d = A^T r with the same factor, and
+// F w (the prediction kernel itself, predict_exact.cu), t - F w in FP64 and float-float
+// products with 1/t (about 2^-45), the correction solves G d = A^T r with the same factor, and
 // x += d.  FP64 is kept to the Cholesky factors, the substitutions and the sums: this
 // GPU's FP64 pipe is narrow.
 #include <cuda_runtime.h>
@@ -22,6 +22,7 @@
 #include <algorithm>
 
 #include "eval_common.cuh"
+#include "float_float.cuh"
 #include "kernels.h"
 #include "pm.h"
 
@@ -54,37 +55,19 @@ __global__ void k_colmax(const int64_t *__restrict__ F, int64_t R, int k, unsign
 // exponent e_c with max |F_c| in [2^(e-1), 2^e) (0 for an all-zero column)
 __device__ __forceinline__ int col_exp(unsigned long long mx) { return mx ? 64 - __clzll((long long)mx) : 0; }
 
-// ---- U = F diag(2^-e) as float-float pairs: Uh = rn(F), Ul = rn(F - Uh), scaled exactly
+// ---- U = F diag(2^-e) as float-float pairs: Uh = rn(F), Ul = rn(F - Uh), scaled exactly;
+// rows of 32 floats, zero beyond column k
 __global__ void k_scale(const int64_t *__restrict__ F, int64_t R, int k, const unsigned long long *cmax,
                         float *__restrict__ Uh, float *__restrict__ Ul) {
-  const int64_t n = R * k;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(i % k);
-    const int64_t v = F[i];
+  const int c = threadIdx.x & 31;
+  const int e = c < k ? col_exp(cmax[c]) : 0;
+  const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < R; r += step) {
+    const int64_t v = c < k ? F[r * k + c] : 0;
     const float h = __ll2float_rn(v);
-    const float l = __ll2float_rn(v - (int64_t)h);
-    const int e = col_exp(cmax[c]);
-    Uh[i] = ldexpf(h, -e);
-    Ul[i] = ldexpf(l, -e);
+    Uh[r * 32 + c] = ldexpf(h, -e);
+    Ul[r * 32 + c] = ldexpf(__ll2float_rn(v - (int64_t)h), -e);
   }
-}
-
-// A double as a float-float pair (hi + lo within 2^-47 of x) with integer operations
-// when its exponent is in [-70, 120] (this GPU's FP64 pipe is narrow; timings,
-// predictions and residuals are well inside that range), else by FP64 conversions.
-__device__ __forceinline__ float2 ff_of_double(double x) {
-  const uint64_t b = (uint64_t)__double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7FF) - 1023;
-  if (e < -70 || e > 120) {
-    const float h = __double2float_rn(x);
-    return make_float2(h, __double2float_rn(x - (double)h));
-  }
-  const uint32_t sgn = (uint32_t)(b >> 32) & 0x80000000u;
-  const uint64_t m = b & 0xFFFFFFFFFFFFFull;                      // 52 fraction bits
-  // hi: the leading one and the next 23 bits (truncated); lo: the 29 bits below, rounded
-  const float h = __uint_as_float(sgn | ((uint32_t)(e + 127) << 23) | (uint32_t)(m >> 29));
-  const float l = __uint2float_rn((uint32_t)(m & 0x1FFFFFFFu)) * __uint_as_float((uint32_t)(e - 52 + 127) << 23);
-  return make_float2(h, sgn ? -l : l);
 }
 
 // 1/t for t > 0 as float-float (within ~2^-46): FP32 reciprocal, one Newton step with
@@ -106,63 +89,97 @@ __device__ __forceinline__ float2 ff_recip(double t) {
   return make_float2(hi, __fsub_rn(lo, __fsub_rn(hi, y)));
 }
 
-// ---- row factors as float-float: 1/t (relative) or 1 (absolute); beta = 1 or t.  The
-// residual kernel reuses the relative row factor as 1/t.
-__global__ void k_rowfac(const double *__restrict__ T, int64_t n, int objective, float2 *__restrict__ rf,
-                         float2 *__restrict__ beta, int *status) {
-  const int64_t big = __double_as_longlong(1e300);
+// ---- row factors as float-float, rows of ld floats: 1/t (relative) or 1 (absolute); beta
+// (if wanted) = 1 or t.  The residual pass reuses the relative row factor as 1/t.  Entries
+// beyond model M are zero.
+__global__ void k_rowfac(const double *__restrict__ T, int64_t R, int M, int ld, int objective, float *__restrict__ rfh,
+                         float *__restrict__ rfl, float *__restrict__ bh, float *__restrict__ bl, int *status) {
+  const int64_t big = __double_as_longlong(1e300), n = R * ld;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double t = T[i];
-    const int64_t tb = __double_as_longlong(t);   // 0 < t <= 1e300 (NaN excluded) by its bits
-    if (tb <= 0 || tb > big) {
-      atomicOr(status, ST_BAD_INPUT);
-      rf[i] = beta[i] = make_float2(0.f, 0.f);
-      continue;
+    const int64_t r = i / ld;
+    const int m = (int)(i - r * ld);
+    float2 f = make_float2(0.f, 0.f), b = f;
+    if (m < M) {
+      const double t = T[r * M + m];
+      const int64_t tb = __double_as_longlong(t);   // 0 < t <= 1e300 (NaN excluded) by its bits
+      if (tb <= 0 || tb > big) {
+        atomicOr(status, ST_BAD_INPUT);
+      } else if (objective == PM_FIT_RELATIVE) {
+        f = ff_recip(t);
+        b = make_float2(1.f, 0.f);
+      } else {
+        f = make_float2(1.f, 0.f);
+        b = ff_of_double(t);
+      }
     }
-    if (objective == PM_FIT_RELATIVE) {
-      rf[i] = ff_recip(t);
-      beta[i] = make_float2(1.f, 0.f);
-    } else {
-      rf[i] = make_float2(1.f, 0.f);
-      beta[i] = ff_of_double(t);
+    rfh[i] = f.x;
+    rfl[i] = f.y;
+    if (bh) {
+      bh[i] = b.x;
+      bl[i] = b.y;
     }
   }
 }
 
-// float-float helpers: error-free product by FMA, compensated accumulation
-__device__ __forceinline__ float2 ff_mul(float ah, float al, float bh, float bl) {
-  const float p = __fmul_rn(ah, bh);
-  float e = __fmaf_rn(ah, bh, -p);
-  e = __fmaf_rn(ah, bl, e);
-  e = __fmaf_rn(al, bh, e);
-  return make_float2(p, e);
-}
-__device__ __forceinline__ void ff_acc(float &s, float &c, float2 p) {
-  const float t = __fadd_rn(s, p.x);
-  const float z = __fsub_rn(t, s);
-  c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p.x, z)), p.y));
-  s = t;
-}
-
-// ---- per (model, column) maxima of |A_rc| = |U_rc| * rowfactor_rm (float bits, atomicMax)
-__global__ void k_acolmax(const float *__restrict__ U, const float2 *__restrict__ rf, int64_t R, int k, int M,
-                          int64_t rows_per_chunk, unsigned *__restrict__ amax) {
-  const int m = blockIdx.y;
-  const int64_t r0 = (int64_t)blockIdx.x * rows_per_chunk;
-  const int64_t r1 = min(R, r0 + rows_per_chunk);
-  const int c = threadIdx.x % 32, lr = threadIdx.x / 32;
-  float mx = 0.f;
-  if (c < k)
-    for (int64_t r = r0 + lr; r < r1; r += FIT_THREADS / 32) {
-      mx = fmaxf(mx, fabsf(__fmul_rn(U[r * k + c], rf[r * M + m].x)));
+// ---- per (model, column) maxima of |A_rc| = |U_rc| * rowfactor_rm, and per model of the
+// row factors (float bits, atomicMax).  A (max, x) matrix product: 32-row stages of U and of
+// the row factors in shared memory, 4 columns x 4 models per thread, the two halves of the
+// CTA on 16 rows each, so one 16-byte read feeds eight products.
+constexpr int AM_ROWS = 32;
+__global__ void __launch_bounds__(FIT_THREADS) k_acolmax(const float *__restrict__ U, const float *__restrict__ rf, int ld,
+                                                         int64_t R, int k, int M, unsigned *__restrict__ amax,
+                                                         unsigned *__restrict__ rmax) {
+  __shared__ __align__(16) float su[AM_ROWS][32], sr[AM_ROWS][64];
+  __shared__ unsigned best[64][33];
+  const int tid = threadIdx.x, cg = tid & 7, mg = (tid >> 3) & 15, half = tid >> 7;
+  for (int i = tid; i < 64 * 33; i += FIT_THREADS) (&best[0][0])[i] = 0;
+  for (int i = tid; i < AM_ROWS * 64; i += FIT_THREADS) (&sr[0][0])[i] = 0.f;
+  float mx[4][4], mr[4];
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    mr[i] = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; j++) mx[i][j] = 0.f;
+  }
+  for (int64_t rb = (int64_t)blockIdx.x * AM_ROWS; rb < R; rb += (int64_t)gridDim.x * AM_ROWS) {
+    const int nr = (int)min((int64_t)AM_ROWS, R - rb);
+    __syncthreads();
+    for (int i = tid; i < AM_ROWS * 8; i += FIT_THREADS) {
+      const int r = i >> 3, c = (i & 7) * 4;
+      const float4 x = r < nr ? *(const float4 *)(U + (rb + r) * 32 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+      *(float4 *)&su[r][c] = make_float4(fabsf(x.x), fabsf(x.y), fabsf(x.z), fabsf(x.w));
     }
-  __shared__ float red[FIT_THREADS];
-  red[threadIdx.x] = mx;
+    for (int i = tid; i < AM_ROWS * (ld / 4); i += FIT_THREADS) {
+      const int r = i / (ld / 4), m = (i - r * (ld / 4)) * 4;
+      *(float4 *)&sr[r][m] = r < nr ? *(const float4 *)(rf + (rb + r) * ld + m) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    if (mg * 4 < ld) {
+#pragma unroll 4
+      for (int r = half * (AM_ROWS / 2); r < (half + 1) * (AM_ROWS / 2); r++) {
+        const float4 u4 = *(const float4 *)&su[r][4 * cg], f4 = *(const float4 *)&sr[r][4 * mg];
+        const float u[4] = {u4.x, u4.y, u4.z, u4.w}, f[4] = {f4.x, f4.y, f4.z, f4.w};
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          mr[i] = fmaxf(mr[i], f[i]);
+#pragma unroll
+          for (int j = 0; j < 4; j++) mx[i][j] = fmaxf(mx[i][j], __fmul_rn(u[j], f[i]));
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    const int m = 4 * mg + i;
+    if (cg == 0) atomicMax(&best[m][32], __float_as_uint(mr[i]));   // non-negative floats order as integers
+#pragma unroll
+    for (int j = 0; j < 4; j++) atomicMax(&best[m][4 * cg + j], __float_as_uint(mx[i][j]));
+  }
   __syncthreads();
-  if (threadIdx.x < 32 && c < k) {
-    float t = 0.f;
-    for (int q = 0; q < FIT_THREADS / 32; q++) t = fmaxf(t, red[q * 32 + threadIdx.x]);
-    atomicMax(&amax[m * FIT_MAXK + c], __float_as_uint(t));   // non-negative floats order as integers
+  for (int i = tid; i < M * 33; i += FIT_THREADS) {
+    const int m = i / 33, c = i - m * 33;
+    if (c == 32) atomicMax(&rmax[m], best[m][32]);
+    else if (c < k) atomicMax(&amax[m * FIT_MAXK + c], best[m][c]);
   }
 }
 
@@ -186,8 +203,9 @@ __device__ __forceinline__ int acol_exp(unsigned bits) {
 // FP64 totals with atomics.
 constexpr int GB_COLS = 36, GB_BLOCKS = 9, GB_TASKS = 45, GB_GROUPS = 5;
 __global__ void __launch_bounds__(FIT_THREADS) k_gram(const float *__restrict__ Uh, const float *__restrict__ Ul,
-                                                      const float2 *__restrict__ rf, const float2 *__restrict__ bt,
-                                                      int64_t R, int k, int M, int64_t rows_per_chunk,
+                                                      const float *__restrict__ rfh, const float *__restrict__ rfl,
+                                                      const float *__restrict__ bh, const float *__restrict__ bl,
+                                                      int ld, int64_t R, int k, int M, int64_t rows_per_chunk,
                                                       const unsigned *__restrict__ amax, double *__restrict__ G,
                                                       double *__restrict__ rhs) {
   __shared__ __align__(16) float vh[FIT_ROWS][GB_COLS], vl[FIT_ROWS][GB_COLS];
@@ -214,13 +232,12 @@ __global__ void __launch_bounds__(FIT_THREADS) k_gram(const float *__restrict__ 
       float2 v = make_float2(0.f, 0.f);
       if (rr < nr) {
         if (cc < k) {
-          const int64_t o = (rb + rr) * k + cc;
-          const float2 r = rf[(rb + rr) * M + m];
-          v = ff_mul(Uh[o], Ul[o], r.x, r.y);
+          const int64_t o = (rb + rr) * 32 + cc, q = (rb + rr) * ld + m;
+          v = ff_mul(Uh[o], Ul[o], rfh[q], rfl[q]);
           v.x = ldexpf(v.x, -f[cc]);
           v.y = ldexpf(v.y, -f[cc]);
         } else if (cc == k) {
-          v = bt[(rb + rr) * M + m];
+          v = make_float2(bh[(rb + rr) * ld + m], bl[(rb + rr) * ld + m]);
         }
       }
       vh[rr][cc] = v.x;
@@ -255,224 +272,181 @@ __global__ void __launch_bounds__(FIT_THREADS) k_gram(const float *__restrict__ 
   }
 }
 
-// ---- Cholesky of each model's Gram (one warp per model), FP64.
+// L L^T d = g of one model by a warp, lane a owning row a: forward and backward substitution
+// column by column, each step one product with the diagonal's reciprocal in lane a and one
+// multiply-add in every lane below (or above) it.  Dead directions give 0.
+__device__ __forceinline__ double chol_substitute(const double (*L)[FIT_MAXK + 1], int k, unsigned dead, double g) {
+  const int a = threadIdx.x & 31;
+  const bool live = a < k && !((dead >> a) & 1);
+  const double inv = live ? 1.0 / L[a][a] : 0.0;
+  double s = live ? g : 0.0, y = 0.0;
+  for (int c = 0; c < k; c++) {
+    if (a == c) y = s * inv;
+    const double yc = __shfl_sync(0xffffffffu, y, c);
+    if (a > c) s -= L[a][c] * yc;
+  }
+  double t = y, d = 0.0;
+  for (int c = k - 1; c >= 0; c--) {
+    if (a == c) d = t * inv;
+    const double dc = __shfl_sync(0xffffffffu, d, c);
+    if (a < c) t -= L[c][a] * dc;
+  }
+  return live ? d : 0.0;
+}
+
+// the weights of scaled coordinates x (w_c = x_c 2^-e_c), and the sums of the pass that
+// follows cleared
+__device__ __forceinline__ void fit_publish(int m, int k, int M, double xa, const unsigned long long *cmax,
+                                            const unsigned *amax, double *W, double *g, double *rr, double *bb) {
+  const int a = threadIdx.x & 31;
+  if (a < k)
+    W[(int64_t)m * k + a] = cmax[a] ? ldexp(xa, -col_exp(cmax[a]) - acol_exp(amax[m * FIT_MAXK + a])) : 0.0;
+  g[(int64_t)m * FIT_MAXK + a] = 0;
+  if (a == 0) rr[m] = bb[m] = 0;
+}
+
+// ---- Cholesky of each model's Gram (one warp per model), FP64, and the first solution.
 // Columns whose scale exponent marks them all-zero are replaced by identity rows
 // (weight 0).  A pivot below tol * (largest diagonal) marks the model rank deficient
-// and its direction is dropped likewise.  Writes L (lower) and the first solution.
-__global__ void k_chol_solve(double *__restrict__ G, const double *__restrict__ rhs, int k, int M,
-                             const unsigned long long *cmax, double *__restrict__ x, int *__restrict__ info,
-                             double *__restrict__ diag_ratio) {
+// and its direction is dropped likewise.  Lane a holds row a; after each column the lanes
+// subtract its outer product from the columns to the right (independent multiply-adds, so
+// the FP64 latency is paid per column, not per term).
+__global__ void __launch_bounds__(32) k_chol_solve(double *__restrict__ G, const double *__restrict__ rhs, int k, int M,
+                                                   const unsigned long long *cmax, const unsigned *__restrict__ amax,
+                                                   double *__restrict__ x, int *__restrict__ info,
+                                                   double *__restrict__ diag_ratio, double *__restrict__ upd,
+                                                   double *__restrict__ W, double *__restrict__ g,
+                                                   double *__restrict__ rr, double *__restrict__ bb) {
   const int m = blockIdx.x;
-  if (m >= M) return;
   __shared__ double L[FIT_MAXK][FIT_MAXK + 1];
-  __shared__ double y[FIT_MAXK];
-  __shared__ int dead[FIT_MAXK];
-  const int lane = threadIdx.x;
+  const int a = threadIdx.x;
   double *Gm = G + (int64_t)m * FIT_MAXK * FIT_MAXK;
-  for (int i = lane; i < k * k; i += 32) {
-    const int a = i / k, b = i - a * k;
-    L[a][b] = a <= b ? Gm[a * FIT_MAXK + b] : Gm[b * FIT_MAXK + a];   // symmetric from the upper triangle
+  for (int i = a; i < FIT_MAXK * FIT_MAXK; i += 32) {
+    const int r = i / FIT_MAXK, c = i % FIT_MAXK;
+    L[r][c] = r < k && c < k ? (r <= c ? Gm[r * FIT_MAXK + c] : Gm[c * FIT_MAXK + r]) : 0.0;   // the upper triangle, mirrored
   }
-  if (lane < k) dead[lane] = cmax[lane] == 0;
+  const unsigned zero = __ballot_sync(0xffffffffu, a < k && cmax[a] == 0);
+  unsigned dead = zero;
   __syncwarp();
-  double dmax = 0;
-  for (int a = 0; a < k; a++) if (!dead[a]) dmax = fmax(dmax, L[a][a]);
+  double row[FIT_MAXK];
+#pragma unroll
+  for (int c = 0; c < FIT_MAXK; c++) row[c] = L[a][c];
+  double dmax = a < k && !((dead >> a) & 1) ? L[a][a] : 0.0;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
   const double tol = dmax * 1e-13;
   int rank = 0;
   double pmin = 1e300, pmax = 0;
-  for (int j = 0; j < k; j++) {
-    // L[j][j] = sqrt(G[j][j] - sum_{p<j} L[j][p]^2)
-    double d = L[j][j];
-    for (int p = 0; p < j; p++) d -= L[j][p] * L[j][p];
-    const bool drop = dead[j] || !(d > tol);
-    __syncwarp();
-    if (drop) {
-      if (lane == 0) { dead[j] = 1; L[j][j] = 1.0; }
-      if (lane < k && lane > j) L[lane][j] = 0.0;
-      if (lane < j) L[j][lane] = 0.0;
+#pragma unroll
+  for (int j = 0; j < FIT_MAXK; j++) {
+    if (j < k) {
+      const double d = __shfl_sync(0xffffffffu, row[j], j);
       __syncwarp();
-      continue;
+      if (((dead >> j) & 1) || !(d > tol)) {
+        dead |= 1u << j;
+        row[j] = 0.0;
+        if (a == j) {
+#pragma unroll
+          for (int c = 0; c <= j; c++) row[c] = c == j ? 1.0 : 0.0;
+        }
+      } else {
+        const double ljj = sqrt(d);
+        rank++;
+        pmin = fmin(pmin, ljj);
+        pmax = fmax(pmax, ljj);
+        row[j] = a > j ? row[j] / ljj : a == j ? ljj : row[j];
+        L[a][j] = row[j];
+        __syncwarp();
+#pragma unroll
+        for (int c = j + 1; c < FIT_MAXK; c++) row[c] -= row[j] * L[c][j];   // used for a >= c
+      }
     }
-    const double ljj = sqrt(d);
-    rank++;
-    pmin = fmin(pmin, ljj);
-    pmax = fmax(pmax, ljj);
-    if (lane > j && lane < k) {
-      double s = L[lane][j];
-      for (int p = 0; p < j; p++) s -= L[lane][p] * L[j][p];
-      L[lane][j] = s / ljj;
-    }
-    __syncwarp();
-    if (lane == 0) L[j][j] = ljj;
-    __syncwarp();
   }
-  // forward and back substitution (one lane), dead directions get 0
-  if (lane == 0) {
-    for (int a = 0; a < k; a++) {
-      double s = dead[a] ? 0.0 : rhs[(int64_t)m * FIT_MAXK + a];
-      for (int p = 0; p < a; p++) s -= L[a][p] * y[p];
-      y[a] = dead[a] ? 0.0 : s / L[a][a];
-    }
-    for (int a = k - 1; a >= 0; a--) {
-      double s = y[a];
-      for (int p = a + 1; p < k; p++) s -= L[p][a] * x[(int64_t)m * FIT_MAXK + p];
-      x[(int64_t)m * FIT_MAXK + a] = dead[a] ? 0.0 : s / L[a][a];
-    }
-    int nz = 0;
-    for (int a = 0; a < k; a++) nz += cmax[a] == 0;
-    unsigned mask = 0;
-    for (int a = 0; a < k; a++) mask |= (unsigned)dead[a] << a;
+  __syncwarp();
+#pragma unroll
+  for (int c = 0; c < FIT_MAXK; c++) L[a][c] = c <= a ? row[c] : 0.0;
+  __syncwarp();
+  const double xa = chol_substitute(L, k, dead, a < k ? rhs[(int64_t)m * FIT_MAXK + a] : 0.0);
+  x[(int64_t)m * FIT_MAXK + a] = xa;
+  fit_publish(m, k, M, xa, cmax, amax, W, g, rr, bb);
+  if (a == 0) {
+    const int nz = __popc(zero);
     info[m * 4 + 0] = rank;
     info[m * 4 + 1] = nz;
     info[m * 4 + 2] = rank < k - nz ? 1 : 0;
-    info[m * 4 + 3] = (int)mask;
+    info[m * 4 + 3] = (int)dead;
     diag_ratio[m] = pmin > 0 ? (pmax / pmin) * (pmax / pmin) : 1e300;
+    upd[m] = 0;
   }
-  __syncwarp();
-  for (int i = lane; i < k * k; i += 32) {
-    const int a = i / k, b = i - a * k;
-    Gm[a * FIT_MAXK + b] = b <= a ? L[a][b] : 0.0;   // keep L for the refinement solves
-  }
-  if (lane < k) Gm[lane * FIT_MAXK + lane] = L[lane][lane];
+  for (int i = a; i < FIT_MAXK * FIT_MAXK; i += 32) Gm[i] = L[i / FIT_MAXK][i % FIT_MAXK];   // L, for the refinement solves
 }
 
-// ---- weights from scaled coordinates: w_c = x_c * 2^-e_c
-__global__ void k_unscale(const double *__restrict__ x, int k, int M, const unsigned long long *cmax,
-                          const unsigned *__restrict__ amax, double *__restrict__ W) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= k * M) return;
-  const int m = i / k, c = i - m * k;
-  W[i] = cmax[c] ? ldexp(x[(int64_t)m * FIT_MAXK + c], -col_exp(cmax[c]) - acol_exp(amax[m * FIT_MAXK + c])) : 0.0;
-}
-
-// ---- residual q = (b - A x) scaled for A^T q, from the exact product p = F w:
-// relative: r = 1 - p / t = (t - p) (1/t), q = r / t;   absolute: r = t - p, q = r.
-// Also sums r^2 and b^2 (b = 1, or t).  Relative objective: t - p in FP64 (exact while
-// p is within a factor 2 of t), then float-float products with the row factor 1/t and
-// a float-float sum of r^2, so that one FP64 operation per element remains.
-__global__ void k_residual(const double *__restrict__ P, const double *__restrict__ T, const float2 *__restrict__ rf,
-                           int64_t R, int M, int objective, float2 *__restrict__ Q, double *__restrict__ rr,
-                           double *__restrict__ bb) {
-  __shared__ double s_r[64], s_b[64];
-  if (threadIdx.x < 64) { s_r[threadIdx.x] = 0; s_b[threadIdx.x] = 0; }
-  __syncthreads();
-  const int64_t n = R * M, stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool fixed_m = stride % M == 0;   // then every element of this thread has model i0 % M
-  float sr = 0.f, cr = 0.f;               // float-float sum of r^2 (relative)
-  double ar = 0, ab = 0;
-  int64_t cnt = 0;
-  for (int64_t i = i0; i < n; i += stride) {
-    const double t = T[i], p = P[i];
-    if (objective == PM_FIT_RELATIVE) {
-      const float2 d = ff_of_double(t - p), it = rf[i];
-      const float2 r = ff_mul(d.x, d.y, it.x, it.y);
-      Q[i] = ff_mul(r.x, r.y, it.x, it.y);
-      const float2 r2 = ff_mul(r.x, r.y, r.x, r.y);
-      if (fixed_m) {
-        ff_acc(sr, cr, r2);
-        cnt++;
-      } else {
-        const int m = (int)(i % M);
-        atomicAdd(&s_r[m], (double)r2.x + (double)r2.y);
-        atomicAdd(&s_b[m], 1.0);
-      }
-    } else {
-      const double r = t - p;
-      Q[i] = ff_of_double(r);
-      if (fixed_m) { ar += r * r; ab += t * t; }
-      else { const int m = (int)(i % M); atomicAdd(&s_r[m], r * r); atomicAdd(&s_b[m], t * t); }
-    }
-  }
-  if (fixed_m && i0 < n) {
-    if (objective == PM_FIT_RELATIVE) { ar = (double)sr + (double)cr; ab = (double)cnt; }
-    atomicAdd(&s_r[i0 % M], ar);
-    atomicAdd(&s_b[i0 % M], ab);
-  }
-  __syncthreads();
-  if (threadIdx.x < M && threadIdx.x < 64) {
-    atomicAdd(&rr[threadIdx.x], s_r[threadIdx.x]);
-    atomicAdd(&bb[threadIdx.x], s_b[threadIdx.x]);
-  }
-}
-
-// ---- g_m = U^T q_m  (float-float products and sums per chunk, FP64 totals).
-// Grid (row chunks, groups of 8 models): each feature value is read once for the 8
-// models of its CTA; thread (column c, row lane) keeps 8 compensated sums.
-constexpr int ATQ_MODELS = 8;
+// ---- g_m = U^T q_m  (float-float products and sums per chunk, FP64 totals): bound by the
+// twelve FP32 operations of each error-free product and compensated sum.  Grid (row chunks,
+// groups of 16 models); a thread owns two columns and eight models (lanes 0-15 and 16-31 of a
+// warp share the columns), so a row's 4 + 16 floats feed 16 products, and the eight warps
+// take every eighth row.
+constexpr int ATQ_MODELS = 16;
 __global__ void __launch_bounds__(FIT_THREADS) k_atq(const float *__restrict__ Uh, const float *__restrict__ Ul,
-                                                     const float2 *__restrict__ Q, int64_t R, int k, int M,
-                                                     int64_t rows_per_chunk, const unsigned *__restrict__ amax,
-                                                     double *__restrict__ g) {
-  const int m0 = blockIdx.y * ATQ_MODELS;
+                                                     const float *__restrict__ Qh, const float *__restrict__ Ql, int ld,
+                                                     int64_t R, int k, int M, int64_t rows_per_chunk,
+                                                     const unsigned *__restrict__ amax, double *__restrict__ g) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int c0 = 2 * (lane & 15), m0 = blockIdx.y * ATQ_MODELS + 8 * (lane >> 4);
   const int64_t r0 = (int64_t)blockIdx.x * rows_per_chunk;
   const int64_t r1 = min(R, r0 + rows_per_chunk);
-  const int c = threadIdx.x % 32, lane_r = threadIdx.x / 32;   // 8 row lanes x 32 columns
-  const int nm = min(ATQ_MODELS, M - m0);
-  float s[ATQ_MODELS], cc[ATQ_MODELS];
+  const bool has = m0 < ld;
+  float s[16], c[16];
 #pragma unroll
-  for (int j = 0; j < ATQ_MODELS; j++) s[j] = cc[j] = 0.f;
-  if (c < k) {
-    for (int64_t r = r0 + lane_r; r < r1; r += FIT_THREADS / 32) {
-      const float uh = Uh[r * k + c], ul = Ul[r * k + c];
-      const float2 *q = Q + r * M + m0;
+  for (int j = 0; j < 16; j++) s[j] = c[j] = 0.f;
+  if (has) {
+    for (int64_t r = r0 + warp; r < r1; r += FIT_THREADS / 32) {
+      const float2 uh = *(const float2 *)(Uh + r * 32 + c0), ul = *(const float2 *)(Ul + r * 32 + c0);
+      const float4 h0 = *(const float4 *)(Qh + r * ld + m0), h1 = *(const float4 *)(Qh + r * ld + m0 + 4);
+      const float4 l0 = *(const float4 *)(Ql + r * ld + m0), l1 = *(const float4 *)(Ql + r * ld + m0 + 4);
+      const float qh[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+      const float ql[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
 #pragma unroll
-      for (int j = 0; j < ATQ_MODELS; j++) {
-        if (j < nm) {
-          const float2 qj = q[j];
-          ff_acc(s[j], cc[j], ff_mul(uh, ul, qj.x, qj.y));
-        }
+      for (int j = 0; j < 8; j++) {
+        ff_acc(s[2 * j], c[2 * j], ff_mul(uh.x, ul.x, qh[j], ql[j]));
+        ff_acc(s[2 * j + 1], c[2 * j + 1], ff_mul(uh.y, ul.y, qh[j], ql[j]));
       }
     }
   }
-  __shared__ double red[FIT_THREADS / 32][ATQ_MODELS][32];
+  // the eight warps' sums of 32 columns x 16 models
+  __shared__ double red[FIT_THREADS / 32][32][17];
 #pragma unroll
-  for (int j = 0; j < ATQ_MODELS; j++) red[lane_r][j][c] = (double)s[j] + (double)cc[j];
+  for (int j = 0; j < 16; j++) red[warp][lane][j] = (double)s[j] + (double)c[j];
   __syncthreads();
-  for (int o = threadIdx.x; o < ATQ_MODELS * 32; o += FIT_THREADS) {
-    const int j = o / 32, col = o % 32;
-    if (j < nm && col < k) {
+  for (int o = tid; o < 32 * 16; o += FIT_THREADS) {
+    const int l = o >> 4, j = o & 15;
+    const int col = 2 * (l & 15) + (j & 1), m = blockIdx.y * ATQ_MODELS + 8 * (l >> 4) + (j >> 1);
+    if (m < M && col < k) {
       double tot = 0;
-      for (int q = 0; q < FIT_THREADS / 32; q++) tot += red[q][j][col];
-      atomicAdd(&g[(int64_t)(m0 + j) * FIT_MAXK + col], ldexp(tot, -acol_exp(amax[(m0 + j) * FIT_MAXK + col])));
+#pragma unroll
+      for (int w = 0; w < FIT_THREADS / 32; w++) tot += red[w][l][j];
+      atomicAdd(&g[(int64_t)m * FIT_MAXK + col], ldexp(tot, -acol_exp(amax[m * FIT_MAXK + col])));
     }
   }
 }
 
-// ---- x += L^-T L^-1 g per model; records |d| / |x|.  One warp per model, lane a owns
-// row a: the forward and backward substitutions run column by column, each step one
-// division by lane a and one multiply-add in every lane below (or above) it, so the
-// FP64 latency of a step is paid once per column, not once per term.
-__global__ void __launch_bounds__(32) k_refine_update(const double *__restrict__ Lall, const double *__restrict__ g,
-                                                      int k, int M, const int *__restrict__ info,
-                                                      double *__restrict__ x, double *__restrict__ upd) {
+// ---- x += L^-T L^-1 g per model (one warp each); records |d| / |x|, and publishes the
+// weights for the next residual pass.
+__global__ void __launch_bounds__(32) k_refine_update(const double *__restrict__ Lall, double *__restrict__ g, int k, int M,
+                                                      const int *__restrict__ info, const unsigned long long *cmax,
+                                                      const unsigned *__restrict__ amax, double *__restrict__ x,
+                                                      double *__restrict__ upd, double *__restrict__ W,
+                                                      double *__restrict__ rr, double *__restrict__ bb) {
   const int m = blockIdx.x, a = threadIdx.x;
-  if (m >= M) return;
-  const unsigned dead = (unsigned)info[m * 4 + 3];
-  const double *L = Lall + (int64_t)m * FIT_MAXK * FIT_MAXK;
-  const bool live = a < k;
-  const double diag = live ? L[a * FIT_MAXK + a] : 1.0;
-  // L y = g: s_a = g_a - sum_{p<a} L[a][p] y_p, subtracted in the order p = 0, 1, ...
-  double s = (live && !((dead >> a) & 1)) ? g[(int64_t)m * FIT_MAXK + a] : 0.0;
-  double y = 0.0;
-  for (int c = 0; c < k; c++) {
-    if (a == c) y = s / diag;
-    const double yc = __shfl_sync(0xffffffffu, y, c);
-    if (live && a > c) s -= L[a * FIT_MAXK + c] * yc;
-  }
-  // L^T d = y: t_a = y_a - sum_{p>a} L[p][a] d_p
-  double t = y, d = 0.0;
-  for (int c = k - 1; c >= 0; c--) {
-    if (a == c) d = t / diag;
-    const double dc = __shfl_sync(0xffffffffu, d, c);
-    if (live && a < c) t -= L[c * FIT_MAXK + a] * dc;
-  }
-  if (!live || ((dead >> a) & 1)) d = 0.0;
-  double xa = 0.0;
-  if (live) {
-    xa = x[(int64_t)m * FIT_MAXK + a] + d;
-    x[(int64_t)m * FIT_MAXK + a] = xa;
-  }
+  __shared__ double L[FIT_MAXK][FIT_MAXK + 1];
+  const double *Lm = Lall + (int64_t)m * FIT_MAXK * FIT_MAXK;
+#pragma unroll 8
+  for (int r = 0; r < FIT_MAXK; r++) L[r][a] = Lm[r * FIT_MAXK + a];
+  __syncwarp();
+  const double d = chol_substitute(L, k, (unsigned)info[m * 4 + 3], a < k ? g[(int64_t)m * FIT_MAXK + a] : 0.0);
+  const double xa = x[(int64_t)m * FIT_MAXK + a] + d;
+  x[(int64_t)m * FIT_MAXK + a] = xa;
+  fit_publish(m, k, M, xa, cmax, amax, W, g, rr, bb);
   double dn = d * d, xn = xa * xa;
   for (int o = 16; o; o >>= 1) {
     dn += __shfl_xor_sync(0xffffffffu, dn, o);
@@ -483,17 +457,17 @@ __global__ void __launch_bounds__(32) k_refine_update(const double *__restrict__
 
 // ------------------------------------------------------------------------------------ host side
 
-size_t fit_scratch_bytes(int64_t R, int k, int M) {
+static int fit_ld(int M) { return (M + 7) & ~7; }   // row length of the row factors and residuals
+
+size_t fit_scratch_bytes(int64_t R, int M) {
   size_t b = 0;
   b += 256;                                        // cmax
-  b += (size_t)M * FIT_MAXK * 4;                   // amax
-  b += (size_t)R * k * 8;                          // Uh, Ul
-  b += (size_t)R * M * 16;                         // row factors, beta
-  b += (size_t)R * M * 8;                          // Q
-  b += (size_t)R * M * 8;                          // P
+  b += (size_t)M * (FIT_MAXK + 1) * 4;             // amax, rmax
+  b += (size_t)R * FIT_MAXK * 8;                   // Uh, Ul
+  b += (size_t)R * fit_ld(M) * 8 * 3;              // row factors, beta, Q (hi and lo)
   b += (size_t)M * FIT_MAXK * FIT_MAXK * 8;        // G / L
   b += (size_t)M * FIT_MAXK * 8 * 3;               // rhs, x, g
-  b += (size_t)M * (4 * 4 + 8 * 4);                // info, ratio, upd, rr, bb
+  b += (size_t)M * FIT_REPORT_BYTES;               // info, ratio, upd, rr, bb
   return b + 32 * 256;                             // every carve rounds up to 256 bytes
 }
 
@@ -504,77 +478,74 @@ static char *carve(char *&p, size_t bytes) {
 }
 
 cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int M, int objective, int gram,
-                       int steps, void *scratch, double *W_out, FitHost *host, int *status, cudaStream_t st) {
+                       int steps, void *scratch, double *W_out, void *h_report, int *status, cudaStream_t st) {
+  const int ld = fit_ld(M);
   char *p = (char *)scratch;
+  // cleared together: cmax, amax, rmax, G, rhs
+  char *zero = p;
   unsigned long long *cmax = (unsigned long long *)carve(p, 256);
   unsigned *amax = (unsigned *)carve(p, (size_t)M * FIT_MAXK * 4);
-  float *U = (float *)carve(p, (size_t)R * k * 4);
-  float *Ul = (float *)carve(p, (size_t)R * k * 4);
-  float2 *rf = (float2 *)carve(p, (size_t)R * M * 8);
-  float2 *bt = (float2 *)carve(p, (size_t)R * M * 8);
-  float2 *Q = (float2 *)carve(p, (size_t)R * M * 8);
-  double *P = (double *)carve(p, (size_t)R * M * 8);
+  unsigned *rmax = (unsigned *)carve(p, (size_t)M * 4);
   double *G = (double *)carve(p, (size_t)M * FIT_MAXK * FIT_MAXK * 8);
   double *rhs = (double *)carve(p, (size_t)M * FIT_MAXK * 8);
+  const size_t zero_bytes = (size_t)(p - zero);
+  float *U = (float *)carve(p, (size_t)R * FIT_MAXK * 4);
+  float *Ul = (float *)carve(p, (size_t)R * FIT_MAXK * 4);
+  float *rfh = (float *)carve(p, (size_t)R * ld * 4);
+  float *rfl = (float *)carve(p, (size_t)R * ld * 4);
+  float *bh = (float *)carve(p, (size_t)R * ld * 4);
+  float *bl = (float *)carve(p, (size_t)R * ld * 4);
+  float *Qh = (float *)carve(p, (size_t)R * ld * 4);
+  float *Ql = (float *)carve(p, (size_t)R * ld * 4);
   double *x = (double *)carve(p, (size_t)M * FIT_MAXK * 8);
   double *g = (double *)carve(p, (size_t)M * FIT_MAXK * 8);
-  int *info = (int *)carve(p, (size_t)M * 16);
-  double *ratio = (double *)carve(p, (size_t)M * 8);
-  double *upd = (double *)carve(p, (size_t)M * 8);
-  double *rr = (double *)carve(p, (size_t)M * 8);
-  double *bb = (double *)carve(p, (size_t)M * 8);
+  void *report = carve(p, (size_t)M * FIT_REPORT_BYTES);
+  const FitHost rep = fit_report(report, M);
   cudaError_t e;
-  cudaMemsetAsync(cmax, 0, 256, st);
-  cudaMemsetAsync(amax, 0, (size_t)M * FIT_MAXK * 4, st);
-  cudaMemsetAsync(G, 0, (size_t)M * FIT_MAXK * FIT_MAXK * 8, st);
-  cudaMemsetAsync(rhs, 0, (size_t)M * FIT_MAXK * 8, st);
-  cudaMemsetAsync(upd, 0, (size_t)M * 8, st);
+  if ((e = cudaMemsetAsync(zero, 0, zero_bytes, st)) != cudaSuccess) return e;
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  k_colmax<<<sms * 2, 256, 0, st>>>(F, R, k, cmax);
+  const bool relative = objective == PM_FIT_RELATIVE;
+  const bool beta = gram == 0 || !relative;   // else beta is 1 and the right-hand side takes the row factors
+  k_colmax<<<sms * 4, 256, 0, st>>>(F, R, k, cmax);
   k_scale<<<sms * 8, 256, 0, st>>>(F, R, k, cmax, U, Ul);
-  k_rowfac<<<sms * 8, 256, 0, st>>>(T, R * M, objective, rf, bt, status);
-  const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>(4 * sms / std::max(1, M) + 1, (R + 255) / 256));
-  const int64_t rpc = (R + chunks - 1) / chunks;
-  const int mchunks = (int)std::max<int64_t>(1, std::min<int64_t>(16 * sms / std::max(1, M) + 1, (R + 255) / 256));
-  k_acolmax<<<dim3(mchunks, M), FIT_THREADS, 0, st>>>(U, rf, R, k, M, (R + mchunks - 1) / mchunks, amax);
+  k_rowfac<<<sms * 8, 256, 0, st>>>(T, R, M, ld, objective, rfh, rfl, beta ? bh : nullptr, beta ? bl : nullptr, status);
+  k_acolmax<<<(int)std::min<int64_t>(sms * 4, (R + AM_ROWS - 1) / AM_ROWS), FIT_THREADS, 0, st>>>(U, rfh, ld, R, k, M, amax, rmax);
   const int groups = (M + ATQ_MODELS - 1) / ATQ_MODELS;
-  // enough row chunks for several CTAs per SM: the float-float sums are load-latency bound
-  const int achunks = (int)std::max<int64_t>(1, std::min<int64_t>(16 * sms / groups + 1, (R + 255) / 256));
+  const int achunks = (int)std::max<int64_t>(1, std::min<int64_t>(3 * sms / groups, (R + 63) / 64));
   const int64_t arpc = (R + achunks - 1) / achunks;
   if (gram != 0) {
-    // Gram on the tensor cores (three bf16 terms of A, or the exact digits of its 47-bit
-    // fixed-point image); right-hand side A^T b = U^T (rowfactor b) with the
+    // the Gram on the tensor cores; the right-hand side A^T b = U^T (rowfactor b) with the
     // float-float product kernel
-    if ((e = launch_gram_tc(U, Ul, rf, R, k, M, amax, G, gram == 2, status, st)) != cudaSuccess) return e;
-    k_atq<<<dim3(achunks, groups), FIT_THREADS, 0, st>>>(U, Ul, objective == PM_FIT_RELATIVE ? rf : bt, R, k, M,
-                                                         arpc, amax, rhs);
+    e = gram == 2 ? launch_gram_tc(U, Ul, rfh, rfl, ld, R, k, M, amax, G, sms, status, st)
+                  : launch_gram_pairs(U, rfh, rfl, ld, R, k, M, amax, rmax, G, sms, status, st);
+    if (e != cudaSuccess) return e;
+    k_atq<<<dim3(achunks, groups), FIT_THREADS, 0, st>>>(U, Ul, relative ? rfh : bh, relative ? rfl : bl, ld, R, k, M, arpc,
+                                                         amax, rhs);
   } else {
-    k_gram<<<dim3(chunks, M), FIT_THREADS, 0, st>>>(U, Ul, rf, bt, R, k, M, rpc, amax, G, rhs);
+    const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>(4 * sms / std::max(1, M) + 1, (R + 255) / 256));
+    k_gram<<<dim3(chunks, M), FIT_THREADS, 0, st>>>(U, Ul, rfh, rfl, bh, bl, ld, R, k, M, (R + chunks - 1) / chunks, amax, G, rhs);
   }
-  k_chol_solve<<<M, 32, 0, st>>>(G, rhs, k, M, cmax, x, info, ratio);
+  k_chol_solve<<<M, 32, 0, st>>>(G, rhs, k, M, cmax, amax, x, rep.info, rep.ratio, rep.upd, W_out, g, rep.rr, rep.bb);
+  FitResidual res;
+  res.T = T;
+  res.rfh = rfh;
+  res.rfl = rfl;
+  res.Qh = Qh;
+  res.Ql = Ql;
+  res.rr = rep.rr;
+  res.bb = rep.bb;
+  res.ld = ld;
+  res.relative = relative;
   for (int it = 0; it < steps; it++) {
-    k_unscale<<<(k * M + 255) / 256, 256, 0, st>>>(x, k, M, cmax, amax, W_out);
-    if ((e = launch_predict(F, R, k, W_out, M, PM_PREC_FP64, P, status, st)) != cudaSuccess) return e;
-    cudaMemsetAsync(rr, 0, (size_t)M * 8, st);
-    cudaMemsetAsync(bb, 0, (size_t)M * 8, st);
-    cudaMemsetAsync(g, 0, (size_t)M * FIT_MAXK * 8, st);
-    k_residual<<<sms * 4, 256, 0, st>>>(P, T, rf, R, M, objective, Q, rr, bb);
-    k_atq<<<dim3(achunks, groups), FIT_THREADS, 0, st>>>(U, Ul, Q, R, k, M, arpc, amax, g);
-    k_refine_update<<<M, 32, 0, st>>>(G, g, k, M, info, x, upd);
+    if ((e = launch_fit_residual(F, R, k, W_out, M, res, false, status, sms, st)) != cudaSuccess) return e;
+    k_atq<<<dim3(achunks, groups), FIT_THREADS, 0, st>>>(U, Ul, Qh, Ql, ld, R, k, M, arpc, amax, g);
+    k_refine_update<<<M, 32, 0, st>>>(G, g, k, M, rep.info, cmax, amax, x, rep.upd, W_out, rep.rr, rep.bb);
   }
-  k_unscale<<<(k * M + 255) / 256, 256, 0, st>>>(x, k, M, cmax, amax, W_out);
-  // final residual for the report
-  if ((e = launch_predict(F, R, k, W_out, M, PM_PREC_FP64, P, status, st)) != cudaSuccess) return e;
-  cudaMemsetAsync(rr, 0, (size_t)M * 8, st);
-  cudaMemsetAsync(bb, 0, (size_t)M * 8, st);
-  k_residual<<<sms * 4, 256, 0, st>>>(P, T, rf, R, M, objective, Q, rr, bb);
-  cudaMemcpyAsync(host->info, info, (size_t)M * 16, cudaMemcpyDeviceToHost, st);
-  cudaMemcpyAsync(host->ratio, ratio, (size_t)M * 8, cudaMemcpyDeviceToHost, st);
-  cudaMemcpyAsync(host->upd, upd, (size_t)M * 8, cudaMemcpyDeviceToHost, st);
-  cudaMemcpyAsync(host->rr, rr, (size_t)M * 8, cudaMemcpyDeviceToHost, st);
-  cudaMemcpyAsync(host->bb, bb, (size_t)M * 8, cudaMemcpyDeviceToHost, st);
+  // the final residual, for the report
+  if ((e = launch_fit_residual(F, R, k, W_out, M, res, true, status, sms, st)) != cudaSuccess) return e;
+  if ((e = cudaMemcpyAsync(h_report, report, (size_t)M * FIT_REPORT_BYTES, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
   return cudaGetLastError();
 }
 

@@ -95,6 +95,18 @@ cudaError_t launch_predict_exact(const int64_t *F, int64_t R, int k, const doubl
                                  int sms, cudaStream_t st);
 cudaError_t launch_argmin_exact(const int64_t *F, int64_t R, int k, const double *W, int M, ArgPart *part, int n_part,
                                 int *status, cudaStream_t st);
+// a residual pass of the fit: predictions p = F w, then the residuals of the measured times
+// T [R][M] as float-float (Qh, Ql), or (sums) the sums rr of their squares and bb of b^2
+struct FitResidual {
+  const double *T = nullptr;
+  const float *rfh = nullptr, *rfl = nullptr;   // 1 / t (relative)
+  float *Qh = nullptr, *Ql = nullptr;
+  double *rr = nullptr, *bb = nullptr;          // [M]
+  int ld = 0;                                   // row length of rf and Q: M rounded up to 8
+  int relative = 0;
+};
+cudaError_t launch_fit_residual(const int64_t *F, int64_t R, int k, const double *W, int M, const FitResidual &res,
+                                bool sums, int *status, int sms, cudaStream_t st);
 
 // top-k rows per (group, model): work units of at most TOPK_CHUNK positions of one
 // group; a group of one unit is written directly (part < 0), the partial lists of the
@@ -139,16 +151,24 @@ struct ServeArgs {
 cudaError_t launch_serve(const ServeArgs &a, int n_blocks, cudaStream_t st);
 
 // fit.cu
-struct FitHost {            // pinned host buffers filled by the fit (per model)
+struct FitHost {            // what the fit reports per model, copied to the host as one block
   int *info;                // [M][4] rank, zero columns, rank deficient, dropped-direction mask
   double *ratio, *upd, *rr, *bb;
 };
-size_t fit_scratch_bytes(int64_t R, int k, int M);
+constexpr size_t FIT_REPORT_BYTES = 16 + 4 * 8;   // per model
+inline FitHost fit_report(void *p, int M) {
+  double *d = (double *)((char *)p + (size_t)M * 16);
+  return FitHost{(int *)p, d, d + M, d + 2 * M, d + 3 * M};
+}
+size_t fit_scratch_bytes(int64_t R, int M);
+// gram: 0 float-float (k_gram), 1 three bf16 terms (k_gram_pairs), 2 exact digits (k_gram_tc)
 cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int M, int objective, int gram,
-                       int steps, void *scratch, double *W_out, FitHost *host, int *status, cudaStream_t st);
-// exact tensor-core Gram matrices of the fit (adds into G, upper triangle, [M][32][32])
-// gram: 0 float-float (k_gram), 1 three bf16 terms on the tensor cores, 2 exact bf16 digits
-cudaError_t launch_gram_tc(const float *Uh, const float *Ul, const float2 *rf, int64_t R, int k, int M,
-                           const unsigned *amax, double *G, int exact, int *status, cudaStream_t st);
+                       int steps, void *scratch, double *W_out, void *h_report, int *status, cudaStream_t st);
+// Gram matrices of the fit on the tensor cores (add into G, upper triangle, [M][32][32])
+cudaError_t launch_gram_pairs(const float *Uh, const float *rfh, const float *rfl, int ld, int64_t R, int k, int M,
+                              const unsigned *amax, const unsigned *rmax, double *G, int sms, int *status,
+                              cudaStream_t st);
+cudaError_t launch_gram_tc(const float *Uh, const float *Ul, const float *rfh, const float *rfl, int ld, int64_t R,
+                           int k, int M, const unsigned *amax, double *G, int sms, int *status, cudaStream_t st);
 
 }  // namespace pmd

@@ -1,4 +1,5 @@
-// FP64-accurate prediction T = F W^T and the per-model argmin on the tensor cores, from
+// FP64-accurate prediction T = F W^T on the tensor cores, as times, per-model argmin or the
+// residuals of the weight fit (Sec. 4.3), from
 // exact digit products (exact_tc.cuh has the number scheme and the operand layouts).
 //
 // One CTA of 16 warps per SM, persistent over 128-row tiles.  Per tile: the counts' digits
@@ -12,6 +13,7 @@
 #include <type_traits>
 
 #include "exact_tc.cuh"
+#include "float_float.cuh"
 #include "kernels.h"
 
 namespace pmd {
@@ -22,13 +24,34 @@ __device__ __forceinline__ int64_t xp_order(double t) {
   return b ^ ((b >> 63) & 0x7fffffffffffffffll);
 }
 
-// ARG false: write T (fp64 [R][M]).  ARG true: per-model minimum over the CTA's rows
-// (smaller time, then smaller row) -> part[blockIdx.x][M].
-template <class G, bool ARG>
+// XP_TIMES: write T (fp64 [R][M]).  XP_ARGMIN: per-model minimum over the CTA's rows
+// (smaller time, then smaller row) -> part[blockIdx.x][M].  The fit's residual passes, with
+// measured times t and predictions p (FitResidual): XP_RESIDUAL writes the residuals for
+// A^T r, relative (t - p) / t^2 or absolute t - p; XP_SUMS_REL and XP_SUMS_ABS add up the
+// squares of the residual, and of t (absolute).
+enum XpMode { XP_TIMES, XP_ARGMIN, XP_RESIDUAL, XP_SUMS_REL, XP_SUMS_ABS };
+
+// what a thread carries over its rows, for its two models of a pass
+template <int MODE> struct XpAcc {};
+template <> struct XpAcc<XP_ARGMIN> {
+  double t[2];
+  int64_t r[2];
+  __device__ XpAcc() { t[0] = t[1] = __longlong_as_double(0x7ff0000000000000ll); r[0] = r[1] = INT64_MAX; }
+};
+template <> struct XpAcc<XP_SUMS_REL> { float s[2] = {0, 0}, c[2] = {0, 0}; };
+template <> struct XpAcc<XP_SUMS_ABS> { double r[2] = {0, 0}, b[2] = {0, 0}; };
+// With two passes these wait in shared memory between tiles: in registers next to a pass's
+// limbs they would spill.
+template <class G, int MODE>
+constexpr size_t xp_stash() {
+  return G::PASSES > 1 && (MODE == XP_ARGMIN || MODE >= XP_SUMS_REL) ? 2 * 32 * XP_WARPS * sizeof(XpAcc<MODE>) : 0;
+}
+
+template <class G, int MODE>
 __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *__restrict__ F, int64_t R, int k,
                                                                  const double *__restrict__ W, int M,
                                                                  double *__restrict__ T, ArgPart *__restrict__ part,
-                                                                 int *status, uint32_t m256) {
+                                                                 int *status, uint32_t m256, FitResidual res) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((128u - (xp_saddr(smem_raw) & 127u)) & 127u);
   __shared__ __align__(8) uint64_t full[XP_RING], empty[XP_RING], digits[2];   // sums ready / read, a tile's digits ready
@@ -42,7 +65,8 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
   const int quarter = warp & 3, slice = warp >> 2;
   const int64_t ntiles = (R + XP_ROWS - 1) / XP_ROWS;
   const bool vec = (k & 1) == 0 && ((uintptr_t)F & 15) == 0;
-  const bool vst = (M & 1) == 0 && ((uintptr_t)T & 15) == 0;
+  const double *meas = MODE >= XP_RESIDUAL ? res.T : T;
+  const bool vst = (M & 1) == 0 && ((uintptr_t)meas & 15) == 0;   // (measured) times move in pairs
   const int row = xp_row<G>();   // this thread's row of a tile when it loads counts
 
   if (tid == 0) {
@@ -78,8 +102,11 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
   uint32_t it = 0;             // tiles so far
   bool ok = true;
   const bool active = warp < XP_WARPS && slice * 8 < G::NB;   // this warp has models
-  double bt[2][2];
-  int64_t br[2][2];
+  XpAcc<MODE> acc;   // one pass: in registers throughout
+  XpAcc<MODE> *stash = (XpAcc<MODE> *)(smem + G::SMEM - 128) + tid;   // [passes][working threads]
+  constexpr bool STASH = xp_stash<G, MODE>() != 0;
+  if (STASH && warp < XP_WARPS)
+    for (int ps = 0; ps < 2; ps++) stash[ps * 32 * XP_WARPS] = XpAcc<MODE>();
   if (warp == XP_WARPS) {
     // one thread issues, ahead of the working warps as far as digits and columns allow
     if (lane == 0) {
@@ -105,10 +132,6 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
     __syncwarp();
   } else {
     const int c0 = slice * 8 + 2 * (lane & 3);   // this thread's models of a pass: c0, c0 + 1
-    if (ARG) {
-#pragma unroll
-      for (int c = 0; c < 4; c++) { bt[c >> 1][c & 1] = __longlong_as_double(0x7ff0000000000000ll); br[c >> 1][c & 1] = INT64_MAX; }
-    }
     const uint32_t tread = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(slice * 8);
     // this warp's digits of the n-th tile are stored
     auto stored = [&](uint32_t n) {
@@ -125,7 +148,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
       seq++;
     };
     // the sums of one (tile, pass): four limbs, then the times
-    auto pass = [&](int ps, int64_t tile, double (&bt)[2], int64_t (&br)[2]) -> bool {
+    auto pass = [&](int ps, int64_t tile, XpAcc<MODE> &acc) -> bool {
       uint32_t limb[4][8];
       uint32_t cy[8];
       if (!wait()) return false;
@@ -158,7 +181,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
       const int64_t r0 = tile * XP_ROWS + quarter * 32 + (lane >> 2);   // this thread's rows: r0 + 8 i, i < 4
       const int left = (int)min((int64_t)XP_ROWS, R - r0);               // row r0 + 8 i exists for 8 i < left
       const int m = 32 * ps + c0;
-      double *out = ARG ? nullptr : T + r0 * M + m;
+      double *out = MODE == XP_TIMES ? T + r0 * M + m : nullptr;
       const int x0[2] = {1150 - s_E[m], 1150 - s_E[m + 1]};
       const bool wide = min(x0[0], x0[1]) < XP_XMIN || max(x0[0], x0[1]) > XP_XMAX;   // times may leave the normal range
       auto emit = [&](auto neg) {
@@ -175,10 +198,51 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
               t[e] = xp_value_rare(limb[0][2 * i + e], limb[1][2 * i + e], limb[2][2 * i + e], limb[3][2 * i + e], 1150 - x0[e]);
           }
           if (8 * i < left) {
-            if (ARG) {
+            if constexpr (MODE == XP_ARGMIN) {
 #pragma unroll
               for (int e = 0; e < 2; e++)   // rows come in increasing order: only a smaller time improves
-                if (xp_order(t[e]) < xp_order(bt[e])) { bt[e] = t[e]; br[e] = r0 + 8 * i; }
+                if (xp_order(t[e]) < xp_order(acc.t[e])) { acc.t[e] = t[e]; acc.r[e] = r0 + 8 * i; }
+            } else if constexpr (MODE != XP_TIMES) {
+              if (m < M) {
+                const double *tin = meas + (r0 + 8 * i) * M + m;
+                double tm[2] = {0, 0};
+                if (vst) {
+                  const double2 x = __ldcs((const double2 *)tin);
+                  tm[0] = x.x;
+                  tm[1] = x.y;
+                } else {
+                  tm[0] = __ldcs(tin);
+                  if (m + 1 < M) tm[1] = __ldcs(tin + 1);
+                }
+                if constexpr (MODE == XP_SUMS_ABS) {
+#pragma unroll
+                  for (int e = 0; e < 2; e++) {
+                    const double r = tm[e] - t[e];
+                    acc.r[e] = fma(r, r, acc.r[e]);
+                    acc.b[e] = fma(tm[e], tm[e], acc.b[e]);
+                  }
+                } else {
+                  const int64_t q = (r0 + 8 * i) * res.ld + m;
+                  // t - p in FP64 (exact while p is within a factor 2 of t), then float-float
+                  float2 d[2] = {ff_of_double(tm[0] - t[0]), ff_of_double(tm[1] - t[1])};
+                  if (MODE == XP_SUMS_REL || res.relative) {
+                    const float2 fh = *(const float2 *)(res.rfh + q), fl = *(const float2 *)(res.rfl + q);
+                    d[0] = ff_mul(d[0].x, d[0].y, fh.x, fl.x);
+                    d[1] = ff_mul(d[1].x, d[1].y, fh.y, fl.y);
+                    if constexpr (MODE == XP_SUMS_REL) {
+                      ff_acc(acc.s[0], acc.c[0], ff_mul(d[0].x, d[0].y, d[0].x, d[0].y));
+                      ff_acc(acc.s[1], acc.c[1], ff_mul(d[1].x, d[1].y, d[1].x, d[1].y));
+                    } else {
+                      d[0] = ff_mul(d[0].x, d[0].y, fh.x, fl.x);
+                      d[1] = ff_mul(d[1].x, d[1].y, fh.y, fl.y);
+                    }
+                  }
+                  if constexpr (MODE == XP_RESIDUAL) {
+                    *(float2 *)(res.Qh + q) = make_float2(d[0].x, d[1].x);
+                    *(float2 *)(res.Ql + q) = make_float2(d[0].y, d[1].y);
+                  }
+                }
+              }
             } else if (vst) {
               if (m < M) __stcs((double2 *)out, make_double2(t[0], t[1]));
             } else {
@@ -186,7 +250,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
               if (m + 1 < M) __stcs(out + 1, t[1]);
             }
           }
-          if (!ARG) out += 8 * M;
+          if (MODE == XP_TIMES) out += 8 * M;
         }
       };
       uint32_t sg = 0;
@@ -205,30 +269,31 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
       const int64_t off = (next * XP_ROWS + warp * (XP_ROWS / XP_WARPS)) * k * 8 + lane * 128;   // bytes: this warp's rows
       if (lane * 128 < (XP_ROWS / XP_WARPS) * k * 8 && off < R * k * 8)
         asm volatile("prefetch.global.L2 [%0];\n" ::"l"((const char *)F + off));
-      if (ARG) {   // the running minima of both passes stay in registers
-        if (!pass(0, tile, bt[0], br[0])) break;
-        if (G::PASSES > 1 && !pass(1, tile, bt[1], br[1])) break;
-      } else {
-        int ps = 0;
+      int ps = 0;
 #pragma unroll 1
-        for (; ps < G::PASSES; ps++)
-          if (!pass(ps, tile, bt[0], br[0])) break;
-        if (ps < G::PASSES) break;
+      for (; ps < G::PASSES; ps++) {
+        if (STASH) acc = stash[ps * 32 * XP_WARPS];
+        if (!pass(ps, tile, acc)) break;
+        if (STASH) stash[ps * 32 * XP_WARPS] = acc;
       }
+      if (ps < G::PASSES) break;
       // every MMA of this tile is complete: its operand buffer takes the tile after the next
       load(next);
       stored(it + 2);
     }
   }
-  if (ARG) {
+  if constexpr (MODE == XP_ARGMIN) {
     // the CTA's minimum per model over the 4 quarters x 8 row lanes, in the operand space
     ArgPart *red = (ArgPart *)smem;   // [32][64], 32 KB
     __syncthreads();
     if (active) {
 #pragma unroll
-      for (int c = 0; c < 4; c++)
-        red[(quarter * 8 + (lane >> 2)) * XP_MAXM + 32 * (c >> 1) + slice * 8 + 2 * (lane & 3) + (c & 1)] =
-            ArgPart{bt[c >> 1][c & 1], br[c >> 1][c & 1]};
+      for (int ps = 0; ps < G::PASSES; ps++) {
+        const XpAcc<MODE> x = STASH ? stash[ps * 32 * XP_WARPS] : acc;
+#pragma unroll
+        for (int e = 0; e < 2; e++)
+          red[(quarter * 8 + (lane >> 2)) * XP_MAXM + 32 * ps + slice * 8 + 2 * (lane & 3) + e] = ArgPart{x.t[e], x.r[e]};
+      }
     }
     __syncthreads();
     if (tid < M) {
@@ -241,6 +306,35 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
       part[(int64_t)blockIdx.x * M + tid] = b;
     }
   }
+  if constexpr (MODE >= XP_SUMS_REL) {
+    // the CTA's sums per model, in the operand space, then added to the totals
+    double *sum = (double *)smem;   // [64][2]
+    __syncthreads();
+    if (tid < 2 * XP_MAXM) sum[tid] = 0;
+    __syncthreads();
+    if (active) {
+#pragma unroll
+      for (int ps = 0; ps < G::PASSES; ps++) {
+        const XpAcc<MODE> x = STASH ? stash[ps * 32 * XP_WARPS] : acc;
+#pragma unroll
+        for (int e = 0; e < 2; e++) {
+          const int m = 32 * ps + slice * 8 + 2 * (lane & 3) + e;
+          if constexpr (MODE == XP_SUMS_REL) {
+            atomicAdd(&sum[2 * m], (double)x.s[e] + (double)x.c[e]);
+          } else {
+            atomicAdd(&sum[2 * m], x.r[e]);
+            atomicAdd(&sum[2 * m + 1], x.b[e]);
+          }
+        }
+      }
+    }
+    __syncthreads();
+    if (tid < M) {
+      atomicAdd(&res.rr[tid], sum[2 * tid]);
+      if (MODE == XP_SUMS_ABS) atomicAdd(&res.bb[tid], sum[2 * tid + 1]);
+      else if (blockIdx.x == 0) res.bb[tid] = (double)R;   // b = 1 in every row
+    }
+  }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
   __syncthreads();
   if (warp == 0)
@@ -249,29 +343,39 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
 
 bool exact_tc_ok(int k, int M) { return k >= 1 && k <= XP_MAXK && M >= 1 && M <= XP_MAXM; }
 
-cudaError_t launch_predict_exact(const int64_t *F, int64_t R, int k, const double *W, int M, double *T, int *status,
-                                 int sms, cudaStream_t st) {
+template <int MODE>
+static cudaError_t launch_mode(const int64_t *F, int64_t R, int k, const double *W, int M, double *T, ArgPart *part,
+                               int grid, int *status, const FitResidual &res, cudaStream_t st) {
   return xp_dispatch(k, M, [&](auto g) {
     using G = decltype(g);
-    cudaError_t e = cudaFuncSetAttribute(k_predict_exact<G, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+    static_assert(G::SMEM >= 32 * XP_MAXM * sizeof(ArgPart) + 128, "the final reductions use the operand space");
+    constexpr size_t smem = G::SMEM + xp_stash<G, MODE>();
+    cudaError_t e = cudaFuncSetAttribute(k_predict_exact<G, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int grid = (int)std::min<int64_t>(sms, (R + XP_ROWS - 1) / XP_ROWS);
-    k_predict_exact<G, false><<<grid, XP_THREADS, G::SMEM, st>>>(F, R, k, W, M, T, nullptr, status, 256u);
+    k_predict_exact<G, MODE><<<grid, XP_THREADS, smem, st>>>(F, R, k, W, M, T, part, status, 256u, res);
     return cudaGetLastError();
   });
+}
+
+static int xp_grid(int64_t R, int sms) { return (int)std::max<int64_t>(1, std::min<int64_t>(sms, (R + XP_ROWS - 1) / XP_ROWS)); }
+
+cudaError_t launch_predict_exact(const int64_t *F, int64_t R, int k, const double *W, int M, double *T, int *status,
+                                 int sms, cudaStream_t st) {
+  return launch_mode<XP_TIMES>(F, R, k, W, M, T, nullptr, xp_grid(R, sms), status, FitResidual{}, st);
 }
 
 // per-CTA minima to part[n_part][M]; every entry is written (n_part CTAs, some without rows)
 cudaError_t launch_argmin_exact(const int64_t *F, int64_t R, int k, const double *W, int M, ArgPart *part, int n_part,
                                 int *status, cudaStream_t st) {
-  return xp_dispatch(k, M, [&](auto g) {
-    using G = decltype(g);
-    static_assert(G::SMEM >= 32 * XP_MAXM * sizeof(ArgPart) + 128, "the final reduction uses the operand space");
-    cudaError_t e = cudaFuncSetAttribute(k_predict_exact<G, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
-    if (e != cudaSuccess) return e;
-    k_predict_exact<G, true><<<n_part, XP_THREADS, G::SMEM, st>>>(F, R, k, W, M, nullptr, part, status, 256u);
-    return cudaGetLastError();
-  });
+  return launch_mode<XP_ARGMIN>(F, R, k, W, M, nullptr, part, n_part, status, FitResidual{}, st);
+}
+
+cudaError_t launch_fit_residual(const int64_t *F, int64_t R, int k, const double *W, int M, const FitResidual &res,
+                                bool sums, int *status, int sms, cudaStream_t st) {
+  const int grid = xp_grid(R, sms);
+  if (!sums) return launch_mode<XP_RESIDUAL>(F, R, k, W, M, nullptr, nullptr, grid, status, res, st);
+  if (res.relative) return launch_mode<XP_SUMS_REL>(F, R, k, W, M, nullptr, nullptr, grid, status, res, st);
+  return launch_mode<XP_SUMS_ABS>(F, R, k, W, M, nullptr, nullptr, grid, status, res, st);
 }
 
 }  // namespace pmd
