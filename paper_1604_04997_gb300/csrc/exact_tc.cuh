@@ -85,12 +85,27 @@ __device__ __forceinline__ uint64_t xp_desc(uint32_t saddr, uint32_t sbo) {
          (uint64_t)1 << 46;
 }
 
+// One MMA, issued by one elected lane of a converged warp.  The whole warp runs the issuing
+// loops with warp-uniform operands: inside a branch of one thread the operands are not known
+// to be uniform, and every MMA then waits about 150 cycles for its registers to be collected.
 __device__ __forceinline__ void xp_mma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+      "{\n.reg .pred p, e;\nsetp.ne.u32 p, %4, 0;\nelect.sync _|e, 0xffffffff;\n"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      : "memory");
 }
+
+// the same lane's commit of its MMAs so far: one arrival at mbar when they are complete
+__device__ __forceinline__ void xp_commit(uint32_t mbar) {
+  asm volatile(
+      "{\n.reg .pred e;\nelect.sync _|e, 0xffffffff;\n"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(mbar)
+      : "memory");
+}
+
+// a value that is the same in all lanes, known as such to the compiler
+__device__ __forceinline__ uint32_t xp_uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
 
 // 16 TMEM lanes x 8 columns: thread t holds lanes t/4 and t/4 + 8, columns 2 (t%4) and + 1
 // as words {0, 1} (lane t/4) and {2, 3} (lane t/4 + 8)
@@ -249,13 +264,12 @@ __device__ __forceinline__ int xp_tile_digits(const int *s_nd) {
 // groups of diagonals that have any digit product, for nd digits (a prefix of the four)
 __device__ __forceinline__ int xp_groups(int nd) { return nd >= 6 ? 4 : nd >= 2 ? 3 : 2; }
 
-// Issue group gr's MMAs into TMEM columns tmem .. (one thread; s0: the operands' shared
-// address, sA: the tile's digits, sB: the pass's weight digits).  Their completion and this thread's own arrival complete
-// one phase of mbar (two arrivals): whoever waits for it sees the sums and everything this
-// thread has seen.
+// Issue group gr's MMAs into TMEM columns tmem .. (a whole warp; s0: the operands' shared
+// address, sA: the tile's digits, sB: the pass's weight digits).  Their completion and the
+// issuing lane's own arrival complete one phase of mbar (two arrivals): whoever waits for it
+// sees the sums and everything the issuing warp has seen.
 template <class G>
-__device__ __forceinline__ void xp_issue(uint32_t s0, uint32_t sA, uint32_t sB, uint32_t tmem, int gr,
-                                         int nd, uint32_t mbar) {
+__device__ __forceinline__ void xp_issue(uint32_t s0, uint32_t sA, uint32_t sB, uint32_t tmem, int gr, int nd, uint32_t mbar) {
   // kind::f16: D fp32, A and B f16, both K-major; the fourth diagonal of group 3 is empty
   const uint32_t n = (uint32_t)((gr == 3 ? 3 : 4) * G::NB);
   const uint32_t idesc = (1u << 4) | (n >> 3) << 17 | (uint32_t)(XP_ROWS >> 4) << 24;
@@ -264,10 +278,12 @@ __device__ __forceinline__ void xp_issue(uint32_t s0, uint32_t sA, uint32_t sB, 
   xp_mma(tmem, xp_desc(s0 + G::OFF_BIAS_A, 256), xp_desc(s0 + G::OFF_BIAS_B, 256), idesc, 0);
   for (int q = q0; q <= q1; q++) {
     const uint32_t a = sA + q * G::A_DIG, b = sB + (uint32_t)(3 + 4 * gr - q) * G::B_BLK;
+#pragma unroll
     for (int kc = 0; kc < G::KS; kc++) xp_mma(tmem, xp_desc(a + kc * 256, G::SBO), xp_desc(b + kc * 256, G::SBO), idesc, 1);
   }
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar));
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(mbar) : "memory");
+  xp_commit(mbar);
+  if ((threadIdx.x & 31) == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(mbar) : "memory");
+  __syncwarp();
 }
 
 // One poll of mbar's phase that lets the hardware suspend the warp for a few microseconds,

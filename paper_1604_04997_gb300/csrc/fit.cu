@@ -90,50 +90,26 @@ __device__ __forceinline__ float2 ff_recip(double t) {
 }
 
 // ---- row factors as float-float, rows of ld floats: 1/t (relative) or 1 (absolute); beta
-// (if wanted) = 1 or t.  The residual pass reuses the relative row factor as 1/t.  Entries
+// (if wanted) = 1 or t.  The residual passes reuse the relative row factor as 1/t.  Entries
 // beyond model M are zero.
-__global__ void k_rowfac(const double *__restrict__ T, int64_t R, int M, int ld, int objective, float *__restrict__ rfh,
-                         float *__restrict__ rfl, float *__restrict__ bh, float *__restrict__ bl, int *status) {
-  const int64_t big = __double_as_longlong(1e300), n = R * ld;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / ld;
-    const int m = (int)(i - r * ld);
-    float2 f = make_float2(0.f, 0.f), b = f;
-    if (m < M) {
-      const double t = T[r * M + m];
-      const int64_t tb = __double_as_longlong(t);   // 0 < t <= 1e300 (NaN excluded) by its bits
-      if (tb <= 0 || tb > big) {
-        atomicOr(status, ST_BAD_INPUT);
-      } else if (objective == PM_FIT_RELATIVE) {
-        f = ff_recip(t);
-        b = make_float2(1.f, 0.f);
-      } else {
-        f = make_float2(1.f, 0.f);
-        b = ff_of_double(t);
-      }
-    }
-    rfh[i] = f.x;
-    rfl[i] = f.y;
-    if (bh) {
-      bh[i] = b.x;
-      bl[i] = b.y;
-    }
-  }
-}
-
-// ---- per (model, column) maxima of |A_rc| = |U_rc| * rowfactor_rm, and per model of the
-// row factors (float bits, atomicMax).  A (max, x) matrix product: 32-row stages of U and of
-// the row factors in shared memory, 4 columns x 4 models per thread, the two halves of the
-// CTA on 16 rows each, so one 16-byte read feeds eight products.
+// From them the maxima per (model, column) of |A_rc| = |U_rc| * rowfactor_rm, and per model
+// of the row factors (float bits, atomicMax): a (max, x) matrix product over 32-row stages of
+// U and of the row factors in shared memory, 4 columns x 4 models per thread, the two halves
+// of the CTA on 16 rows each, so one 16-byte read feeds eight products.
 constexpr int AM_ROWS = 32;
-__global__ void __launch_bounds__(FIT_THREADS) k_acolmax(const float *__restrict__ U, const float *__restrict__ rf, int ld,
-                                                         int64_t R, int k, int M, unsigned *__restrict__ amax,
-                                                         unsigned *__restrict__ rmax) {
+__global__ void __launch_bounds__(FIT_THREADS) k_rowfac(const float *__restrict__ U, const double *__restrict__ T, int ld,
+                                                        int64_t R, int k, int M, int objective, float *__restrict__ rfh,
+                                                        float *__restrict__ rfl, float *__restrict__ bh,
+                                                        float *__restrict__ bl, unsigned *__restrict__ amax,
+                                                        unsigned *__restrict__ rmax, int *status) {
   __shared__ __align__(16) float su[AM_ROWS][32], sr[AM_ROWS][64];
   __shared__ unsigned best[64][33];
   const int tid = threadIdx.x, cg = tid & 7, mg = (tid >> 3) & 15, half = tid >> 7;
   for (int i = tid; i < 64 * 33; i += FIT_THREADS) (&best[0][0])[i] = 0;
   for (int i = tid; i < AM_ROWS * 64; i += FIT_THREADS) (&sr[0][0])[i] = 0.f;
+  const int64_t big = __double_as_longlong(1e300);
+  const int m4 = ld / 4, inv4 = (65536 + m4 - 1) / m4;   // i / m4 = i inv4 / 2^16 for i < 512
+  const bool vec = (M & 1) == 0 && ((uintptr_t)T & 15) == 0;
   float mx[4][4], mr[4];
 #pragma unroll
   for (int i = 0; i < 4; i++) {
@@ -149,9 +125,47 @@ __global__ void __launch_bounds__(FIT_THREADS) k_acolmax(const float *__restrict
       const float4 x = r < nr ? *(const float4 *)(U + (rb + r) * 32 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
       *(float4 *)&su[r][c] = make_float4(fabsf(x.x), fabsf(x.y), fabsf(x.z), fabsf(x.w));
     }
-    for (int i = tid; i < AM_ROWS * (ld / 4); i += FIT_THREADS) {
-      const int r = i / (ld / 4), m = (i - r * (ld / 4)) * 4;
-      *(float4 *)&sr[r][m] = r < nr ? *(const float4 *)(rf + (rb + r) * ld + m) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = tid; i < AM_ROWS * m4; i += FIT_THREADS) {   // four models of a row per thread
+      const int r = (i * inv4) >> 16, m = (i - r * m4) * 4;
+      double t[4] = {1, 1, 1, 1};
+      if (r < nr) {
+        const double *src = T + (rb + r) * M + m;
+        if (vec && m + 3 < M) {
+          const double2 x = __ldcs((const double2 *)src), y = __ldcs((const double2 *)src + 1);
+          t[0] = x.x, t[1] = x.y, t[2] = y.x, t[3] = y.y;
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; e++)
+            if (m + e < M) t[e] = __ldcs(src + e);
+        }
+      }
+      float fh[4], fl[4], gh[4], gl[4];
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        float2 x = make_float2(0.f, 0.f), b = x;
+        const int64_t tb = __double_as_longlong(t[e]);   // 0 < t <= 1e300 (NaN excluded) by its bits
+        if (r >= nr || m + e >= M) {
+        } else if (tb <= 0 || tb > big) {
+          atomicOr(status, ST_BAD_INPUT);
+        } else if (objective == PM_FIT_RELATIVE) {
+          x = ff_recip(t[e]);
+          b = make_float2(1.f, 0.f);
+        } else {
+          x = make_float2(1.f, 0.f);
+          b = ff_of_double(t[e]);
+        }
+        fh[e] = x.x, fl[e] = x.y, gh[e] = b.x, gl[e] = b.y;
+      }
+      *(float4 *)&sr[r][m] = make_float4(fh[0], fh[1], fh[2], fh[3]);
+      if (r < nr) {
+        const int64_t o = (rb + r) * ld + m;
+        *(float4 *)(rfh + o) = make_float4(fh[0], fh[1], fh[2], fh[3]);
+        *(float4 *)(rfl + o) = make_float4(fl[0], fl[1], fl[2], fl[3]);
+        if (bh) {
+          *(float4 *)(bh + o) = make_float4(gh[0], gh[1], gh[2], gh[3]);
+          *(float4 *)(bl + o) = make_float4(gl[0], gl[1], gl[2], gl[3]);
+        }
+      }
     }
     __syncthreads();
     if (mg * 4 < ld) {
@@ -305,12 +319,27 @@ __device__ __forceinline__ void fit_publish(int m, int k, int M, double xa, cons
   if (a == 0) rr[m] = bb[m] = 0;
 }
 
+// 1/sqrt(d) to FP64 accuracy from the FP32 value by Newton's iteration (each step squares
+// the relative error: 2^-22, 2^-43, below 2^-52), a fraction of the FP64 root and quotient on
+// this GPU.  Pivots lie in FP32's normal range: above 1e-13 of the largest diagonal entry,
+// which is at least 1/4 (scaled columns) and at most the row count.
+__device__ __forceinline__ double rsqrt_newton(double d) {
+  double y = (double)rsqrtf((float)d);
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    const double e = fma(-d * y, y, 1.0);
+    y = fma(0.5 * y, e, y);
+  }
+  return y;
+}
+
 // ---- Cholesky of each model's Gram (one warp per model), FP64, and the first solution.
 // Columns whose scale exponent marks them all-zero are replaced by identity rows
 // (weight 0).  A pivot below tol * (largest diagonal) marks the model rank deficient
-// and its direction is dropped likewise.  Lane a holds row a; after each column the lanes
+// and its direction is dropped likewise.  Lane a owns row a; after each column the lanes
 // subtract its outer product from the columns to the right (independent multiply-adds, so
-// the FP64 latency is paid per column, not per term).
+// the FP64 latency is paid per column, not per term; unrolled over all columns the code
+// outgrows the instruction cache).
 __global__ void __launch_bounds__(32) k_chol_solve(double *__restrict__ G, const double *__restrict__ rhs, int k, int M,
                                                    const unsigned long long *cmax, const unsigned *__restrict__ amax,
                                                    double *__restrict__ x, int *__restrict__ info,
@@ -328,43 +357,45 @@ __global__ void __launch_bounds__(32) k_chol_solve(double *__restrict__ G, const
   const unsigned zero = __ballot_sync(0xffffffffu, a < k && cmax[a] == 0);
   unsigned dead = zero;
   __syncwarp();
-  double row[FIT_MAXK];
-#pragma unroll
-  for (int c = 0; c < FIT_MAXK; c++) row[c] = L[a][c];
   double dmax = a < k && !((dead >> a) & 1) ? L[a][a] : 0.0;
 #pragma unroll
   for (int o = 16; o; o >>= 1) dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
   const double tol = dmax * 1e-13;
   int rank = 0;
   double pmin = 1e300, pmax = 0;
-#pragma unroll
-  for (int j = 0; j < FIT_MAXK; j++) {
-    if (j < k) {
-      const double d = __shfl_sync(0xffffffffu, row[j], j);
+#pragma unroll 1
+  for (int j = 0; j < k; j++) {
+    const double d = L[j][j];
+    __syncwarp();
+    if (((dead >> j) & 1) || !(d > tol)) {
+      dead |= 1u << j;
+      if (a > j) L[a][j] = 0.0;
+      if (a <= j) L[j][a] = a == j ? 1.0 : 0.0;
+    } else {
+      const double inv = rsqrt_newton(d), ljj = d * inv;
+      rank++;
+      pmin = fmin(pmin, ljj);
+      pmax = fmax(pmax, ljj);
+      const double l = a > j ? L[a][j] * inv : a == j ? ljj : 0.0;
+      if (a >= j) L[a][j] = l;
       __syncwarp();
-      if (((dead >> j) & 1) || !(d > tol)) {
-        dead |= 1u << j;
-        row[j] = 0.0;
-        if (a == j) {
+      for (int c0 = j + 1; c0 < k; c0 += 8) {   // eight columns at a time, their loads ahead of the stores
+        double own[8], col[8];
 #pragma unroll
-          for (int c = 0; c <= j; c++) row[c] = c == j ? 1.0 : 0.0;
+        for (int i = 0; i < 8; i++) {
+          const int c = min(c0 + i, FIT_MAXK - 1);
+          own[i] = L[a][c];
+          col[i] = L[c][j];
         }
-      } else {
-        const double ljj = sqrt(d);
-        rank++;
-        pmin = fmin(pmin, ljj);
-        pmax = fmax(pmax, ljj);
-        row[j] = a > j ? row[j] / ljj : a == j ? ljj : row[j];
-        L[a][j] = row[j];
-        __syncwarp();
 #pragma unroll
-        for (int c = j + 1; c < FIT_MAXK; c++) row[c] -= row[j] * L[c][j];   // used for a >= c
+        for (int i = 0; i < 8; i++)
+          if (c0 + i < k && a >= c0 + i) L[a][c0 + i] = own[i] - l * col[i];
       }
     }
+    __syncwarp();
   }
-  __syncwarp();
-#pragma unroll
-  for (int c = 0; c < FIT_MAXK; c++) L[a][c] = c <= a ? row[c] : 0.0;
+#pragma unroll 4
+  for (int c = a + 1; c < FIT_MAXK; c++) L[a][c] = 0.0;
   __syncwarp();
   const double xa = chol_substitute(L, k, dead, a < k ? rhs[(int64_t)m * FIT_MAXK + a] : 0.0);
   x[(int64_t)m * FIT_MAXK + a] = xa;
@@ -387,7 +418,7 @@ __global__ void __launch_bounds__(32) k_chol_solve(double *__restrict__ G, const
 // warp share the columns), so a row's 4 + 16 floats feed 16 products, and the eight warps
 // take every eighth row.
 constexpr int ATQ_MODELS = 16;
-__global__ void __launch_bounds__(FIT_THREADS) k_atq(const float *__restrict__ Uh, const float *__restrict__ Ul,
+__global__ void __launch_bounds__(FIT_THREADS, 2) k_atq(const float *__restrict__ Uh, const float *__restrict__ Ul,
                                                      const float *__restrict__ Qh, const float *__restrict__ Ql, int ld,
                                                      int64_t R, int k, int M, int64_t rows_per_chunk,
                                                      const unsigned *__restrict__ amax, double *__restrict__ g) {
@@ -396,11 +427,18 @@ __global__ void __launch_bounds__(FIT_THREADS) k_atq(const float *__restrict__ U
   const int64_t r0 = (int64_t)blockIdx.x * rows_per_chunk;
   const int64_t r1 = min(R, r0 + rows_per_chunk);
   const bool has = m0 < ld;
-  float s[16], c[16];
+  // this thread's sums so far; a compensated sum's error grows with the square of its length,
+  // so runs of 64 rows are added up in float-float
+  __shared__ float2 red[FIT_THREADS / 32][32][17];
 #pragma unroll
-  for (int j = 0; j < 16; j++) s[j] = c[j] = 0.f;
-  if (has) {
-    for (int64_t r = r0 + warp; r < r1; r += FIT_THREADS / 32) {
+  for (int j = 0; j < 16; j++) red[warp][lane][j] = make_float2(0.f, 0.f);
+  for (int64_t rb = r0 + warp; has && rb < r1; rb += 64 * (FIT_THREADS / 32)) {
+    const int64_t re = min(r1, rb + 64 * (FIT_THREADS / 32));
+    float s[16], c[16];
+#pragma unroll
+    for (int j = 0; j < 16; j++) s[j] = c[j] = 0.f;
+#pragma unroll 2
+    for (int64_t r = rb; r < re; r += FIT_THREADS / 32) {
       const float2 uh = *(const float2 *)(Uh + r * 32 + c0), ul = *(const float2 *)(Ul + r * 32 + c0);
       const float4 h0 = *(const float4 *)(Qh + r * ld + m0), h1 = *(const float4 *)(Qh + r * ld + m0 + 4);
       const float4 l0 = *(const float4 *)(Ql + r * ld + m0), l1 = *(const float4 *)(Ql + r * ld + m0 + 4);
@@ -412,20 +450,24 @@ __global__ void __launch_bounds__(FIT_THREADS) k_atq(const float *__restrict__ U
         ff_acc(s[2 * j + 1], c[2 * j + 1], ff_mul(uh.y, ul.y, qh[j], ql[j]));
       }
     }
-  }
-  // the eight warps' sums of 32 columns x 16 models
-  __shared__ double red[FIT_THREADS / 32][32][17];
 #pragma unroll
-  for (int j = 0; j < 16; j++) red[warp][lane][j] = (double)s[j] + (double)c[j];
+    for (int j = 0; j < 16; j++) {
+      float2 t = red[warp][lane][j];
+      ff_acc(t.x, t.y, make_float2(s[j], c[j]));
+      red[warp][lane][j] = t;
+    }
+  }
   __syncthreads();
+  // the eight warps' sums of 32 columns x 16 models
   for (int o = tid; o < 32 * 16; o += FIT_THREADS) {
     const int l = o >> 4, j = o & 15;
     const int col = 2 * (l & 15) + (j & 1), m = blockIdx.y * ATQ_MODELS + 8 * (l >> 4) + (j >> 1);
     if (m < M && col < k) {
-      double tot = 0;
+      float ts = 0.f, tc = 0.f;
 #pragma unroll
-      for (int w = 0; w < FIT_THREADS / 32; w++) tot += red[w][l][j];
-      atomicAdd(&g[(int64_t)m * FIT_MAXK + col], ldexp(tot, -acol_exp(amax[m * FIT_MAXK + col])));
+      for (int w = 0; w < FIT_THREADS / 32; w++) ff_acc(ts, tc, red[w][l][j]);
+      atomicAdd(&g[(int64_t)m * FIT_MAXK + col],
+                ldexp((double)ts + (double)tc, -acol_exp(amax[m * FIT_MAXK + col])));
     }
   }
 }
@@ -510,10 +552,11 @@ cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int 
   const bool beta = gram == 0 || !relative;   // else beta is 1 and the right-hand side takes the row factors
   k_colmax<<<sms * 4, 256, 0, st>>>(F, R, k, cmax);
   k_scale<<<sms * 8, 256, 0, st>>>(F, R, k, cmax, U, Ul);
-  k_rowfac<<<sms * 8, 256, 0, st>>>(T, R, M, ld, objective, rfh, rfl, beta ? bh : nullptr, beta ? bl : nullptr, status);
-  k_acolmax<<<(int)std::min<int64_t>(sms * 4, (R + AM_ROWS - 1) / AM_ROWS), FIT_THREADS, 0, st>>>(U, rfh, ld, R, k, M, amax, rmax);
+  k_rowfac<<<(int)std::min<int64_t>(sms * 4, (R + AM_ROWS - 1) / AM_ROWS), FIT_THREADS, 0, st>>>(
+      U, T, ld, R, k, M, objective, rfh, rfl, beta ? bh : nullptr, beta ? bl : nullptr, amax, rmax, status);
   const int groups = (M + ATQ_MODELS - 1) / ATQ_MODELS;
-  const int achunks = (int)std::max<int64_t>(1, std::min<int64_t>(3 * sms / groups, (R + 63) / 64));
+  // one wave of two CTAs per SM: the sums are issue-bound, and a partial second wave idles
+  const int achunks = (int)std::max<int64_t>(1, std::min<int64_t>(2 * sms / groups, (R + 63) / 64));
   const int64_t arpc = (R + achunks - 1) / achunks;
   if (gram != 0) {
     // the Gram on the tensor cores; the right-hand side A^T b = U^T (rowfactor b) with the

@@ -13,10 +13,11 @@
 // well below 1; else it falls back to the exact Gram (gram_tc.cu).
 //
 // One CTA per SM takes one contiguous range of rows, in stages of 16 rows (one K-step): 16
-// warps write the stage's operands (pairs at rows 0 .. 639 in five 128-row tiles, models as
-// the N operand, K-major without swizzle, three terms each, 66 KB) into a ring of three, and
-// one thread issues its 30 MMAs (M = 128, N = models); bound by the shared-memory reads of
-// the MMAs (a 4 KB A tile per 48 cycles) and the split arithmetic.
+// warps write the stage's pairs (rows 0 .. 639 in five 128-row tiles), four its models (the N
+// operand), K-major without swizzle, three terms each, 66 KB, into a ring of three, and a
+// warp issues its 30 MMAs (M = 128, N = models).  Bound by the split arithmetic and the
+// shared-memory reads of the MMAs (a 4 KB A tile per 48 cycles); the inputs of later stages
+// are prefetched into L2 and, one or two stages ahead, into registers.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -30,7 +31,10 @@ namespace pmd {
 
 namespace {
 
-constexpr int GP_WARPS = 16, GP_WORK = 32 * GP_WARPS, GP_THREADS = GP_WORK + 32;
+constexpr int GP_WARPS = 16, GP_WORK = 32 * GP_WARPS;   // warps that write pairs
+constexpr int GP_BWARPS = 4;                            // warps that write models
+constexpr int GP_ISSUER = GP_WARPS + GP_BWARPS, GP_THREADS = 32 * (GP_ISSUER + 1);
+constexpr int GP_AHEAD = 8;           // stages whose inputs are on their way into L2
 constexpr int GP_K = 16;              // rows per stage
 constexpr int GP_RING = 3;
 constexpr int GP_SUB = 42 * GP_K;     // rows accumulated in FP32
@@ -107,7 +111,7 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
   }
   if (tid == 0) {
     for (int b = 0; b < GP_RING; b++) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(xp_saddr(&ready[b])), "n"(GP_WARPS));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(xp_saddr(&ready[b])), "n"(GP_WARPS + GP_BWARPS));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(xp_saddr(&freed[b])));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(xp_saddr(&summed)));
@@ -123,39 +127,84 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-  const uint32_t tmem = tmem_base;
+  const uint32_t tmem = xp_uniform(tmem_base), s0 = xp_uniform(xp_saddr(smem));
   bool ok = true;
   uint32_t n = 0, sub = 0;   // stages and FP32 sums so far
 
-  if (warp == GP_WARPS) {
-    if (lane == 0) {
-      // kind::f16: D fp32, A and B bf16, both K-major
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t)(nb >> 3) << 17 | (128u >> 4) << 24;
-      for (int64_t rb = r0; rb < r1 && ok; rb += GP_SUB, sub++) {
-        if (sub && !(ok = xp_wait_one(xp_saddr(&drained), (sub - 1) & 1, &s_abort))) break;
-        for (int64_t rs = rb; rs < min(r1, rb + GP_SUB); rs += GP_K, n++) {
-          const uint32_t b = n % GP_RING;
-          if (!(ok = xp_wait_one(xp_saddr(&ready[b]), (n / GP_RING) & 1, &s_abort))) break;
-          const uint32_t sa = xp_saddr(smem) + b * GP_STAGE, sb = sa + 3 * GP_ATERM;
-          for (int p = 0; p < 6; p++) {   // term products 11, 12, 21, 13, 22, 31
-            const uint32_t pa = p == 2 || p == 4 ? 1 : (p == 5 ? 2 : 0), pb = p == 1 || p == 4 ? 1 : (p == 3 ? 2 : 0);
-            for (int t = 0; t < tiles; t++)
+  if (warp == GP_ISSUER) {
+    // kind::f16: D fp32, A and B bf16, both K-major
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t)(nb >> 3) << 17 | (128u >> 4) << 24;
+    for (int64_t rb = r0; rb < r1 && ok; rb += GP_SUB, sub++) {
+      if (sub && !(ok = xp_wait(xp_saddr(&drained), (sub - 1) & 1, &s_abort))) break;
+      for (int64_t rs = rb; rs < min(r1, rb + GP_SUB); rs += GP_K, n++) {
+        const uint32_t b = n % GP_RING;
+        if (!(ok = xp_wait(xp_saddr(&ready[b]), (n / GP_RING) & 1, &s_abort))) break;
+        const uint32_t sa = s0 + b * GP_STAGE, sb = sa + 3 * GP_ATERM;
+#pragma unroll
+        for (int p = 0; p < 6; p++) {   // term products 11, 12, 21, 13, 22, 31
+          const uint32_t pa = p == 2 || p == 4 ? 1 : (p == 5 ? 2 : 0), pb = p == 1 || p == 4 ? 1 : (p == 3 ? 2 : 0);
+#pragma unroll
+          for (int t = 0; t < GP_TILES; t++)
+            if (t < tiles)
               xp_mma(tmem + t * 64, xp_desc(sa + pa * GP_ATERM + t * 4096, 256), xp_desc(sb + pb * GP_BTERM, 256), idesc,
-                     rs != rb || p != 0);
-          }
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(xp_saddr(&freed[b])));
+                     p != 0 || rs != rb);
         }
-        if (ok) asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(xp_saddr(&summed)));
+        xp_commit(xp_saddr(&freed[b]));
       }
-      if (!ok) {
-        if (status) atomicOr(status, ST_TIMEOUT);
-        // let the MMAs in flight finish before TMEM is freed (bounded)
-        const unsigned long long t0 = globaltimer_ns();
-        for (uint32_t i = n >= GP_RING ? n - GP_RING : 0; i < n; i++)
-          while (!xp_try(xp_saddr(&freed[i % GP_RING]), (i / GP_RING) & 1) && globaltimer_ns() - t0 < MBAR_WAIT_NS) {}
-      }
+      if (ok) xp_commit(xp_saddr(&summed));
+    }
+    if (!ok) {
+      if (lane == 0 && status) atomicOr(status, ST_TIMEOUT);
+      // let the MMAs in flight finish before TMEM is freed (bounded)
+      const unsigned long long t0 = globaltimer_ns();
+      for (uint32_t i = n >= GP_RING ? n - GP_RING : 0; i < n; i++)
+        while (!xp_try(xp_saddr(&freed[i % GP_RING]), (i / GP_RING) & 1) && globaltimer_ns() - t0 < MBAR_WAIT_NS) {}
     }
     __syncwarp();
+  } else if (warp >= GP_WARPS) {
+    // one row (8 rows of U of one model) of the N operand per thread: 64 models x 2 K-groups
+    const int mop = tid - GP_WORK, mm = mop & 63, mkg = mop >> 6;
+    const bool has = mm < M;
+    const float msc = has ? __uint_as_float((uint32_t)(127 - s_sh[mm]) << 23) : 0.f;   // 2^-sh
+    float nh[2][8], nl[2][8];   // two stages ahead
+    auto fetch = [&](int64_t rs, float (&h)[8], float (&l)[8]) {
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        const int64_t q = rs + mkg * 8 + i;
+        const bool in = has && q < r1;
+        h[i] = in ? rfh[q * ld + mm] : 0.f;
+        l[i] = in ? rfl[q * ld + mm] : 0.f;
+      }
+    };
+    auto stage = [&](int64_t rs, float (&h)[8], float (&l)[8]) {
+      const uint32_t buf = n % GP_RING;
+      float w[8];
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        const float x = __fmul_rn(h[i], msc), y = __fmul_rn(l[i], msc);
+        w[i] = __fmaf_rn(x, x, __fmul_rn(2.f, __fmul_rn(x, y)));
+      }
+      fetch(rs + 2 * GP_K, h, l);
+      if (n >= GP_RING) ok = xp_wait(xp_saddr(&freed[buf]), (n / GP_RING - 1) & 1, &s_abort);
+      if (!ok) return;
+      if (has) gp_store(w, smem + buf * GP_STAGE + 3 * GP_ATERM + (mm >> 3) * 256 + mkg * 128 + (mm & 7) * 16, GP_BTERM);
+      asm volatile("fence.proxy.async.shared::cta;\n" ::);
+      __syncwarp();
+      if (lane == 0) xp_arrive(xp_saddr(&ready[buf]));
+      n++;
+    };
+    fetch(r0, nh[0], nl[0]);
+    fetch(r0 + GP_K, nh[1], nl[1]);
+    for (int64_t rs = r0; rs < r1 && ok; rs += 2 * GP_K) {
+      // the row factors of a later pair of stages on their way: 32 rows, 128 bytes per prefetch
+      const int64_t off = ((rs + GP_AHEAD * GP_K) * ld + (int64_t)mop * 32) * 4;
+      if (mop < ld && off < R * ld * 4) {
+        asm volatile("prefetch.global.L2 [%0];\n" ::"l"((const char *)rfh + off));
+        asm volatile("prefetch.global.L2 [%0];\n" ::"l"((const char *)rfl + off));
+      }
+      stage(rs, nh[0], nl[0]);
+      if (rs + GP_K < r1 && ok) stage(rs + GP_K, nh[1], nl[1]);
+    }
   } else {
     // this thread's pair operations of a stage: 8 rows (K-group) of one pair; operation i
     // is pair 8 (i / 16) + i % 8, K-group (i / 8) % 2
@@ -169,36 +218,21 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
       op_src[j] = p < np ? (uint32_t)(a * GP_USTRIDE + kg * 8) | (uint32_t)(b * GP_USTRIDE + kg * 8) << 16 : 0xFFFFFFFFu;
       op_dst[j] = (uint32_t)((p >> 3) * 256 + kg * 128 + (p & 7) * 16);
     }
-    // models: the last four warps each write 32 of the 64 x 2 (model, K-group) rows
-    const int mop = tid - (GP_WORK - 128), mm = mop & 63, mkg = mop >> 6;
-    const bool has_m = mop >= 0 && mm < M;
-    const float msc = has_m ? __uint_as_float((uint32_t)(127 - s_sh[mm]) << 23) : 0.f;   // 2^-sh
-    float nu = 0.f, nh[8], nl[8];
-    auto fetch = [&](int64_t rs, int64_t re) {   // the stage at row rs: this thread's entry of U, its model's factors
+    auto fetch = [&](int64_t rs) {   // this thread's entry of the stage at row rs
       const int64_t r = rs + (tid >> 5);
-      nu = r < re ? Uh[r * 32 + lane] : 0.f;
-      if (has_m) {
-#pragma unroll
-        for (int i = 0; i < 8; i++) {
-          const int64_t q = rs + mkg * 8 + i;
-          nh[i] = q < re ? rfh[q * ld + mm] : 0.f;
-          nl[i] = q < re ? rfl[q * ld + mm] : 0.f;
-        }
-      }
+      return r < r1 ? Uh[r * 32 + lane] : 0.f;
     };
-    fetch(r0, r1);
+    float nu = fetch(r0), nu2 = fetch(r0 + GP_K);
     bool dead = false;   // some warp's wait ran out: all working warps leave at the next stage's barrier
     for (int64_t rb = r0; rb < r1 && !dead; rb += GP_SUB, sub++) {
       const int64_t re = min(r1, rb + GP_SUB);
       for (int64_t rs = rb; rs < re; rs += GP_K, n++) {
         const uint32_t buf = n % GP_RING;
         su[n & 1][lane][tid >> 5] = nu;
-        float w[8];
-#pragma unroll
-        for (int i = 0; i < 8; i++) {
-          const float x = __fmul_rn(nh[i], msc), y = __fmul_rn(nl[i], msc);
-          w[i] = __fmaf_rn(x, x, __fmul_rn(2.f, __fmul_rn(x, y)));
-        }
+        nu = nu2;
+        nu2 = fetch(rs + 2 * GP_K);
+        if (lane == 0 && rs + GP_AHEAD * GP_K + (tid >> 5) < R)   // one 128-byte row of U per warp
+          asm volatile("prefetch.global.L2 [%0];\n" ::"l"(Uh + (rs + GP_AHEAD * GP_K + (tid >> 5)) * 32));
         if (n >= GP_RING) ok = xp_wait(xp_saddr(&freed[buf]), (n / GP_RING - 1) & 1, &s_abort) && ok;
         uint32_t any;   // the stage's U is complete once all have arrived
         asm volatile(
@@ -207,8 +241,6 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
             : "r"((uint32_t)!ok), "n"(GP_WORK)
             : "memory");
         if ((dead = any != 0)) break;
-        const int64_t nx = rs + GP_K;
-        if (nx < r1) fetch(nx, r1);
         uint8_t *st = smem + buf * GP_STAGE;
         const float *u = &su[n & 1][0][0];
 #pragma unroll
@@ -220,7 +252,6 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
                               a1.x * b1.x, a1.y * b1.y, a1.z * b1.z, a1.w * b1.w};
           gp_store(x, st + op_dst[j], GP_ATERM);
         }
-        if (has_m) gp_store(w, st + 3 * GP_ATERM + (mm >> 3) * 256 + mkg * 128 + (mm & 7) * 16, GP_BTERM);
         asm volatile("fence.proxy.async.shared::cta;\n" ::);
         __syncwarp();
         if (lane == 0) xp_arrive(xp_saddr(&ready[buf]));

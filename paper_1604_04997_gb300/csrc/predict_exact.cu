@@ -4,7 +4,7 @@
 //
 // One CTA of 16 warps per SM, persistent over 128-row tiles.  Per tile: the counts' digits
 // go to shared memory (the loads are issued before the previous tile's times are formed),
-// one thread issues the MMAs of the groups of diagonals, and every thread gathers 16 exact
+// one warp issues the MMAs of the groups of diagonals, and every thread gathers 16 exact
 // sums limb by limb, turns them into times and hands them on.
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
   __syncthreads();   // the staged weights in sA have been read
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-  const uint32_t tmem = tmem_base, s0 = xp_saddr(smem);
+  const uint32_t tmem = xp_uniform(tmem_base), s0 = xp_uniform(xp_saddr(smem));
   uint32_t seq = 0;            // groups so far: columns seq % XP_RING, their (seq / XP_RING)-th use
   uint32_t it = 0;             // tiles so far
   bool ok = true;
@@ -108,26 +108,24 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
   if (STASH && warp < XP_WARPS)
     for (int ps = 0; ps < 2; ps++) stash[ps * 32 * XP_WARPS] = XpAcc<MODE>();
   if (warp == XP_WARPS) {
-    // one thread issues, ahead of the working warps as far as digits and columns allow
-    if (lane == 0) {
-      for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, it++) {
-        if (!(ok = xp_wait_one(xp_saddr(&digits[it & 1]), (it >> 1) & 1, &s_abort))) break;
-        const int nd = xp_tile_digits(s_nd[it & 3]), ng = xp_groups(nd);
-        for (int n = 0; n < G::PASSES * ng && ok; n++, seq++) {
-          const uint32_t b = seq % XP_RING;
-          const int ps = n >= ng;
-          if (seq >= XP_RING && !(ok = xp_wait_one(xp_saddr(&empty[b]), (seq / XP_RING - 1) & 1, &s_abort))) break;
-          xp_issue<G>(s0, s0 + (it & 1) * G::A_BUF, s0 + G::OFF_B + ps * G::B_PASS, tmem + b * G::RANGE, n - ps * ng, nd,
-                   xp_saddr(&full[b]));
-        }
+    // this warp issues, ahead of the working warps as far as digits and columns allow
+    for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, it++) {
+      if (!(ok = xp_wait(xp_saddr(&digits[it & 1]), (it >> 1) & 1, &s_abort))) break;
+      const int nd = (int)xp_uniform((uint32_t)xp_tile_digits(s_nd[it & 3])), ng = xp_groups(nd);
+      for (int n = 0; n < G::PASSES * ng && ok; n++, seq++) {
+        const uint32_t b = seq % XP_RING;
+        const int ps = n >= ng;
+        if (seq >= XP_RING && !(ok = xp_wait(xp_saddr(&empty[b]), (seq / XP_RING - 1) & 1, &s_abort))) break;
+        xp_issue<G>(s0, s0 + (it & 1) * G::A_BUF, s0 + G::OFF_B + ps * G::B_PASS, tmem + b * G::RANGE, n - ps * ng, nd,
+                    xp_saddr(&full[b]));
       }
-      if (!ok) {
-        if (status) atomicOr(status, ST_TIMEOUT);
-        // let the MMAs in flight finish before TMEM is freed (bounded)
-        const unsigned long long t0 = globaltimer_ns();
-        for (uint32_t n = seq >= XP_RING ? seq - XP_RING : 0; n < seq; n++)
-          while (!xp_try(xp_saddr(&full[n % XP_RING]), (n / XP_RING) & 1) && globaltimer_ns() - t0 < MBAR_WAIT_NS) {}
-      }
+    }
+    if (!ok) {
+      if (lane == 0 && status) atomicOr(status, ST_TIMEOUT);
+      // let the MMAs in flight finish before TMEM is freed (bounded)
+      const unsigned long long t0 = globaltimer_ns();
+      for (uint32_t n = seq >= XP_RING ? seq - XP_RING : 0; n < seq; n++)
+        while (!xp_try(xp_saddr(&full[n % XP_RING]), (n / XP_RING) & 1) && globaltimer_ns() - t0 < MBAR_WAIT_NS) {}
     }
     __syncwarp();
   } else {
@@ -184,6 +182,29 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
       double *out = MODE == XP_TIMES ? T + r0 * M + m : nullptr;
       const int x0[2] = {1150 - s_E[m], 1150 - s_E[m + 1]};
       const bool wide = min(x0[0], x0[1]) < XP_XMIN || max(x0[0], x0[1]) > XP_XMAX;   // times may leave the normal range
+      // the residual passes' inputs, on their way while the times are formed
+      double2 tm[4];
+      float2 fh[4], fl[4];
+      if constexpr (MODE >= XP_RESIDUAL) {
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          tm[i] = make_double2(0, 0);
+          fh[i] = fl[i] = make_float2(0, 0);
+          if (m < M && 8 * i < left) {
+            const double *tin = res.T + (r0 + 8 * i) * M + m;
+            if (vst) {
+              tm[i] = __ldcs((const double2 *)tin);
+            } else {
+              tm[i].x = __ldcs(tin);
+              if (m + 1 < M) tm[i].y = __ldcs(tin + 1);
+            }
+            if (MODE == XP_SUMS_REL || (MODE == XP_RESIDUAL && res.relative)) {
+              fh[i] = *(const float2 *)(res.rfh + (r0 + 8 * i) * res.ld + m);
+              fl[i] = *(const float2 *)(res.rfl + (r0 + 8 * i) * res.ld + m);
+            }
+          }
+        }
+      }
       auto emit = [&](auto neg) {
 #pragma unroll
         for (int i = 0; i < 4; i++) {
@@ -204,40 +225,29 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
                 if (xp_order(t[e]) < xp_order(acc.t[e])) { acc.t[e] = t[e]; acc.r[e] = r0 + 8 * i; }
             } else if constexpr (MODE != XP_TIMES) {
               if (m < M) {
-                const double *tin = meas + (r0 + 8 * i) * M + m;
-                double tm[2] = {0, 0};
-                if (vst) {
-                  const double2 x = __ldcs((const double2 *)tin);
-                  tm[0] = x.x;
-                  tm[1] = x.y;
-                } else {
-                  tm[0] = __ldcs(tin);
-                  if (m + 1 < M) tm[1] = __ldcs(tin + 1);
-                }
                 if constexpr (MODE == XP_SUMS_ABS) {
 #pragma unroll
                   for (int e = 0; e < 2; e++) {
-                    const double r = tm[e] - t[e];
+                    const double b = e ? tm[i].y : tm[i].x, r = b - t[e];
                     acc.r[e] = fma(r, r, acc.r[e]);
-                    acc.b[e] = fma(tm[e], tm[e], acc.b[e]);
+                    acc.b[e] = fma(b, b, acc.b[e]);
                   }
                 } else {
-                  const int64_t q = (r0 + 8 * i) * res.ld + m;
                   // t - p in FP64 (exact while p is within a factor 2 of t), then float-float
-                  float2 d[2] = {ff_of_double(tm[0] - t[0]), ff_of_double(tm[1] - t[1])};
+                  float2 d[2] = {ff_of_double(tm[i].x - t[0]), ff_of_double(tm[i].y - t[1])};
                   if (MODE == XP_SUMS_REL || res.relative) {
-                    const float2 fh = *(const float2 *)(res.rfh + q), fl = *(const float2 *)(res.rfl + q);
-                    d[0] = ff_mul(d[0].x, d[0].y, fh.x, fl.x);
-                    d[1] = ff_mul(d[1].x, d[1].y, fh.y, fl.y);
+                    d[0] = ff_mul(d[0].x, d[0].y, fh[i].x, fl[i].x);
+                    d[1] = ff_mul(d[1].x, d[1].y, fh[i].y, fl[i].y);
                     if constexpr (MODE == XP_SUMS_REL) {
                       ff_acc(acc.s[0], acc.c[0], ff_mul(d[0].x, d[0].y, d[0].x, d[0].y));
                       ff_acc(acc.s[1], acc.c[1], ff_mul(d[1].x, d[1].y, d[1].x, d[1].y));
                     } else {
-                      d[0] = ff_mul(d[0].x, d[0].y, fh.x, fl.x);
-                      d[1] = ff_mul(d[1].x, d[1].y, fh.y, fl.y);
+                      d[0] = ff_mul(d[0].x, d[0].y, fh[i].x, fl[i].x);
+                      d[1] = ff_mul(d[1].x, d[1].y, fh[i].y, fl[i].y);
                     }
                   }
                   if constexpr (MODE == XP_RESIDUAL) {
+                    const int64_t q = (r0 + 8 * i) * res.ld + m;
                     *(float2 *)(res.Qh + q) = make_float2(d[0].x, d[1].x);
                     *(float2 *)(res.Ql + q) = make_float2(d[0].y, d[1].y);
                   }
