@@ -117,6 +117,29 @@ __global__ void __launch_bounds__(FIT_THREADS) k_rowfac(const float *__restrict_
 #pragma unroll
     for (int j = 0; j < 4; j++) mx[i][j] = 0.f;
   }
+  // this thread's items of a stage: four models of a row each, their timings one stage ahead
+  constexpr int ITEMS = AM_ROWS * 16 / FIT_THREADS;
+  double tn[ITEMS][4];
+  auto fetch = [&](int64_t rb) {
+#pragma unroll
+    for (int q = 0; q < ITEMS; q++) {
+      const int i = tid + q * FIT_THREADS, r = (i * inv4) >> 16, m = (i - r * m4) * 4;
+#pragma unroll
+      for (int e = 0; e < 4; e++) tn[q][e] = 1.0;
+      if (r < AM_ROWS && rb + r < R) {
+        const double *src = T + (rb + r) * M + m;
+        if (vec && m + 3 < M) {
+          const double2 x = __ldcs((const double2 *)src), y = __ldcs((const double2 *)src + 1);
+          tn[q][0] = x.x, tn[q][1] = x.y, tn[q][2] = y.x, tn[q][3] = y.y;
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; e++)
+            if (m + e < M) tn[q][e] = __ldcs(src + e);
+        }
+      }
+    }
+  };
+  fetch((int64_t)blockIdx.x * AM_ROWS);
   for (int64_t rb = (int64_t)blockIdx.x * AM_ROWS; rb < R; rb += (int64_t)gridDim.x * AM_ROWS) {
     const int nr = (int)min((int64_t)AM_ROWS, R - rb);
     __syncthreads();
@@ -125,20 +148,11 @@ __global__ void __launch_bounds__(FIT_THREADS) k_rowfac(const float *__restrict_
       const float4 x = r < nr ? *(const float4 *)(U + (rb + r) * 32 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
       *(float4 *)&su[r][c] = make_float4(fabsf(x.x), fabsf(x.y), fabsf(x.z), fabsf(x.w));
     }
-    for (int i = tid; i < AM_ROWS * m4; i += FIT_THREADS) {   // four models of a row per thread
-      const int r = (i * inv4) >> 16, m = (i - r * m4) * 4;
-      double t[4] = {1, 1, 1, 1};
-      if (r < nr) {
-        const double *src = T + (rb + r) * M + m;
-        if (vec && m + 3 < M) {
-          const double2 x = __ldcs((const double2 *)src), y = __ldcs((const double2 *)src + 1);
-          t[0] = x.x, t[1] = x.y, t[2] = y.x, t[3] = y.y;
-        } else {
 #pragma unroll
-          for (int e = 0; e < 4; e++)
-            if (m + e < M) t[e] = __ldcs(src + e);
-        }
-      }
+    for (int q = 0; q < ITEMS; q++) {
+      const int i = tid + q * FIT_THREADS, r = (i * inv4) >> 16, m = (i - r * m4) * 4;
+      if (r >= AM_ROWS) continue;
+      const double(&t)[4] = tn[q];
       float fh[4], fl[4], gh[4], gl[4];
 #pragma unroll
       for (int e = 0; e < 4; e++) {
@@ -167,6 +181,7 @@ __global__ void __launch_bounds__(FIT_THREADS) k_rowfac(const float *__restrict_
         }
       }
     }
+    fetch(rb + (int64_t)gridDim.x * AM_ROWS);
     __syncthreads();
     if (mg * 4 < ld) {
 #pragma unroll 4
@@ -416,32 +431,68 @@ __global__ void __launch_bounds__(32) k_chol_solve(double *__restrict__ G, const
 // twelve FP32 operations of each error-free product and compensated sum.  Grid (row chunks,
 // groups of 16 models); a thread owns two columns and eight models (lanes 0-15 and 16-31 of a
 // warp share the columns), so a row's 4 + 16 floats feed 16 products, and the eight warps
-// take every eighth row.
-constexpr int ATQ_MODELS = 16;
+// take every eighth row.  Stages of 64 rows come through shared memory, two ahead (cp.async):
+// read straight from L2, the loads' latency took half of the time (242 us for 200,000 x 32 x
+// 64 with 16 warps per SM).
+constexpr int ATQ_MODELS = 16, ATQ_ROWS = 64, ATQ_RING = 3;
+struct AtqStage { float u[ATQ_ROWS][2][32], q[ATQ_ROWS][2][ATQ_MODELS]; };   // [hi, lo]
+struct AtqSmem { AtqStage st[ATQ_RING]; float2 red[FIT_THREADS / 32][32][17]; };
+
+__device__ __forceinline__ void cp_async16_zfill(void *dst, const void *src, bool in) {   // 16 bytes, zeros if !in
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(in ? 16 : 0));
+}
+
 __global__ void __launch_bounds__(FIT_THREADS, 2) k_atq(const float *__restrict__ Uh, const float *__restrict__ Ul,
-                                                     const float *__restrict__ Qh, const float *__restrict__ Ql, int ld,
-                                                     int64_t R, int k, int M, int64_t rows_per_chunk,
-                                                     const unsigned *__restrict__ amax, double *__restrict__ g) {
+                                                        const float *__restrict__ Qh, const float *__restrict__ Ql, int ld,
+                                                        int64_t R, int k, int M, int64_t rows_per_chunk,
+                                                        const unsigned *__restrict__ amax, double *__restrict__ g) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  AtqSmem &S = *(AtqSmem *)smem_raw;
+  auto &red = S.red;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int c0 = 2 * (lane & 15), m0 = blockIdx.y * ATQ_MODELS + 8 * (lane >> 4);
+  const int c0 = 2 * (lane & 15), mg = 8 * (lane >> 4), mb = blockIdx.y * ATQ_MODELS;
   const int64_t r0 = (int64_t)blockIdx.x * rows_per_chunk;
   const int64_t r1 = min(R, r0 + rows_per_chunk);
-  const bool has = m0 < ld;
+  const int nst = (int)max((int64_t)0, (r1 - r0 + ATQ_ROWS - 1) / ATQ_ROWS);
+  auto fetch = [&](int s) {   // stage s on its way; rows and models that do not exist are zero
+    if (s < nst) {
+      AtqStage &T = S.st[s % ATQ_RING];
+      const int64_t rb = r0 + (int64_t)s * ATQ_ROWS;
+#pragma unroll
+      for (int i = 0; i < ATQ_ROWS * 16 / FIT_THREADS; i++) {
+        const int x = tid + i * FIT_THREADS, row = x >> 4, h = (x >> 3) & 1, c = (x & 7) * 4;
+        const bool in = rb + row < r1;
+        cp_async16_zfill(&T.u[row][h][c], (h ? Ul : Uh) + (in ? (rb + row) * 32 + c : 0), in);
+      }
+#pragma unroll
+      for (int i = 0; i < ATQ_ROWS * 8 / FIT_THREADS; i++) {
+        const int x = tid + i * FIT_THREADS, row = x >> 3, h = (x >> 2) & 1, m = (x & 3) * 4;
+        const bool in = rb + row < r1 && mb + m < ld;
+        cp_async16_zfill(&T.q[row][h][m], (h ? Ql : Qh) + (in ? (rb + row) * ld + mb + m : 0), in);
+      }
+    }
+    asm volatile("cp.async.commit_group;\n" ::);
+  };
+  fetch(0);
+  fetch(1);
   // this thread's sums so far; a compensated sum's error grows with the square of its length,
-  // so runs of 64 rows are added up in float-float
-  __shared__ float2 red[FIT_THREADS / 32][32][17];
+  // so runs of 64 rows (8 stages) are added up in float-float
 #pragma unroll
   for (int j = 0; j < 16; j++) red[warp][lane][j] = make_float2(0.f, 0.f);
-  for (int64_t rb = r0 + warp; has && rb < r1; rb += 64 * (FIT_THREADS / 32)) {
-    const int64_t re = min(r1, rb + 64 * (FIT_THREADS / 32));
-    float s[16], c[16];
+  float s[16], c[16];
 #pragma unroll
-    for (int j = 0; j < 16; j++) s[j] = c[j] = 0.f;
+  for (int j = 0; j < 16; j++) s[j] = c[j] = 0.f;
+  for (int st = 0; st < nst; st++) {
+    asm volatile("cp.async.wait_group 1;\n" ::);
+    __syncthreads();   // stage st is complete, and the buffer of stage st - 1 is free
+    fetch(st + 2);
+    const AtqStage &T = S.st[st % ATQ_RING];
 #pragma unroll 2
-    for (int64_t r = rb; r < re; r += FIT_THREADS / 32) {
-      const float2 uh = *(const float2 *)(Uh + r * 32 + c0), ul = *(const float2 *)(Ul + r * 32 + c0);
-      const float4 h0 = *(const float4 *)(Qh + r * ld + m0), h1 = *(const float4 *)(Qh + r * ld + m0 + 4);
-      const float4 l0 = *(const float4 *)(Ql + r * ld + m0), l1 = *(const float4 *)(Ql + r * ld + m0 + 4);
+    for (int row = warp; row < ATQ_ROWS; row += FIT_THREADS / 32) {
+      const float2 uh = *(const float2 *)&T.u[row][0][c0], ul = *(const float2 *)&T.u[row][1][c0];
+      const float4 h0 = *(const float4 *)&T.q[row][0][mg], h1 = *(const float4 *)&T.q[row][0][mg + 4];
+      const float4 l0 = *(const float4 *)&T.q[row][1][mg], l1 = *(const float4 *)&T.q[row][1][mg + 4];
       const float qh[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
       const float ql[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
 #pragma unroll
@@ -450,18 +501,21 @@ __global__ void __launch_bounds__(FIT_THREADS, 2) k_atq(const float *__restrict_
         ff_acc(s[2 * j + 1], c[2 * j + 1], ff_mul(uh.y, ul.y, qh[j], ql[j]));
       }
     }
+    if ((st & 7) == 7 || st + 1 == nst) {
 #pragma unroll
-    for (int j = 0; j < 16; j++) {
-      float2 t = red[warp][lane][j];
-      ff_acc(t.x, t.y, make_float2(s[j], c[j]));
-      red[warp][lane][j] = t;
+      for (int j = 0; j < 16; j++) {
+        float2 t = red[warp][lane][j];
+        ff_acc(t.x, t.y, make_float2(s[j], c[j]));
+        red[warp][lane][j] = t;
+        s[j] = c[j] = 0.f;
+      }
     }
   }
   __syncthreads();
   // the eight warps' sums of 32 columns x 16 models
   for (int o = tid; o < 32 * 16; o += FIT_THREADS) {
     const int l = o >> 4, j = o & 15;
-    const int col = 2 * (l & 15) + (j & 1), m = blockIdx.y * ATQ_MODELS + 8 * (l >> 4) + (j >> 1);
+    const int col = 2 * (l & 15) + (j & 1), m = mb + 8 * (l >> 4) + (j >> 1);
     if (m < M && col < k) {
       float ts = 0.f, tc = 0.f;
 #pragma unroll
@@ -556,15 +610,16 @@ cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int 
       U, T, ld, R, k, M, objective, rfh, rfl, beta ? bh : nullptr, beta ? bl : nullptr, amax, rmax, status);
   const int groups = (M + ATQ_MODELS - 1) / ATQ_MODELS;
   // one wave of two CTAs per SM: the sums are issue-bound, and a partial second wave idles
-  const int achunks = (int)std::max<int64_t>(1, std::min<int64_t>(2 * sms / groups, (R + 63) / 64));
+  const int achunks = (int)std::max<int64_t>(1, std::min<int64_t>(2 * sms / groups, (R + ATQ_ROWS - 1) / ATQ_ROWS));
   const int64_t arpc = (R + achunks - 1) / achunks;
+  if ((e = cudaFuncSetAttribute(k_atq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(AtqSmem))) != cudaSuccess) return e;
   if (gram != 0) {
     // the Gram on the tensor cores; the right-hand side A^T b = U^T (rowfactor b) with the
     // float-float product kernel
     e = gram == 2 ? launch_gram_tc(U, Ul, rfh, rfl, ld, R, k, M, amax, G, sms, status, st)
                   : launch_gram_pairs(U, rfh, rfl, ld, R, k, M, amax, rmax, G, sms, status, st);
     if (e != cudaSuccess) return e;
-    k_atq<<<dim3(achunks, groups), FIT_THREADS, 0, st>>>(U, Ul, relative ? rfh : bh, relative ? rfl : bl, ld, R, k, M, arpc,
+    k_atq<<<dim3(achunks, groups), FIT_THREADS, sizeof(AtqSmem), st>>>(U, Ul, relative ? rfh : bh, relative ? rfl : bl, ld, R, k, M, arpc,
                                                          amax, rhs);
   } else {
     const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>(4 * sms / std::max(1, M) + 1, (R + 255) / 256));
@@ -583,7 +638,7 @@ cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int 
   res.relative = relative;
   for (int it = 0; it < steps; it++) {
     if ((e = launch_fit_residual(F, R, k, W_out, M, res, false, status, sms, st)) != cudaSuccess) return e;
-    k_atq<<<dim3(achunks, groups), FIT_THREADS, 0, st>>>(U, Ul, Qh, Ql, ld, R, k, M, arpc, amax, g);
+    k_atq<<<dim3(achunks, groups), FIT_THREADS, sizeof(AtqSmem), st>>>(U, Ul, Qh, Ql, ld, R, k, M, arpc, amax, g);
     k_refine_update<<<M, 32, 0, st>>>(G, g, k, M, rep.info, cmax, amax, x, rep.upd, W_out, rep.rr, rep.bb);
   }
   // the final residual, for the report
