@@ -313,14 +313,16 @@ extern "C" pm_status pm_predict_topk(pm_ctx *c, const int64_t *F, int64_t R, int
   for (int32_t i = 0; i < G; i++)
     if (h_seg_off[i + 1] < h_seg_off[i]) return pm_set_error(PM_ERR_INVALID_ARG, "group offsets must be non-decreasing");
   if (!d_rows && h_seg_off[G] > R) return pm_set_error(PM_ERR_INVALID_ARG, "without a row list the groups must lie in [0, R)");
-  // work units: groups cut into chunks of TOPK_CHUNK positions; a one-chunk group
+  // work units: groups cut into even chunks; a one-chunk group
   // (an empty one too) is written directly, the others through partial lists
   std::vector<pmd::TopkUnit> units;
   std::vector<pmd::TopkMerge> merges;
   int64_t parts = 0;
+  const int64_t most = pmd::topk_chunk(k, M, h_seg_off[G] - h_seg_off[0]);
   for (int32_t i = 0; i < G; i++) {
     const int64_t p0 = h_seg_off[i], p1 = h_seg_off[i + 1];
-    const int64_t nch = std::max<int64_t>(1, (p1 - p0 + pmd::TOPK_CHUNK - 1) / pmd::TOPK_CHUNK);
+    const int64_t nch = std::max<int64_t>(1, (p1 - p0 + most - 1) / most);
+    const int64_t each = ((p1 - p0 + nch - 1) / nch + 31) & ~(int64_t)31;   // a multiple of 32, at most `most`
     if (nch == 1) {
       units.push_back(pmd::TopkUnit{p0, p1, i, -1});
       continue;
@@ -328,7 +330,7 @@ extern "C" pm_status pm_predict_topk(pm_ctx *c, const int64_t *F, int64_t R, int
     if (parts + nch > INT32_MAX) return pm_set_error(PM_ERR_INVALID_ARG, "too many rows");
     merges.push_back(pmd::TopkMerge{i, (int32_t)parts, (int32_t)nch, 0});
     for (int64_t q = 0; q < nch; q++)
-      units.push_back(pmd::TopkUnit{p0 + q * pmd::TOPK_CHUNK, std::min(p1, p0 + (q + 1) * pmd::TOPK_CHUNK), i,
+      units.push_back(pmd::TopkUnit{std::min(p1, p0 + q * each), std::min(p1, p0 + (q + 1) * each), i,
                                     (int32_t)(parts + q)});
     parts += nch;
   }

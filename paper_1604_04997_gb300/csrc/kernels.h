@@ -108,11 +108,13 @@ struct FitResidual {
 cudaError_t launch_fit_residual(const int64_t *F, int64_t R, int k, const double *W, int M, const FitResidual &res,
                                 bool sums, int *status, int sms, cudaStream_t st);
 
-// top-k rows per (group, model): work units of at most TOPK_CHUNK positions of one
+// top-k rows per (group, model): work units of at most topk_chunk(...) positions of one
 // group; a group of one unit is written directly (part < 0), the partial lists of the
 // others ([part][M][topk]) are merged per group (TopkMerge)
 constexpr int TOPK_MAX = 16;
-constexpr int64_t TOPK_CHUNK = 1024;
+constexpr int64_t TOPK_CHUNK = 1024;   // the smallest unit a group is cut into
+// the largest unit for M models and `total` positions in all
+int64_t topk_chunk(int k, int M, int64_t total);
 struct TopkUnit { int64_t p0, p1; int32_t g, part; };
 struct TopkMerge { int32_t g, part0, n_parts, pad; };
 cudaError_t launch_predict_topk(const int64_t *F, int64_t R, int k, const double *W, int M, const int64_t *rows,

@@ -15,6 +15,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "eval_common.cuh"
 #include "kernels.h"
@@ -434,11 +435,19 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_predict_topk(const int64_t *_
 
 // The same top-k for few models (M <= 8): the 64-model tile above would leave most of
 // its products and warps idle, so here each lane owns one row (a warp takes 32
-// consecutive positions of the unit, the CTA 256) and computes its M exact sums; each
+// consecutive positions of the unit, the CTA 128) and computes its M exact sums; each
 // warp keeps its own sorted lists per model, and at the end of the unit warp m merges
-// the eight warps' lists of model m.  Same products, same keys, same (time, row) order.
-template <int MN>
-__global__ void __launch_bounds__(PR_WARPS * 32) k_predict_topk_rows(const int64_t *__restrict__ F, int64_t R, int k,
+// the four warps' lists of model m.  Same products, same keys, same (time, row) order.
+//
+// STAGED (k even, at most 32, F 16-byte aligned): a warp copies its 32 rows to shared memory
+// with 16-byte asynchronous copies, whole rows at a time, and each lane then reads its own
+// row; the chunk index is XORed with the row's low bits, which keeps the 16-byte reads of
+// eight lanes on distinct banks.  Lanes reading their rows straight from global memory touch
+// 32 lines per instruction, and the kernel waited for L1 (1.02 ms for 4.5 M rows x 32, one
+// model; with the copies the multiply-adds and the reads from HBM bound it).
+constexpr int TR_WARPS = 4;
+template <int MN, bool STAGED>
+__global__ void __launch_bounds__(TR_WARPS * 32) k_predict_topk_rows(const int64_t *__restrict__ F, int64_t R, int k,
                                                                      const double *__restrict__ W, int M,
                                                                      const int64_t *__restrict__ rows,
                                                                      const TopkUnit *__restrict__ units, int n_units,
@@ -448,22 +457,36 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_predict_topk_rows(const int64
                                                                      double *__restrict__ top_t, int *status) {
   __shared__ int64_t sw[PR_MAXK][MN];
   __shared__ int sE[MN];
-  __shared__ double st[PR_WARPS][MN][32];
-  __shared__ int64_t sr[PR_WARPS][MN][32];
-  for (int m = threadIdx.x; m < MN; m += blockDim.x) {
-    const int E = m < M ? weight_exponent(W + (int64_t)m * k, k) : 0;
-    for (int i = 0; i < PR_MAXK; i++) sw[i][m] = (m < M && i < k) ? llrint(ldexp(W[(int64_t)m * k + i], E)) : 0;
-    sE[m] = E;
+  // the staged rows [warp][row][chunk ^ (row & 15)]; at the end of a unit the warps' lists
+  constexpr int LISTS = TR_WARPS * MN * 32, STAGE = STAGED ? TR_WARPS * 32 * 16 : 0;
+  __shared__ __align__(16) longlong2 stage[STAGE > LISTS ? STAGE : LISTS];
+  double(*st)[MN][32] = (double(*)[MN][32])stage;
+  int64_t(*sr)[MN][32] = (int64_t(*)[MN][32])((double *)stage + LISTS);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < MN * k; i += TR_WARPS * 32) {
+    const int m = i / k;
+    sw[i - m * k][m] = m < M ? __double_as_longlong(W[i]) : 0;
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x < MN) {   // the serial loop of weight_exponent over the staged weights
+    double w[PR_MAXK];
+    for (int c = 0; c < k; c++) w[c] = __longlong_as_double(sw[c][threadIdx.x]);
+    sE[threadIdx.x] = (int)threadIdx.x < M ? weight_exponent(w, k) : 0;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < MN * k; i += TR_WARPS * 32) {
+    const int m = i / k, c = i - m * k;
+    if (m < M) sw[c][m] = fixed_weight(__longlong_as_double(sw[c][m]), sE[m]);
+  }
+  __syncthreads();
+  const int cpr = k / 2, inv = (65536 + cpr - 1) / max(cpr, 1);   // 16-byte chunks per row; x / cpr = x inv / 2^16 for x < 512
   for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
     const TopkUnit U = units[u];
     double lt[MN];
     int64_t lr[MN];
 #pragma unroll
     for (int m = 0; m < MN; m++) { lt[m] = TK_INF; lr[m] = INT64_MAX; }
-    for (int64_t t0 = U.p0 + 32 * warp; t0 < U.p1; t0 += 32 * PR_WARPS) {   // warp-uniform
+    for (int64_t t0 = U.p0 + 32 * warp; t0 < U.p1; t0 += 32 * TR_WARPS) {   // warp-uniform
       const int64_t pos = t0 + lane;
       int64_t row = -1;
       if (pos < U.p1) {
@@ -476,7 +499,26 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_predict_topk_rows(const int64
       uint32_t a[MN][4];
 #pragma unroll
       for (int m = 0; m < MN; m++) a[m][0] = a[m][1] = a[m][2] = a[m][3] = 0;
-      if (row >= 0) {
+      if (STAGED) {
+        longlong2 *S = stage + warp * (32 * 16);
+        __syncwarp();   // the batch before has been read
+        for (int j = 0; j < cpr; j++) {
+          const int x = lane + 32 * j, r = (x * inv) >> 16, c = x - r * cpr;
+          const int64_t src = __shfl_sync(0xffffffffu, row, r);
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
+                           (unsigned)__cvta_generic_to_shared(S + r * 16 + (c ^ (r & 15)))),
+                       "l"(F + (src >= 0 ? src : 0) * k + 2 * c), "r"(src >= 0 ? 16 : 0));
+        }
+        asm volatile("cp.async.wait_all;\n" ::);
+        __syncwarp();
+        for (int c = 0; c < cpr; c++) {
+          const longlong2 v = S[lane * 16 + (c ^ (lane & 15))];
+#pragma unroll
+          for (int m = 0; m < MN; m++) acc_mad(a[m], v.x, sw[2 * c][m]);
+#pragma unroll
+          for (int m = 0; m < MN; m++) acc_mad(a[m], v.y, sw[2 * c + 1][m]);
+        }
+      } else if (row >= 0) {
         const int64_t *f = F + row * k;
         for (int i = 0; i < k; i++) {
           const int64_t v = __ldg(f + i);
@@ -494,18 +536,17 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_predict_topk_rows(const int64
         }
       }
     }
-    __syncthreads();   // the previous unit's merge has read st / sr
+    __syncthreads();   // every warp has read its rows
 #pragma unroll
     for (int m = 0; m < MN; m++) {
       st[warp][m][lane] = lt[m];
       sr[warp][m][lane] = lr[m];
     }
     __syncthreads();
-    if (warp < M && warp < MN) {
-      const int m = warp;
+    for (int m = warp; m < M && m < MN; m += TR_WARPS) {
       double ft = TK_INF;
       int64_t fr = INT64_MAX;
-      for (int w = 0; w < PR_WARPS; w++) {
+      for (int w = 0; w < TR_WARPS; w++) {
         const double t = st[w][m][lane];
         const int64_t r = sr[w][m][lane];
         warp_list_merge(ft, fr, t, r, lane < topk && r != INT64_MAX, topk, lane);
@@ -522,19 +563,24 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_predict_topk_rows(const int64
         }
       }
     }
+    __syncthreads();   // the lists have been read
   }
 }
 
-template <int MN>
+template <int MN, bool STAGED>
 static void launch_topk_rows(const int64_t *F, int64_t R, int k, const double *W, int M, const int64_t *rows,
                              const TopkUnit *units, int n_units, int topk, double *part_t, int64_t *part_r,
                              int64_t *top_idx, double *top_t, int *status, cudaStream_t st) {
   int per_sm = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_predict_topk_rows<MN>, PR_WARPS * 32, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_predict_topk_rows<MN, STAGED>, TR_WARPS * 32, 0);
   const int grid = std::min(n_units, num_sms() * std::max(1, per_sm));
-  k_predict_topk_rows<MN><<<grid, PR_WARPS * 32, 0, st>>>(F, R, k, W, M, rows, units, n_units, topk, part_t, part_r,
-                                                          top_idx, top_t, status);
+  k_predict_topk_rows<MN, STAGED><<<grid, TR_WARPS * 32, 0, st>>>(F, R, k, W, M, rows, units, n_units, topk, part_t, part_r,
+                                                                  top_idx, top_t, status);
 }
+
+// A unit of the few-model kernel may take 2,048 positions (a tuning space's variants of one
+// template and point fit in one unit, so nothing is merged across units).
+int64_t topk_chunk(int k, int M, int64_t total) { return M <= 8 ? 2 * TOPK_CHUNK : TOPK_CHUNK; }
 
 // Groups split over several units: one CTA per (group, model) merges the units' sorted
 // lists of that model; its warps take every eighth block of 32 candidates, then warp 0
@@ -588,10 +634,16 @@ cudaError_t launch_predict_topk(const int64_t *F, int64_t R, int k, const double
   if (k > PR_MAXK || M > PR_MAXM || topk < 1 || topk > TOPK_MAX) return cudaErrorInvalidValue;
   if (n_units <= 0) return cudaSuccess;
   if (M <= 8) {   // few models: one row per lane
-    if (M == 1) launch_topk_rows<1>(F, R, k, W, M, rows, units, n_units, topk, part_t, part_r, top_idx, top_t, status, st);
-    else if (M == 2) launch_topk_rows<2>(F, R, k, W, M, rows, units, n_units, topk, part_t, part_r, top_idx, top_t, status, st);
-    else if (M <= 4) launch_topk_rows<4>(F, R, k, W, M, rows, units, n_units, topk, part_t, part_r, top_idx, top_t, status, st);
-    else launch_topk_rows<8>(F, R, k, W, M, rows, units, n_units, topk, part_t, part_r, top_idx, top_t, status, st);
+    const bool staged = k % 2 == 0 && k <= 32 && ((uintptr_t)F & 15) == 0;
+    auto go = [&](auto mn) {
+      constexpr int MN = decltype(mn)::value;
+      if (staged) launch_topk_rows<MN, true>(F, R, k, W, M, rows, units, n_units, topk, part_t, part_r, top_idx, top_t, status, st);
+      else launch_topk_rows<MN, false>(F, R, k, W, M, rows, units, n_units, topk, part_t, part_r, top_idx, top_t, status, st);
+    };
+    if (M == 1) go(std::integral_constant<int, 1>{});
+    else if (M == 2) go(std::integral_constant<int, 2>{});
+    else if (M <= 4) go(std::integral_constant<int, 4>{});
+    else go(std::integral_constant<int, 8>{});
   } else {
     const size_t sm = predict_topk_smem();
     cudaFuncSetAttribute(k_predict_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
