@@ -117,6 +117,10 @@ constexpr int64_t TOPK_CHUNK = 1024;   // the smallest unit a group is cut into
 int64_t topk_chunk(int k, int M, int64_t total);
 struct TopkUnit { int64_t p0, p1; int32_t g, part; };
 struct TopkMerge { int32_t g, part0, n_parts, pad; };
+// topk_exact.cu: more than a few models, k <= 32, on the tensor cores
+cudaError_t launch_topk_exact(const int64_t *F, int64_t R, int k, const double *W, int M, const int64_t *rows,
+                              const TopkUnit *units, int n_units, int topk, double *part_t, int64_t *part_r,
+                              int64_t *top_idx, double *top_t, int *status, int sms, cudaStream_t st);
 cudaError_t launch_predict_topk(const int64_t *F, int64_t R, int k, const double *W, int M, const int64_t *rows,
                                 const TopkUnit *units, int n_units, const TopkMerge *merges, int n_merges, int topk,
                                 double *part_t, int64_t *part_r, int64_t *top_idx, double *top_t, int *status,

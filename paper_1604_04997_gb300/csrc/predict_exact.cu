@@ -15,14 +15,9 @@
 #include "exact_tc.cuh"
 #include "float_float.cuh"
 #include "kernels.h"
+#include "topk_list.cuh"
 
 namespace pmd {
-
-// the order of times as integers (no NaN, no -0.0 among them)
-__device__ __forceinline__ int64_t xp_order(double t) {
-  const int64_t b = __double_as_longlong(t);
-  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
-}
 
 // XP_TIMES: write T (fp64 [R][M]).  XP_ARGMIN: per-model minimum over the CTA's rows
 // (smaller time, then smaller row) -> part[blockIdx.x][M].  The fit's residual passes, with
@@ -222,7 +217,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
             if constexpr (MODE == XP_ARGMIN) {
 #pragma unroll
               for (int e = 0; e < 2; e++)   // rows come in increasing order: only a smaller time improves
-                if (xp_order(t[e]) < xp_order(acc.t[e])) { acc.t[e] = t[e]; acc.r[e] = r0 + 8 * i; }
+                if (time_order(t[e]) < time_order(acc.t[e])) { acc.t[e] = t[e]; acc.r[e] = r0 + 8 * i; }
             } else if constexpr (MODE != XP_TIMES) {
               if (m < M) {
                 if constexpr (MODE == XP_SUMS_ABS) {
@@ -310,7 +305,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
       ArgPart b = red[tid];
       for (int w = 1; w < 32; w++) {
         const ArgPart x = red[w * XP_MAXM + tid];
-        const int64_t kx = xp_order(x.t), kb = xp_order(b.t);
+        const int64_t kx = time_order(x.t), kb = time_order(b.t);
         if (kx < kb || (kx == kb && x.r < b.r)) b = x;
       }
       part[(int64_t)blockIdx.x * M + tid] = b;
