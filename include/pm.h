@@ -162,8 +162,9 @@ pm_status pm_predict_argmin(pm_ctx *ctx, const int64_t *d_F, int64_t R, int32_t 
  * at PM_PREC_FP64 (the only precision accepted here); 1 <= topk <= 16, k <= 40,
  * M <= 64.  A listed row outside [0, R) is skipped and makes pm_sync_status return
  * PM_ERR_INVALID_ARG.  A row listed twice in a group may be returned twice.
- * Groups of more than 1,024 positions use context scratch memory (16 bytes per
- * (1,024 positions, model, k-entry)). */
+ * Groups that are cut into several work units use context scratch memory (16 bytes per
+ * (unit, model, k-entry); units hold at least 128 positions, and from a few thousand units
+ * on at least 1,024). */
 pm_status pm_predict_topk(pm_ctx *ctx, const int64_t *d_F, int64_t R, int32_t k, const double *d_W,
                           int32_t M, int32_t precision, const int64_t *h_seg_off, int32_t G,
                           const int64_t *d_rows, int32_t topk, int64_t *d_top_idx, double *d_top_t,

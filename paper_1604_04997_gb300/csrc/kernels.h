@@ -112,9 +112,11 @@ cudaError_t launch_fit_residual(const int64_t *F, int64_t R, int k, const double
 // group; a group of one unit is written directly (part < 0), the partial lists of the
 // others ([part][M][topk]) are merged per group (TopkMerge)
 constexpr int TOPK_MAX = 16;
-constexpr int64_t TOPK_CHUNK = 1024;   // the smallest unit a group is cut into
-// the largest unit for M models and `total` positions in all
-int64_t topk_chunk(int k, int M, int64_t total);
+constexpr int64_t TOPK_CHUNK = 1024;
+// whether M models over `total` positions in G groups take the row-per-lane kernel, and the
+// largest unit
+bool topk_rows_path(int k, int M, int64_t total, int64_t G);
+int64_t topk_chunk(int k, int M, int64_t total, int64_t G);
 struct TopkUnit { int64_t p0, p1; int32_t g, part; };
 struct TopkMerge { int32_t g, part0, n_parts, pad; };
 // topk_exact.cu: more than a few models, k <= 32, on the tensor cores
@@ -123,8 +125,8 @@ cudaError_t launch_topk_exact(const int64_t *F, int64_t R, int k, const double *
                               int64_t *top_idx, double *top_t, int *status, int sms, cudaStream_t st);
 cudaError_t launch_predict_topk(const int64_t *F, int64_t R, int k, const double *W, int M, const int64_t *rows,
                                 const TopkUnit *units, int n_units, const TopkMerge *merges, int n_merges, int topk,
-                                double *part_t, int64_t *part_r, int64_t *top_idx, double *top_t, int *status,
-                                cudaStream_t st);
+                                double *part_t, int64_t *part_r, int64_t *top_idx, double *top_t, bool rows_path,
+                                int *status, cudaStream_t st);
 
 // predict_tc.cu (tensor cores, three-term bf16 split)
 int tc_parts(int sms);

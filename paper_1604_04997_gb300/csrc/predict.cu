@@ -75,6 +75,37 @@ __device__ __forceinline__ void acc_mad(uint32_t (&A)[4], int64_t v, int64_t W) 
   if (W < 0) asm("sub.cc.u32 %0, %0, %2;\n\tsubc.u32 %1, %1, %3;\n\t" : "+r"(A[2]), "+r"(A[3]) : "r"(v0), "r"(v1));
 }
 
+// The same for 0 <= v < 2^32: four multiply-adds.
+__device__ __forceinline__ void acc_mad_u32(uint32_t (&A)[4], uint32_t v, int64_t W) {
+  const uint32_t w0 = (uint32_t)W, w1 = (uint32_t)((uint64_t)W >> 32);
+  asm("mad.lo.cc.u32  %0, %4, %5, %0;\n\t"
+      "madc.lo.cc.u32 %1, %4, %6, %1;\n\t"
+      "madc.hi.cc.u32 %2, %4, %6, %2;\n\t"
+      "addc.u32       %3, %3, 0;\n\t"
+      "mad.hi.cc.u32  %1, %4, %5, %1;\n\t"
+      "addc.cc.u32    %2, %2, 0;\n\t"
+      "addc.u32       %3, %3, 0;\n\t"
+      : "+r"(A[0]), "+r"(A[1]), "+r"(A[2]), "+r"(A[3])
+      : "r"(v), "r"(w0), "r"(w1));
+  if (W < 0) asm("sub.cc.u32 %0, %0, %2;\n\tsubc.u32 %1, %1, 0;\n\t" : "+r"(A[2]), "+r"(A[3]) : "r"(v));
+}
+
+// One feature of a warp's 32 rows, with every model's weight.  Most features are zero in all
+// rows of a batch (a kernel has a few properties), many are below 2^32: what the whole warp
+// can leave out, it does.
+template <int MN>
+__device__ __forceinline__ void acc_feature(uint32_t (&a)[MN][4], int64_t v, const int64_t *w) {
+  if (__any_sync(0xffffffffu, v != 0)) {
+    if (__any_sync(0xffffffffu, (uint64_t)v >> 32 != 0)) {
+#pragma unroll
+      for (int m = 0; m < MN; m++) acc_mad(a[m], v, w[m]);
+    } else {
+#pragma unroll
+      for (int m = 0; m < MN; m++) acc_mad_u32(a[m], (uint32_t)v, w[m]);
+    }
+  }
+}
+
 // Each thread: rows warp + 8 q (q < 4), models lane + 32 j (j < 2).
 __device__ __forceinline__ void tile_fixed(const PredictSmem &S, int k, Acc128 acc[4][2]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -363,13 +394,16 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_predict_topk(const int64_t *_
 // warp keeps its own sorted lists per model, and at the end of the unit warp m merges
 // the four warps' lists of model m.  Same products, same keys, same (time, row) order.
 //
-// STAGED (k even, at most 32, F 16-byte aligned): a warp copies its 32 rows to shared memory
+// STAGED (k even, 24 to 32, F 16-byte aligned): a warp copies its 32 rows to shared memory
 // with 16-byte asynchronous copies, whole rows at a time, and each lane then reads its own
 // row; the chunk index is XORed with the row's low bits, which keeps the 16-byte reads of
 // eight lanes on distinct banks.  Lanes reading their rows straight from global memory touch
 // 32 lines per instruction, and the kernel waited for L1 (1.02 ms for 4.5 M rows x 32, one
 // model; with the copies the multiply-adds and the reads from HBM bound it).
 constexpr int TR_WARPS = 4;
+// the time of an exact sum, once in the code
+static __device__ __noinline__ double time_of(Acc128 A, int E) { return key_value(acc_key(A), E); }
+
 template <int MN, bool STAGED>
 __global__ void __launch_bounds__(TR_WARPS * 32) k_predict_topk_rows(const int64_t *__restrict__ F, int64_t R, int k,
                                                                      const double *__restrict__ W, int M,
@@ -381,11 +415,14 @@ __global__ void __launch_bounds__(TR_WARPS * 32) k_predict_topk_rows(const int64
                                                                      double *__restrict__ top_t, int *status) {
   __shared__ int64_t sw[PR_MAXK][MN];
   __shared__ int sE[MN];
-  // the staged rows [warp][row][chunk ^ (row & 15)]; at the end of a unit the warps' lists
-  constexpr int LISTS = TR_WARPS * MN * 32, STAGE = STAGED ? TR_WARPS * 32 * 16 : 0;
-  __shared__ __align__(16) longlong2 stage[STAGE > LISTS ? STAGE : LISTS];
-  double(*st)[MN][32] = (double(*)[MN][32])stage;
-  int64_t(*sr)[MN][32] = (int64_t(*)[MN][32])((double *)stage + LISTS);
+  // the warps' lists, then the staged rows [warp][row][chunk ^ (row & 15)].  One buffer per
+  // warp: with two, half the warps fit, and 12 warps per SM are slower (four models, 4,096
+  // groups of 244 rows: 782 us).
+  constexpr int LISTS = TR_WARPS * MN * 32;
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  longlong2 *stage = (longlong2 *)smem_raw + LISTS;
+  double(*st)[MN][32] = (double(*)[MN][32])smem_raw;
+  int64_t(*sr)[MN][32] = (int64_t(*)[MN][32])((double *)smem_raw + LISTS);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int i = threadIdx.x; i < MN * k; i += TR_WARPS * 32) {
     const int m = i / k;
@@ -406,10 +443,10 @@ __global__ void __launch_bounds__(TR_WARPS * 32) k_predict_topk_rows(const int64
   const int cpr = k / 2, inv = (65536 + cpr - 1) / max(cpr, 1);   // 16-byte chunks per row; x / cpr = x inv / 2^16 for x < 512
   for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
     const TopkUnit U = units[u];
-    double lt[MN];
-    int64_t lr[MN];
+    // this warp's lists, one model's entry i in lane i
 #pragma unroll
-    for (int m = 0; m < MN; m++) { lt[m] = TK_INF; lr[m] = INT64_MAX; }
+    for (int m = 0; m < MN; m++) { st[warp][m][lane] = TK_INF; sr[warp][m][lane] = INT64_MAX; }
+    __syncwarp();
     for (int64_t t0 = U.p0 + 32 * warp; t0 < U.p1; t0 += 32 * TR_WARPS) {   // warp-uniform
       const int64_t pos = t0 + lane;
       int64_t row = -1;
@@ -437,34 +474,35 @@ __global__ void __launch_bounds__(TR_WARPS * 32) k_predict_topk_rows(const int64
         __syncwarp();
         for (int c = 0; c < cpr; c++) {
           const longlong2 v = S[lane * 16 + (c ^ (lane & 15))];
-#pragma unroll
-          for (int m = 0; m < MN; m++) acc_mad(a[m], v.x, sw[2 * c][m]);
-#pragma unroll
-          for (int m = 0; m < MN; m++) acc_mad(a[m], v.y, sw[2 * c + 1][m]);
+          acc_feature(a, v.x, sw[2 * c]);
+          acc_feature(a, v.y, sw[2 * c + 1]);
         }
-      } else if (row >= 0) {
-        const int64_t *f = F + row * k;
-        for (int i = 0; i < k; i++) {
-          const int64_t v = __ldg(f + i);
-#pragma unroll
-          for (int m = 0; m < MN; m++) acc_mad(a[m], v, sw[i][m]);
-        }
+      } else {
+        const int64_t *f = F + (row >= 0 ? row : 0) * k;
+#pragma unroll 4
+        for (int i = 0; i < k; i++) acc_feature(a, row >= 0 ? __ldg(f + i) : 0, sw[i]);
       }
+      // one merge in the code for all models: unrolled, it outgrows the instruction cache (four
+      // models: 8.5 of 15 stall cycles per instruction)
+      double t[MN];
 #pragma unroll
       for (int m = 0; m < MN; m++) {
-        if (m < M) {   // warp-uniform
-          Acc128 A;
-          A.lo = (uint64_t)a[m][0] | ((uint64_t)a[m][1] << 32);
-          A.hi = (uint64_t)a[m][2] | ((uint64_t)a[m][3] << 32);
-          warp_list_merge(lt[m], lr[m], key_value(acc_key(A), sE[m]), row, row >= 0, topk, lane);
-        }
+        Acc128 A;
+        A.lo = (uint64_t)a[m][0] | ((uint64_t)a[m][1] << 32);
+        A.hi = (uint64_t)a[m][2] | ((uint64_t)a[m][3] << 32);
+        t[m] = time_of(A, sE[m]);
       }
-    }
-    __syncthreads();   // every warp has read its rows
+#pragma unroll 1
+      for (int m = 0; m < M && m < MN; m++) {
+        double x = t[0];
 #pragma unroll
-    for (int m = 0; m < MN; m++) {
-      st[warp][m][lane] = lt[m];
-      sr[warp][m][lane] = lr[m];
+        for (int q = 1; q < MN; q++) x = m == q ? t[q] : x;
+        double lt = st[warp][m][lane];
+        int64_t lr = sr[warp][m][lane];
+        warp_list_merge(lt, lr, x, row, row >= 0, topk, lane);
+        st[warp][m][lane] = lt;
+        sr[warp][m][lane] = lr;
+      }
     }
     __syncthreads();
     for (int m = warp; m < M && m < MN; m += TR_WARPS) {
@@ -495,21 +533,40 @@ template <int MN, bool STAGED>
 static void launch_topk_rows(const int64_t *F, int64_t R, int k, const double *W, int M, const int64_t *rows,
                              const TopkUnit *units, int n_units, int topk, double *part_t, int64_t *part_r,
                              int64_t *top_idx, double *top_t, int *status, cudaStream_t st) {
+  const size_t sm = sizeof(longlong2) * (TR_WARPS * MN * 32 + (STAGED ? TR_WARPS * 32 * 16 : 0));
   int per_sm = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_predict_topk_rows<MN, STAGED>, TR_WARPS * 32, 0);
+  cudaFuncSetAttribute(k_predict_topk_rows<MN, STAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_predict_topk_rows<MN, STAGED>, TR_WARPS * 32, sm);
   const int grid = std::min(n_units, num_sms() * std::max(1, per_sm));
-  k_predict_topk_rows<MN, STAGED><<<grid, TR_WARPS * 32, 0, st>>>(F, R, k, W, M, rows, units, n_units, topk, part_t, part_r,
+  k_predict_topk_rows<MN, STAGED><<<grid, TR_WARPS * 32, sm, st>>>(F, R, k, W, M, rows, units, n_units, topk, part_t, part_r,
                                                                   top_idx, top_t, status);
 }
 
-// A unit of the few-model kernel may take 2,048 positions (a tuning space's variants of one
-// template and point fit in one unit, so nothing is merged across units).
-// The tensor-core kernel keeps one list per CTA and unit: one unit per SM for large groups.
-int64_t topk_chunk(int k, int M, int64_t total) {
-  if (M <= 8) return 2 * TOPK_CHUNK;
+// Which kernel, and how large a unit may be.  The row-per-lane kernel's cost grows with the
+// models, the tensor cores' hardly (they pad to a tile) but with the lists' ends, so the line
+// is in models and rows per group.  1e6 x 32, us, row-per-lane | tensor cores: 4 models 303 |
+// 360 (one group), 447 | 1,010 (4,096 groups); 5 models 585 (600 groups) | 768 (400), 647
+// (200), 624 (10); 8 models 900 | 1,174 (4,096), 716 (600) | 696 (400), 367 (one).  Rows of 12
+// counts have fewer than half the products to do: 8 models in 100 groups 451 | 554.  The tensor
+// cores take k up to 32.
+bool topk_rows_path(int k, int M, int64_t total, int64_t G) {
+  if (M <= 4) return true;
+  if (M > 8) return false;
+  return k <= 16 || !exact_tc_ok(k, M) || total < (M == 5 ? int64_t(1) << 17 : 2048) * G;
+}
+// The row-per-lane kernel's units fill its resident CTAs once (six per SM, four with eight
+// models' lists): of 977 units of 1,024 positions on 912 CTAs the last 65 took as
+// long as the rest (1e6 rows, 4 models).  At most 2,048 positions, so that larger problems
+// balance over many units while the variants of one template and point stay one unit.  The
+// tensor-core kernel keeps one list per CTA and unit: one unit per SM.
+int64_t topk_chunk(int k, int M, int64_t total, int64_t G) {
+  auto split = [&](int64_t ctas, int64_t grain, int64_t lo, int64_t hi) {
+    const int64_t each = ((total + ctas - 1) / ctas + grain - 1) / grain * grain;
+    return std::min(hi, std::max(lo, each));
+  };
+  if (topk_rows_path(k, M, total, G)) return split((int64_t)num_sms() * (M <= 2 ? 6 : M <= 4 ? 5 : 4), 32, 32 * TR_WARPS, 2048);
   if (!exact_tc_ok(k, M)) return TOPK_CHUNK;
-  const int64_t each = (total + num_sms() - 1) / num_sms();
-  return std::min<int64_t>(int64_t(1) << 20, std::max<int64_t>(TOPK_CHUNK, (each + 127) & ~(int64_t)127));
+  return split(num_sms(), 128, TOPK_CHUNK, int64_t(1) << 20);
 }
 
 // Groups split over several units: one CTA per (group, model) merges the units' sorted
@@ -559,12 +616,13 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_topk_merge(const TopkMerge *_
 
 cudaError_t launch_predict_topk(const int64_t *F, int64_t R, int k, const double *W, int M, const int64_t *rows,
                                 const TopkUnit *units, int n_units, const TopkMerge *merges, int n_merges, int topk,
-                                double *part_t, int64_t *part_r, int64_t *top_idx, double *top_t, int *status,
-                                cudaStream_t st) {
+                                double *part_t, int64_t *part_r, int64_t *top_idx, double *top_t, bool rows_path,
+                                int *status, cudaStream_t st) {
   if (k > PR_MAXK || M > PR_MAXM || topk < 1 || topk > TOPK_MAX) return cudaErrorInvalidValue;
   if (n_units <= 0) return cudaSuccess;
-  if (M <= 8) {   // few models: one row per lane
-    const bool staged = k % 2 == 0 && k <= 32 && ((uintptr_t)F & 15) == 0;
+  if (rows_path) {   // few models: one row per lane
+    // rows of 12 counts are read well enough as they are (1e6 x 12, 4 models: staged 331 us)
+    const bool staged = k % 2 == 0 && k >= 24 && k <= 32 && ((uintptr_t)F & 15) == 0;
     auto go = [&](auto mn) {
       constexpr int MN = decltype(mn)::value;
       if (staged) launch_topk_rows<MN, true>(F, R, k, W, M, rows, units, n_units, topk, part_t, part_r, top_idx, top_t, status, st);

@@ -3,12 +3,14 @@
 // the times are those of k_predict_exact, bit for bit.
 //
 // One CTA of 16 working warps and an issuing warp per SM; the CTA takes units (up to
-// topk_chunk positions of one group) in turn, in tiles of 128 positions.  A time that is not
-// above the model's current 16th is offered to the model's buffer of TX_BUF candidates in
-// shared memory; when some buffer is half full (or cannot take a candidate), all warps meet
-// and warp w merges the buffers of models w, w + 16, .. into their sorted lists (entry i in
-// lane i, predict.cu's merge).  After the first tiles of a unit few candidates pass, so the
-// warps rarely meet: the products bound the kernel, not the lists.
+// topk_chunk positions of one group) in turn, in tiles of 128 positions.  Each model has one
+// sorted list and a buffer of TX_BUF candidates in shared memory.  A time that is not above
+// the list's last entry reserves a slot of its model's buffer; the warp that fills the buffer
+// merges it into the list (topk_list.cuh) and empties it, and warps that find it full wait for
+// that.  The warps meet only where a unit ends.  Kept in step by barriers around the buffers
+// they could not hide each other's latencies (0.84 ms for 1e6 x 32 x 64, against 0.32 for the
+// times alone), and merging each candidate as it came cost 400 instructions for one or two
+// (1.19 ms).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -22,46 +24,52 @@
 namespace pmd {
 
 constexpr int TX_BUF = 16;           // buffered candidates per model
-
-struct TxSmem {                      // beyond the operands of XpGeom
-  int64_t lt[XP_MAXM][TOPK_MAX];     // sorted lists: times (as bits), rows
-  int64_t lr[XP_MAXM][TOPK_MAX];
-  int64_t ct[XP_MAXM][TX_BUF];       // candidates: times, positions within the unit
-  int32_t cp[XP_MAXM][TX_BUF];
-  int64_t thr[XP_MAXM];              // time_order of the list's last entry
-  int32_t cnt[XP_MAXM];
-  int64_t rows[4][XP_ROWS];          // rows of the tiles in flight (by tile modulo 4), -1: none
-};
+constexpr int TX_TRIES = 1 << 22;    // polls of a buffer before giving up
 
 // The tiles of a CTA, in order: units blockIdx.x, blockIdx.x + gridDim.x, .., each cut into
 // 128 positions (a unit without positions is one empty tile).
 struct TxCursor {
-  const TopkUnit *units;
-  int n_units, u;
-  int64_t p, p1;
-  int32_t g, part;
-  __device__ void open() {
+  int64_t p, p0, p1;   // this tile; its unit
+  int32_t u, g, part, pad;
+  __device__ void open(const TopkUnit *units, int n_units) {
     if (u < n_units) {
       const TopkUnit U = units[u];
-      p = U.p0;
+      p = p0 = U.p0;
       p1 = U.p1;
       g = U.g;
       part = U.part;
     }
   }
-  __device__ TxCursor(const TopkUnit *units, int n_units) : units(units), n_units(n_units), u(blockIdx.x), p(0), p1(0), g(0), part(0) {
-    open();
+  __device__ void start(const TopkUnit *units, int n_units) {
+    p = p0 = p1 = 0;
+    g = part = pad = 0;
+    u = blockIdx.x;
+    open(units, n_units);
   }
-  __device__ bool more() const { return u < n_units; }
+  __device__ bool more(int n_units) const { return u < n_units; }
   __device__ bool last() const { return p + XP_ROWS >= p1; }   // of its unit
-  __device__ void next() {
+  __device__ void next(const TopkUnit *units, int n_units) {
+    if (!more(n_units)) return;
     if (last()) {
       u += gridDim.x;
-      open();
+      open(units, n_units);
     } else {
       p += XP_ROWS;
     }
   }
+};
+
+constexpr int TX_ROWRING = 8;
+struct TxSmem {                      // beyond the operands of XpGeom
+  int64_t lt[XP_MAXM][TOPK_MAX];     // sorted lists: times (as bits), rows
+  int64_t lr[XP_MAXM][TOPK_MAX];
+  int64_t thr[XP_MAXM];              // time_order of the list's last entry, and its row
+  int64_t thr_row[XP_MAXM];
+  int64_t ct[XP_MAXM][TX_BUF];       // candidates: times, positions within the unit
+  int32_t cp[XP_MAXM][TX_BUF];
+  int32_t cnt[XP_MAXM], wr[XP_MAXM]; // slots reserved and written
+  uint8_t live[TX_ROWRING][XP_ROWS]; // positions of the tiles in flight (by tile modulo 8) that have a row
+  TxCursor cursor[2][XP_WARPS + 1];  // per warp: its tile, and the tile it loads for
 };
 
 template <class G>
@@ -105,7 +113,8 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
     }
     if (lane == 0) {
       X.thr[m] = INF;
-      X.cnt[m] = 0;
+      X.thr_row[m] = INT64_MAX;
+      X.cnt[m] = X.wr[m] = 0;
     }
   };
   if (warp < XP_WARPS)
@@ -123,10 +132,22 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
   const uint32_t tmem = xp_uniform(tmem_base), s0 = xp_uniform(xp_saddr(smem));
   uint32_t seq = 0, it = 0;
   bool ok = true;
-  TxCursor cur(units, n_units);
+  // a warp's cursors, in shared memory: held in registers next to the limbs they make the
+  // kernel spill, and shared memory leaves L1 too little room for that
+  TxCursor &cur = X.cursor[0][warp], &ahead = X.cursor[1][warp];
+  if (lane == 0) {
+    cur.start(units, n_units);
+    ahead.start(units, n_units);
+  }
+  __syncwarp();
+  auto advance = [&](TxCursor &c) {
+    __syncwarp();
+    if (lane == 0) c.next(units, n_units);
+    __syncwarp();
+  };
   if (warp == XP_WARPS) {
     // this warp issues, ahead of the working warps as far as digits and columns allow
-    for (; cur.more() && ok; cur.next(), it++) {
+    for (; cur.more(n_units) && ok; advance(cur), it++) {
       if (!(ok = xp_wait(xp_saddr(&digits[it & 1]), (it >> 1) & 1, &s_abort))) break;
       const int nd = (int)xp_uniform((uint32_t)xp_tile_digits(s_nd[it & 3])), ng = xp_groups(nd);
       for (int n = 0; n < G::PASSES * ng && ok; n++, seq++) {
@@ -149,67 +170,74 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
     const bool active = slice * 8 < G::NB;   // this warp has models
     const int c0 = slice * 8 + 2 * (lane & 3);
     const uint32_t tread = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(slice * 8);
-    // the working warps meet; true if any of their threads says so
-    auto meet = [&](bool say) -> bool {
-      uint32_t any;
-      asm volatile(
-          "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbar.red.or.pred q, 1, %2, p;\nselp.u32 %0, 1, 0, q;\n}\n"
-          : "=r"(any)
-          : "r"((uint32_t)say), "n"(32 * XP_WARPS)
-          : "memory");
-      return any != 0;
+    auto meet = [&]() { asm volatile("bar.sync 1, %0;\n" ::"n"(32 * XP_WARPS) : "memory"); };   // all working warps
+    // find the rows of this warp's share of the n-th tile (at cursor ahead), and prefetch
+    // them into L2, 128 bytes per instruction
+    int64_t nrow = -1;
+    auto locate = [&](uint32_t n) {
+      nrow = -1;
+      if (row < XP_ROWS) {
+        const int64_t pos = ahead.p + row;
+        int64_t r = -1;
+        if (ahead.more(n_units) && pos < ahead.p1) {
+          r = rows ? rows[pos] : pos;
+          if (r < 0 || r >= R) {
+            if (xp_kg<G>() == 0) atomicOr(status, ST_BAD_ROW);
+            r = -1;
+          }
+        }
+        if (xp_kg<G>() == 0) X.live[n % TX_ROWRING][row] = r >= 0;
+        nrow = r;
+        if (r >= 0 && (xp_kg<G>() & 1) == 0 && xp_kg<G>() * 64 < k * 8)
+          asm volatile("prefetch.global.L2 [%0];\n" ::"l"((const char *)(F + r * k) + xp_kg<G>() * 64));
+      }
+      advance(ahead);
     };
-    // the feature row of this thread's share of the tile at cursor c, or -1
-    auto locate = [&](const TxCursor &c) -> int64_t {
-      const int64_t pos = c.p + row;
-      if (row >= XP_ROWS || !c.more() || pos >= c.p1) return -1;
-      const int64_t r = rows ? rows[pos] : pos;
-      if (r >= 0 && r < R) return r;
-      if (xp_kg<G>() == 0) atomicOr(status, ST_BAD_ROW);
-      return -1;
-    };
-    // load this thread's share of the n-th tile, from row r, and store its digits
-    auto feed = [&](int64_t r, uint32_t n) {
+    // load this thread's share of the n-th tile and store its digits
+    auto feed = [&](uint32_t n) {
       int64_t v[8];
 #pragma unroll
       for (int i = 0; i < 8; i++) v[i] = 0;
-      if (row < XP_ROWS) {
-        if (xp_kg<G>() == 0) X.rows[n & 3][row] = r;
-        if (r >= 0) xp_load_row<G>(F + r * k, k, vec, v);
-      }
+      if (nrow >= 0) xp_load_row<G>(F + nrow * k, k, vec, v);
       xp_store_digits<G>(v, sA + (n & 1) * G::A_BUF, s_nd[n & 3]);
       asm volatile("fence.proxy.async.shared::cta;\n" ::);
       __syncwarp();
       if (lane == 0) xp_arrive(xp_saddr(&digits[n & 1]));
     };
-    // the candidates of this warp's models into their lists
-    int64_t base = 0;   // first position of the current unit
-    auto merge = [&]() {
-      for (int m = warp; m < M; m += XP_WARPS) {
-        const int n = min(X.cnt[m], TX_BUF);
-        if (n == 0) continue;   // warp-uniform
-        double t = TK_INF, lt = TK_INF;
-        int64_t r = INT64_MAX, lr = INT64_MAX;
-        if (lane < n) {
-          t = __longlong_as_double(X.ct[m][lane]);
-          const int64_t pos = base + X.cp[m][lane];
-          r = rows ? rows[pos] : pos;
-        }
-        if (lane < TOPK_MAX) {
-          lt = __longlong_as_double(X.lt[m][lane]);
-          lr = X.lr[m][lane];
-        }
-        warp_list_merge(lt, lr, t, r, lane < n, topk, lane);
-        if (lane < TOPK_MAX) {
-          X.lt[m][lane] = __double_as_longlong(lt);
-          X.lr[m][lane] = lr;
-        }
-        const int64_t th = time_order(__shfl_sync(0xffffffffu, lt, topk - 1));
-        if (lane == 0) {
-          X.thr[m] = th;
-          X.cnt[m] = 0;
-        }
-        __syncwarp();
+    // whether the time o (as ordered bits) of position pos may be among model m's topk
+    auto below = [&](int64_t o, int64_t pos, int m) {
+      const int64_t th = *(volatile int64_t *)&X.thr[m];
+      if (o != th) return o < th;
+      return (rows ? rows[pos] : pos) < *(volatile int64_t *)&X.thr_row[m];
+    };
+    // model m's n candidates into its list (a warp; all n are written)
+    auto merge = [&](int m, int n) {
+      double t = TK_INF, lt = TK_INF;
+      int64_t r = INT64_MAX, lr = INT64_MAX;
+      if (lane < n) {
+        t = __longlong_as_double(*(volatile int64_t *)&X.ct[m][lane]);
+        const int64_t pos = cur.p0 + *(volatile int32_t *)&X.cp[m][lane];
+        r = rows ? rows[pos] : pos;
+      }
+      if (lane < TOPK_MAX) {
+        lt = __longlong_as_double(*(volatile int64_t *)&X.lt[m][lane]);
+        lr = *(volatile int64_t *)&X.lr[m][lane];
+      }
+      warp_list_merge(lt, lr, t, r, lane < n, topk, lane);
+      if (lane < TOPK_MAX) {
+        X.lt[m][lane] = __double_as_longlong(lt);
+        X.lr[m][lane] = lr;
+      }
+      const int64_t th = time_order(__shfl_sync(0xffffffffu, lt, topk - 1)), thr = __shfl_sync(0xffffffffu, lr, topk - 1);
+      __threadfence_block();
+      __syncwarp();
+      if (lane == 0) {
+        *(volatile int64_t *)&X.thr_row[m] = thr;   // the row first: who reads the time and then the row (above)
+        __threadfence_block();                      // never compares with a looser pair's row
+        *(volatile int64_t *)&X.thr[m] = th;
+        *(volatile int32_t *)&X.wr[m] = 0;
+        __threadfence_block();
+        atomicExch(&X.cnt[m], 0);   // the buffer is open again
       }
     };
     auto wait = [&]() { return xp_wait(xp_saddr(&full[seq % XP_RING]), (seq / XP_RING) & 1, &s_abort); };
@@ -219,11 +247,11 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
       if (lane == 0) xp_arrive(xp_saddr(&empty[seq % XP_RING]));
       seq++;
     };
-    // one (tile, pass): the exact sums, the times, the candidates.  On a wait that ran out the
-    // warp goes on without sums to the meeting point, where all leave together (false).
-    auto pass = [&](int ps) -> bool {
+    // one (tile, pass): the exact sums, the times, the candidates.  After a wait that ran out
+    // the warp only keeps the order of the meetings.
+    auto pass = [&](int ps) {
       uint32_t limb[4][8], cy[8];
-      ok = wait();
+      ok = ok && wait();
       int ng = 4;
       if (ok) {
         ng = xp_groups(xp_tile_digits(s_nd[it & 3]));
@@ -258,81 +286,100 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
 #pragma unroll
         for (int o = 0; o < 8; o++) limb[3][o] = cy[o] - XP_HI;
       }
+      if (!ok || !active) return;
       const int m = 32 * ps + c0;
-      const int rl = quarter * 32 + (lane >> 2);   // this thread's rows of the tile: rl + 8 i, i < 4
-      int64_t t[8];
-      uint32_t pending = 0;   // bit 2 i + e: the time of row rl + 8 i, model m + e is still to be offered
-      if (ok && active) {
-        const int x0[2] = {1150 - s_E[m], 1150 - s_E[m + 1]};
-        const bool wide = min(x0[0], x0[1]) < XP_XMIN || max(x0[0], x0[1]) > XP_XMAX;
-        uint32_t sg = 0;
-#pragma unroll
-        for (int o = 0; o < 8; o++) sg |= limb[3][o];
-        const bool neg = __any_sync(0xffffffffu, (int32_t)sg < 0);
+      int64_t t[8];           // row quarter 32 + lane / 4 + 8 i, model m + e: 2 i + e
+      uint32_t pending = 0;   // bit 2 i + e: a candidate
+      const int x0[2] = {1150 - s_E[m], 1150 - s_E[m + 1]};
+      const bool wide = min(x0[0], x0[1]) < XP_XMIN || max(x0[0], x0[1]) > XP_XMAX;
+      const int64_t th[2] = {*(volatile int64_t *)&X.thr[m], *(volatile int64_t *)&X.thr[m + 1]};
+      const uint8_t *tile_live = X.live[it % TX_ROWRING] + quarter * 32 + (lane >> 2);
+      const int32_t off = (int32_t)(cur.p - cur.p0) + quarter * 32 + (lane >> 2);   // of this thread's first row in the unit
+      auto emit = [&](auto neg) {
 #pragma unroll
         for (int i = 0; i < 4; i++) {
-          const bool live = X.rows[it & 3][rl + 8 * i] >= 0;
+          const bool live = tile_live[8 * i];
+          double x[2];
+          bool bad = wide;
+#pragma unroll
+          for (int e = 0; e < 2; e++)
+            x[e] = xp_value<decltype(neg)::value>(limb[0][2 * i + e], limb[1][2 * i + e], limb[2][2 * i + e], limb[3][2 * i + e], x0[e], bad);
+          if (bad) {
+#pragma unroll
+            for (int e = 0; e < 2; e++)
+              x[e] = xp_value_rare(limb[0][2 * i + e], limb[1][2 * i + e], limb[2][2 * i + e], limb[3][2 * i + e], 1150 - x0[e]);
+          }
 #pragma unroll
           for (int e = 0; e < 2; e++) {
-            const int o = 2 * i + e;
-            bool bad = wide;
-            double x = neg ? xp_value<true>(limb[0][o], limb[1][o], limb[2][o], limb[3][o], x0[e], bad)
-                           : xp_value<false>(limb[0][o], limb[1][o], limb[2][o], limb[3][o], x0[e], bad);
-            if (bad) x = xp_value_rare(limb[0][o], limb[1][o], limb[2][o], limb[3][o], 1150 - x0[e]);
-            t[o] = __double_as_longlong(x);
-            if (live && m + e < M && time_order(x) <= X.thr[m + e]) pending |= 1u << o;
+            t[2 * i + e] = __double_as_longlong(x[e]);
+            if (live && m + e < M && time_order(x[e]) <= th[e]) pending |= 1u << (2 * i + e);
           }
         }
-      }
-      // offer; when a buffer is half full, or full, merge and offer the rest
-      while (true) {
-        bool call = false;
+      };
+      uint32_t sg = 0;
 #pragma unroll
-        for (int o = 0; o < 8; o++) {
-          if (pending & (1u << o)) {
-            const int mm = m + (o & 1);
-            if (time_order(__longlong_as_double(t[o])) > X.thr[mm]) {   // tightened since
-              pending &= ~(1u << o);
-            } else {
-              const int slot = atomicAdd(&X.cnt[mm], 1);
-              if (slot < TX_BUF) {
-                X.ct[mm][slot] = t[o];
-                X.cp[mm][slot] = (int32_t)(cur.p - base) + rl + 8 * (o >> 1);
-                pending &= ~(1u << o);
-              }
-              call |= slot >= TX_BUF / 2;
+      for (int o = 0; o < 8; o++) sg |= limb[3][o];
+      if (__any_sync(0xffffffffu, (int32_t)sg < 0)) emit(std::true_type{});
+      else emit(std::false_type{});
+      // offer the candidates; the warp that fills a buffer merges it
+      for (int tries = 0; __any_sync(0xffffffffu, pending); tries++) {
+        if (tries == TX_TRIES) s_abort = 1;   // never: a full buffer's owner empties it
+        if (__any_sync(0xffffffffu, s_abort)) {
+          ok = false;
+          break;
+        }
+        // one candidate of every lane that has any (unrolled over the eight, the code outgrows
+        // the instruction cache)
+        int mm = 0;
+        bool filled = false;
+        if (pending) {
+          const int o = __ffs(pending) - 1;
+          mm = m + (o & 1);
+          int64_t x = t[0];
+#pragma unroll
+          for (int n = 1; n < 8; n++) x = o == n ? t[n] : x;
+          const int32_t at = off + 8 * (o >> 1);
+          bool gone = !below(time_order(__longlong_as_double(x)), cur.p0 + at, mm);   // tightened since, or a tie with a larger row
+          if (!gone && *(volatile int32_t *)&X.cnt[mm] < TX_BUF) {
+            const int slot = atomicAdd(&X.cnt[mm], 1);
+            if (slot < TX_BUF) {
+              *(volatile int64_t *)&X.ct[mm][slot] = x;
+              *(volatile int32_t *)&X.cp[mm][slot] = at;
+              __threadfence_block();
+              atomicAdd(&X.wr[mm], 1);
+              gone = true;
+              filled = slot == TX_BUF - 1;
             }
           }
+          if (gone) pending &= pending - 1;
         }
-        if (meet(!ok)) return false;          // (also: every offer is written)
-        if (!meet(call || pending)) break;
-        merge();
-        meet(false);                          // lists, thresholds and counts are up to date
-        if (!meet(pending != 0)) break;
+        unsigned who;
+        while ((who = __ballot_sync(0xffffffffu, filled)) != 0) {
+          const int from = __ffs(who) - 1;
+          const int full_m = __shfl_sync(0xffffffffu, mm, from);
+          if (lane == from) filled = false;
+          int polls = 0;   // the other writers of the buffer are between reserving and writing
+          while (*(volatile int32_t *)&X.wr[full_m] < TX_BUF && ++polls < TX_TRIES) {}
+          __threadfence_block();
+          __syncwarp();
+          merge(full_m, TX_BUF);
+        }
       }
-      return true;
     };
-    TxCursor ahead(units, n_units);
-    feed(locate(ahead), 0);
-    if (ahead.more()) ahead.next();
-    feed(locate(ahead), 1);
-    if (ahead.more()) ahead.next();
-    base = cur.p;
-    for (; cur.more(); it++) {
-      // the rows of the tile after the next on their way into L2, 128 bytes per prefetch
-      const int64_t next = locate(ahead);
-      if (next >= 0 && (xp_kg<G>() & 1) == 0 && xp_kg<G>() * 64 < k * 8)
-        asm volatile("prefetch.global.L2 [%0];\n" ::"l"((const char *)(F + next * k) + xp_kg<G>() * 64));
-      int ps = 0;
+    locate(0);
+    feed(0);
+    locate(1);
+    feed(1);
+    for (; cur.more(n_units); it++) {
+      locate(it + 2);
 #pragma unroll 1
-      for (; ps < G::PASSES; ps++)
-        if (!pass(ps)) break;
-      if (ps < G::PASSES) break;
+      for (int ps = 0; ps < G::PASSES; ps++) pass(ps);
       const bool end = cur.last();
       if (end) {
-        // the unit's lists
-        merge();
+        meet();   // every candidate of the unit is in a buffer or merged
         for (int m = warp; m < M; m += XP_WARPS) {
+          merge(m, min(X.cnt[m], TX_BUF));
+          __syncwarp();
           if (lane < topk) {
             const int64_t r = X.lr[m][lane];
             const double t = __longlong_as_double(X.lt[m][lane]);
@@ -351,15 +398,10 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
         }
       }
       // every MMA of this tile is complete: its operand buffer takes the tile after the next
-      feed(next, it + 2);
-      if (ahead.more()) ahead.next();
-      cur.next();
-      if (end) {
-        base = cur.p;
-        meet(false);   // the lists are reset
-      }
+      if (ok) feed(it + 2);
+      advance(cur);
+      if (end) meet();   // the lists are reset
     }
-    if (!ok) s_abort = 1;
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
   __syncthreads();
