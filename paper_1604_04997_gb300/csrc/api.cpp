@@ -114,6 +114,7 @@ pm_status ctx_dcopy(pm_ctx *c, const void *h, size_t bytes, void **d) {
     CU(cudaDeviceSynchronize());
     for (auto &kv : c->dcache) cudaFree(kv.second);
     c->dcache.clear();
+    c->eval_plans.clear();   // their device arrays are in dcache
   }
   void *p = nullptr;
   CU(cudaMalloc(&p, std::max<size_t>(bytes, 16)));
@@ -138,6 +139,10 @@ pm_status ctx_scratch(pm_ctx *c, size_t bytes, void **d) {
 
 static pm_status upload_table(pm_ctx *c, int id) {
   const auto &w = c->tables[id];
+  if (c->canon[id] != id) {   // the same words are there already
+    c->dev_off[id] = c->dev_off[c->canon[id]];
+    return PM_OK;
+  }
   size_t need = c->arena_used + w.size();
   if (need > c->arena_cap) {
     size_t cap = std::max<size_t>(need * 2, size_t(1) << 20);
@@ -157,17 +162,33 @@ static pm_status upload_table(pm_ctx *c, int id) {
 
 // ------------------------------------------------------------------------------------- counting
 
-// Upload the newly added table id (the last one) to the device arena; on failure the
-// table is taken back out, so that no id refers to a table without device words.
-static pm_status register_on_device(pm_ctx *c, int id) {
-  if (c->device < 0) return PM_OK;
-  pm_status s = ctx_device_guard(c);
-  if (!s) s = upload_table(c, id);
-  if (s) {
-    c->tables.pop_back();
-    c->dev_off.pop_back();
+// Add a table's image: its id, and the first table with the same image (tables of equal
+// images are evaluated once, and share their device words).
+static pm_status add_table(pm_ctx *c, std::vector<uint32_t> words, int *out_id) {
+  const int id = (int)c->tables.size();
+  uint64_t h = 1469598103934665603ull;   // FNV-1a over the words
+  for (uint32_t w : words) h = (h ^ w) * 1099511628211ull;
+  auto &same = c->by_hash[h];
+  int canon = id;
+  for (int t : same)
+    if (c->tables[t] == words) { canon = t; break; }
+  c->tables.push_back(std::move(words));
+  c->dev_off.push_back(-1);
+  c->canon.push_back(canon);
+  if (canon == id) same.push_back(id);
+  if (c->device >= 0) {
+    pm_status s = ctx_device_guard(c);
+    if (!s) s = upload_table(c, id);
+    if (s) {   // taken back out, so that no id refers to a table without device words
+      if (canon == id) c->by_hash[h].pop_back();
+      c->tables.pop_back();
+      c->dev_off.pop_back();
+      c->canon.pop_back();
+      return s;
+    }
   }
-  return s;
+  *out_id = id;
+  return PM_OK;
 }
 
 extern "C" pm_status pm_compile_counts(pm_ctx *c, const char *ir, size_t len, int32_t layout, const int64_t *lo,
@@ -181,11 +202,7 @@ extern "C" pm_status pm_compile_counts(pm_ctx *c, const char *ir, size_t len, in
   int rc = pm_compile_table(ir, len, layout, lo, hi, words, inf, msg);
   if (rc) return pm_set_error(rc, msg);
   std::lock_guard<std::mutex> lk(c->mu);
-  int id = (int)c->tables.size();
-  c->tables.push_back(std::move(words));
-  c->dev_off.push_back(-1);
-  if (pm_status u = register_on_device(c, id)) return u;
-  *out_id = id;
+  if (pm_status u = add_table(c, std::move(words), out_id)) return u;
   if (info) {
     info->n_params = inf[0]; info->n_atoms = inf[1]; info->n_conds = inf[2]; info->n_pieces = inf[3];
     info->n_monomials = inf[4]; info->n_columns = inf[5]; info->n_words = inf[6]; info->degree = inf[7];
@@ -201,12 +218,7 @@ extern "C" pm_status pm_table_load(pm_ctx *c, const uint32_t *words, size_t n_wo
   std::string why;
   if (!pm_table_valid(words, n_words, why)) return pm_set_error(PM_ERR_INVALID_ARG, "table image rejected: " + why);
   std::lock_guard<std::mutex> lk(c->mu);
-  int id = (int)c->tables.size();
-  c->tables.emplace_back(words, words + n_words);
-  c->dev_off.push_back(-1);
-  if (pm_status u = register_on_device(c, id)) return u;
-  *out_id = id;
-  return PM_OK;
+  return add_table(c, std::vector<uint32_t>(words, words + n_words), out_id);
 }
 
 extern "C" pm_status pm_table_image(pm_ctx *c, int32_t id, uint32_t *buf, size_t cap, size_t *out_words) {
@@ -220,25 +232,51 @@ extern "C" pm_status pm_table_image(pm_ctx *c, int32_t id, uint32_t *buf, size_t
   return PM_OK;
 }
 
-pm_status ctx_table_offsets(pm_ctx *c, const int32_t *ids, int n, int *P, int *K, const int64_t **d_off) {
-  std::vector<int64_t> off(n);
-  *P = -1;
-  *K = -1;
+// The work list of a table list: per distinct table the output positions it fills, in items
+// of at most `per_item` positions.
+static pm_status eval_plan(pm_ctx *c, const int32_t *ids, int n, int per_item, const EvalPlan **out) {
+  std::string key((const char *)ids, (size_t)n * sizeof(int32_t));
+  key.append((const char *)&per_item, sizeof per_item);
+  auto it = c->eval_plans.find(key);
+  if (it != c->eval_plans.end()) { *out = &it->second; return PM_OK; }
+  EvalPlan p;
+  std::unordered_map<int, int> slot;             // canonical table -> its members
+  std::vector<std::vector<int32_t>> members;
+  std::vector<int> tab;
   for (int i = 0; i < n; i++) {
-    int id = ids[i];
+    const int id = ids[i];
     if (id < 0 || id >= (int)c->tables.size()) return pm_set_error(PM_ERR_NOT_FOUND, "unknown table id");
     const auto &w = c->tables[id];
-    int p = (int)w[pmt::H_NPARAMS], k = (int)w[pmt::H_K];
-    if (*P < 0) { *P = p; *K = k; }
-    if (P && *P != p) return pm_set_error(PM_ERR_INVALID_ARG, "tables differ in parameter count");
-    if (*K != k) return pm_set_error(PM_ERR_INVALID_ARG, "tables differ in layout");
-    if (c->device >= 0 && c->dev_off[id] < 0) return pm_set_error(PM_ERR_INVALID_ARG, "table not on the device");
-    off[i] = c->dev_off[id];
+    if (i == 0) { p.P = (int)w[pmt::H_NPARAMS]; p.K = (int)w[pmt::H_K]; }
+    if (p.P != (int)w[pmt::H_NPARAMS]) return pm_set_error(PM_ERR_INVALID_ARG, "tables differ in parameter count");
+    if (p.K != (int)w[pmt::H_K]) return pm_set_error(PM_ERR_INVALID_ARG, "tables differ in layout");
+    if (c->dev_off[id] < 0) return pm_set_error(PM_ERR_INVALID_ARG, "table not on the device");
+    const auto at = slot.emplace(c->canon[id], (int)tab.size());
+    if (at.second) {
+      tab.push_back(c->canon[id]);
+      members.emplace_back();
+      p.max_words = std::max(p.max_words, (int)w.size());
+    }
+    members[at.first->second].push_back(i);
   }
+  std::vector<int32_t> items, list;
+  for (size_t t = 0; t < tab.size(); t++) {
+    const int cnt = (int)members[t].size();
+    for (int m = 0; m < cnt; m += per_item) {
+      const int k = std::min(per_item, cnt - m);
+      const int64_t off = c->dev_off[tab[t]];
+      items.insert(items.end(), {(int32_t)(uint32_t)off, (int32_t)list.size(), k, (int32_t)(off >> 32)});
+      list.insert(list.end(), members[t].begin() + m, members[t].begin() + m + k);
+    }
+  }
+  p.n_items = (int)items.size() / 4;
+  items.insert(items.end(), list.begin(), list.end());
   void *d = nullptr;
-  pm_status s = ctx_dcopy(c, off.data(), off.size() * 8, &d);
-  *d_off = (const int64_t *)d;
-  return s;
+  pm_status s = ctx_dcopy(c, items.data(), items.size() * sizeof(int32_t), &d);
+  if (s) return s;
+  p.d_items = (const int32_t *)d;
+  *out = &(c->eval_plans[key] = p);
+  return PM_OK;
 }
 
 extern "C" pm_status pm_eval_counts(pm_ctx *c, const int32_t *ids, int32_t n_tables, const int64_t *d_points,
@@ -249,18 +287,22 @@ extern "C" pm_status pm_eval_counts(pm_ctx *c, const int32_t *ids, int32_t n_tab
   if (n_tables < 0 || n_points < 0 || (n_tables && !ids)) return pm_set_error(PM_ERR_INVALID_ARG, "bad sizes");
   if (n_tables == 0 || n_points == 0) return PM_OK;
   if (!d_points || !d_counts) return pm_set_error(PM_ERR_INVALID_ARG, "null device buffer");
-  // the launch puts points on grid x (128 per block) and tables on grid y (at most 65,535)
+  // the launch puts points on grid x (128 per block) and work items on grid y (at most 65,535)
   if (n_points > (int64_t(1) << 37)) return pm_set_error(PM_ERR_INVALID_ARG, "too many points");
-  int P, K;
-  const int64_t *d_off;
-  pm_status s = ctx_table_offsets(c, ids, n_tables, &P, &K, &d_off);
+  // A block evaluates 128 points of one table and writes the rows of up to eight positions
+  // that name it: about 2,800 blocks of eight take 109 us where 21,248 of one took 201 (2,656
+  // tables x 1,024 points).  Fewer positions a block where that would leave fewer than 16
+  // blocks per SM (three are resident): small calls keep one block per position.
+  const int64_t chunks = (n_points + 127) / 128;
+  const int per_item = (int)std::min<int64_t>(8, std::max<int64_t>(1, chunks * n_tables / ((int64_t)c->n_sms * 16)));
+  const EvalPlan *p = nullptr;
+  pm_status s = eval_plan(c, ids, n_tables, per_item, &p);
   if (s) return s;
   constexpr int64_t MAX_GRID_Y = 65535;
-  for (int64_t t0 = 0; t0 < n_tables; t0 += MAX_GRID_Y) {
-    const int nt = (int)std::min<int64_t>(MAX_GRID_Y, n_tables - t0);
-    CU(pmd::launch_eval_counts(c->arena, d_off + t0, nt, d_points, n_points, P, K,
-                               d_counts + (int64_t)t0 * n_points * K, c->d_status, (cudaStream_t)stream));
-  }
+  for (int64_t t0 = 0; t0 < p->n_items; t0 += MAX_GRID_Y)
+    CU(pmd::launch_eval_counts(c->arena, p->d_items + 4 * t0, p->d_items + 4 * (int64_t)p->n_items,
+                               (int)std::min<int64_t>(MAX_GRID_Y, p->n_items - t0), p->max_words, d_points, n_points, p->P, p->K,
+                               d_counts, c->d_status, (cudaStream_t)stream));
   return PM_OK;
 }
 

@@ -14,19 +14,28 @@ namespace pmd {
 
 constexpr int K1_THREADS = 128;
 
+// One block: 128 points of one distinct table, one thread per point; the rows are staged in
+// shared memory and written to every output position that names the table, as contiguous
+// 16-byte pieces (the counts of a tuning space repeat: 2,656 matmul variants have 32 distinct
+// tables).  Bound by the HBM writes where tables repeat (2,656 tables x 1,024 points, 696 MB:
+// 201 us with every position evaluated, 109 now, 6.4 TB/s); else by the evaluation's latency,
+// at the warps that the staged rows and slots (57 KB per block, and the largest table's words)
+// leave room for.
 template <int K>
 __global__ void __launch_bounds__(K1_THREADS) k_eval_counts(const uint32_t *__restrict__ arena,
-                                                           const int64_t *__restrict__ tab_off,
+                                                           const int4 *__restrict__ items,
+                                                           const int32_t *__restrict__ members, int table_words,
                                                            const int64_t *__restrict__ points, int64_t n_points,
                                                            int P, int64_t *__restrict__ out, int *status) {
   extern __shared__ __align__(16) uint8_t smem[];
-  uint32_t *sT = (uint32_t *)smem;                                   // table, <= 16 KB
-  int64_t *stage = (int64_t *)(smem + pmt::MAX_TABLE_WORDS * 4);     // [threads][K+1]
+  uint32_t *sT = (uint32_t *)smem;                                   // the table
+  int64_t *stage = (int64_t *)(smem + table_words * 4);              // [threads][K+1]
   int64_t *slots = stage + K1_THREADS * (K + 1);                     // [24][threads]
   const int tid = threadIdx.x;
-  const uint32_t *gT = arena + tab_off[blockIdx.y];
+  const int4 item = items[blockIdx.y];
+  const uint32_t *gT = arena + ((int64_t)item.w << 32 | (uint32_t)item.x);
   const int words = (int)gT[pmt::H_WORDS];
-  if (gT[pmt::H_MAGIC] != pmt::MAGIC || words > pmt::MAX_TABLE_WORDS || (int)gT[pmt::H_K] != K) {
+  if (gT[pmt::H_MAGIC] != pmt::MAGIC || words > table_words || (int)gT[pmt::H_K] != K) {
     if (tid == 0) atomicOr(status, ST_BAD_TABLE);
     return;
   }
@@ -54,35 +63,42 @@ __global__ void __launch_bounds__(K1_THREADS) k_eval_counts(const uint32_t *__re
     }
   }
   __syncthreads();
-  const int64_t nvalid = min((int64_t)K1_THREADS, n_points - p0);
-  int64_t *dst = out + ((int64_t)blockIdx.y * n_points + p0) * K;
-  const int total = (int)nvalid * K;
-  for (int i = tid; i < total; i += K1_THREADS) {   // streaming stores: the rows are not reread
-    int r = i / K, c = i - r * K;
-    __stcs(dst + i, stage[r * (K + 1) + c]);
-  }
-}
-
-size_t k1_smem_bytes(int K) {
-  return (size_t)pmt::MAX_TABLE_WORDS * 4 + (size_t)K1_THREADS * (K + 1) * 8 +
-         (size_t)pmt::MAX_SLOTS * K1_THREADS * 8;
-}
-
-cudaError_t launch_eval_counts(const uint32_t *arena, const int64_t *d_tab_off, int n_tables, const int64_t *points,
-                               int64_t n_points, int P, int K, int64_t *out, int *status, cudaStream_t st) {
-  if (n_points == 0 || n_tables == 0) return cudaSuccess;
-  dim3 grid((unsigned)((n_points + K1_THREADS - 1) / K1_THREADS), (unsigned)n_tables);
-  size_t sm = k1_smem_bytes(K);
-  if (K == 32) {
-    cudaFuncSetAttribute(k_eval_counts<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_eval_counts<32><<<grid, K1_THREADS, sm, st>>>(arena, d_tab_off, points, n_points, P, out, status);
-  } else if (K == 12) {
-    cudaFuncSetAttribute(k_eval_counts<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_eval_counts<12><<<grid, K1_THREADS, sm, st>>>(arena, d_tab_off, points, n_points, P, out, status);
+  // streaming stores: the rows are not reread.  This thread's columns 2 c2 and + 1 of rows
+  // r0, r0 + K1_THREADS / (K / 2), ..
+  const int nvalid = (int)min((int64_t)K1_THREADS, n_points - p0);
+  constexpr int H = K / 2;
+  if (((uintptr_t)out & 15) == 0) {
+    for (int i = tid; i < nvalid * H; i += K1_THREADS) {
+      const int r = i / H, c2 = i - r * H;
+      const longlong2 v = make_longlong2(stage[r * (K + 1) + 2 * c2], stage[r * (K + 1) + 2 * c2 + 1]);
+      for (int m = 0; m < item.z; m++)
+        __stcs((longlong2 *)(out + ((int64_t)members[item.y + m] * n_points + p0) * K) + i, v);
+    }
   } else {
-    return cudaErrorInvalidValue;
+    for (int i = tid; i < nvalid * K; i += K1_THREADS) {
+      const int r = i / K, c = i - r * K;
+      for (int m = 0; m < item.z; m++)
+        __stcs(out + ((int64_t)members[item.y + m] * n_points + p0) * K + i, stage[r * (K + 1) + c]);
+    }
   }
-  return cudaGetLastError();
+}
+
+cudaError_t launch_eval_counts(const uint32_t *arena, const int32_t *items, const int32_t *members, int n_items,
+                               int max_words, const int64_t *points, int64_t n_points, int P, int K, int64_t *out,
+                               int *status, cudaStream_t st) {
+  if (n_points == 0 || n_items == 0) return cudaSuccess;
+  const dim3 grid((unsigned)((n_points + K1_THREADS - 1) / K1_THREADS), (unsigned)n_items);
+  const int words = (max_words + 3) & ~3;
+  const size_t sm = (size_t)words * 4 + (size_t)K1_THREADS * (K + 1) * 8 + (size_t)pmt::MAX_SLOTS * K1_THREADS * 8;
+  auto launch = [&](auto kernel) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    kernel<<<grid, K1_THREADS, sm, st>>>(arena, (const int4 *)items, members, words, points, n_points, P, out, status);
+    return cudaGetLastError();
+  };
+  if (K == 32) return launch(k_eval_counts<32>);
+  if (K == 12) return launch(k_eval_counts<12>);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace pmd

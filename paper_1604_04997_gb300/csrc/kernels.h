@@ -9,8 +9,11 @@ namespace pmd {
 enum StatusBits { ST_OUT_OF_BOX = 1, ST_BAD_TABLE = 2, ST_TIMEOUT = 4, ST_BAD_INPUT = 8, ST_BAD_ROW = 16 };
 
 // K1 (eval.cu)
-cudaError_t launch_eval_counts(const uint32_t *arena, const int64_t *d_tab_off, int n_tables, const int64_t *points,
-                               int64_t n_points, int P, int K, int64_t *out, int *status, cudaStream_t st);
+// items: [n_items][4] (arena word offset low, first member, members, offset high); members: the table
+// positions an item's rows are written to; max_words: the largest table
+cudaError_t launch_eval_counts(const uint32_t *arena, const int32_t *items, const int32_t *members, int n_items,
+                               int max_words, const int64_t *points, int64_t n_points, int P, int K, int64_t *out,
+                               int *status, cudaStream_t st);
 
 // Fused ranking (rank.cu).  A ranking group's image (32-bit words, 16-byte aligned
 // sections; built by plan.cpp):

@@ -686,16 +686,7 @@ static pm_status build_host_plan(pm_ctx *c, const int32_t *tables, const int32_t
     if (var_off[t + 1] < var_off[t] || var_off[t + 1] - var_off[t] > 65536)
       return pm_set_error(PM_ERR_INVALID_ARG, "at most 65,536 variants per template");
   // Tables with the same image evaluate alike; they share one program in a group.
-  std::map<std::vector<uint32_t>, int> image_id;
-  std::vector<int> canon(c->tables.size(), -1);
-  auto canonical = [&](int id) {
-    if (canon[id] < 0) {
-      auto it = image_id.find(c->tables[id]);
-      if (it == image_id.end()) it = image_id.emplace(c->tables[id], id).first;
-      canon[id] = it->second;
-    }
-    return canon[id];
-  };
+  auto canonical = [&](int id) { return c->canon[id]; };
   try {
     for (int t = 0; t < T; t++) {
       first_group[t] = (int)groups.size() / 2;

@@ -6,6 +6,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "pm.h"
@@ -41,6 +42,13 @@ struct Plan {
   int g_topk = 0, g_nw = 0, g_grid = 0;
 };
 
+// Device work list of one pm_eval_counts table list: distinct tables, each with the output
+// positions it fills.
+struct EvalPlan {
+  int P = 0, K = 0, n_items = 0, max_words = 0;
+  const int32_t *d_items = nullptr;   // [n_items][4] (arena word offset low, first member, members, offset high), then the members
+};
+
 struct pm_ctx {
   int device = -1;
   int n_sms = 0;
@@ -48,6 +56,9 @@ struct pm_ctx {
   std::mutex mu;
   std::vector<std::vector<uint32_t>> tables;  // host images
   std::vector<int64_t> dev_off;               // word offset of each table in the arena
+  std::vector<int> canon;                     // the first table with the same image (they share device words)
+  std::unordered_map<uint64_t, std::vector<int>> by_hash;   // first tables by their image's hash
+  std::map<std::string, EvalPlan> eval_plans; // pm_eval_counts argument lists seen (device arrays in dcache)
   uint32_t *arena = nullptr;
   size_t arena_cap = 0, arena_used = 0;       // in words
   int *d_status = nullptr;
@@ -70,7 +81,6 @@ pm_status pm_set_error_c(pm_status code, const char *m);
 pm_status ctx_device_guard(pm_ctx *c);
 pm_status ctx_dcopy(pm_ctx *c, const void *h, size_t bytes, void **d);
 pm_status ctx_scratch(pm_ctx *c, size_t bytes, void **d);
-pm_status ctx_table_offsets(pm_ctx *c, const int32_t *ids, int n, int *P, int *K, const int64_t **d_off);
 pm_status ctx_plan_k2(pm_ctx *c, const int32_t *tables, const int32_t *var_off, int n_templates,
                       const int64_t *pt_off, Plan **out);
 pm_status ctx_run_k2(pm_ctx *c, Plan *p, const int32_t *tables, const int32_t *var_off, const int64_t *pt_off,
