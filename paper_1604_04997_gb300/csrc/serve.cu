@@ -9,28 +9,26 @@
 //   k_serve_topk  one CTA per query -> topk (key, candidate) pairs, ordered by
 //                 (time, candidate index), converted to times.
 #include "eval_common.cuh"
+#include "topk_list.cuh"
 
 namespace pmd {
 
 constexpr int SV_THREADS = 128;      // candidates per k_serve_eval CTA
-constexpr int SV_TOPK_THREADS = 256;
+constexpr int SV_TOPK_WARPS = 16;
 
 // Per-model fixed-point weights W_i = round(w_i 2^E) (sum |W_i| <= 2^62) as 28-bit limb
-// triples; thread 0 finds E with the same serial loop in every CTA of a batch, so every
-// CTA derives the same values.
-__device__ __forceinline__ void load_model_limbs(const double *w, Limbs3 *s_w, int *s_E) {
-  if (threadIdx.x == 0) *s_E = weight_exponent(w, 32);
-  __syncthreads();
-  if (threadIdx.x < 32) s_w[threadIdx.x] = to_limbs3(llrint(ldexp(w[threadIdx.x], *s_E)));
+// triples, by the block's first warp (E by weight_exponent_warp: one thread's chain of 32
+// FP64 additions cost every block of a batch more than the rest of its prologue).
+__device__ __forceinline__ void load_model_limbs(const double *w, Limbs3 *s_w) {
+  if (threadIdx.x < 32) s_w[threadIdx.x] = to_limbs3(llrint(ldexp(w[threadIdx.x], weight_exponent_warp(w))));
 }
 
 __global__ void __launch_bounds__(SV_THREADS) k_serve_eval(ServeArgs a) {
   __shared__ int64_t slots[pmt::MAX_SLOTS * SV_THREADS];
   __shared__ Limbs3 s_w[32];
-  __shared__ int s_E;
   const int2 b = a.blocks[blockIdx.x];
   const SQuery q = a.queries[b.x];
-  load_model_limbs(a.models + (int64_t)q.model * 32, s_w, &s_E);
+  load_model_limbs(a.models + (int64_t)q.model * 32, s_w);
   __syncthreads();
   const int i = b.y * SV_THREADS + threadIdx.x;
   if (i >= q.n) return;
@@ -53,81 +51,72 @@ __global__ void __launch_bounds__(SV_THREADS) k_serve_eval(ServeArgs a) {
   a.keys[c] = key;
 }
 
-// Sorted (key, index) list of the 16 smallest pairs seen by one thread.
-struct SvList {
-  int64_t k[SV_MAX_TOPK];
-  int32_t id[SV_MAX_TOPK];
-  __device__ __forceinline__ void init() {
-#pragma unroll
-    for (int j = 0; j < SV_MAX_TOPK; j++) { k[j] = INT64_MAX; id[j] = 0x7fffffff; }
-  }
-  // indices arrive in increasing order: an equal key ranks after the ones already held
-  __device__ __forceinline__ void insert(int64_t key, int32_t idx) {
-    if (!(key < k[SV_MAX_TOPK - 1])) return;
-#pragma unroll
-    for (int j = SV_MAX_TOPK - 1; j > 0; j--) {
-      const bool shift = key < k[j - 1];
-      const bool here = !shift && key < k[j];
-      if (shift) { k[j] = k[j - 1]; id[j] = id[j - 1]; }
-      else if (here) { k[j] = key; id[j] = idx; }
-    }
-    if (key < k[0]) { k[0] = key; id[0] = idx; }
-  }
-  __device__ __forceinline__ void pop() {
-#pragma unroll
-    for (int j = 0; j < SV_MAX_TOPK - 1; j++) { k[j] = k[j + 1]; id[j] = id[j + 1]; }
-    k[SV_MAX_TOPK - 1] = INT64_MAX;
-    id[SV_MAX_TOPK - 1] = 0x7fffffff;
-  }
-};
-
-__device__ __forceinline__ bool pair_less(int64_t ka, int32_t ia, int64_t kb, int32_t ib) {
-  return ka < kb || (ka == kb && ia < ib);
-}
-
-__global__ void __launch_bounds__(SV_TOPK_THREADS) k_serve_topk(ServeArgs a) {
-  __shared__ Limbs3 s_w[32];
-  __shared__ int s_E;
-  __shared__ int64_t r_k[SV_TOPK_THREADS / 32];
-  __shared__ int32_t r_i[SV_TOPK_THREADS / 32];
+// One CTA per query.  Each warp keeps one sorted list of its smallest (key, index) pairs, an
+// entry per lane, and merges 32 keys at a time into it.  Bound by the issue of those merges
+// (some 400 instructions each), so the warps share the least of their lists' last entries:
+// after the first batches nearly every key falls to one comparison and a vote.  Largest and
+// smallest query of a burst, by the kernel's time: 126 and 12.6 us with a list of 16 per
+// thread (every lane inserting on its own, then topk rounds over the block), 80 and 6.1 with
+// 32 warps and no shared bound, 58 and 5.3 now; one query of 16 candidates from submission to
+// result 51 -> 37 us.
+//
+// Keys ride through the list as the doubles whose time_order they are; they stay below that
+// of +inf (|S| < 2^126, so a key's top byte is at most 0x7e).
+__global__ void __launch_bounds__(SV_TOPK_WARPS * 32) k_serve_topk(ServeArgs a) {
+  __shared__ double s_k[SV_TOPK_WARPS][SV_MAX_TOPK];
+  __shared__ int64_t s_i[SV_TOPK_WARPS][SV_MAX_TOPK];
+  __shared__ long long s_thr;   // no key above it is among the topk: the least of the warps' last entries
+  static_assert(SV_MAX_TOPK == 16 && SV_TOPK_WARPS % 2 == 0, "two warps' lists are merged at a time");
   const SQuery q = a.queries[blockIdx.x];
-  load_model_limbs(a.models + (int64_t)q.model * 32, s_w, &s_E);
-  SvList L;
-  L.init();
-  for (int i = threadIdx.x; i < q.n; i += SV_TOPK_THREADS) L.insert(a.keys[q.begin + i], i);
-  __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int r = 0; r < q.topk; r++) {
-    // block-wide smallest head; every index is held by exactly one thread
-    int64_t bk = L.k[0];
-    int32_t bi = L.id[0];
+  const int64_t *keys = a.keys + q.begin;
+  if (threadIdx.x == 0) s_thr = INT64_MAX;
+  __syncthreads();
+  double lt = TK_INF;
+  int64_t lr = INT64_MAX;
+  for (int64_t b = 32 * warp; b < q.n; b += 4 * 32 * SV_TOPK_WARPS) {   // warp-uniform
+    int64_t k[4];
 #pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      const int64_t ok = __shfl_xor_sync(0xffffffffu, bk, o);
-      const int32_t oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (pair_less(ok, oi, bk, bi)) { bk = ok; bi = oi; }
+    for (int u = 0; u < 4; u++) {
+      const int64_t i = b + u * 32 * SV_TOPK_WARPS + lane;
+      k[u] = i < q.n ? keys[i] : INT64_MAX;
     }
-    if (lane == 0) { r_k[warp] = bk; r_i[warp] = bi; }
-    __syncthreads();
-    bk = r_k[0];
-    bi = r_i[0];
-#pragma unroll
-    for (int w = 1; w < SV_TOPK_THREADS / 32; w++)
-      if (pair_less(r_k[w], r_i[w], bk, bi)) { bk = r_k[w]; bi = r_i[w]; }
-    __syncthreads();
-    if (L.id[0] == bi && bi != 0x7fffffff) L.pop();
-    if (threadIdx.x == 0) {
-      const bool real = bi != 0x7fffffff;
-      a.out_idx[(int64_t)blockIdx.x * SV_MAX_TOPK + r] = real ? bi : -1;
-      a.out_t[(int64_t)blockIdx.x * SV_MAX_TOPK + r] =
-          real ? key_value(bk, s_E) : __longlong_as_double(0x7ff0000000000000ll);
+#pragma unroll 1
+    for (int u = 0; u < 4; u++) {   // one copy of the merge's code
+      const bool ok = k[0] != INT64_MAX && k[0] <= *(volatile long long *)&s_thr;
+      if (__any_sync(0xffffffffu, ok)) {
+        const double t = __longlong_as_double(k[0] ^ ((k[0] >> 63) & 0x7fffffffffffffffll));
+        warp_list_merge(lt, lr, t, b + u * 32 * SV_TOPK_WARPS + lane, ok, q.topk, lane);
+        if (lane == q.topk - 1 && lr != INT64_MAX && time_order(lt) < *(volatile long long *)&s_thr)
+          atomicMin(&s_thr, (long long)time_order(lt));
+      }
+      k[0] = k[1], k[1] = k[2], k[2] = k[3], k[3] = INT64_MAX;
     }
+  }
+  if (lane < SV_MAX_TOPK) {
+    s_k[warp][lane] = lt;
+    s_i[warp][lane] = lr;
+  }
+  __syncthreads();
+  if (warp) return;
+  const int E = weight_exponent_warp(a.models + (int64_t)q.model * 32);
+#pragma unroll 1
+  for (int w = 0; w < SV_TOPK_WARPS; w += 2) {
+    const int64_t r = w ? s_i[w + (lane >> 4)][lane & 15] : s_i[1][lane & 15];
+    const double t = w ? s_k[w + (lane >> 4)][lane & 15] : s_k[1][lane & 15];
+    warp_list_merge(lt, lr, t, r, r != INT64_MAX && (w || lane < 16), q.topk, lane);   // the warp's own list is held
+  }
+  if (lane < q.topk) {
+    const bool real = lr != INT64_MAX;
+    a.out_idx[(int64_t)blockIdx.x * SV_MAX_TOPK + lane] = real ? (int32_t)lr : -1;
+    a.out_t[(int64_t)blockIdx.x * SV_MAX_TOPK + lane] =
+        real ? key_value(time_order(lt), E) : __longlong_as_double(0x7ff0000000000000ll);
   }
 }
 
 cudaError_t launch_serve(const ServeArgs &a, int n_blocks, cudaStream_t st) {
   if (n_blocks > 0) k_serve_eval<<<n_blocks, SV_THREADS, 0, st>>>(a);
-  if (a.n_queries > 0) k_serve_topk<<<a.n_queries, SV_TOPK_THREADS, 0, st>>>(a);
+  if (a.n_queries > 0) k_serve_topk<<<a.n_queries, SV_TOPK_WARPS * 32, 0, st>>>(a);
   return cudaGetLastError();
 }
 
