@@ -260,7 +260,7 @@ def _plain_form(ctx, bp, d_w, dev, stream, fused_idx, reps=2):
     return {"ms": eval_ms + rank_ms, "eval_counts_ms": eval_ms, "predict_topk_ms": rank_ms,
             "points_with_identical_top16": same / max(1, total),
             "note": "per template: pm_eval_counts (all 32 counts to HBM, 10.5 GB) then pm_predict_topk "
-                    "(PM_PREC_FP64, one model, per-point row lists; one row per lane for M <= 8): "
+                    "(PM_PREC_FP64, one model, per-point row lists; one row per lane for few models): "
                     "the same exact arithmetic and ranking as the fused launch"}
 
 
@@ -425,6 +425,8 @@ def run_ours(args):
                          "unit": "T lane-ops/s", "frac": achieved / peak_ops, "traffic": traffic,
                          "kernel": "k_rank",
                          "ops_per_eval": info["work_per_eval"],
+                         "ops_note": "integer operations of each variant's own exact sum; variants whose tables are "
+                                     "equal share one evaluation, so fewer are executed",
                          "peak_note": f"{sms} SMs x 128 lanes x {max_mhz:.0f} MHz (issue bound, derived)",
                          "measured_peak": measured_ops / 1e12, "frac_of_measured": achieved / measured_ops,
                          "measured_peak_note": "integer issue-rate probe (pmm_int_issue_rate): independent "
@@ -590,11 +592,7 @@ def run_other(args):
                             "bytes_per_step": nbytes, "l2": "inputs (256 MB) and output (512 MB) larger than L2",
                             "argmin_only_ms": ms_arg, "argmin_only_gbs": nb_arg / (ms_arg / 1e3) / 1e9,
                             "fp64_accurate_ms": times["fp64_T"][0],
-                            # the exact path's integer work: ten 32-bit multiply-adds per 64 x 64-bit product
-                            "fp64_accurate_frac_of_lane_op_peak":
-                                R * M * 32 * 10 / (times["fp64_T"][0] / 1e3) /
-                                (torch.cuda.get_device_properties(dev).multi_processor_count * 128 *
-                                 float(_peaks().get("sm_max_mhz", 2070.0)) * 1e6),
+                            "fp64_accurate_gbs": nbytes / (times["fp64_T"][0] / 1e3) / 1e9,
                             "fp64_accurate_top16_ms": {"one group of 1e6 rows": times["fp64_topk16_one_group"][0],
                                                        "4096 groups of ~244 rows":
                                                            times["fp64_topk16_4096_groups"][0]}},
@@ -619,15 +617,15 @@ def run_other(args):
         gram_flops = 2.0 * 32 * 32 * R * M          # the 64 Gram matrices' useful flops
         line = dict(base, metric="weight fits/s (200,000 rows x 32 features, 64 models, 3 refinement steps)",
                     value=M / (ms / 1e3), unit="model fits/s", ms_per_step=ms, higher_is_better=True,
-                    dtype="Gram on tcgen05 from three bf16 terms of A, fp32 accumulation per 4096-row chunk "
+                    dtype="Gram on tcgen05 from three bf16 terms, fp32 accumulation over at most 672 rows "
                           "(exact bf16-digit Gram if refinement stalls), FP64 Cholesky, exact residual products",
                     config={"workload": "200,000 x 32 int64 features, 64 device models, relative objective",
                             "float_float_gram_ms_per_step": ms_ff},
                     roofline={"bound": "tensor", "achieved": gram_flops / (ms / 1e3) / 1e12, "peak": peak_tc,
                               "unit": "TFLOP/s", "frac": gram_flops / (ms / 1e3) / 1e12 / peak_tc, "traffic": None,
-                              "kernel": "pm_fit_weights (whole call; the Gram kernel is a third of it)",
-                              "note": "useful Gram flops 2 k^2 R M over the whole fit; the three-term split "
-                                      "executes 9 bf16 term-pair products (one 128 x 96 MMA tile) per useful product"},
+                              "kernel": "pm_fit_weights (whole call; the Gram kernel is a tenth of it)",
+                              "note": "useful Gram flops 2 k^2 R M over the whole fit; one product [pairs x rows] "
+                                      "[rows x models] of six bf16 term products serves all models"},
                     clocks=ck, gpu_launches=None)
     print(json.dumps(line))
     ctx.close()
