@@ -298,15 +298,18 @@ __device__ __forceinline__ bool xp_try(uint32_t mbar, uint32_t parity) {
   return done != 0;
 }
 
-// Wait for one phase of mbar: false if it took longer than MBAR_WAIT_NS, or if another
-// thread has given up (*s_abort).
-__device__ __forceinline__ bool xp_wait_one(uint32_t mbar, uint32_t parity, volatile int *s_abort) {
+constexpr unsigned long long XP_HELD_NS = 2000000ull;   // the waits of the HELD kernels (tests)
+
+// Wait for one phase of mbar: false if it took longer than limit_ns, or if another thread has
+// given up; *s_abort is set in both cases.
+__device__ __forceinline__ bool xp_wait_one(uint32_t mbar, uint32_t parity, volatile int *s_abort,
+                                            unsigned long long limit_ns) {
   bool ok = xp_try(mbar, parity);
   if (!ok) {
     const unsigned long long t0 = globaltimer_ns();
     while (!ok && !*s_abort) {
       ok = xp_try(mbar, parity);
-      if (!ok && globaltimer_ns() - t0 > MBAR_WAIT_NS) *s_abort = 1;
+      if (!ok && globaltimer_ns() - t0 > limit_ns) *s_abort = 1;
     }
   }
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
@@ -314,8 +317,28 @@ __device__ __forceinline__ bool xp_wait_one(uint32_t mbar, uint32_t parity, vola
 }
 
 // the same for a whole warp, with the same result in all lanes
-__device__ __forceinline__ bool xp_wait(uint32_t mbar, uint32_t parity, volatile int *s_abort) {
-  return __all_sync(0xffffffffu, xp_wait_one(mbar, parity, s_abort));
+__device__ __forceinline__ bool xp_wait(uint32_t mbar, uint32_t parity, volatile int *s_abort,
+                                        unsigned long long limit_ns = MBAR_WAIT_NS) {
+  return __all_sync(0xffffffffu, xp_wait_one(mbar, parity, s_abort, limit_ns));
+}
+
+// What a kernel does before it frees its TMEM: after a wait of any warp ran out, the status
+// bit, and the MMAs in flight finish (bounded).  Every thread of the CTA calls it, past all of
+// its waits; the issuing warp (issuer) gives the number n of commits that it made in turn to
+// the `ring` barriers mbar[0 .. ring).  The issuing warp cannot report alone: it runs ahead of
+// the others, and has left when they wait for the last sums.
+__device__ __forceinline__ void xp_finish(volatile int *s_abort, int *status, bool issuer, const uint64_t *mbar,
+                                          uint32_t ring, uint32_t n) {
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
+  __syncthreads();
+  if (!*s_abort) return;   // the same for all threads
+  if (threadIdx.x == 0 && status) atomicOr(status, ST_TIMEOUT);
+  if (issuer) {
+    const unsigned long long t0 = globaltimer_ns();
+    for (uint32_t i = n >= ring ? n - ring : 0; i < n; i++)
+      while (!xp_try(xp_saddr(&mbar[i % ring]), (i / ring) & 1) && globaltimer_ns() - t0 < MBAR_WAIT_NS) {}
+  }
+  __syncthreads();
 }
 
 __device__ __forceinline__ void xp_arrive(uint32_t mbar) {

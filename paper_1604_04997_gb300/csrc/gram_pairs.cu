@@ -26,6 +26,7 @@
 
 #include "exact_tc.cuh"
 #include "kernels.h"
+#include "pm.h"
 
 namespace pmd {
 
@@ -81,12 +82,15 @@ __device__ __forceinline__ void gp_pair(int p, int k, int &a, int &b) {
 }  // namespace
 
 // Uh: [R][32] (zero columns beyond k); rfh, rfl: row factors as float-float [R][ld];
-// rmax: their column maxima (float bits)
+// rmax: their column maxima (float bits).  HELD: the issuing warp leaves without reporting its
+// sums and the waits are short (pmx_gram_held).
+template <bool HELD>
 __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__restrict__ Uh, const float *__restrict__ rfh,
                                                               const float *__restrict__ rfl, int ld, int64_t R, int k,
                                                               int M, int64_t rows_per_cta, const unsigned *__restrict__ amax,
                                                               const unsigned *__restrict__ rmax,
                                                               double *__restrict__ G, int *status) {
+  constexpr unsigned long long LIMIT = HELD ? XP_HELD_NS : MBAR_WAIT_NS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((128u - (xp_saddr(smem_raw) & 127u)) & 127u);
   float(*su)[32][GP_USTRIDE] = (float(*)[32][GP_USTRIDE])(smem + GP_RING * GP_STAGE);
@@ -135,10 +139,10 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
     // kind::f16: D fp32, A and B bf16, both K-major
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t)(nb >> 3) << 17 | (128u >> 4) << 24;
     for (int64_t rb = r0; rb < r1 && ok; rb += GP_SUB, sub++) {
-      if (sub && !(ok = xp_wait(xp_saddr(&drained), (sub - 1) & 1, &s_abort))) break;
+      if (sub && !(ok = xp_wait(xp_saddr(&drained), (sub - 1) & 1, &s_abort, LIMIT))) break;
       for (int64_t rs = rb; rs < min(r1, rb + GP_SUB); rs += GP_K, n++) {
         const uint32_t b = n % GP_RING;
-        if (!(ok = xp_wait(xp_saddr(&ready[b]), (n / GP_RING) & 1, &s_abort))) break;
+        if (!(ok = xp_wait(xp_saddr(&ready[b]), (n / GP_RING) & 1, &s_abort, LIMIT))) break;
         const uint32_t sa = s0 + b * GP_STAGE, sb = sa + 3 * GP_ATERM;
 #pragma unroll
         for (int p = 0; p < 6; p++) {   // term products 11, 12, 21, 13, 22, 31
@@ -151,14 +155,7 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
         }
         xp_commit(xp_saddr(&freed[b]));
       }
-      if (ok) xp_commit(xp_saddr(&summed));
-    }
-    if (!ok) {
-      if (lane == 0 && status) atomicOr(status, ST_TIMEOUT);
-      // let the MMAs in flight finish before TMEM is freed (bounded)
-      const unsigned long long t0 = globaltimer_ns();
-      for (uint32_t i = n >= GP_RING ? n - GP_RING : 0; i < n; i++)
-        while (!xp_try(xp_saddr(&freed[i % GP_RING]), (i / GP_RING) & 1) && globaltimer_ns() - t0 < MBAR_WAIT_NS) {}
+      if (ok && !HELD) xp_commit(xp_saddr(&summed));
     }
     __syncwarp();
   } else if (warp >= GP_WARPS) {
@@ -185,7 +182,7 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
         w[i] = __fmaf_rn(x, x, __fmul_rn(2.f, __fmul_rn(x, y)));
       }
       fetch(rs + 2 * GP_K, h, l);
-      if (n >= GP_RING) ok = xp_wait(xp_saddr(&freed[buf]), (n / GP_RING - 1) & 1, &s_abort);
+      if (n >= GP_RING) ok = xp_wait(xp_saddr(&freed[buf]), (n / GP_RING - 1) & 1, &s_abort, LIMIT);
       if (!ok) return;
       if (has) gp_store(w, smem + buf * GP_STAGE + 3 * GP_ATERM + (mm >> 3) * 256 + mkg * 128 + (mm & 7) * 16, GP_BTERM);
       asm volatile("fence.proxy.async.shared::cta;\n" ::);
@@ -233,7 +230,7 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
         nu2 = fetch(rs + 2 * GP_K);
         if (lane == 0 && rs + GP_AHEAD * GP_K + (tid >> 5) < R)   // one 128-byte row of U per warp
           asm volatile("prefetch.global.L2 [%0];\n" ::"l"(Uh + (rs + GP_AHEAD * GP_K + (tid >> 5)) * 32));
-        if (n >= GP_RING) ok = xp_wait(xp_saddr(&freed[buf]), (n / GP_RING - 1) & 1, &s_abort) && ok;
+        if (n >= GP_RING) ok = xp_wait(xp_saddr(&freed[buf]), (n / GP_RING - 1) & 1, &s_abort, LIMIT) && ok;
         uint32_t any;   // the stage's U is complete once all have arrived
         asm volatile(
             "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbar.red.or.pred q, 1, %2, p;\nselp.u32 %0, 1, 0, q;\n}\n"
@@ -257,7 +254,7 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
         if (lane == 0) xp_arrive(xp_saddr(&ready[buf]));
       }
       if (dead) break;
-      if (!xp_wait(xp_saddr(&summed), sub & 1, &s_abort)) {
+      if (!xp_wait(xp_saddr(&summed), sub & 1, &s_abort, LIMIT)) {
         ok = false;
         continue;
       }
@@ -302,22 +299,37 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
       if (lane == 0) xp_arrive(xp_saddr(&drained));
     }
   }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
-  __syncthreads();
+  xp_finish(&s_abort, status, warp == GP_ISSUER, freed, GP_RING, n);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
+}
+
+template <bool HELD>
+static cudaError_t launch(const float *Uh, const float *rfh, const float *rfl, int ld, int64_t R, int k, int M,
+                          int64_t rows, const unsigned *amax, const unsigned *rmax, double *G, int *status,
+                          cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(k_gram_pairs<HELD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GP_SMEM);
+  if (e != cudaSuccess) return e;
+  k_gram_pairs<HELD><<<(unsigned)((R + rows - 1) / rows), GP_THREADS, GP_SMEM, st>>>(Uh, rfh, rfl, ld, R, k, M, rows, amax,
+                                                                                  rmax, G, status);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_gram_pairs(const float *Uh, const float *rfh, const float *rfl, int ld, int64_t R, int k, int M,
                               const unsigned *amax, const unsigned *rmax, double *G, int sms, int *status,
                               cudaStream_t st) {
   if (R <= 0 || M <= 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(k_gram_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GP_SMEM);
-  if (e != cudaSuccess) return e;
   // one range of rows per SM, at least eight stages of them
   const int64_t rows = std::max<int64_t>(8 * GP_K, ((R + sms - 1) / sms + GP_K - 1) / GP_K * GP_K);
-  k_gram_pairs<<<(unsigned)((R + rows - 1) / rows), GP_THREADS, GP_SMEM, st>>>(Uh, rfh, rfl, ld, R, k, M, rows, amax, rmax, G,
-                                                                            status);
-  return cudaGetLastError();
+  return launch<false>(Uh, rfh, rfl, ld, R, k, M, rows, amax, rmax, G, status, st);
 }
 
 }  // namespace pmd
+
+// Test hook: the Gram of one CTA whose issuing warp leaves without reporting its sums.  U, rfh,
+// rfl: [R][32]; amax [M][32], rmax [M]; G [M][32][32]; R <= 1,024, k <= 32, M <= 32.
+extern "C" int pmx_gram_held(const float *U, const float *rfh, const float *rfl, int64_t R, int k, int M,
+                             const unsigned *amax, const unsigned *rmax, double *G, int *status, void *stream) {
+  if (R < 1 || R > 1024 || k < 1 || k > 32 || M < 1 || M > 32) return PM_ERR_INVALID_ARG;
+  return pmd::launch<true>(U, rfh, rfl, 32, R, k, M, 1024, amax, rmax, G, status, (cudaStream_t)stream) == cudaSuccess
+             ? PM_OK : PM_ERR_CUDA;
+}

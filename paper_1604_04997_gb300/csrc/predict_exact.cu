@@ -15,6 +15,7 @@
 #include "exact_tc.cuh"
 #include "float_float.cuh"
 #include "kernels.h"
+#include "pm.h"
 #include "topk_list.cuh"
 
 namespace pmd {
@@ -42,11 +43,14 @@ constexpr size_t xp_stash() {
   return G::PASSES > 1 && (MODE == XP_ARGMIN || MODE >= XP_SUMS_REL) ? 2 * 32 * XP_WARPS * sizeof(XpAcc<MODE>) : 0;
 }
 
-template <class G, int MODE>
+// HELD: the issuing warp leaves after its first tile and the waits are short, so that the
+// working warps' waits for the second tile run out (pmx_predict_held).
+template <class G, int MODE, bool HELD = false>
 __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *__restrict__ F, int64_t R, int k,
                                                                  const double *__restrict__ W, int M,
                                                                  double *__restrict__ T, ArgPart *__restrict__ part,
                                                                  int *status, uint32_t m256, FitResidual res) {
+  constexpr unsigned long long LIMIT = HELD ? XP_HELD_NS : MBAR_WAIT_NS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((128u - (xp_saddr(smem_raw) & 127u)) & 127u);
   __shared__ __align__(8) uint64_t full[XP_RING], empty[XP_RING], digits[2];   // sums ready / read, a tile's digits ready
@@ -104,23 +108,16 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
     for (int ps = 0; ps < 2; ps++) stash[ps * 32 * XP_WARPS] = XpAcc<MODE>();
   if (warp == XP_WARPS) {
     // this warp issues, ahead of the working warps as far as digits and columns allow
-    for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, it++) {
-      if (!(ok = xp_wait(xp_saddr(&digits[it & 1]), (it >> 1) & 1, &s_abort))) break;
+    for (int64_t tile = blockIdx.x; tile < ntiles && ok && !(HELD && it); tile += gridDim.x, it++) {
+      if (!(ok = xp_wait(xp_saddr(&digits[it & 1]), (it >> 1) & 1, &s_abort, LIMIT))) break;
       const int nd = (int)xp_uniform((uint32_t)xp_tile_digits(s_nd[it & 3])), ng = xp_groups(nd);
       for (int n = 0; n < G::PASSES * ng && ok; n++, seq++) {
         const uint32_t b = seq % XP_RING;
         const int ps = n >= ng;
-        if (seq >= XP_RING && !(ok = xp_wait(xp_saddr(&empty[b]), (seq / XP_RING - 1) & 1, &s_abort))) break;
+        if (seq >= XP_RING && !(ok = xp_wait(xp_saddr(&empty[b]), (seq / XP_RING - 1) & 1, &s_abort, LIMIT))) break;
         xp_issue<G>(s0, s0 + (it & 1) * G::A_BUF, s0 + G::OFF_B + ps * G::B_PASS, tmem + b * G::RANGE, n - ps * ng, nd,
                     xp_saddr(&full[b]));
       }
-    }
-    if (!ok) {
-      if (lane == 0 && status) atomicOr(status, ST_TIMEOUT);
-      // let the MMAs in flight finish before TMEM is freed (bounded)
-      const unsigned long long t0 = globaltimer_ns();
-      for (uint32_t n = seq >= XP_RING ? seq - XP_RING : 0; n < seq; n++)
-        while (!xp_try(xp_saddr(&full[n % XP_RING]), (n / XP_RING) & 1) && globaltimer_ns() - t0 < MBAR_WAIT_NS) {}
     }
     __syncwarp();
   } else {
@@ -133,7 +130,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
       __syncwarp();
       if (lane == 0) xp_arrive(xp_saddr(&digits[n & 1]));
     };
-    auto wait = [&]() { return xp_wait(xp_saddr(&full[seq % XP_RING]), (seq / XP_RING) & 1, &s_abort); };
+    auto wait = [&]() { return xp_wait(xp_saddr(&full[seq % XP_RING]), (seq / XP_RING) & 1, &s_abort, LIMIT); };
     auto done = [&]() {   // this warp has read its share of a group
       asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
       __syncwarp();
@@ -340,8 +337,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
       else if (blockIdx.x == 0) res.bb[tid] = (double)R;   // b = 1 in every row
     }
   }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
-  __syncthreads();
+  xp_finish(&s_abort, status, warp == XP_WARPS, full, XP_RING, seq);
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(G::TMEM_COLS));
 }
@@ -384,3 +380,15 @@ cudaError_t launch_fit_residual(const int64_t *F, int64_t R, int k, const double
 }
 
 }  // namespace pmd
+
+// Test hook: the prediction of one CTA whose issuing warp leaves after the first of its tiles.
+// F [R][k], T [R][M]; k <= 16, M <= 16.
+extern "C" int pmx_predict_held(const int64_t *F, int64_t R, int k, const double *W, int M, double *T, int *status,
+                                void *stream) {
+  using G = pmd::XpGeom<1, 16, 1>;
+  if (R < 1 || k < 1 || k > 16 || M < 1 || M > 16) return PM_ERR_INVALID_ARG;
+  const auto kernel = pmd::k_predict_exact<G, pmd::XP_TIMES, true>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM) != cudaSuccess) return PM_ERR_CUDA;
+  kernel<<<1, pmd::XP_THREADS, G::SMEM, (cudaStream_t)stream>>>(F, R, k, W, M, T, nullptr, status, 256u, pmd::FitResidual{});
+  return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ERR_CUDA;
+}

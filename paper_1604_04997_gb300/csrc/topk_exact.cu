@@ -19,6 +19,7 @@
 
 #include "exact_tc.cuh"
 #include "kernels.h"
+#include "pm.h"
 #include "topk_list.cuh"
 
 namespace pmd {
@@ -72,7 +73,8 @@ struct TxSmem {                      // beyond the operands of XpGeom
   TxCursor cursor[2][XP_WARPS + 1];  // per warp: its tile, and the tile it loads for
 };
 
-template <class G>
+// HELD: the issuing warp leaves after its first tile and the waits are short (pmx_topk_held).
+template <class G, bool HELD = false>
 __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__restrict__ F, int64_t R, int k,
                                                               const double *__restrict__ W, int M,
                                                               const int64_t *__restrict__ rows,
@@ -80,6 +82,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
                                                               double *__restrict__ part_t, int64_t *__restrict__ part_r,
                                                               int64_t *__restrict__ top_idx, double *__restrict__ top_t,
                                                               int *status, uint32_t m256) {
+  constexpr unsigned long long LIMIT = HELD ? XP_HELD_NS : MBAR_WAIT_NS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((128u - (xp_saddr(smem_raw) & 127u)) & 127u);
   TxSmem &X = *(TxSmem *)(smem + G::SMEM - 128);
@@ -147,23 +150,16 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
   };
   if (warp == XP_WARPS) {
     // this warp issues, ahead of the working warps as far as digits and columns allow
-    for (; cur.more(n_units) && ok; advance(cur), it++) {
-      if (!(ok = xp_wait(xp_saddr(&digits[it & 1]), (it >> 1) & 1, &s_abort))) break;
+    for (; cur.more(n_units) && ok && !(HELD && it); advance(cur), it++) {
+      if (!(ok = xp_wait(xp_saddr(&digits[it & 1]), (it >> 1) & 1, &s_abort, LIMIT))) break;
       const int nd = (int)xp_uniform((uint32_t)xp_tile_digits(s_nd[it & 3])), ng = xp_groups(nd);
       for (int n = 0; n < G::PASSES * ng && ok; n++, seq++) {
         const uint32_t b = seq % XP_RING;
         const int ps = n >= ng;
-        if (seq >= XP_RING && !(ok = xp_wait(xp_saddr(&empty[b]), (seq / XP_RING - 1) & 1, &s_abort))) break;
+        if (seq >= XP_RING && !(ok = xp_wait(xp_saddr(&empty[b]), (seq / XP_RING - 1) & 1, &s_abort, LIMIT))) break;
         xp_issue<G>(s0, s0 + (it & 1) * G::A_BUF, s0 + G::OFF_B + ps * G::B_PASS, tmem + b * G::RANGE, n - ps * ng, nd,
                     xp_saddr(&full[b]));
       }
-    }
-    if (!ok) {
-      if (lane == 0) atomicOr(status, ST_TIMEOUT);
-      // let the MMAs in flight finish before TMEM is freed (bounded)
-      const unsigned long long t0 = globaltimer_ns();
-      for (uint32_t n = seq >= XP_RING ? seq - XP_RING : 0; n < seq; n++)
-        while (!xp_try(xp_saddr(&full[n % XP_RING]), (n / XP_RING) & 1) && globaltimer_ns() - t0 < MBAR_WAIT_NS) {}
     }
     __syncwarp();
   } else {
@@ -240,7 +236,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
         atomicExch(&X.cnt[m], 0);   // the buffer is open again
       }
     };
-    auto wait = [&]() { return xp_wait(xp_saddr(&full[seq % XP_RING]), (seq / XP_RING) & 1, &s_abort); };
+    auto wait = [&]() { return xp_wait(xp_saddr(&full[seq % XP_RING]), (seq / XP_RING) & 1, &s_abort, LIMIT); };
     auto done = [&]() {   // this warp has read its share of a group
       asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
       __syncwarp();
@@ -403,8 +399,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
       if (end) meet();   // the lists are reset
     }
   }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
-  __syncthreads();
+  xp_finish(&s_abort, status, warp == XP_WARPS, full, XP_RING, seq);
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(G::TMEM_COLS));
 }
@@ -425,3 +420,18 @@ cudaError_t launch_topk_exact(const int64_t *F, int64_t R, int k, const double *
 }
 
 }  // namespace pmd
+
+// Test hook: the top-k of one CTA whose issuing warp leaves after the first of its tiles.
+// F [R][k]; units [n_units] (each of one whole group: part -1); outputs [groups][M][topk];
+// k <= 16, M <= 16.
+extern "C" int pmx_topk_held(const int64_t *F, int64_t R, int k, const double *W, int M, const void *units, int n_units,
+                             int topk, int64_t *idx, double *t, int *status, void *stream) {
+  using G = pmd::XpGeom<1, 16, 1>;
+  if (R < 1 || k < 1 || k > 16 || M < 1 || M > 16 || topk < 1 || topk > pmd::TOPK_MAX) return PM_ERR_INVALID_ARG;
+  constexpr size_t smem = G::SMEM + sizeof(pmd::TxSmem);
+  const auto kernel = pmd::k_topk_exact<G, true>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return PM_ERR_CUDA;
+  kernel<<<1, pmd::XP_THREADS, smem, (cudaStream_t)stream>>>(F, R, k, W, M, nullptr, (const pmd::TopkUnit *)units, n_units, topk,
+                                                             nullptr, nullptr, idx, t, status, 256u);
+  return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ERR_CUDA;
+}
