@@ -73,8 +73,11 @@ struct TxSmem {                      // beyond the operands of XpGeom
   TxCursor cursor[2][XP_WARPS + 1];  // per warp: its tile, and the tile it loads for
 };
 
-// HELD: the issuing warp leaves after its first tile and the waits are short (pmx_topk_held).
-template <class G, bool HELD = false>
+// For tests, with short waits: HELD: the issuing warp leaves after its first tile
+// (pmx_topk_held); UNWRITTEN: every buffer has a slot that is never counted as written
+// (pmx_topk_unwritten).
+enum TxTest { TX_NORMAL, TX_HELD, TX_UNWRITTEN };
+template <class G, TxTest TEST = TX_NORMAL>
 __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__restrict__ F, int64_t R, int k,
                                                               const double *__restrict__ W, int M,
                                                               const int64_t *__restrict__ rows,
@@ -82,7 +85,8 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
                                                               double *__restrict__ part_t, int64_t *__restrict__ part_r,
                                                               int64_t *__restrict__ top_idx, double *__restrict__ top_t,
                                                               int *status, uint32_t m256) {
-  constexpr unsigned long long LIMIT = HELD ? XP_HELD_NS : MBAR_WAIT_NS;
+  constexpr unsigned long long LIMIT = TEST != TX_NORMAL ? XP_HELD_NS : MBAR_WAIT_NS;
+  constexpr int TRIES = TEST != TX_NORMAL ? 1 << 10 : TX_TRIES;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((128u - (xp_saddr(smem_raw) & 127u)) & 127u);
   TxSmem &X = *(TxSmem *)(smem + G::SMEM - 128);
@@ -117,7 +121,8 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
     if (lane == 0) {
       X.thr[m] = INF;
       X.thr_row[m] = INT64_MAX;
-      X.cnt[m] = X.wr[m] = 0;
+      X.cnt[m] = 0;
+      X.wr[m] = TEST == TX_UNWRITTEN ? -1 : 0;
     }
   };
   if (warp < XP_WARPS)
@@ -150,7 +155,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
   };
   if (warp == XP_WARPS) {
     // this warp issues, ahead of the working warps as far as digits and columns allow
-    for (; cur.more(n_units) && ok && !(HELD && it); advance(cur), it++) {
+    for (; cur.more(n_units) && ok && !(TEST == TX_HELD && it); advance(cur), it++) {
       if (!(ok = xp_wait(xp_saddr(&digits[it & 1]), (it >> 1) & 1, &s_abort, LIMIT))) break;
       const int nd = (int)xp_uniform((uint32_t)xp_tile_digits(s_nd[it & 3])), ng = xp_groups(nd);
       for (int n = 0; n < G::PASSES * ng && ok; n++, seq++) {
@@ -319,7 +324,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
       else emit(std::false_type{});
       // offer the candidates; the warp that fills a buffer merges it
       for (int tries = 0; __any_sync(0xffffffffu, pending); tries++) {
-        if (tries == TX_TRIES) s_abort = 1;   // never: a full buffer's owner empties it
+        if (tries == TRIES) s_abort = 1;   // never: a full buffer's owner empties it
         if (__any_sync(0xffffffffu, s_abort)) {
           ok = false;
           break;
@@ -355,7 +360,11 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
           const int full_m = __shfl_sync(0xffffffffu, mm, from);
           if (lane == from) filled = false;
           int polls = 0;   // the other writers of the buffer are between reserving and writing
-          while (*(volatile int32_t *)&X.wr[full_m] < TX_BUF && ++polls < TX_TRIES) {}
+          while (*(volatile int32_t *)&X.wr[full_m] < TX_BUF && ++polls < TRIES) {}
+          if (__any_sync(0xffffffffu, polls == TRIES)) {   // never; a buffer with unwritten slots is not merged
+            s_abort = 1;
+            break;
+          }
           __threadfence_block();
           __syncwarp();
           merge(full_m, TX_BUF);
@@ -421,17 +430,26 @@ cudaError_t launch_topk_exact(const int64_t *F, int64_t R, int k, const double *
 
 }  // namespace pmd
 
-// Test hook: the top-k of one CTA whose issuing warp leaves after the first of its tiles.
-// F [R][k]; units [n_units] (each of one whole group: part -1); outputs [groups][M][topk];
-// k <= 16, M <= 16.
-extern "C" int pmx_topk_held(const int64_t *F, int64_t R, int k, const double *W, int M, const void *units, int n_units,
-                             int topk, int64_t *idx, double *t, int *status, void *stream) {
+// Test hooks: the top-k of one CTA whose issuing warp leaves after the first of its tiles
+// (held), or whose buffers never count as written.  F [R][k]; units [n_units] (each of one
+// whole group: part -1); outputs [groups][M][topk]; k <= 16, M <= 16.
+template <pmd::TxTest TEST>
+static int topk_test(const int64_t *F, int64_t R, int k, const double *W, int M, const void *units, int n_units, int topk,
+                     int64_t *idx, double *t, int *status, void *stream) {
   using G = pmd::XpGeom<1, 16, 1>;
   if (R < 1 || k < 1 || k > 16 || M < 1 || M > 16 || topk < 1 || topk > pmd::TOPK_MAX) return PM_ERR_INVALID_ARG;
   constexpr size_t smem = G::SMEM + sizeof(pmd::TxSmem);
-  const auto kernel = pmd::k_topk_exact<G, true>;
+  const auto kernel = pmd::k_topk_exact<G, TEST>;
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return PM_ERR_CUDA;
   kernel<<<1, pmd::XP_THREADS, smem, (cudaStream_t)stream>>>(F, R, k, W, M, nullptr, (const pmd::TopkUnit *)units, n_units, topk,
                                                              nullptr, nullptr, idx, t, status, 256u);
   return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ERR_CUDA;
+}
+extern "C" int pmx_topk_held(const int64_t *F, int64_t R, int k, const double *W, int M, const void *units, int n_units,
+                             int topk, int64_t *idx, double *t, int *status, void *stream) {
+  return topk_test<pmd::TX_HELD>(F, R, k, W, M, units, n_units, topk, idx, t, status, stream);
+}
+extern "C" int pmx_topk_unwritten(const int64_t *F, int64_t R, int k, const double *W, int M, const void *units,
+                                  int n_units, int topk, int64_t *idx, double *t, int *status, void *stream) {
+  return topk_test<pmd::TX_UNWRITTEN>(F, R, k, W, M, units, n_units, topk, idx, t, status, stream);
 }

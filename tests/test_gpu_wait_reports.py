@@ -57,8 +57,9 @@ def test_predict_reports(env):
     assert bool(((T[:128] - ref[:128]).abs() <= 1e-12 * ref[:128]).all())   # the tile that was issued
 
 
+@pytest.mark.parametrize("hook", ["pmx_topk_held", "pmx_topk_unwritten"])
 @pytest.mark.parametrize("cuts", [[0, 400], [0, 100, 100, 130, 400]], ids=["tiles", "units"])
-def test_topk_reports(env, cuts):
+def test_topk_reports(env, cuts, hook):
     import torch
     _, F, w = env
     G = len(cuts) - 1
@@ -68,7 +69,7 @@ def test_topk_reports(env, cuts):
     u = torch.from_numpy(units).to("cuda:0")
     idx = torch.zeros((G, 5, 4), dtype=torch.int64, device="cuda:0")
     tt = torch.zeros((G, 5, 4), dtype=torch.float64, device="cuda:0")
-    status, s = _hook("pmx_topk_held", F, ctypes.c_int64(400), 12, w, 5, u, G, 4, idx, tt)
+    status, s = _hook(hook, F, ctypes.c_int64(400), 12, w, 5, u, G, 4, idx, tt)
     assert status & TIMEOUT and s < 5
 
 
