@@ -184,7 +184,8 @@ pm_status pm_predict_topk(pm_ctx *ctx, const int64_t *d_F, int64_t R, int32_t k,
  * stream capture.  All calls share the one array: calls whose work overlaps on the
  * GPU (different streams, or different host threads) race and must be serialised by
  * the caller.  Each launch writes every partial entry before reading it, so no
- * clearing is needed between calls. */
+ * clearing is needed between calls.  There is no status: if a device wait ran out,
+ * d_arg is -1 and d_min NaN for every model. */
 pm_status pm_predict_argmin_static(const int64_t *d_F, int64_t R, int32_t k, const double *d_W, int32_t M,
                                    int64_t *d_arg, double *d_min, void *stream);
 

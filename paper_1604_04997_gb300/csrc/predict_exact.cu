@@ -305,6 +305,8 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_predict_exact(const int64_t *
         const int64_t kx = time_order(x.t), kb = time_order(b.t);
         if (kx < kb || (kx == kb && x.r < b.r)) b = x;
       }
+      // a wait ran out: NaN (ordered below every time) and no row, for callers without a status
+      if (s_abort) b = ArgPart{__longlong_as_double(-1ll), -1};
       part[(int64_t)blockIdx.x * M + tid] = b;
     }
   }
@@ -381,14 +383,27 @@ cudaError_t launch_fit_residual(const int64_t *F, int64_t R, int k, const double
 
 }  // namespace pmd
 
-// Test hook: the prediction of one CTA whose issuing warp leaves after the first of its tiles.
-// F [R][k], T [R][M]; k <= 16, M <= 16.
+// Test hooks: the prediction, or the argmin, of one CTA whose issuing warp leaves after the
+// first of its tiles.  F [R][k], T [R][M], part: M pairs; k <= 16, M <= 16.
+template <int MODE>
+static cudaError_t launch_held(const int64_t *F, int64_t R, int k, const double *W, int M, double *T, void *part,
+                               int *status, void *stream) {
+  using G = pmd::XpGeom<1, 16, 1>;
+  if (R < 1 || k < 1 || k > 16 || M < 1 || M > 16) return cudaErrorInvalidValue;
+  const auto kernel = pmd::k_predict_exact<G, MODE, true>;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+  if (e != cudaSuccess) return e;
+  kernel<<<1, pmd::XP_THREADS, G::SMEM, (cudaStream_t)stream>>>(F, R, k, W, M, T, (pmd::ArgPart *)part, status, 256u,
+                                                                pmd::FitResidual{});
+  return cudaGetLastError();
+}
 extern "C" int pmx_predict_held(const int64_t *F, int64_t R, int k, const double *W, int M, double *T, int *status,
                                 void *stream) {
-  using G = pmd::XpGeom<1, 16, 1>;
-  if (R < 1 || k < 1 || k > 16 || M < 1 || M > 16) return PM_ERR_INVALID_ARG;
-  const auto kernel = pmd::k_predict_exact<G, pmd::XP_TIMES, true>;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM) != cudaSuccess) return PM_ERR_CUDA;
-  kernel<<<1, pmd::XP_THREADS, G::SMEM, (cudaStream_t)stream>>>(F, R, k, W, M, T, nullptr, status, 256u, pmd::FitResidual{});
-  return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ERR_CUDA;
+  return launch_held<pmd::XP_TIMES>(F, R, k, W, M, T, nullptr, status, stream) == cudaSuccess ? PM_OK : PM_ERR_CUDA;
+}
+extern "C" int pmx_argmin_held(const int64_t *F, int64_t R, int k, const double *W, int M, void *part, int64_t *arg,
+                               double *mn, int *status, void *stream) {
+  if (launch_held<pmd::XP_ARGMIN>(F, R, k, W, M, nullptr, part, status, stream) != cudaSuccess) return PM_ERR_CUDA;
+  return pmd::launch_argmin_reduce((const pmd::ArgPart *)part, 1, M, arg, mn, (cudaStream_t)stream) == cudaSuccess ? PM_OK
+                                                                                                             : PM_ERR_CUDA;
 }

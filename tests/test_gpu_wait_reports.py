@@ -57,6 +57,18 @@ def test_predict_reports(env):
     assert bool(((T[:128] - ref[:128]).abs() <= 1e-12 * ref[:128]).all())   # the tile that was issued
 
 
+def test_argmin_without_a_status_reports(env):
+    """pm_predict_argmin_static has no status: a timeout gives row -1 and NaN."""
+    import torch
+    _, F, w = env
+    part = torch.zeros((5, 2), dtype=torch.int64, device="cuda:0")
+    arg = torch.zeros(5, dtype=torch.int64, device="cuda:0")
+    mn = torch.zeros(5, dtype=torch.float64, device="cuda:0")
+    status, s = _hook("pmx_argmin_held", F, ctypes.c_int64(400), 12, w, 5, part, arg, mn)
+    assert status & TIMEOUT and s < 5
+    assert (arg.cpu() == -1).all() and mn.cpu().isnan().all()
+
+
 @pytest.mark.parametrize("hook", ["pmx_topk_held", "pmx_topk_unwritten"])
 @pytest.mark.parametrize("cuts", [[0, 400], [0, 100, 100, 130, 400]], ids=["tiles", "units"])
 def test_topk_reports(env, cuts, hook):
