@@ -232,11 +232,8 @@ extern "C" pm_status pm_table_image(pm_ctx *c, int32_t id, uint32_t *buf, size_t
   return PM_OK;
 }
 
-// The work list of a table list: per distinct table the output positions it fills, in items
-// of at most `per_item` positions.
-static pm_status eval_plan(pm_ctx *c, const int32_t *ids, int n, int per_item, const EvalPlan **out) {
+static pm_status eval_plan(pm_ctx *c, const int32_t *ids, int n, const EvalPlan **out) {
   std::string key((const char *)ids, (size_t)n * sizeof(int32_t));
-  key.append((const char *)&per_item, sizeof per_item);
   auto it = c->eval_plans.find(key);
   if (it != c->eval_plans.end()) { *out = &it->second; return PM_OK; }
   EvalPlan p;
@@ -259,22 +256,33 @@ static pm_status eval_plan(pm_ctx *c, const int32_t *ids, int n, int per_item, c
     }
     members[at.first->second].push_back(i);
   }
-  std::vector<int32_t> items, list;
-  for (size_t t = 0; t < tab.size(); t++) {
-    const int cnt = (int)members[t].size();
-    for (int m = 0; m < cnt; m += per_item) {
-      const int k = std::min(per_item, cnt - m);
+  std::vector<int32_t> list, first;              // the members, table by table
+  int most = 0;
+  for (auto &m : members) {
+    first.push_back((int32_t)list.size());
+    list.insert(list.end(), m.begin(), m.end());
+    most = std::max(most, (int)m.size());
+  }
+  list.resize((list.size() + 3) & ~(size_t)3);   // the items are read as 16-byte records
+  size_t at[EVAL_ITEM];
+  for (int per = 1; per <= EVAL_ITEM; per++) {
+    p.n_items[per - 1] = per > 1 && per > most ? p.n_items[per - 2] : 0;   // the same items again
+    at[per - 1] = p.n_items[per - 1] ? at[per - 2] : list.size();
+    if (p.n_items[per - 1]) continue;
+    for (size_t t = 0; t < tab.size(); t++) {
+      const int cnt = (int)members[t].size();
       const int64_t off = c->dev_off[tab[t]];
-      items.insert(items.end(), {(int32_t)(uint32_t)off, (int32_t)list.size(), k, (int32_t)(off >> 32)});
-      list.insert(list.end(), members[t].begin() + m, members[t].begin() + m + k);
+      for (int m = 0; m < cnt; m += per) {
+        list.insert(list.end(), {(int32_t)(uint32_t)off, first[t] + m, std::min(per, cnt - m), (int32_t)(off >> 32)});
+        p.n_items[per - 1]++;
+      }
     }
   }
-  p.n_items = (int)items.size() / 4;
-  items.insert(items.end(), list.begin(), list.end());
   void *d = nullptr;
-  pm_status s = ctx_dcopy(c, items.data(), items.size() * sizeof(int32_t), &d);
+  pm_status s = ctx_dcopy(c, list.data(), list.size() * sizeof(int32_t), &d);
   if (s) return s;
-  p.d_items = (const int32_t *)d;
+  p.members = (const int32_t *)d;
+  for (int i = 0; i < EVAL_ITEM; i++) p.items[i] = p.members + at[i];
   *out = &(c->eval_plans[key] = p);
   return PM_OK;
 }
@@ -294,15 +302,15 @@ extern "C" pm_status pm_eval_counts(pm_ctx *c, const int32_t *ids, int32_t n_tab
   // tables x 1,024 points).  Fewer positions a block where that would leave fewer than 16
   // blocks per SM (three are resident): small calls keep one block per position.
   const int64_t chunks = (n_points + 127) / 128;
-  const int per_item = (int)std::min<int64_t>(8, std::max<int64_t>(1, chunks * n_tables / ((int64_t)c->n_sms * 16)));
+  const int per = (int)std::min<int64_t>(EVAL_ITEM, std::max<int64_t>(1, chunks * n_tables / ((int64_t)c->n_sms * 16)));
   const EvalPlan *p = nullptr;
-  pm_status s = eval_plan(c, ids, n_tables, per_item, &p);
+  pm_status s = eval_plan(c, ids, n_tables, &p);
   if (s) return s;
   constexpr int64_t MAX_GRID_Y = 65535;
-  for (int64_t t0 = 0; t0 < p->n_items; t0 += MAX_GRID_Y)
-    CU(pmd::launch_eval_counts(c->arena, p->d_items + 4 * t0, p->d_items + 4 * (int64_t)p->n_items,
-                               (int)std::min<int64_t>(MAX_GRID_Y, p->n_items - t0), p->max_words, d_points, n_points, p->P, p->K,
-                               d_counts, c->d_status, (cudaStream_t)stream));
+  const int n_items = p->n_items[per - 1];
+  for (int64_t t0 = 0; t0 < n_items; t0 += MAX_GRID_Y)
+    CU(pmd::launch_eval_counts(c->arena, p->items[per - 1] + 4 * t0, p->members, (int)std::min<int64_t>(MAX_GRID_Y, n_items - t0),
+                               p->max_words, d_points, n_points, p->P, p->K, d_counts, c->d_status, (cudaStream_t)stream));
   return PM_OK;
 }
 

@@ -42,11 +42,15 @@ struct Plan {
   int g_topk = 0, g_nw = 0, g_grid = 0;
 };
 
-// Device work list of one pm_eval_counts table list: distinct tables, each with the output
-// positions it fills.
+// Device work lists of one pm_eval_counts table list: distinct tables, each with the output
+// positions it fills, in items of at most n positions for every n of 1 .. EVAL_ITEM.  The point
+// count chooses among them, so a list that was seen is on the device for any number of points.
+constexpr int EVAL_ITEM = 8;
 struct EvalPlan {
-  int P = 0, K = 0, n_items = 0, max_words = 0;
-  const int32_t *d_items = nullptr;   // [n_items][4] (arena word offset low, first member, members, offset high), then the members
+  int P = 0, K = 0, max_words = 0;
+  int n_items[EVAL_ITEM] = {};
+  const int32_t *items[EVAL_ITEM] = {};   // [n_items][4] (arena word offset low, first member, members, offset high)
+  const int32_t *members = nullptr;
 };
 
 struct pm_ctx {
