@@ -233,7 +233,13 @@ extern "C" pm_status pm_table_image(pm_ctx *c, int32_t id, uint32_t *buf, size_t
 }
 
 static pm_status eval_plan(pm_ctx *c, const int32_t *ids, int n, const EvalPlan **out) {
-  std::string key((const char *)ids, (size_t)n * sizeof(int32_t));
+  // by the first tables of equal images: a list of other ids with the same images is the same,
+  // so there are no more plans than device arrays in dcache, which is bounded
+  std::string key((size_t)n * sizeof(int), 0);
+  for (int i = 0; i < n; i++) {
+    if (ids[i] < 0 || ids[i] >= (int)c->tables.size()) return pm_set_error(PM_ERR_NOT_FOUND, "unknown table id");
+    memcpy(&key[i * sizeof(int)], &c->canon[ids[i]], sizeof(int));
+  }
   auto it = c->eval_plans.find(key);
   if (it != c->eval_plans.end()) { *out = &it->second; return PM_OK; }
   EvalPlan p;
@@ -241,16 +247,15 @@ static pm_status eval_plan(pm_ctx *c, const int32_t *ids, int n, const EvalPlan 
   std::vector<std::vector<int32_t>> members;
   std::vector<int> tab;
   for (int i = 0; i < n; i++) {
-    const int id = ids[i];
-    if (id < 0 || id >= (int)c->tables.size()) return pm_set_error(PM_ERR_NOT_FOUND, "unknown table id");
+    const int id = c->canon[ids[i]];
     const auto &w = c->tables[id];
     if (i == 0) { p.P = (int)w[pmt::H_NPARAMS]; p.K = (int)w[pmt::H_K]; }
     if (p.P != (int)w[pmt::H_NPARAMS]) return pm_set_error(PM_ERR_INVALID_ARG, "tables differ in parameter count");
     if (p.K != (int)w[pmt::H_K]) return pm_set_error(PM_ERR_INVALID_ARG, "tables differ in layout");
     if (c->dev_off[id] < 0) return pm_set_error(PM_ERR_INVALID_ARG, "table not on the device");
-    const auto at = slot.emplace(c->canon[id], (int)tab.size());
+    const auto at = slot.emplace(id, (int)tab.size());
     if (at.second) {
-      tab.push_back(c->canon[id]);
+      tab.push_back(id);
       members.emplace_back();
       p.max_words = std::max(p.max_words, (int)w.size());
     }
@@ -286,6 +291,9 @@ static pm_status eval_plan(pm_ctx *c, const int32_t *ids, int n, const EvalPlan 
   *out = &(c->eval_plans[key] = p);
   return PM_OK;
 }
+
+// Test hook: the work lists that pm_eval_counts keeps.
+extern "C" int pmx_eval_plans(const pm_ctx *c) { return c ? (int)c->eval_plans.size() : -1; }
 
 extern "C" pm_status pm_eval_counts(pm_ctx *c, const int32_t *ids, int32_t n_tables, const int64_t *d_points,
                                     int64_t n_points, int64_t *d_counts, void *stream) {

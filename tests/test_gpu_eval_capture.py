@@ -41,3 +41,31 @@ def test_a_seen_list_can_be_captured_for_any_point_count(repeats):
             assert bool((out[at] == out[at[0]]).all())
             assert torch.equal(out[at[0], :1], one[at[0]])
     ctx.close()
+
+
+def test_lists_of_equal_images_share_one_plan():
+    """Tables compiled again and again (new ids, equal images) leave one work list behind."""
+    import ctypes
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    ctx, dev = B.Context(0), torch.device("cuda:0")
+    f = B.lib().pmx_eval_plans
+    f.restype, f.argtypes = ctypes.c_int, [ctypes.c_void_p]
+    vs = [v for v in W.all_variants() if v.template == "vecadd"][:3]
+    P = len(W.TEMPLATE_PARAMS["vecadd"])
+    pts = torch.from_numpy(W.draw_points(P, 40, 3)).to(dev)
+    out = torch.empty((3, 40, 32), dtype=torch.int64, device=dev)
+    first = None
+    for _ in range(20):
+        ids = [ctx.compile_counts(W.variant_ir(v), 32, [W.BOX_LO] * P, [W.BOX_HI] * P)[0] for v in vs]
+        ctx.eval_counts(ids, pts, out)
+        ctx.sync_status()
+        first = out.clone() if first is None else first
+        assert torch.equal(out, first)
+    assert f(ctx.h) == 1
+    with pytest.raises(B.PMError):
+        ctx.eval_counts([ids[0], 10 ** 6], pts, out)
+    with pytest.raises(B.PMError):
+        ctx.eval_counts([-1], pts, out)
+    ctx.close()
