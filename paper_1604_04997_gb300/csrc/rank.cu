@@ -599,10 +599,13 @@ __global__ void __maxnreg__(96) k_rank(RankArgs a) {
           const int64_t e = lists[i * 32 + lane];
           if (e == RK_EMPTY) break;
           const int64_t key = entry_key(e);
+          const uint32_t sp = span[entry_vid(e)], off = sp & 0xFFFF;
+          // A program of one variant comes before all that follow, in a tie too: programs with
+          // equal keys are in the order of their first variants.
           int j = i + 1;
-          while (j < RK_TOPK && entry_key(lists[j * 32 + lane]) == key) j++;
+          if (sp >> 16 > 1)
+            while (j < RK_TOPK && entry_key(lists[j * 32 + lane]) == key) j++;
           if (j == i + 1) {
-            const uint32_t sp = span[entry_vid(e)], off = sp & 0xFFFF;
             const int n = min((int)(sp >> 16), RK_TOPK - o);
             for (int c = 0; c < n; c++) ranked[(o + c) * 32 + lane] = key | (uint32_t)(vbase + pvid[off + c]);
             o += n;
