@@ -572,9 +572,12 @@ int64_t topk_chunk(int k, int M, int64_t total, int64_t G) {
   return split(num_sms(), 128, TOPK_CHUNK, int64_t(1) << 20);
 }
 
-// Groups split over several units: one CTA per (group, model) merges the units' sorted
-// lists of that model; its warps take every eighth block of 32 candidates, then warp 0
-// merges the eight warp lists.
+// Groups split over several units: one CTA per (group, model) merges the units' sorted lists
+// of that model in rounds: the first entries of all lists, then the next ones, until no entry
+// of a round is below the warps' shared bound (the lists are sorted, so later ones are not
+// either).  Then warp 0 merges the eight warp lists.  A round is one entry of many lists or
+// several of few, about four candidates a thread.  With every entry of 782 lists merged, one
+// group of 100,000 rows x 32 took 79 us (one model, 16 entries), 46 now.
 __global__ void __launch_bounds__(PR_WARPS * 32) k_topk_merge(const TopkMerge *__restrict__ merges, int M, int topk,
                                                               const double *__restrict__ part_t,
                                                               const int64_t *__restrict__ part_r,
@@ -585,19 +588,44 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_topk_merge(const TopkMerge *_
   const TopkMerge G = merges[blockIdx.x];
   const int m = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t n = (int64_t)G.n_parts * topk;
   double lt = TK_INF;
   int64_t lr = INT64_MAX;
-  for (int64_t c0 = 32 * warp; c0 < n; c0 += 32 * PR_WARPS) {   // warp-uniform
-    const int64_t c = c0 + lane;
-    double t = TK_INF;
-    int64_t r = INT64_MAX;
-    if (c < n) {
-      const int64_t o = (((int64_t)G.part0 + c / topk) * M + m) * topk + c % topk;
-      t = part_t[o];
-      r = part_r[o];
+  __shared__ long long s_thr;   // no time above it is among the topk: the least of the warps' last entries
+  if (threadIdx.x == 0) s_thr = INT64_MAX;
+  __syncthreads();
+  int sh = 0;   // 2^sh entries of a list per round
+  while (sh < 4 && ((int64_t)G.n_parts << (sh + 1)) <= 4 * 32 * PR_WARPS) sh++;
+  const int64_t n = (int64_t)G.n_parts << sh;
+  for (int j = 0; j < topk; j += 1 << sh) {
+    bool some = false;
+    for (int64_t c0 = 32 * warp; c0 < n; c0 += 4 * 32 * PR_WARPS) {   // warp-uniform
+      double t[4];
+      int64_t r[4];
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        const int64_t c = c0 + u * 32 * PR_WARPS + lane, q = j + (c & ((1 << sh) - 1));
+        t[u] = TK_INF;
+        r[u] = INT64_MAX;
+        if (c < n && q < topk) {
+          const int64_t o = ((G.part0 + (c >> sh)) * M + m) * topk + q;
+          t[u] = part_t[o];
+          r[u] = part_r[o];
+        }
+      }
+#pragma unroll 1
+      for (int u = 0; u < 4; u++) {   // one copy of the merge's code
+        const bool ok = r[0] != INT64_MAX && time_order(t[0]) <= *(volatile long long *)&s_thr;
+        if (__any_sync(0xffffffffu, ok)) {
+          some = true;
+          warp_list_merge(lt, lr, t[0], r[0], ok, topk, lane);
+          if (lane == topk - 1 && lr != INT64_MAX && time_order(lt) < *(volatile long long *)&s_thr)
+            atomicMin(&s_thr, (long long)time_order(lt));
+        }
+        t[0] = t[1], t[1] = t[2], t[2] = t[3];
+        r[0] = r[1], r[1] = r[2], r[2] = r[3], r[3] = INT64_MAX;
+      }
     }
-    warp_list_merge(lt, lr, t, r, r != INT64_MAX, topk, lane);
+    if (j + (1 << sh) >= topk || !__syncthreads_or(some)) break;
   }
   st[warp][lane] = lt;
   sr[warp][lane] = lr;
