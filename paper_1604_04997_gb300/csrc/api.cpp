@@ -408,7 +408,7 @@ extern "C" pm_status pm_predict_topk(pm_ctx *c, const int64_t *F, int64_t R, int
   CU(pmd::launch_predict_topk(F, R, k, W, M, d_rows, (const pmd::TopkUnit *)d_meta, (int)units.size(),
                               (const pmd::TopkMerge *)((uint8_t *)d_meta + ub), (int)merges.size(), topk,
                               (double *)scr, (int64_t *)((uint8_t *)scr + pb), d_top_idx, d_top_t,
-                              pmd::topk_rows_path(k, M, total, G), c->d_status, (cudaStream_t)stream));
+                              pmd::topk_path(k, M, total, G), c->d_status, (cudaStream_t)stream));
   return PM_OK;
 }
 

@@ -116,9 +116,10 @@ cudaError_t launch_fit_residual(const int64_t *F, int64_t R, int k, const double
 // others ([part][M][topk]) are merged per group (TopkMerge)
 constexpr int TOPK_MAX = 16;
 constexpr int64_t TOPK_CHUNK = 1024;
-// whether M models over `total` positions in G groups take the row-per-lane kernel, and the
-// largest unit
-bool topk_rows_path(int k, int M, int64_t total, int64_t G);
+// the kernel that M models over `total` positions in G groups take (row per lane, tensor
+// cores, integer tile), and its largest unit
+enum class TopkPath { ROWS, TENSOR, INTEGER };
+TopkPath topk_path(int k, int M, int64_t total, int64_t G);
 int64_t topk_chunk(int k, int M, int64_t total, int64_t G);
 struct TopkUnit { int64_t p0, p1; int32_t g, part; };
 struct TopkMerge { int32_t g, part0, n_parts, pad; };
@@ -128,7 +129,7 @@ cudaError_t launch_topk_exact(const int64_t *F, int64_t R, int k, const double *
                               int64_t *top_idx, double *top_t, int *status, int sms, cudaStream_t st);
 cudaError_t launch_predict_topk(const int64_t *F, int64_t R, int k, const double *W, int M, const int64_t *rows,
                                 const TopkUnit *units, int n_units, const TopkMerge *merges, int n_merges, int topk,
-                                double *part_t, int64_t *part_r, int64_t *top_idx, double *top_t, bool rows_path,
+                                double *part_t, int64_t *part_r, int64_t *top_idx, double *top_t, TopkPath path,
                                 int *status, cudaStream_t st);
 
 // predict_tc.cu (tensor cores, three-term bf16 split)

@@ -552,10 +552,20 @@ static void launch_topk_rows(const int64_t *F, int64_t R, int k, const double *W
 // (200), 624 (10); 8 models 900 | 1,174 (4,096), 716 (600) | 696 (400), 367 (one).  Rows of 12
 // counts have fewer than half the products to do: 8 models in 100 groups 451 | 554.  The tensor
 // cores take k up to 32.
-bool topk_rows_path(int k, int M, int64_t total, int64_t G) {
-  if (M <= 4) return true;
-  if (M > 8) return false;
-  return k <= 16 || !exact_tc_ok(k, M) || total < (M == 5 ? int64_t(1) << 17 : 2048) * G;
+//
+// More than eight models take the tensor cores unless the groups are short: each group fills M
+// empty lists there, some 15 merges a model, where the integer tile's lists are its warps' own,
+// but the integer tile pays for every product.  So the line is in a group's rows times what a
+// row costs, k + M / 4, against the lists, 600 + 50 M.  100,000 rows, us, integer | tensor
+// cores: 9 models x 12 columns 270 | 343 (64 rows a group), 268 | 245 (100); 64 models x 12
+// 558 | 642 (100), 566 | 423 (256); 64 x 32 800 | 879 (64), 782 | 632 (100); 33 x 32 629 | 886
+// (32), 650 | 577 (64).
+TopkPath topk_path(int k, int M, int64_t total, int64_t G) {
+  if (M <= 4) return TopkPath::ROWS;
+  if (M <= 8)
+    return k <= 16 || !exact_tc_ok(k, M) || total < (M == 5 ? int64_t(1) << 17 : 2048) * G ? TopkPath::ROWS : TopkPath::TENSOR;
+  return exact_tc_ok(k, M) && (double)total * (k + 0.25 * M) >= (double)G * (600 + 50.0 * M) ? TopkPath::TENSOR
+                                                                                          : TopkPath::INTEGER;
 }
 // The row-per-lane kernel's units fill its resident CTAs once (six per SM, four with eight
 // models' lists): of 977 units of 1,024 positions on 912 CTAs the last 65 took as
@@ -567,8 +577,9 @@ int64_t topk_chunk(int k, int M, int64_t total, int64_t G) {
     const int64_t each = ((total + ctas - 1) / ctas + grain - 1) / grain * grain;
     return std::min(hi, std::max(lo, each));
   };
-  if (topk_rows_path(k, M, total, G)) return split((int64_t)num_sms() * (M <= 2 ? 6 : M <= 4 ? 5 : 4), 32, 32 * TR_WARPS, 2048);
-  if (!exact_tc_ok(k, M)) return TOPK_CHUNK;
+  const TopkPath path = topk_path(k, M, total, G);
+  if (path == TopkPath::ROWS) return split((int64_t)num_sms() * (M <= 2 ? 6 : M <= 4 ? 5 : 4), 32, 32 * TR_WARPS, 2048);
+  if (path == TopkPath::INTEGER) return TOPK_CHUNK;
   return split(num_sms(), 128, TOPK_CHUNK, int64_t(1) << 20);
 }
 
@@ -647,11 +658,11 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_topk_merge(const TopkMerge *_
 
 cudaError_t launch_predict_topk(const int64_t *F, int64_t R, int k, const double *W, int M, const int64_t *rows,
                                 const TopkUnit *units, int n_units, const TopkMerge *merges, int n_merges, int topk,
-                                double *part_t, int64_t *part_r, int64_t *top_idx, double *top_t, bool rows_path,
+                                double *part_t, int64_t *part_r, int64_t *top_idx, double *top_t, TopkPath path,
                                 int *status, cudaStream_t st) {
   if (k > PR_MAXK || M > PR_MAXM || topk < 1 || topk > TOPK_MAX) return cudaErrorInvalidValue;
   if (n_units <= 0) return cudaSuccess;
-  if (rows_path) {   // few models: one row per lane
+  if (path == TopkPath::ROWS) {   // few models: one row per lane
     // rows of 12 counts are read well enough as they are (1e6 x 12, 4 models: staged 331 us)
     const bool staged = k % 2 == 0 && k >= 24 && k <= 32 && ((uintptr_t)F & 15) == 0;
     auto go = [&](auto mn) {
@@ -663,7 +674,7 @@ cudaError_t launch_predict_topk(const int64_t *F, int64_t R, int k, const double
     else if (M == 2) go(std::integral_constant<int, 2>{});
     else if (M <= 4) go(std::integral_constant<int, 4>{});
     else go(std::integral_constant<int, 8>{});
-  } else if (exact_tc_ok(k, M)) {
+  } else if (path == TopkPath::TENSOR) {
     const cudaError_t x = launch_topk_exact(F, R, k, W, M, rows, units, n_units, topk, part_t, part_r, top_idx, top_t, status,
                                             num_sms(), st);
     if (x != cudaSuccess) return x;
