@@ -545,13 +545,15 @@ static void launch_topk_rows(const int64_t *F, int64_t R, int k, const double *W
                                                                   top_idx, top_t, status);
 }
 
-// Which kernel, and how large a unit may be.  The row-per-lane kernel's cost grows with the
-// models, the tensor cores' hardly (they pad to a tile) but with the lists' ends, so the line
-// is in models and rows per group.  1e6 x 32, us, row-per-lane | tensor cores: 4 models 303 |
-// 360 (one group), 447 | 1,010 (4,096 groups); 5 models 585 (600 groups) | 768 (400), 647
-// (200), 624 (10); 8 models 900 | 1,174 (4,096), 716 (600) | 696 (400), 367 (one).  Rows of 12
-// counts have fewer than half the products to do: 8 models in 100 groups 451 | 554.  The tensor
-// cores take k up to 32.
+// Which kernel, and how large a unit may be.
+//
+// Up to eight models, 1e6 x 32, us, row-per-lane | tensor cores: one group 303 | 360 for 4 models,
+// 440 | 388 for 5, 471 | 358 for 6, 501 | 402 for 7, 531 | 363 for 8; 10 groups 407 | 648, 439 | 587,
+// 469 | 653, 497 | 574 for 5 to 8; 400 groups 535 | 791, 575 | 721, 614 | 804, 650 | 709; between them
+// eight models are as fast on either (200 groups 615 | 573).  100,000 rows in one group 81 | 108,
+// 86 | 108, 90 | 117, 96 | 112.  The end of a group costs the tensor-core kernel as much as many
+// of its tiles: from 2^17 rows a group on it takes five to eight models.  Rows of 16 counts and
+// fewer have at most half the products to do: 8 models x 12 in 10 groups 408 | 547.
 //
 // More than eight models take the tensor cores unless the groups are short: each group fills M
 // empty lists there, some 15 merges a model, where the integer tile's lists are its warps' own,
@@ -563,7 +565,7 @@ static void launch_topk_rows(const int64_t *F, int64_t R, int k, const double *W
 TopkPath topk_path(int k, int M, int64_t total, int64_t G) {
   if (M <= 4) return TopkPath::ROWS;
   if (M <= 8)
-    return k <= 16 || !exact_tc_ok(k, M) || total < (M == 5 ? int64_t(1) << 17 : 2048) * G ? TopkPath::ROWS : TopkPath::TENSOR;
+    return k <= 16 || !exact_tc_ok(k, M) || total < (int64_t(1) << 17) * G ? TopkPath::ROWS : TopkPath::TENSOR;
   return exact_tc_ok(k, M) && (double)total * (k + 0.25 * M) >= (double)G * (600 + 50.0 * M) ? TopkPath::TENSOR
                                                                                           : TopkPath::INTEGER;
 }

@@ -23,8 +23,8 @@ def env():
 
 @pytest.mark.parametrize("longest,groups", [(400, 700), (60, 900)], ids=["long", "short"])
 @pytest.mark.parametrize("listed", [False, True], ids=["rows", "list"])
-@pytest.mark.parametrize("k,M,topk", [(12, 9, 16), (31, 64, 5), (32, 33, 16), (32, 64, 16), (12, 64, 1), (8, 9, 3),
-                                      (32, 2, 16)])
+@pytest.mark.parametrize("k,M,topk", [(12, 9, 16), (31, 64, 5), (32, 33, 16), (32, 64, 16), (12, 64, 1), (8, 9, 3), (32, 6, 4),
+                                      (32, 7, 16), (32, 2, 16)])
 def test_many_units_per_block(env, k, M, topk, listed, longest, groups):
     import torch
     ctx, dev = env
@@ -64,3 +64,25 @@ def test_many_units_per_block(env, k, M, topk, listed, longest, groups):
             order = np.lexsort((mem, T[mem, m]))[:real]
             assert np.array_equal(idx[g, m, :real], mem[order]), (g, m)
             assert np.array_equal(tt[g, m, :real], T[mem[order], m]), (g, m)
+
+
+@pytest.mark.parametrize("R", [130001, 131072, 140003])
+@pytest.mark.parametrize("M", [5, 6, 7, 8])
+def test_one_group_around_the_line_of_five_to_eight_models(env, M, R):
+    import torch
+    ctx, dev = env
+    rng = np.random.default_rng(R + M)
+    F = rng.integers(0, 1 << 30, size=(R, 32))
+    F[rng.integers(0, R, size=R // 2)] = F[rng.integers(0, R, size=R // 2)]
+    dF = torch.from_numpy(F).to(dev)
+    dW = torch.from_numpy(rng.random((M, 32)) * 1e-9).to(dev)
+    idx = torch.full((1, M, 16), -5, dtype=torch.int64, device=dev)
+    tt = torch.full((1, M, 16), np.nan, dtype=torch.float64, device=dev)
+    ctx.predict_topk(dF, dW, np.array([0, R], dtype=np.int64), 16, idx, tt)
+    T = torch.empty((R, M), dtype=torch.float64, device=dev)
+    ctx.predict(dF, dW, T)
+    ctx.sync_status()
+    idx, tt, T = idx.cpu().numpy(), tt.cpu().numpy(), T.cpu().numpy()
+    for m in range(M):
+        order = np.lexsort((np.arange(R), T[:, m]))[:16]
+        assert np.array_equal(idx[0, m], order) and np.array_equal(tt[0, m], T[order, m]), m
