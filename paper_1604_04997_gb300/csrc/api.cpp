@@ -458,7 +458,7 @@ extern "C" pm_status pm_fit_weights(pm_ctx *c, const int64_t *F, int64_t R, int3
   if (objective != PM_FIT_RELATIVE && objective != PM_FIT_ABSOLUTE) return pm_set_error(PM_ERR_INVALID_ARG, "objective");
   if (precision != PM_PREC_FP64 && precision != PM_PREC_BF16X3) return pm_set_error(PM_ERR_INVALID_ARG, "precision");
   void *scr = nullptr;
-  pm_status s = ctx_scratch(c, pmd::fit_scratch_bytes(R, M), &scr);
+  pm_status s = ctx_scratch(c, pmd::fit_scratch_bytes(R, k, M), &scr);
   if (s) return s;
   if (!c->fit_host) CU(cudaMallocHost(&c->fit_host, 64 * pmd::FIT_REPORT_BYTES));
   const pmd::FitHost h = pmd::fit_report(c->fit_host, M);

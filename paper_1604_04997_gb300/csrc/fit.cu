@@ -56,8 +56,8 @@ __global__ void k_colmax(const int64_t *__restrict__ F, int64_t R, int k, unsign
 __device__ __forceinline__ int col_exp(unsigned long long mx) { return mx ? 64 - __clzll((long long)mx) : 0; }
 
 // ---- U = F diag(2^-e) as float-float pairs: Uh = rn(F), Ul = rn(F - Uh), scaled exactly;
-// rows of 32 floats, zero beyond column k
-__global__ void k_scale(const int64_t *__restrict__ F, int64_t R, int k, const unsigned long long *cmax,
+// rows of ldu floats (k rounded up to 4), zero beyond column k
+__global__ void k_scale(const int64_t *__restrict__ F, int64_t R, int k, int ldu, const unsigned long long *cmax,
                         float *__restrict__ Uh, float *__restrict__ Ul) {
   const int c = threadIdx.x & 31;
   const int e = c < k ? col_exp(cmax[c]) : 0;
@@ -65,8 +65,10 @@ __global__ void k_scale(const int64_t *__restrict__ F, int64_t R, int k, const u
   for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < R; r += step) {
     const int64_t v = c < k ? F[r * k + c] : 0;
     const float h = __ll2float_rn(v);
-    Uh[r * 32 + c] = ldexpf(h, -e);
-    Ul[r * 32 + c] = ldexpf(__ll2float_rn(v - (int64_t)h), -e);
+    if (c < ldu) {
+      Uh[r * ldu + c] = ldexpf(h, -e);
+      Ul[r * ldu + c] = ldexpf(__ll2float_rn(v - (int64_t)h), -e);
+    }
   }
 }
 
@@ -97,7 +99,7 @@ __device__ __forceinline__ float2 ff_recip(double t) {
 // U and of the row factors in shared memory, 4 columns x 4 models per thread, the two halves
 // of the CTA on 16 rows each, so one 16-byte read feeds eight products.
 constexpr int AM_ROWS = 32;
-__global__ void __launch_bounds__(FIT_THREADS) k_rowfac(const float *__restrict__ U, const double *__restrict__ T, int ld,
+__global__ void __launch_bounds__(FIT_THREADS) k_rowfac(const float *__restrict__ U, int ldu, const double *__restrict__ T, int ld,
                                                         int64_t R, int k, int M, int objective, float *__restrict__ rfh,
                                                         float *__restrict__ rfl, float *__restrict__ bh,
                                                         float *__restrict__ bl, unsigned *__restrict__ amax,
@@ -145,7 +147,7 @@ __global__ void __launch_bounds__(FIT_THREADS) k_rowfac(const float *__restrict_
     __syncthreads();
     for (int i = tid; i < AM_ROWS * 8; i += FIT_THREADS) {
       const int r = i >> 3, c = (i & 7) * 4;
-      const float4 x = r < nr ? *(const float4 *)(U + (rb + r) * 32 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float4 x = r < nr && c < ldu ? *(const float4 *)(U + (rb + r) * ldu + c) : make_float4(0.f, 0.f, 0.f, 0.f);
       *(float4 *)&su[r][c] = make_float4(fabsf(x.x), fabsf(x.y), fabsf(x.z), fabsf(x.w));
     }
 #pragma unroll
@@ -231,7 +233,7 @@ __device__ __forceinline__ int acol_exp(unsigned bits) {
 // products, accumulated with TwoSum compensation.  Chunk results are added to the
 // FP64 totals with atomics.
 constexpr int GB_COLS = 36, GB_BLOCKS = 9, GB_TASKS = 45, GB_GROUPS = 5;
-__global__ void __launch_bounds__(FIT_THREADS) k_gram(const float *__restrict__ Uh, const float *__restrict__ Ul,
+__global__ void __launch_bounds__(FIT_THREADS) k_gram(const float *__restrict__ Uh, const float *__restrict__ Ul, int ldu,
                                                       const float *__restrict__ rfh, const float *__restrict__ rfl,
                                                       const float *__restrict__ bh, const float *__restrict__ bl,
                                                       int ld, int64_t R, int k, int M, int64_t rows_per_chunk,
@@ -256,17 +258,18 @@ __global__ void __launch_bounds__(FIT_THREADS) k_gram(const float *__restrict__ 
   for (int64_t rb = r0; rb < r1; rb += FIT_ROWS) {
     __syncthreads();
     const int nr = (int)min((int64_t)FIT_ROWS, r1 - rb);
+    const int64_t u0 = rb * ldu, m0 = rb * ld + m;
     for (int i = threadIdx.x; i < FIT_ROWS * GB_COLS; i += FIT_THREADS) {
       const int rr = i / GB_COLS, cc = i - rr * GB_COLS;
       float2 v = make_float2(0.f, 0.f);
       if (rr < nr) {
+        const int o = rr * ldu + cc, q = rr * ld;
         if (cc < k) {
-          const int64_t o = (rb + rr) * 32 + cc, q = (rb + rr) * ld + m;
-          v = ff_mul(Uh[o], Ul[o], rfh[q], rfl[q]);
+          v = ff_mul(Uh[u0 + o], Ul[u0 + o], rfh[m0 + q], rfl[m0 + q]);
           v.x = ldexpf(v.x, -f[cc]);
           v.y = ldexpf(v.y, -f[cc]);
         } else if (cc == k) {
-          v = make_float2(bh[(rb + rr) * ld + m], bl[(rb + rr) * ld + m]);
+          v = make_float2(bh[m0 + q], bl[m0 + q]);
         }
       }
       vh[rr][cc] = v.x;
@@ -443,7 +446,7 @@ __device__ __forceinline__ void cp_async16_zfill(void *dst, const void *src, boo
                "r"(in ? 16 : 0));
 }
 
-__global__ void __launch_bounds__(FIT_THREADS, 2) k_atq(const float *__restrict__ Uh, const float *__restrict__ Ul,
+__global__ void __launch_bounds__(FIT_THREADS, 2) k_atq(const float *__restrict__ Uh, const float *__restrict__ Ul, int ldu,
                                                         const float *__restrict__ Qh, const float *__restrict__ Ql, int ld,
                                                         int64_t R, int k, int M, int64_t rows_per_chunk,
                                                         const unsigned *__restrict__ amax, double *__restrict__ g) {
@@ -462,8 +465,8 @@ __global__ void __launch_bounds__(FIT_THREADS, 2) k_atq(const float *__restrict_
 #pragma unroll
       for (int i = 0; i < ATQ_ROWS * 16 / FIT_THREADS; i++) {
         const int x = tid + i * FIT_THREADS, row = x >> 4, h = (x >> 3) & 1, c = (x & 7) * 4;
-        const bool in = rb + row < r1;
-        cp_async16_zfill(&T.u[row][h][c], (h ? Ul : Uh) + (in ? (rb + row) * 32 + c : 0), in);
+        const bool in = rb + row < r1 && c < ldu;
+        cp_async16_zfill(&T.u[row][h][c], (h ? Ul : Uh) + (in ? (rb + row) * ldu + c : 0), in);
       }
 #pragma unroll
       for (int i = 0; i < ATQ_ROWS * 8 / FIT_THREADS; i++) {
@@ -553,14 +556,16 @@ __global__ void __launch_bounds__(32) k_refine_update(const double *__restrict__
 
 // ------------------------------------------------------------------------------------ host side
 
-static int fit_ld(int M) { return (M + 7) & ~7; }   // row length of the row factors and residuals
+// row lengths of the row factors and residuals, and of the scaled counts: whole 16-byte pieces
+static int fit_ld(int M) { return (M + 3) & ~3; }
+static int fit_ldu(int k) { return (k + 3) & ~3; }
 
-size_t fit_scratch_bytes(int64_t R, int M) {
+size_t fit_scratch_bytes(int64_t R, int k, int M) {
   size_t b = 0;
   b += 256;                                        // cmax
   b += (size_t)M * (FIT_MAXK + 1) * 4;             // amax, rmax
-  b += (size_t)R * FIT_MAXK * 8;                   // Uh, Ul
-  b += (size_t)R * fit_ld(M) * 8 * 3;              // row factors, beta, Q (hi and lo)
+  b += (size_t)R * fit_ldu(k) * 8;                 // Uh, Ul
+  b += (size_t)R * fit_ld(M) * 8 * 2;              // row factors; beta, then Q (hi and lo)
   b += (size_t)M * FIT_MAXK * FIT_MAXK * 8;        // G / L
   b += (size_t)M * FIT_MAXK * 8 * 3;               // rhs, x, g
   b += (size_t)M * FIT_REPORT_BYTES;               // info, ratio, upd, rr, bb
@@ -575,7 +580,7 @@ static char *carve(char *&p, size_t bytes) {
 
 cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int M, int objective, int gram,
                        int steps, void *scratch, double *W_out, void *h_report, int *status, cudaStream_t st) {
-  const int ld = fit_ld(M);
+  const int ld = fit_ld(M), ldu = fit_ldu(k);
   char *p = (char *)scratch;
   // cleared together: cmax, amax, rmax, G, rhs
   char *zero = p;
@@ -585,14 +590,13 @@ cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int 
   double *G = (double *)carve(p, (size_t)M * FIT_MAXK * FIT_MAXK * 8);
   double *rhs = (double *)carve(p, (size_t)M * FIT_MAXK * 8);
   const size_t zero_bytes = (size_t)(p - zero);
-  float *U = (float *)carve(p, (size_t)R * FIT_MAXK * 4);
-  float *Ul = (float *)carve(p, (size_t)R * FIT_MAXK * 4);
+  float *U = (float *)carve(p, (size_t)R * ldu * 4);
+  float *Ul = (float *)carve(p, (size_t)R * ldu * 4);
   float *rfh = (float *)carve(p, (size_t)R * ld * 4);
   float *rfl = (float *)carve(p, (size_t)R * ld * 4);
   float *bh = (float *)carve(p, (size_t)R * ld * 4);
   float *bl = (float *)carve(p, (size_t)R * ld * 4);
-  float *Qh = (float *)carve(p, (size_t)R * ld * 4);
-  float *Ql = (float *)carve(p, (size_t)R * ld * 4);
+  float *Qh = bh, *Ql = bl;   // the residuals: beta has been read when the first are written
   double *x = (double *)carve(p, (size_t)M * FIT_MAXK * 8);
   double *g = (double *)carve(p, (size_t)M * FIT_MAXK * 8);
   void *report = carve(p, (size_t)M * FIT_REPORT_BYTES);
@@ -605,9 +609,9 @@ cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int 
   const bool relative = objective == PM_FIT_RELATIVE;
   const bool beta = gram == 0 || !relative;   // else beta is 1 and the right-hand side takes the row factors
   k_colmax<<<sms * 4, 256, 0, st>>>(F, R, k, cmax);
-  k_scale<<<sms * 8, 256, 0, st>>>(F, R, k, cmax, U, Ul);
+  k_scale<<<sms * 8, 256, 0, st>>>(F, R, k, ldu, cmax, U, Ul);
   k_rowfac<<<(int)std::min<int64_t>(sms * 4, (R + AM_ROWS - 1) / AM_ROWS), FIT_THREADS, 0, st>>>(
-      U, T, ld, R, k, M, objective, rfh, rfl, beta ? bh : nullptr, beta ? bl : nullptr, amax, rmax, status);
+      U, ldu, T, ld, R, k, M, objective, rfh, rfl, beta ? bh : nullptr, beta ? bl : nullptr, amax, rmax, status);
   const int groups = (M + ATQ_MODELS - 1) / ATQ_MODELS;
   // one wave of two CTAs per SM: the sums are issue-bound, and a partial second wave idles
   const int achunks = (int)std::max<int64_t>(1, std::min<int64_t>(2 * sms / groups, (R + ATQ_ROWS - 1) / ATQ_ROWS));
@@ -616,14 +620,14 @@ cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int 
   if (gram != 0) {
     // the Gram on the tensor cores; the right-hand side A^T b = U^T (rowfactor b) with the
     // float-float product kernel
-    e = gram == 2 ? launch_gram_tc(U, Ul, rfh, rfl, ld, R, k, M, amax, G, sms, status, st)
-                  : launch_gram_pairs(U, rfh, rfl, ld, R, k, M, amax, rmax, G, sms, status, st);
+    e = gram == 2 ? launch_gram_tc(U, Ul, ldu, rfh, rfl, ld, R, k, M, amax, G, sms, status, st)
+                  : launch_gram_pairs(U, ldu, rfh, rfl, ld, R, k, M, amax, rmax, G, sms, status, st);
     if (e != cudaSuccess) return e;
-    k_atq<<<dim3(achunks, groups), FIT_THREADS, sizeof(AtqSmem), st>>>(U, Ul, relative ? rfh : bh, relative ? rfl : bl, ld, R, k, M, arpc,
+    k_atq<<<dim3(achunks, groups), FIT_THREADS, sizeof(AtqSmem), st>>>(U, Ul, ldu, relative ? rfh : bh, relative ? rfl : bl, ld, R, k, M, arpc,
                                                          amax, rhs);
   } else {
     const int chunks = (int)std::max<int64_t>(1, std::min<int64_t>(4 * sms / std::max(1, M) + 1, (R + 255) / 256));
-    k_gram<<<dim3(chunks, M), FIT_THREADS, 0, st>>>(U, Ul, rfh, rfl, bh, bl, ld, R, k, M, (R + chunks - 1) / chunks, amax, G, rhs);
+    k_gram<<<dim3(chunks, M), FIT_THREADS, 0, st>>>(U, Ul, ldu, rfh, rfl, bh, bl, ld, R, k, M, (R + chunks - 1) / chunks, amax, G, rhs);
   }
   k_chol_solve<<<M, 32, 0, st>>>(G, rhs, k, M, cmax, amax, x, rep.info, rep.ratio, rep.upd, W_out, g, rep.rr, rep.bb);
   FitResidual res;
@@ -638,7 +642,7 @@ cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int 
   res.relative = relative;
   for (int it = 0; it < steps; it++) {
     if ((e = launch_fit_residual(F, R, k, W_out, M, res, false, status, sms, st)) != cudaSuccess) return e;
-    k_atq<<<dim3(achunks, groups), FIT_THREADS, sizeof(AtqSmem), st>>>(U, Ul, Qh, Ql, ld, R, k, M, arpc, amax, g);
+    k_atq<<<dim3(achunks, groups), FIT_THREADS, sizeof(AtqSmem), st>>>(U, Ul, ldu, Qh, Ql, ld, R, k, M, arpc, amax, g);
     k_refine_update<<<M, 32, 0, st>>>(G, g, k, M, rep.info, cmax, amax, x, rep.upd, W_out, rep.rr, rep.bb);
   }
   // the final residual, for the report
@@ -648,3 +652,6 @@ cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int 
 }
 
 }  // namespace pmd
+
+// Test hook: bytes of context scratch that a fit takes.
+extern "C" size_t pmx_fit_scratch(int64_t R, int k, int M) { return pmd::fit_scratch_bytes(R, k, M); }

@@ -81,11 +81,11 @@ __device__ __forceinline__ void gp_pair(int p, int k, int &a, int &b) {
 
 }  // namespace
 
-// Uh: [R][32] (zero columns beyond k); rfh, rfl: row factors as float-float [R][ld];
+// Uh: [R][ldu] (zero columns beyond k); rfh, rfl: row factors as float-float [R][ld];
 // rmax: their column maxima (float bits).  HELD: the issuing warp leaves without reporting its
 // sums and the waits are short (pmx_gram_held).
 template <bool HELD>
-__global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__restrict__ Uh, const float *__restrict__ rfh,
+__global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__restrict__ Uh, int ldu, const float *__restrict__ rfh,
                                                               const float *__restrict__ rfl, int ld, int64_t R, int k,
                                                               int M, int64_t rows_per_cta, const unsigned *__restrict__ amax,
                                                               const unsigned *__restrict__ rmax,
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
     }
     auto fetch = [&](int64_t rs) {   // this thread's entry of the stage at row rs
       const int64_t r = rs + (tid >> 5);
-      return r < r1 ? Uh[r * 32 + lane] : 0.f;
+      return r < r1 && lane < ldu ? Uh[r * ldu + lane] : 0.f;
     };
     float nu = fetch(r0), nu2 = fetch(r0 + GP_K);
     bool dead = false;   // some warp's wait ran out: all working warps leave at the next stage's barrier
@@ -228,8 +228,8 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
         su[n & 1][lane][tid >> 5] = nu;
         nu = nu2;
         nu2 = fetch(rs + 2 * GP_K);
-        if (lane == 0 && rs + GP_AHEAD * GP_K + (tid >> 5) < R)   // one 128-byte row of U per warp
-          asm volatile("prefetch.global.L2 [%0];\n" ::"l"(Uh + (rs + GP_AHEAD * GP_K + (tid >> 5)) * 32));
+        if (lane == 0 && rs + GP_AHEAD * GP_K + (tid >> 5) < R)   // one row of U per warp
+          asm volatile("prefetch.global.L2 [%0];\n" ::"l"(Uh + (rs + GP_AHEAD * GP_K + (tid >> 5)) * ldu));
         if (n >= GP_RING) ok = xp_wait(xp_saddr(&freed[buf]), (n / GP_RING - 1) & 1, &s_abort, LIMIT) && ok;
         uint32_t any;   // the stage's U is complete once all have arrived
         asm volatile(
@@ -304,23 +304,23 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
 }
 
 template <bool HELD>
-static cudaError_t launch(const float *Uh, const float *rfh, const float *rfl, int ld, int64_t R, int k, int M,
+static cudaError_t launch(const float *Uh, int ldu, const float *rfh, const float *rfl, int ld, int64_t R, int k, int M,
                           int64_t rows, const unsigned *amax, const unsigned *rmax, double *G, int *status,
                           cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k_gram_pairs<HELD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GP_SMEM);
   if (e != cudaSuccess) return e;
-  k_gram_pairs<HELD><<<(unsigned)((R + rows - 1) / rows), GP_THREADS, GP_SMEM, st>>>(Uh, rfh, rfl, ld, R, k, M, rows, amax,
+  k_gram_pairs<HELD><<<(unsigned)((R + rows - 1) / rows), GP_THREADS, GP_SMEM, st>>>(Uh, ldu, rfh, rfl, ld, R, k, M, rows, amax,
                                                                                   rmax, G, status);
   return cudaGetLastError();
 }
 
-cudaError_t launch_gram_pairs(const float *Uh, const float *rfh, const float *rfl, int ld, int64_t R, int k, int M,
+cudaError_t launch_gram_pairs(const float *Uh, int ldu, const float *rfh, const float *rfl, int ld, int64_t R, int k, int M,
                               const unsigned *amax, const unsigned *rmax, double *G, int sms, int *status,
                               cudaStream_t st) {
   if (R <= 0 || M <= 0) return cudaSuccess;
   // one range of rows per SM, at least eight stages of them
   const int64_t rows = std::max<int64_t>(8 * GP_K, ((R + sms - 1) / sms + GP_K - 1) / GP_K * GP_K);
-  return launch<false>(Uh, rfh, rfl, ld, R, k, M, rows, amax, rmax, G, status, st);
+  return launch<false>(Uh, ldu, rfh, rfl, ld, R, k, M, rows, amax, rmax, G, status, st);
 }
 
 }  // namespace pmd
@@ -330,6 +330,6 @@ cudaError_t launch_gram_pairs(const float *Uh, const float *rfh, const float *rf
 extern "C" int pmx_gram_held(const float *U, const float *rfh, const float *rfl, int64_t R, int k, int M,
                              const unsigned *amax, const unsigned *rmax, double *G, int *status, void *stream) {
   if (R < 1 || R > 1024 || k < 1 || k > 32 || M < 1 || M > 32) return PM_ERR_INVALID_ARG;
-  return pmd::launch<true>(U, rfh, rfl, 32, R, k, M, 1024, amax, rmax, G, status, (cudaStream_t)stream) == cudaSuccess
+  return pmd::launch<true>(U, 32, rfh, rfl, 32, R, k, M, 1024, amax, rmax, G, status, (cudaStream_t)stream) == cudaSuccess
              ? PM_OK : PM_ERR_CUDA;
 }

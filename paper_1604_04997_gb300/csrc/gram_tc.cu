@@ -153,8 +153,8 @@ __device__ __forceinline__ void gt_digits(int64_t a, int (&d)[7]) {
 
 }  // namespace
 
-// Uh, Ul: [R][32]; rfh, rfl: [R][ld]
-__global__ void __launch_bounds__(GT_THREADS, 1) k_gram_tc(const float *__restrict__ Uh, const float *__restrict__ Ul,
+// Uh, Ul: [R][ldu]; rfh, rfl: [R][ld]
+__global__ void __launch_bounds__(GT_THREADS, 1) k_gram_tc(const float *__restrict__ Uh, const float *__restrict__ Ul, int ldu,
                                                            const float *__restrict__ rfh,
                                                            const float *__restrict__ rfl, int ld, int64_t R, int k, int M,
                                                            const unsigned *__restrict__ amax, double *__restrict__ G,
@@ -202,13 +202,16 @@ __global__ void __launch_bounds__(GT_THREADS, 1) k_gram_tc(const float *__restri
     float nh[8], nl[8];
     float2 nf[8];
     auto fetch = [&](int64_t rb) {
+      // a stage's rows start at an address that is the same for all threads; 32-bit offsets from it
+      const char *uh = (const char *)(Uh + rb * ldu), *ul = (const char *)(Ul + rb * ldu);
+      const char *fh = (const char *)(rfh + rb * ld + m), *fl = (const char *)(rfl + rb * ld + m);
 #pragma unroll
       for (int i = 0; i < 8; i++) {
-        const int64_t r = rb + 8 * warp + i;
-        const bool ok = r < r1 && c < k;
-        nh[i] = ok ? Uh[r * 32 + c] : 0.f;
-        nl[i] = ok ? Ul[r * 32 + c] : 0.f;
-        nf[i] = ok ? make_float2(rfh[r * ld + m], rfl[r * ld + m]) : make_float2(0.f, 0.f);
+        const uint32_t r = 8 * warp + i, u = (r * ldu + c) * 4, f = r * ld * 4;
+        const bool ok = rb + r < r1 && c < k;
+        nh[i] = ok ? *(const float *)(uh + u) : 0.f;
+        nl[i] = ok ? *(const float *)(ul + u) : 0.f;
+        nf[i] = ok ? make_float2(*(const float *)(fh + f), *(const float *)(fl + f)) : make_float2(0.f, 0.f);
       }
     };
     fetch(r0);
@@ -318,7 +321,7 @@ __global__ void __launch_bounds__(GT_THREADS, 1) k_gram_tc(const float *__restri
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512));
 }
 
-cudaError_t launch_gram_tc(const float *Uh, const float *Ul, const float *rfh, const float *rfl, int ld, int64_t R,
+cudaError_t launch_gram_tc(const float *Uh, const float *Ul, int ldu, const float *rfh, const float *rfl, int ld, int64_t R,
                            int k, int M, const unsigned *amax, double *G, int sms, int *status, cudaStream_t st) {
   if (R <= 0 || M <= 0) return cudaSuccess;
   const int64_t items = ((R + GT_CHUNK - 1) / GT_CHUNK) * M;
@@ -326,7 +329,7 @@ cudaError_t launch_gram_tc(const float *Uh, const float *Ul, const float *rfh, c
   const size_t sm = 2 * GT_STAGE + GT_CONTRIB + 128;
   cudaError_t e = cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k_gram_tc<<<grid, GT_THREADS, sm, st>>>(Uh, Ul, rfh, rfl, ld, R, k, M, amax, G, status);
+  k_gram_tc<<<grid, GT_THREADS, sm, st>>>(Uh, Ul, ldu, rfh, rfl, ld, R, k, M, amax, G, status);
   return cudaGetLastError();
 }
 

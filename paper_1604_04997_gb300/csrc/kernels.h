@@ -105,7 +105,7 @@ struct FitResidual {
   const float *rfh = nullptr, *rfl = nullptr;   // 1 / t (relative)
   float *Qh = nullptr, *Ql = nullptr;
   double *rr = nullptr, *bb = nullptr;          // [M]
-  int ld = 0;                                   // row length of rf and Q: M rounded up to 8
+  int ld = 0;                                   // row length of rf and Q: M rounded up to 4
   int relative = 0;
 };
 cudaError_t launch_fit_residual(const int64_t *F, int64_t R, int k, const double *W, int M, const FitResidual &res,
@@ -172,15 +172,15 @@ inline FitHost fit_report(void *p, int M) {
   double *d = (double *)((char *)p + (size_t)M * 16);
   return FitHost{(int *)p, d, d + M, d + 2 * M, d + 3 * M};
 }
-size_t fit_scratch_bytes(int64_t R, int M);
+size_t fit_scratch_bytes(int64_t R, int k, int M);
 // gram: 0 float-float (k_gram), 1 three bf16 terms (k_gram_pairs), 2 exact digits (k_gram_tc)
 cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int M, int objective, int gram,
                        int steps, void *scratch, double *W_out, void *h_report, int *status, cudaStream_t st);
 // Gram matrices of the fit on the tensor cores (add into G, upper triangle, [M][32][32])
-cudaError_t launch_gram_pairs(const float *Uh, const float *rfh, const float *rfl, int ld, int64_t R, int k, int M,
+cudaError_t launch_gram_pairs(const float *Uh, int ldu, const float *rfh, const float *rfl, int ld, int64_t R, int k, int M,
                               const unsigned *amax, const unsigned *rmax, double *G, int sms, int *status,
                               cudaStream_t st);
-cudaError_t launch_gram_tc(const float *Uh, const float *Ul, const float *rfh, const float *rfl, int ld, int64_t R,
+cudaError_t launch_gram_tc(const float *Uh, const float *Ul, int ldu, const float *rfh, const float *rfl, int ld, int64_t R,
                            int k, int M, const unsigned *amax, double *G, int sms, int *status, cudaStream_t st);
 
 }  // namespace pmd
