@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(32) k_chol_solve(double *__restrict__ G, const
   for (int i = a; i < FIT_MAXK * FIT_MAXK; i += 32) Gm[i] = L[i / FIT_MAXK][i % FIT_MAXK];   // L, for the refinement solves
 }
 
-// ---- g_m = U^T q_m  (float-float products and sums per chunk, FP64 totals): bound by the
+// ---- g_m = U^T q_m  (float-float products and sums per warp, FP64 totals): bound by the
 // twelve FP32 operations of each error-free product and compensated sum.  Grid (row chunks,
 // groups of 16 models); a thread owns two columns and eight models (lanes 0-15 and 16-31 of a
 // warp share the columns), so a row's 4 + 16 floats feed 16 products, and the eight warps
@@ -515,16 +515,16 @@ __global__ void __launch_bounds__(FIT_THREADS, 2) k_atq(const float *__restrict_
     }
   }
   __syncthreads();
-  // the eight warps' sums of 32 columns x 16 models
+  // the eight warps' sums of 32 columns x 16 models, added up no worse than in FP64
   for (int o = tid; o < 32 * 16; o += FIT_THREADS) {
     const int l = o >> 4, j = o & 15;
     const int col = 2 * (l & 15) + (j & 1), m = mb + 8 * (l >> 4) + (j >> 1);
     if (m < M && col < k) {
-      float ts = 0.f, tc = 0.f;
+      float ts = 0.f, tc = 0.f, td = 0.f;
 #pragma unroll
-      for (int w = 0; w < FIT_THREADS / 32; w++) ff_acc(ts, tc, red[w][l][j]);
+      for (int w = 0; w < FIT_THREADS / 32; w++) ff_acc3(ts, tc, td, red[w][l][j]);
       atomicAdd(&g[(int64_t)m * FIT_MAXK + col],
-                ldexp((double)ts + (double)tc, -acol_exp(amax[m * FIT_MAXK + col])));
+                ldexp(((double)ts + (double)tc) + (double)td, -acol_exp(amax[m * FIT_MAXK + col])));
     }
   }
 }
@@ -655,3 +655,14 @@ cudaError_t launch_fit(const int64_t *F, int64_t R, int k, const double *T, int 
 
 // Test hook: bytes of context scratch that a fit takes.
 extern "C" size_t pmx_fit_scratch(int64_t R, int k, int M) { return pmd::fit_scratch_bytes(R, k, M); }
+
+// Test hook: g [M][32] += U^T q of one row chunk (columns unscaled).  Uh, Ul [R][32]; Qh, Ql
+// [R][16]; M <= 16; amax [M][32]: 1.0f each.
+extern "C" int pmx_atq(const float *Uh, const float *Ul, const float *Qh, const float *Ql, int64_t R, int k, int M,
+                       const unsigned *amax, double *g, void *stream) {
+  if (R < 1 || k < 1 || k > 32 || M < 1 || M > 16) return PM_ERR_INVALID_ARG;
+  if (cudaFuncSetAttribute(pmd::k_atq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(pmd::AtqSmem)) != cudaSuccess)
+    return PM_ERR_CUDA;
+  pmd::k_atq<<<dim3(1, 1), pmd::FIT_THREADS, sizeof(pmd::AtqSmem), (cudaStream_t)stream>>>(Uh, Ul, 32, Qh, Ql, 16, R, k, M, R, amax, g);
+  return cudaGetLastError() == cudaSuccess ? PM_OK : PM_ERR_CUDA;
+}

@@ -39,4 +39,20 @@ __device__ __forceinline__ void ff_acc(float &s, float &c, float2 p) {
   s = t;
 }
 
+// The same with the sum's own rounding errors kept: s + c + d holds the exact sum to some 2^-66
+// of the largest part, so one FP64 sum of the three is no worse than adding in FP64.
+__device__ __forceinline__ void two_sum(float &s, float x, float &err) {   // s + x = (new s) + err
+  const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
+  err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z));
+  s = t;
+}
+__device__ __forceinline__ void ff_acc3(float &s, float &c, float &d, float2 p) {
+  float e0, e1, e2, e3;
+  two_sum(p.x, p.y, e0);   // the leading bits in the first part, also where sums cancelled
+  two_sum(s, p.x, e1);
+  two_sum(c, e1, e2);
+  two_sum(c, e0, e3);
+  d = __fadd_rn(d, __fadd_rn(e2, e3));
+}
+
 }  // namespace pmd
