@@ -463,18 +463,20 @@ extern "C" pm_status pm_fit_weights(pm_ctx *c, const int64_t *F, int64_t R, int3
   if (!c->fit_host) CU(cudaMallocHost(&c->fit_host, 64 * pmd::FIT_REPORT_BYTES));
   const pmd::FitHost h = pmd::fit_report(c->fit_host, M);
   cudaStream_t st = (cudaStream_t)stream;
-  // PM_PREC_BF16X3: the Gram from three bf16 terms first; refinement with exact residuals
-  // makes it accurate when cond(G) 2^-24 is well below one.  If some model's last
-  // correction is still large (or its factor reports a rank drop the exact Gram may not
-  // have), the fit is repeated with the exact digit Gram.
+  // PM_PREC_BF16X3: the Gram from three bf16 terms first, within 2^-21 (1,000 rows) to 2^-18
+  // (200,000) of its diagonal; refinement with exact residuals makes the weights accurate when
+  // cond(G) 2^-18 is well below one.  If some model's last correction is still large, or
+  // without refinement its smallest pivot is known to less than a hundredth, or its factor reports a rank
+  // drop that the exact Gram may not have, the fit is repeated with the exact digit Gram.
   int gram = precision == PM_PREC_BF16X3 ? 1 : 0;
   for (;;) {
     CU(pmd::launch_fit(F, R, k, T, M, objective, gram, refine_steps, scr, W_out, c->fit_host, c->d_status, st));
     s = pm_sync_status(c, stream);
     if (s) return s;
-    if (gram != 1 || refine_steps == 0) break;
+    if (gram != 1) break;
     bool converged = true;
-    for (int m = 0; m < M; m++) converged &= h.upd[m] < 1e-10 && h.info[m * 4 + 2] == 0;
+    for (int m = 0; m < M; m++)
+      converged &= h.info[m * 4 + 2] == 0 && (refine_steps ? h.upd[m] < 1e-10 : h.ratio[m] < 0x1p12);
     if (converged) break;
     gram = 2;
   }

@@ -8,9 +8,12 @@
 //
 // Products and squares are rounded to FP32 and split into three bf16 terms each (24
 // significant bits); the six term products down to 2^-24 accumulate in FP32 in tensor memory
-// over at most GP_SUB rows (252 accumulation steps), then in FP64 into G.  The fit's
-// refinement with exact residuals recovers full accuracy as long as cond(G) 2^-20 or so is
-// well below 1; else it falls back to the exact Gram (gram_tc.cu).
+// over at most GP_SUB rows (252 accumulation steps), then in FP64 into G.  The FP32 accumulation
+// is what limits G: weights without refinement are off by 8e-7 (1,000 to 20,000 rows, cond(A)
+// 20), 2.2e-6 (60,000) and 3.6e-6 (200,000 rows), where entries split into three terms per
+// model and chunks of 4,096 rows gave 2e-6 (1,000) to 2e-5 (60,000); the rounding of the
+// products alone is 2e-8.  Refinement with exact residuals recovers full accuracy as long as
+// cond(G) 2^-18 is well below 1; else the fit falls back to the exact Gram (gram_tc.cu).
 //
 // One CTA per SM takes one contiguous range of rows, in stages of 16 rows (one K-step): 16
 // warps write the stage's pairs (rows 0 .. 639 in five 128-row tiles), four its models (the N
