@@ -943,13 +943,14 @@ static void default_shape(pm_ctx *c, Plan *p, int nw) {
 static constexpr int DEFAULT_SLICE = 1 << 30;   // one group per template unless a limit splits it
 // Warps per CTA.  While all units are resident at once with eight warps each (two CTAs per SM),
 // eight shorten the chain that one unit is (us with eight | four: 64 distinct matmul tables, 512
-// points 25 | 31; 10,000 variants, 1,001 points of 8 templates 22.6 | 24.7).  With more units it
-// is by the programs of the largest group: with few a unit is mostly its fixed steps (staging,
-// basis, ranking), so four warps and twice the CTAs per SM are faster (137 programs over 8
-// groups, 1,024 units: 41 | 47); with more than 16 per warp of eight the walk over the programs
-// dominates and all eight share one basis.
+// points 25 | 31; 10,000 variants, 1,001 points of 8 templates 22.6 | 24.7); with at most four
+// programs per warp of four they take as long (coupled templates, up to ten programs: 17.1 to
+// 19.4 | 18.5).  With more units it is by the programs of the largest group: with few a unit is
+// mostly its fixed steps (staging, basis, ranking), so four warps and twice the CTAs per SM are
+// faster (137 programs over 8 groups, 1,024 units: 41 | 47); with more than 16 per warp of eight
+// the walk over the programs dominates and all eight share one basis.
 static int default_nw(const pm_ctx *c, const Plan *p) {
-  if (p->n_units <= c->n_sms * pmd::rank_max_blocks_per_sm(8, p->img_words, p->basis_cap)) return 8;
+  if (p->max_progs > 16 && p->n_units <= c->n_sms * pmd::rank_max_blocks_per_sm(8, p->img_words, p->basis_cap)) return 8;
   return p->max_progs <= 128 ? 4 : 8;
 }
 
