@@ -322,22 +322,25 @@ __device__ __forceinline__ bool xp_wait(uint32_t mbar, uint32_t parity, volatile
   return __all_sync(0xffffffffu, xp_wait_one(mbar, parity, s_abort, limit_ns));
 }
 
-// What a kernel does before it frees its TMEM: after a wait of any warp ran out, the status
-// bit, and the MMAs in flight finish (bounded).  Every thread of the CTA calls it, past all of
-// its waits; the issuing warp (issuer) gives the number n of commits that it made in turn to
-// the `ring` barriers mbar[0 .. ring).  The issuing warp cannot report alone: it runs ahead of
-// the others, and has left when they wait for the last sums.
+// The n-th commit that a warp made in turn to the `ring` barriers mbar[0 .. ring), and all
+// before it, complete (bounded): the MMAs in flight, before their TMEM is freed.
+__device__ __forceinline__ void xp_drain(const uint64_t *mbar, uint32_t ring, uint32_t n) {
+  const unsigned long long t0 = globaltimer_ns();
+  for (uint32_t i = n >= ring ? n - ring : 0; i < n; i++)
+    while (!xp_try(xp_saddr(&mbar[i % ring]), (i / ring) & 1) && globaltimer_ns() - t0 < MBAR_WAIT_NS) {}
+}
+
+// What a kernel does before it frees its TMEM, after a wait of any warp ran out: the status bit,
+// and the issuing warp's (issuer) n commits complete.  Every thread of the CTA calls it, past
+// all of its waits.  The issuing warp cannot report alone: it runs ahead of the others, and has
+// left when they wait for the last sums.
 __device__ __forceinline__ void xp_finish(volatile int *s_abort, int *status, bool issuer, const uint64_t *mbar,
                                           uint32_t ring, uint32_t n) {
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
   __syncthreads();
   if (!*s_abort) return;   // the same for all threads
   if (threadIdx.x == 0 && status) atomicOr(status, ST_TIMEOUT);
-  if (issuer) {
-    const unsigned long long t0 = globaltimer_ns();
-    for (uint32_t i = n >= ring ? n - ring : 0; i < n; i++)
-      while (!xp_try(xp_saddr(&mbar[i % ring]), (i / ring) & 1) && globaltimer_ns() - t0 < MBAR_WAIT_NS) {}
-  }
+  if (issuer) xp_drain(mbar, ring, n);
   __syncthreads();
 }
 

@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(GP_THREADS, 1) k_gram_pairs(const float *__res
       }
       if (ok && !HELD) xp_commit(xp_saddr(&summed));
     }
+    if (!ok) xp_drain(freed, GP_RING, n);
     __syncwarp();
   } else if (warp >= GP_WARPS) {
     // one row (8 rows of U of one model) of the N operand per thread: 64 models x 2 K-groups

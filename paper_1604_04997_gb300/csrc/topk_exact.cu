@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(XP_THREADS, 1) k_topk_exact(const int64_t *__r
                     xp_saddr(&full[b]));
       }
     }
+    if (!ok) xp_drain(full, XP_RING, seq);
     __syncwarp();
   } else {
     const bool active = slice * 8 < G::NB;   // this warp has models
