@@ -397,9 +397,10 @@ def run_ours(args):
     peak_ops = sms * 128 * max_mhz * 1e6           # lane-instruction issue rate at the maximum clock
     achieved = evals * info["work_per_eval"] / (ms / 1e3)
     measured_ops = B.pmm_int_issue_rate()          # integer multiply-add / xor / add chains, every lane
-    traffic = _profile_traffic("rank_coupled_10000x4096.md" if coupled else
-                               "rank_batched_10000x4096.md",
-                               ("rank.cu", "eval_common.cuh", "kernels.h", "plan.cpp"))
+    rank_profile = ("rank_coupled_10000x4096.md" if coupled else "rank_batched_10000x4096.md",
+                    ("rank.cu", "eval_common.cuh", "kernels.h", "plan.cpp"))
+    traffic = _profile_value("traffic_bytes_per_launch", *rank_profile)
+    issue = _profile_value("issue_active_pct", *rank_profile)
 
     if rank == 0:
         line = {
@@ -422,13 +423,14 @@ def run_ours(args):
                     "d2h_bytes_per_step": int(n * 16 * (4 + 8))},
             "gpu_launches": 2 * args.steps,   # per step: the weight prepass and the fused ranking kernel
             "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12,
-                         "unit": "T lane-ops/s", "frac": achieved / peak_ops, "traffic": traffic,
-                         "kernel": "k_rank",
+                         "unit": "T lane-ops/s", "frac": None, "traffic": traffic,
+                         "issue_active_pct": issue, "kernel": "k_rank",
                          "ops_per_eval": info["work_per_eval"],
                          "ops_note": "integer operations of each variant's own exact sum; variants whose tables are "
-                                     "equal share one evaluation, so fewer are executed",
+                                     "equal share one evaluation, so fewer are executed and their rate is no "
+                                     "fraction of the peak: issue_active_pct is the profile's (ncu) instead",
                          "peak_note": f"{sms} SMs x 128 lanes x {max_mhz:.0f} MHz (issue bound, derived)",
-                         "measured_peak": measured_ops / 1e12, "frac_of_measured": achieved / measured_ops,
+                         "measured_peak": measured_ops / 1e12,
                          "measured_peak_note": "integer issue-rate probe (pmm_int_issue_rate): independent "
                                                "32-bit multiply-add, xor and add chains in every lane"},
             "clocks": ck,
@@ -493,18 +495,19 @@ def _tuning_summary(ctx, bp):
         return None
 
 
-def _profile_traffic(md: str, sources) -> "int | None":
-    """DRAM bytes per launch recorded in a committed ncu summary under profiles/, or
-    None when the kernel's sources changed since the capture (fingerprint mismatch)."""
+def _profile_value(name: str, md: str, sources) -> "int | float | None":
+    """A figure of one launch recorded in a committed ncu summary under profiles/ (DRAM
+    bytes, issue slots used), or None when the kernel's sources changed since the
+    capture (fingerprint mismatch)."""
     import hashlib
     import re
     try:
         text = open(os.path.join(ROOT, "profiles", md)).read()
-        t = int(re.search(r"^traffic_bytes_per_launch: (\d+)", text, re.M).group(1))
+        t = re.search(rf"^{name}: ([0-9.]+)", text, re.M).group(1)
         want = re.search(r"^source_sha256_16: ([0-9a-f]{16})", text, re.M).group(1)
         csrc = os.path.join(ROOT, "paper_1604_04997_gb300", "csrc")
         h = hashlib.sha256(b"".join(open(os.path.join(csrc, f), "rb").read() for f in sources)).hexdigest()[:16]
-        return t if h == want else None
+        return None if h != want else float(t) if "." in t else int(t)
     except Exception:
         return None
 
@@ -598,7 +601,8 @@ def run_other(args):
                                                            times["fp64_topk16_4096_groups"][0]}},
                     roofline={"bound": "hbm", "achieved": nbytes / (ms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
                               "frac": nbytes / (ms / 1e3) / 1e9 / hbm,
-                              "traffic": _profile_traffic("predict_tc_1e6x32x64.md", ("predict_tc.cu", "mbar_wait.cuh")),
+                              "traffic": _profile_value("traffic_bytes_per_launch", "predict_tc_1e6x32x64.md",
+                                                         ("predict_tc.cu", "mbar_wait.cuh")),
                               "kernel": "k_predict_tc",
                               "algorithmic_bytes": "256 B read + 8 B written per (row, model)"},
                     clocks=ck, gpu_launches=args.steps)
