@@ -604,12 +604,25 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_topk_merge(const TopkMerge *_
   double lt = TK_INF;
   int64_t lr = INT64_MAX;
   __shared__ long long s_thr;   // no time above it is among the topk: the least of the warps' last entries
-  if (threadIdx.x == 0) s_thr = INT64_MAX;
-  __syncthreads();
+  const bool few = (int64_t)G.n_parts * topk <= 32 * PR_WARPS;   // one candidate a thread: no rounds
+  if (few) {
+    const int p = (int)threadIdx.x / topk, q = (int)threadIdx.x - p * topk;
+    double t = TK_INF;
+    int64_t r = INT64_MAX;
+    if (p < G.n_parts) {
+      const int64_t o = (((int64_t)G.part0 + p) * M + m) * topk + q;
+      t = part_t[o];
+      r = part_r[o];
+    }
+    warp_list_merge(lt, lr, t, r, r != INT64_MAX, topk, lane);
+  } else {
+    if (threadIdx.x == 0) s_thr = INT64_MAX;
+    __syncthreads();
+  }
   int sh = 0;   // 2^sh entries of a list per round
-  while (sh < 4 && ((int64_t)G.n_parts << (sh + 1)) <= 4 * 32 * PR_WARPS) sh++;
+  while ((1 << sh) < topk && ((int64_t)G.n_parts << (sh + 1)) <= 4 * 32 * PR_WARPS) sh++;
   const int64_t n = (int64_t)G.n_parts << sh;
-  for (int j = 0; j < topk; j += 1 << sh) {
+  for (int j = 0; j < topk && !few; j += 1 << sh) {
     bool some = false;
     for (int64_t c0 = 32 * warp; c0 < n; c0 += 4 * 32 * PR_WARPS) {   // warp-uniform
       double t[4];
