@@ -376,7 +376,7 @@ extern "C" pm_status pm_predict_topk(pm_ctx *c, const int64_t *F, int64_t R, int
   std::vector<pmd::TopkUnit> units;
   std::vector<pmd::TopkMerge> merges;
   int64_t parts = 0;
-  const int64_t total = h_seg_off[G] - h_seg_off[0], most = pmd::topk_chunk(k, M, total, G);
+  const int64_t total = h_seg_off[G] - h_seg_off[0], most = pmd::topk_chunk(k, M, topk, total, G);
   for (int32_t i = 0; i < G; i++) {
     const int64_t p0 = h_seg_off[i], p1 = h_seg_off[i + 1];
     const int64_t nch = std::max<int64_t>(1, (p1 - p0 + most - 1) / most);
@@ -408,7 +408,7 @@ extern "C" pm_status pm_predict_topk(pm_ctx *c, const int64_t *F, int64_t R, int
   CU(pmd::launch_predict_topk(F, R, k, W, M, d_rows, (const pmd::TopkUnit *)d_meta, (int)units.size(),
                               (const pmd::TopkMerge *)((uint8_t *)d_meta + ub), (int)merges.size(), topk,
                               (double *)scr, (int64_t *)((uint8_t *)scr + pb), d_top_idx, d_top_t,
-                              pmd::topk_path(k, M, total, G), c->d_status, (cudaStream_t)stream));
+                              pmd::topk_path(k, M, topk, total, G), c->d_status, (cudaStream_t)stream));
   return PM_OK;
 }
 

@@ -119,8 +119,8 @@ constexpr int64_t TOPK_CHUNK = 1024;
 // the kernel that M models over `total` positions in G groups take (row per lane, tensor
 // cores, integer tile), and its largest unit
 enum class TopkPath { ROWS, TENSOR, INTEGER };
-TopkPath topk_path(int k, int M, int64_t total, int64_t G);
-int64_t topk_chunk(int k, int M, int64_t total, int64_t G);
+TopkPath topk_path(int k, int M, int topk, int64_t total, int64_t G);
+int64_t topk_chunk(int k, int M, int topk, int64_t total, int64_t G);
 struct TopkUnit { int64_t p0, p1; int32_t g, part; };
 struct TopkMerge { int32_t g, part0, n_parts, pad; };
 // topk_exact.cu: more than a few models, k <= 32, on the tensor cores

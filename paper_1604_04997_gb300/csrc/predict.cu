@@ -555,31 +555,38 @@ static void launch_topk_rows(const int64_t *F, int64_t R, int k, const double *W
 // of its tiles: from 2^17 rows a group on it takes five to eight models.  Rows of 16 counts and
 // fewer have at most half the products to do: 8 models x 12 in 10 groups 408 | 547.
 //
-// More than eight models take the tensor cores unless the groups are short: each group fills M
-// empty lists there, some 15 merges a model, where the integer tile's lists are its warps' own,
-// but the integer tile pays for every product.  So the line is in a group's rows times what a
-// row costs, k + M / 4, against the lists, 600 + 50 M.  100,000 rows, us, integer | tensor
+// More than eight models take the tensor cores unless there are many short groups: each group
+// fills M empty lists there, some 15 merges a model, where the integer tile's lists are its warps'
+// own, but the integer tile pays for every product.  So the line is in a group's rows times what
+// a row costs, k + M / 4, against the lists, 600 + 50 M.  100,000 rows, us, integer | tensor
 // cores: 9 models x 12 columns 270 | 343 (64 rows a group), 268 | 245 (100); 64 models x 12
 // 558 | 642 (100), 566 | 423 (256); 64 x 32 800 | 879 (64), 782 | 632 (100); 33 x 32 629 | 886
-// (32), 650 | 577 (64).
-TopkPath topk_path(int k, int M, int64_t total, int64_t G) {
+// (32), 650 | 577 (64).  One CTA per SM takes a group, so what counts is how many each SM takes in
+// turn: one alone is faster on the tensor cores whatever its length (10 groups of 100 rows, 64 x
+// 12: 140 | 110), and so are two (64 x 12, 50 rows: 201 | 198); with three the line lies at two
+// thirds (37 x 12: 267 | 259 at 100 rows, 158 | 212 at 50), from four on where it is above.  Short
+// rankings fill their lists sooner (64 x 32, 64 rows: the fastest row 435 | 376), and wide rows
+// cost the integer tile more than their width (9 x 32, 30 rows: 207 | 173).
+TopkPath topk_path(int k, int M, int topk, int64_t total, int64_t G) {
   if (M <= 4) return TopkPath::ROWS;
   if (M <= 8)
     return k <= 16 || !exact_tc_ok(k, M) || total < (int64_t(1) << 17) * G ? TopkPath::ROWS : TopkPath::TENSOR;
-  return exact_tc_ok(k, M) && (double)total * (k + 0.25 * M) >= (double)G * (600 + 50.0 * M) ? TopkPath::TENSOR
-                                                                                          : TopkPath::INTEGER;
+  if (!exact_tc_ok(k, M)) return TopkPath::INTEGER;
+  const double turns = std::min(1.0, std::max(0.0, ((double)G / num_sms() - 1) / 3));
+  const double row = (k + 0.25 * M) * std::max(1.0, k / 24.0), lists = (600 + 50.0 * M) * (0.75 + 0.25 * (topk - 1) / (TOPK_MAX - 1));
+  return (double)total * row >= turns * G * lists ? TopkPath::TENSOR : TopkPath::INTEGER;
 }
 // The row-per-lane kernel's units fill its resident CTAs once (six per SM, four with eight
 // models' lists): of 977 units of 1,024 positions on 912 CTAs the last 65 took as
 // long as the rest (1e6 rows, 4 models).  At most 2,048 positions, so that larger problems
 // balance over many units while the variants of one template and point stay one unit.  The
 // tensor-core kernel keeps one list per CTA and unit: one unit per SM.
-int64_t topk_chunk(int k, int M, int64_t total, int64_t G) {
+int64_t topk_chunk(int k, int M, int topk, int64_t total, int64_t G) {
   auto split = [&](int64_t ctas, int64_t grain, int64_t lo, int64_t hi) {
     const int64_t each = ((total + ctas - 1) / ctas + grain - 1) / grain * grain;
     return std::min(hi, std::max(lo, each));
   };
-  const TopkPath path = topk_path(k, M, total, G);
+  const TopkPath path = topk_path(k, M, topk, total, G);
   if (path == TopkPath::ROWS) return split((int64_t)num_sms() * (M <= 2 ? 6 : M <= 4 ? 5 : 4), 32, 32 * TR_WARPS, 2048);
   if (path == TopkPath::INTEGER) return TOPK_CHUNK;
   return split(num_sms(), 128, TOPK_CHUNK, int64_t(1) << 20);
